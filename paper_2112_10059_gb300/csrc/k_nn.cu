@@ -22,6 +22,7 @@
 #include <algorithm>
 
 #include "nn_kernels.cuh"
+#include "nn_pack.cuh"
 #include "tc_sm103.cuh"
 
 namespace sph {
@@ -29,150 +30,13 @@ namespace nn {
 
 using namespace tc;
 
-constexpr int STAGES = 4, LAG = 2;
 constexpr uint32_t A_STAGE = 128 * 128;     // 128 rows x 64 BF16
 constexpr uint32_t NN_WAIT = 1u << 22;
 
-__host__ __device__ constexpr uint32_t conv_smem(int N) { return 1024 + STAGES * (A_STAGE + N * 128) + 64; }
 __host__ __device__ constexpr uint32_t wgrad_smem(int N) { return 1024 + 2 * (A_STAGE + N * 128) + 64; }
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
     return reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
-}
-
-__device__ __forceinline__ void unpack8(const uint4 &q, float *f) {
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        f[2 * i] = __uint_as_float(w[i] << 16);
-        f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-    }
-}
-__device__ __forceinline__ uint4 pack8(const float *f) {
-    uint32_t w[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = (uint32_t)f2bf(f[2 * i]) | ((uint32_t)f2bf(f[2 * i + 1]) << 16);
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-// ---------------------------------------------------------------- convolution (forward / data gradient)
-template <int C, int N>
-__global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
-    constexpr int T = 64 / C;                 // taps per K chunk
-    constexpr int NCH = conv_chunks(C);
-    constexpr int GPR = C / 8;                // 16-byte groups per tap
-    constexpr uint32_t STAGE = A_STAGE + N * 128;
-    extern __shared__ uint8_t raw[];
-    uint8_t *base = align1024(raw);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(base + STAGES * STAGE);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + STAGES);
-    int *eflag = reinterpret_cast<int *>(tslot + 1);
-
-    const int r = threadIdx.x;
-    const int m = blockIdx.x * 128 + r;
-    const bool valid = m < a.nvox;
-    const int lg = a.lg, D = 1 << lg, dm = D - 1;
-    const int x0 = m & dm, y0 = (m >> lg) & dm, z0 = (m >> (2 * lg)) & dm;
-
-    if (r < 32) {
-        tmem_alloc(smem_u32(tslot), 32);
-        tmem_relinquish();
-    }
-    if (r == 0) {
-        for (int s = 0; s < STAGES; ++s) mbar_init(smem_u32(&bar[s]), 1);
-        *eflag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    const uint32_t tmem = *tslot;
-    const uint32_t sbase = smem_u32(base);
-    const uint32_t idesc = idesc_bf16_f32(128, N);
-
-    for (int kc = 0; kc < NCH + LAG; ++kc) {
-        if (kc < NCH) {
-            const int s = kc % STAGES;
-            if (kc >= STAGES && !mbar_wait_bounded(smem_u32(&bar[s]), ((kc / STAGES) - 1) & 1, NN_WAIT)) *eflag = 1;
-            const uint32_t sa = sbase + s * STAGE, sb = sa + A_STAGE;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int tap = kc * T + u / GPR, cg = u % GPR;
-                const void *src = a.x;
-                uint32_t bytes = 0;
-                if (valid && tap < NTAPS) {
-                    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                    if ((unsigned)(x0 + dx) < (unsigned)D && (unsigned)(y0 + dy) < (unsigned)D &&
-                        (unsigned)(z0 + dz) < (unsigned)D) {
-                        src = a.x + (size_t)(m + (dz * D + dy) * D + dx) * C + cg * 8;
-                        bytes = 16;
-                    }
-                }
-                cp_async16(sa + r * 128 + ((u ^ (r & 7)) << 4), src, bytes);
-            }
-            const uint16_t *wsrc = a.w + (size_t)kc * N * 64;
-#pragma unroll
-            for (int i = r; i < N * 8; i += 128) cp_async16(sb + i * 16, wsrc + i * 8, 16);
-        }
-        cp_async_commit();
-        if (kc >= LAG) {
-            cp_async_wait<LAG>();
-            fence_proxy_async_smem();
-            __syncthreads();
-            if (r == 0) {
-                fence_after_sync();
-                const int c = kc - LAG, s = c % STAGES;
-                const uint32_t sa = sbase + s * STAGE, sb = sa + A_STAGE;
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_bf16(tmem, sdesc_sw128(sa + 32 * ks), sdesc_sw128(sb + 32 * ks), idesc,
-                             (c > 0 || ks > 0) ? 1u : 0u);
-                mma_commit(smem_u32(&bar[s]));
-            }
-        }
-    }
-    // the last use of every stage (the final one covers every MMA)
-#pragma unroll
-    for (int s = 0; s < STAGES && s < NCH; ++s) {
-        const int last = s + STAGES * ((NCH - 1 - s) / STAGES);
-        if (!mbar_wait_bounded(smem_u32(&bar[s]), (last / STAGES) & 1, NN_WAIT)) *eflag = 1;
-    }
-    fence_after_sync();
-    const int warp = r >> 5;
-    float v[N];
-    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16), v);
-    if constexpr (N == 32) tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + 16, v + 16);
-    if (valid) {
-        const size_t o = (size_t)m * N;
-#pragma unroll
-        for (int g = 0; g < N / 8; ++g) {
-            float f[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                float x = v[8 * g + j];
-                if (a.bias) x += a.bias[8 * g + j];
-                if (a.relu) x = fmaxf(x, 0.f);
-                f[j] = x;
-            }
-            if (a.add) {
-                float ad[8];
-                unpack8(*reinterpret_cast<const uint4 *>(a.add + o + 8 * g), ad);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) f[j] += ad[j];
-            }
-            if (a.mask) {
-                float mk[8];
-                unpack8(*reinterpret_cast<const uint4 *>(a.mask + o + 8 * g), mk);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) f[j] = mk[j] > 0.f ? f[j] : 0.f;
-            }
-            *reinterpret_cast<uint4 *>(a.out + o + 8 * g) = pack8(f);
-        }
-    }
-    fence_before_sync();
-    __syncthreads();
-    if (r == 0 && *eflag) atomicOr(a.err, 1);
-    if (r < 32) tmem_dealloc(tmem, 32);
 }
 
 // ---------------------------------------------------------------- weight gradient
@@ -300,33 +164,18 @@ __global__ void k_wgrad_sum(const float *__restrict__ part, float *__restrict__ 
 
 template <int C, int N>
 static void set_attrs() {
-    cudaFuncSetAttribute(k_conv_tc<C, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(N));
     cudaFuncSetAttribute(k_wgrad_tc<C, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, wgrad_smem(N));
 }
 
 void init_attributes() {
     static bool done = false;
     if (done) return;
+    init_conv();
     set_attrs<16, 16>();
     set_attrs<16, 32>();
     set_attrs<32, 16>();
     set_attrs<32, 32>();
     done = true;
-}
-
-template <int C, int N>
-static void launch_conv(const ConvArgs &a, cudaStream_t st) {
-    const int grid = (a.nvox + 127) / 128;
-    if (grid > 0) k_conv_tc<C, N><<<grid, 128, conv_smem(N), st>>>(a);
-}
-
-int conv(const ConvArgs &a, int C, int N, cudaStream_t st) {
-    if (C == 16 && N == 16) launch_conv<16, 16>(a, st);
-    else if (C == 16 && N == 32) launch_conv<16, 32>(a, st);
-    else if (C == 32 && N == 16) launch_conv<32, 16>(a, st);
-    else if (C == 32 && N == 32) launch_conv<32, 32>(a, st);
-    else return -1;
-    return 0;
 }
 
 template <int C, int N>

@@ -34,6 +34,7 @@ struct ConvArgs {
     int relu;
     int nvox, lg;
     int *err;                // bit 0: a bounded wait expired
+    int up = 0;              // 1: x holds the grid of half the edge, read at each voxel's parent
 };
 
 struct WgradArgs {
@@ -53,6 +54,7 @@ constexpr int HEAD_MAX_BLOCKS = 8192;  // blocks of the head's loss / gradient k
 
 // set the shared-memory limits of every instantiation (call once, outside graph capture)
 void init_attributes();
+void init_conv();   // the part of it in k_conv.cu
 // C, N in {16, 32}; returns 0, or -1 for an unsupported shape
 int conv(const ConvArgs &a, int C, int N, cudaStream_t st);
 int wgrad(const WgradArgs &a, int C, int N, cudaStream_t st);

@@ -37,6 +37,14 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
     return d;
 }
 
+// The same without a swizzle: core matrices of 8 rows x 16 bytes (128 contiguous bytes), any
+// 16-byte start address.  K-major: `lbo` bytes from one core matrix to the next along K, `sbo`
+// along M or N.
+__device__ __forceinline__ uint64_t sdesc_none(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)(lbo >> 4) << 16 | (uint64_t)(sbo >> 4) << 32 |
+           (uint64_t)1u << 46;
+}
+
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9,
 // 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
 __host__ __device__ __forceinline__ uint32_t idesc_bf16_f32(int M, int N) {

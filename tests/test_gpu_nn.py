@@ -62,6 +62,20 @@ def test_conv_forward(sur, C, N, edge, batch):
 
 
 @pytest.mark.parametrize("C,N", SHAPES)
+@pytest.mark.parametrize("edge,batch", [(1, 3), (2, 2), (32, 5), (64, 2)])
+def test_conv_tile_columns(sur, C, N, edge, batch):
+    """Grids smaller than one 8 x 16 tile, and marches in z that cross from one column of tiles to
+    the next (and from one sample to the next) with the ring of planes wrapping."""
+    rng = np.random.default_rng(900 + C + N + edge)
+    x = _bf(rng.standard_normal((batch, edge, edge, edge, C)))
+    w = _bf(rng.standard_normal((N, 27, C)) * 0.2)
+    b = rng.standard_normal(N).astype(np.float32).astype(np.float64)
+    out = sur.conv3d(0, C, N, edge, batch, _to_dev_bf16(x), _to_dev_f32(w), bias=_to_dev_f32(b), relu=True)
+    ref = nn.relu(nn.conv3d(x, w, b))
+    _close_bf16(_host(out).reshape(ref.shape), ref, "columns C%d N%d e%d" % (C, N, edge))
+
+
+@pytest.mark.parametrize("C,N", SHAPES)
 def test_conv_forward_add_and_mask(sur, C, N):
     rng = np.random.default_rng(7 + C * N)
     edge, batch = 8, 1
