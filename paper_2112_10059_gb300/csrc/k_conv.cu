@@ -42,6 +42,9 @@ __host__ __device__ constexpr uint32_t weight_bytes(int C, int N) { return (uint
 __host__ __device__ constexpr uint32_t conv_smem(int C, int N) {
     return 1024 + weight_bytes(C, N) + RING * plane_bytes(C) + 64;
 }
+__host__ __device__ constexpr uint32_t conv_smem(int C, int N, int epi) {   // a tile's results staged for their children
+    return conv_smem(C, N) + (epi == CONV_EXPAND ? 128u * N * 2 : 0u);
+}
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
     return reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
@@ -54,34 +57,45 @@ __device__ __forceinline__ void cp_async_wait_upto(int pending) {
     else cp_async_wait<2>();
 }
 
-template <int C, int N>
-__global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
+template <int C, int N, int EPI>
+__global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
     pdl_enter();
     constexpr int CG = C / 8;
     constexpr uint32_t GB = group_bytes(C), PB = plane_bytes(C), WB = weight_bytes(C, N);
     constexpr int NU = (PX * PY * CG + 127) / 128;   // units copied per thread and plane
     extern __shared__ uint8_t raw[];
     uint8_t *base = align1024(raw);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(base + WB + RING * PB);   // [0], [1]: accumulators; [2]: weights
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 3);
+    // [0], [1]: accumulator done; [2], [3]: planes of the tile in shared memory; [4]: weights
+    uint64_t *bar = reinterpret_cast<uint64_t *>(base + WB + RING * PB);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 5);
     int *eflag = reinterpret_cast<int *>(tslot + 1);
     __shared__ float sbias[N];
+    __shared__ float shead[EPI == CONV_HEAD ? 34 : 1];
 
-    const int r = threadIdx.x;
+    const int r = threadIdx.x, warp = r >> 5;
     const int lg = a.lg, D = 1 << lg, dm = D - 1;
     const int ltx = lg > 3 ? lg - 3 : 0, lty = lg > 4 ? lg - 4 : 0;   // tiles per row and plane (log2)
     const int ntiles = (a.nvox >> (2 * lg)) << (ltx + lty);           // (batch x D) planes of tiles
-    const int t0 = (int)((long long)ntiles * blockIdx.x / gridDim.x);
-    const int t1 = (int)((long long)ntiles * (blockIdx.x + 1) / gridDim.x);
+    // equal shares of consecutive tiles (z fastest); whole z-pairs where the epilogue pools
+    const int g2 = EPI == CONV_POOL ? 1 : 0;
+    const int t0 = (int)((long long)(ntiles >> g2) * blockIdx.x / gridDim.x) << g2;
+    const int t1 = (int)((long long)(ntiles >> g2) * (blockIdx.x + 1) / gridDim.x) << g2;
     if (t0 >= t1) return;                     // uniform over the CTA, before any allocation
 
-    if (r < N) sbias[r] = a.bias ? a.bias[r] : 0.f;
-    if (r < 32) {
+    if (warp == 4) {
         tmem_alloc(smem_u32(tslot), 2 * N);
         tmem_relinquish();
     }
+    if (r < N) sbias[r] = a.bias ? a.bias[r] : 0.f;
+    if constexpr (EPI == CONV_HEAD) {
+        if (r < 34) shead[r] = a.hw[r];
+    }
     if (r == 0) {
-        for (int s = 0; s < 3; ++s) mbar_init(smem_u32(&bar[s]), 1);
+        mbar_init(smem_u32(&bar[0]), 1);
+        mbar_init(smem_u32(&bar[1]), 1);
+        mbar_init(smem_u32(&bar[2]), 128);
+        mbar_init(smem_u32(&bar[3]), 128);
+        mbar_init(smem_u32(&bar[4]), 1);
         *eflag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -90,66 +104,93 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
     fence_after_sync();
     const uint32_t tmem = *tslot;
     const uint32_t wbase = smem_u32(base), ring = wbase + WB;
-    const uint32_t idesc = idesc_bf16_f32(128, N);
-    if (r == 0) {
-        mbar_expect_tx(smem_u32(&bar[2]), WB);
-        bulk_g2s(wbase, a.w, WB, smem_u32(&bar[2]));
-    }
 
-    // ---- load cursor: the planes zs - 1 .. zs + len of each column's run of tiles, in order
-    const int up = a.up, lgi = lg - up, Di = 1 << lgi;   // input grid (half the edge when up-sampled on load)
-    int off[NU];
-    const uint16_t *xcol = a.x;
-    int ltile = t0, lz = 0, lze = -2, loaded = -1;
-    auto load_next = [&]() {                  // the next plane, one copy group; false when none is left
-        if (lz > lze) {                       // next column
-            if (ltile >= t1) return false;
-            const int col = ltile >> lg, zs = ltile & dm, len = min(D - zs, t1 - ltile);
-            const int x0 = (col & ((1 << ltx) - 1)) * CX - 1, y0 = ((col >> ltx) & ((1 << lty) - 1)) * CY - 1;
-            xcol = a.x + ((size_t)(col >> (ltx + lty)) << (3 * lgi)) * C;
+    if (warp == 4) {                          // ---- one thread issues every MMA
+        if (r == 128) {
+            const uint32_t idesc = idesc_bf16_f32(128, N);
+            const uint64_t ad0 = sdesc_none(0, GB, PX * 16), bd0 = sdesc_sw128(0);
+            mbar_expect_tx(smem_u32(&bar[4]), WB);
+            bulk_g2s(wbase, a.w, WB, smem_u32(&bar[4]));
+            if (!mbar_wait_bounded(smem_u32(&bar[4]), 0, NN_WAIT)) *eflag = 1;
+            int f = 0;
+            for (int it = 0; it < t1 - t0; ++it) {
+                if (it > 0) f += ((t0 + it) & dm) ? 1 : 3;
+                if (!mbar_wait_bounded(smem_u32(&bar[2 + (it & 1)]), (it >> 1) & 1, NN_WAIT)) *eflag = 1;
+                fence_after_sync();
+                const uint32_t acc = tmem + (uint32_t)((it & 1) * N);
+#pragma unroll
+                for (int dz = 0; dz < 3; ++dz) {
+                    const uint32_t sp = ring + (uint32_t)((f + dz) % RING) * PB;
+#pragma unroll
+                    for (int tap = 9 * dz; tap < 9 * dz + 9; ++tap) {
+                        const uint32_t sv = sp + (uint32_t)((tap / 3 % 3) * PX + tap % 3) * 16;
+#pragma unroll
+                        for (int h = 0; h < C / 16; ++h) {
+                            const int k = tap * (C / 16) + h;   // K = 16 slice of the weight image
+                            mma_bf16(acc, ad0 + ((sv + 2 * h * GB) >> 4),
+                                     bd0 + ((wbase + (uint32_t)(k / 4) * N * 128 + (uint32_t)(k % 4) * 32) >> 4), idesc,
+                                     k > 0 ? 1u : 0u);
+                        }
+                    }
+                }
+                mma_commit(smem_u32(&bar[it & 1]));
+            }
+        }
+    } else {                                  // ---- four warps copy planes and write results
+        // load cursor: the planes zs - 1 .. zs + len of each column's run of tiles, in order
+        const int up = a.up, lgi = lg - up;   // input grid (half the edge when up-sampled on load)
+        int off[NU];
+        const uint16_t *xcol = a.x;
+        int ltile = t0, lz = 0, lze = -2, loaded = -1;
+        auto load_next = [&]() {              // the next plane, one copy group; false when none is left
+            if (lz > lze) {                   // next column
+                const int col = ltile >> lg, zs = ltile & dm, len = min(D - zs, t1 - ltile);
+                const int x0 = (col & ((1 << ltx) - 1)) * CX - 1, y0 = ((col >> ltx) & ((1 << lty) - 1)) * CY - 1;
+                xcol = a.x + ((size_t)(col >> (ltx + lty)) << (3 * lgi)) * C;
+#pragma unroll
+                for (int j = 0; j < NU; ++j) {
+                    const int u = r + 128 * j, v = u / CG, cg = u % CG;
+                    const int x = x0 + v % PX, y = y0 + v / PX;
+                    off[j] = ((unsigned)x < (unsigned)D && (unsigned)y < (unsigned)D)
+                                 ? (((y >> up) << lgi) + (x >> up)) * C + cg * 8
+                                 : -1;
+                }
+                lz = zs - 1;
+                lze = zs + len;
+                ltile += len;
+            }
+            ++loaded;
+            const uint32_t dst = ring + (uint32_t)(loaded % RING) * PB;
+            const bool zin = (unsigned)lz < (unsigned)D;
+            const uint16_t *xp = xcol + ((size_t)((zin ? lz : 0) >> up) << (2 * lgi)) * C;
 #pragma unroll
             for (int j = 0; j < NU; ++j) {
-                const int u = r + 128 * j, v = u / CG, cg = u % CG;
-                const int x = x0 + v % PX, y = y0 + v / PX;
-                off[j] = ((unsigned)x < (unsigned)D && (unsigned)y < (unsigned)D)
-                             ? (((y >> up) << lgi) + (x >> up)) * C + cg * 8
-                             : -1;
+                const int u = r + 128 * j;
+                if (u < PX * PY * CG) {
+                    const bool in = zin && off[j] >= 0;
+                    cp_async16(dst + (uint32_t)(u % CG) * GB + (uint32_t)(u / CG) * 16, in ? xp + off[j] : a.x, in ? 16 : 0);
+                }
             }
-            lz = zs - 1;
-            lze = zs + len;
-            ltile += len;
-        }
-        ++loaded;
-        const uint32_t dst = ring + (uint32_t)(loaded % RING) * PB;
-        const bool zin = (unsigned)lz < (unsigned)D;
-        const uint16_t *xp = xcol + ((size_t)((zin ? lz : 0) >> up) << (2 * lgi)) * C;
-#pragma unroll
-        for (int j = 0; j < NU; ++j) {
-            const int u = r + 128 * j;
-            if (u < PX * PY * CG) {
-                const bool in = zin && off[j] >= 0;
-                cp_async16(dst + (uint32_t)(u % CG) * GB + (uint32_t)(u / CG) * 16, in ? xp + off[j] : a.x, in ? 16 : 0);
-            }
-        }
-        cp_async_commit();
-        ++lz;
-        return lz <= lze || ltile < t1;
-    };
+            cp_async_commit();
+            ++lz;
+            return lz <= lze || ltile < t1;
+        };
 
-    const int warp = r >> 5;
-    auto epilogue = [&](int t, int it) {
-        const int col = t >> lg, z = t & dm;
-        const int x = (col & ((1 << ltx) - 1)) * CX + (r & 7), y = ((col >> ltx) & ((1 << lty) - 1)) * CY + (r >> 3);
-        const size_t m = ((((size_t)(col >> (ltx + lty)) << lg) + z) << (2 * lg)) + ((size_t)y << lg) + x;
-        if (!mbar_wait_bounded(smem_u32(&bar[it & 1]), (it >> 1) & 1, NN_WAIT)) *eflag = 1;
-        fence_after_sync();
-        float v[N];
-        const uint32_t acc = tmem + (uint32_t)((it & 1) * N) + ((uint32_t)(warp * 32) << 16);
-        tmem_ld16(acc, v);
-        if constexpr (N == 32) tmem_ld16(acc + 16, v + 16);
-        fence_before_sync();                  // ordered before the MMAs that overwrite it by the next barrier
-        if (x < D && y < D) {
-            const size_t o = m * N;
+        float pool[EPI == CONV_POOL ? N : 1];
+        auto epilogue = [&](int t, int it) {
+            const int col = t >> lg, z = t & dm;
+            const int x = (col & ((1 << ltx) - 1)) * CX + (r & 7), y = ((col >> ltx) & ((1 << lty) - 1)) * CY + (r >> 3);
+            const size_t bz = ((size_t)(col >> (ltx + lty)) << lg) + z;   // sample and plane
+            const bool valid = x < D && y < D;
+            if (!mbar_wait_bounded(smem_u32(&bar[it & 1]), (it >> 1) & 1, NN_WAIT)) *eflag = 1;
+            fence_after_sync();
+            float v[N];
+            const uint32_t acc = tmem + (uint32_t)((it & 1) * N) + ((uint32_t)(warp * 32) << 16);
+            tmem_ld16(acc, v);
+            if constexpr (N == 32) tmem_ld16(acc + 16, v + 16);
+            fence_before_sync();              // read before this thread's next arrival frees the accumulator
+            const size_t o = ((bz << (2 * lg)) + ((size_t)y << lg) + x) * N;
+            uint4 q[N / 8];
 #pragma unroll
             for (int g = 0; g < N / 8; ++g) {
                 float f[8];
@@ -160,98 +201,478 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
                     if (a.relu) s = fmaxf(s, 0.f);
                     f[j] = s;
                 }
-                if (a.add) {
-                    float ad[8];
-                    unpack8(*reinterpret_cast<const uint4 *>(a.add + o + 8 * g), ad);
+                if constexpr (EPI == CONV_PLAIN) {
+                    if (a.add && valid) {
+                        float ad[8];
+                        unpack8(*reinterpret_cast<const uint4 *>(a.add + o + 8 * g), ad);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) f[j] += ad[j];
-                }
-                if (a.mask) {
-                    float mk[8];
-                    unpack8(*reinterpret_cast<const uint4 *>(a.mask + o + 8 * g), mk);
+                        for (int j = 0; j < 8; ++j) f[j] += ad[j];
+                    }
+                    if (a.mask && valid) {
+                        float mk[8];
+                        unpack8(*reinterpret_cast<const uint4 *>(a.mask + o + 8 * g), mk);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) f[j] = mk[j] > 0.f ? f[j] : 0.f;
+                        for (int j = 0; j < 8; ++j) f[j] = mk[j] > 0.f ? f[j] : 0.f;
+                    }
                 }
-                const uint4 q = pack8(f);
-                *reinterpret_cast<uint4 *>(a.out + o + 8 * g) = q;
+                q[g] = pack8(f);
+                if (valid && (EPI == CONV_PLAIN || a.out)) *reinterpret_cast<uint4 *>(a.out + o + 8 * g) = q[g];
             }
-        }
-    };
-
-    int f = 0, fprev = 0;                     // sequence number of the tile's first plane
-    bool more = true;
-    for (int it = 0; it < t1 - t0; ++it) {
-        const int t = t0 + it;
-        if (it > 0) {
-            fprev = f;
-            f += (t & dm) ? 1 : 3;
-        }
-        // a slot is free once the last tile that read it is done: the previous tile, whose MMAs
-        // may still run, reads the planes from fprev on
-        const int lim = min(f + 2 + AHEAD, fprev + RING - 1);
-        while (more && loaded < lim) more = load_next();
-        cp_async_wait_upto(loaded - (f + 2));
-        fence_proxy_async_smem();
-        __syncthreads();
-        if (r == 0) {
-            if (it == 0 && !mbar_wait_bounded(smem_u32(&bar[2]), 0, NN_WAIT)) *eflag = 1;
-            fence_after_sync();
-            const uint64_t ad0 = sdesc_none(0, GB, PX * 16), bd0 = sdesc_sw128(0);
-            const uint32_t acc = tmem + (uint32_t)((it & 1) * N);
+            if constexpr (EPI == CONV_PAIR) {
+                if (valid) {
 #pragma unroll
-            for (int dz = 0; dz < 3; ++dz) {
-                const uint32_t sp = ring + (uint32_t)((f + dz) % RING) * PB;
+                    for (int g = 0; g < N / 8; ++g) {
+                        float f[8], s[8];
+                        unpack8(q[g], f);
+                        unpack8(__ldg(reinterpret_cast<const uint4 *>((a.add2 ? a.add2 : a.mask2) + o + 8 * g)), s);
 #pragma unroll
-                for (int tap = 9 * dz; tap < 9 * dz + 9; ++tap) {
-                    const uint32_t sv = sp + (uint32_t)((tap / 3 % 3) * PX + tap % 3) * 16;
-#pragma unroll
-                    for (int h = 0; h < C / 16; ++h) {
-                        const int k = tap * (C / 16) + h;   // K = 16 slice of the weight image
-                        mma_bf16(acc, ad0 + ((sv + 2 * h * GB) >> 4),
-                                 bd0 + ((wbase + (uint32_t)(k / 4) * N * 128 + (uint32_t)(k % 4) * 32) >> 4), idesc,
-                                 k > 0 ? 1u : 0u);
+                        for (int j = 0; j < 8; ++j) f[j] = a.add2 ? f[j] + s[j] : (s[j] > 0.f ? f[j] : 0.f);
+                        *reinterpret_cast<uint4 *>(a.out2 + o + 8 * g) = pack8(f);
                     }
                 }
             }
-            mma_commit(smem_u32(&bar[it & 1]));
+            if constexpr (EPI == CONV_EXPAND) {
+                // through shared memory, so that the four warps walk the children's 16-byte units in
+                // the order they lie (with a thread per parent, every lane of an access is a line of
+                // its own and the unrolled code misses the instruction cache: 30 against 8 us at 8^3)
+                constexpr int G = N / 8;
+                uint4 *tile = reinterpret_cast<uint4 *>(bar + 6);
+#pragma unroll
+                for (int g = 0; g < G; ++g) tile[r * G + g] = q[g];
+                named_sync(1, 128);
+                const int cx0 = 2 * (x - (r & 7)), cy0 = 2 * (y - (r >> 3));
+#pragma unroll 4
+                for (int i = 0; i < N; ++i) {
+                    const int e = r + 128 * i, g = e % G, cx = e / G % 16, cy = e / G / 16 % 32, cz = e / G / 512;
+                    if (cx0 + cx < 2 * D && cy0 + cy < 2 * D) {
+                        const size_t oc = (((2 * bz + cz) << (2 * lg + 2)) + ((size_t)(cy0 + cy) << (lg + 1)) + cx0 + cx) * N + 8 * g;
+                        float f[8], s[8], m[8];
+                        unpack8(__ldg(reinterpret_cast<const uint4 *>(a.add2 + oc)), s);
+                        if (a.mask2) unpack8(__ldg(reinterpret_cast<const uint4 *>(a.mask2 + oc)), m);
+                        unpack8(tile[((cy >> 1) * 8 + (cx >> 1)) * G + g], f);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            f[j] = !a.mask2 ? f[j] + s[j] : (m[j] > 0.f ? s[j] + 0.125f * f[j] : 0.f);
+                        *reinterpret_cast<uint4 *>(a.out2 + oc) = pack8(f);
+                    }
+                }
+                named_sync(1, 128);           // read before the next tile is staged
+            }
+            if constexpr (EPI == CONV_POOL) {
+                // children in the order x, y, z: this lane, its x, y and diagonal neighbour (lanes
+                // r + 1, r + 8, r + 9 of the same warp), then the next plane's four
+#pragma unroll
+                for (int g = 0; g < N / 8; ++g) {
+                    float s[8], f[8];
+                    unpack8(q[g], s);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int src = (c & 1) + 8 * (c >> 1);
+                        if (c > 0) {
+                            uint4 n;
+                            n.x = __shfl_down_sync(0xffffffffu, q[g].x, src);
+                            n.y = __shfl_down_sync(0xffffffffu, q[g].y, src);
+                            n.z = __shfl_down_sync(0xffffffffu, q[g].z, src);
+                            n.w = __shfl_down_sync(0xffffffffu, q[g].w, src);
+                            unpack8(n, f);
+                        } else {
+                            unpack8(q[g], f);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) pool[8 * g + j] = c == 0 && !(z & 1) ? 0.f + s[j] : pool[8 * g + j] + f[j];
+                    }
+                }
+                if ((z & 1) && valid && !(r & 1) && !(r & 8)) {
+                    const size_t op = ((((bz >> 1) << (2 * lg - 2)) + ((size_t)(y >> 1) << (lg - 1))) + (x >> 1)) * N;
+#pragma unroll
+                    for (int g = 0; g < N / 8; ++g) {
+                        float f[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) f[j] = a.scale * pool[8 * g + j];
+                        if (a.mask2) {
+                            float mk[8];
+                            unpack8(__ldg(reinterpret_cast<const uint4 *>(a.mask2 + op + 8 * g)), mk);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) f[j] = mk[j] > 0.f ? f[j] : 0.f;
+                        }
+                        *reinterpret_cast<uint4 *>(a.out2 + op + 8 * g) = pack8(f);
+                    }
+                }
+            }
+            if constexpr (EPI == CONV_HEAD) {
+                float f[16], r0 = shead[32], e0 = shead[33];
+                unpack8(q[0], f);
+                unpack8(q[1], f + 8);
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    r0 = fmaf(shead[c], f[c], r0);
+                    e0 = fmaf(shead[16 + c], f[c], e0);
+                }
+                if (valid) *reinterpret_cast<float2 *>(a.y + o / N * 2) = make_float2(r0, e0);
+            }
+        };
+
+        int f = 0, fprev = 0;                 // sequence number of the tile's first plane
+        bool more = true;
+        for (int it = 0; it < t1 - t0; ++it) {
+            const int t = t0 + it;
+            if (it > 0) {
+                fprev = f;
+                f += (t & dm) ? 1 : 3;
+            }
+            // a slot is free once the last tile that read it is done: the previous tile, whose MMAs
+            // may still run, reads the planes from fprev on
+            const int lim = min(f + 2 + AHEAD, fprev + RING - 1);
+            while (more && loaded < lim) more = load_next();
+            cp_async_wait_upto(loaded - (f + 2));
+            fence_proxy_async_smem();
+            mbar_arrive(smem_u32(&bar[2 + (it & 1)]));
+            if (it > 0) epilogue(t - 1, it - 1);
         }
-        if (it > 0) epilogue(t - 1, it - 1);
+        epilogue(t1 - 1, t1 - 1 - t0);
     }
-    epilogue(t1 - 1, t1 - 1 - t0);
     fence_before_sync();
     __syncthreads();
     if (r == 0 && *eflag) atomicOr(a.err, 1);
-    if (r < 32) tmem_dealloc(tmem, 2 * N);
+    if (warp == 4) tmem_dealloc(tmem, 2 * N);
+}
+
+// ---------------------------------------------------------------- weight gradient
+// dW[n][tap][c] = sum over voxels m of dz[m][n] x[m + off(tap)][c]: M = (tap, c), N = out
+// channels, K = voxels.  Both operands are K x M (N) with the channels contiguous, i.e. MN-major
+// as the tensors lie: a core matrix is 8 x-neighbours of one 8-channel group, the same 16-byte
+// units as above, so nothing is transposed or repeated.  Shared memory holds, per y row, the
+// units of [z - 1, z, z + 1][channel group][x] at one stride; the core matrices of three
+// neighbouring rows then follow each other at that stride in the order (dy, dz, group), which
+// makes M tiles of 128 rows that cover the nine (dy, dz) taps (a tenth of the rows is padding),
+// and the three dx are start addresses one unit apart.  A constant plane of ones behind the
+// three z gives the bias gradient as one more row.
+// CTAs march in y through equal shares of the (sample, z, x segment) columns, 64 voxels an
+// iteration, rows in a ring whose first slots are mirrored behind its last so that three rows
+// always follow each other.  Each CTA's sums go to its own slice of `part`; k_wgrad_sum adds
+// the slices in order (training is reproducible bit for bit).
+// What bounds it: 4 KB of x read from shared memory per MMA, as above.
+__host__ __device__ constexpr int wg_block(int C) { return 3 * (C / 8) + 1; }               // core-matrix columns per row
+__host__ __device__ constexpr int wg_tiles(int C) { return (3 * wg_block(C) + 15) / 16; }   // M tiles per dx
+__host__ __device__ constexpr int wg_cols(int C, int N) {                                   // TMEM columns (power of 2)
+    return 3 * wg_tiles(C) * N <= 128 ? 128 : 3 * wg_tiles(C) * N <= 256 ? 256 : 512;
+}
+constexpr uint32_t wg_dz_slot(int N) { return (uint32_t)(N / 8) * 1024 + 128; }
+
+struct WgradShape {      // how a layer's voxels are cut, from its edge alone
+    int lgx;             // x segment of a row: 2^lgx voxels, 8 .. 64
+    int rpi, lipc;       // rows per iteration, iterations per column (log2)
+    int ring, mirror;    // rows in the ring, slots repeated behind it
+    uint32_t stride;     // bytes between core-matrix columns
+    int cols;            // core-matrix columns in shared memory
+    int iters;           // iterations in all
+};
+static WgradShape wgrad_shape(int C, int lg, int nvox) {
+    WgradShape s;
+    const int lge = lg < 3 ? 3 : lg;
+    s.lgx = lge > 6 ? 6 : lge;
+    s.rpi = 64 >> s.lgx;
+    s.lipc = lge - (6 - s.lgx);
+    s.ring = 2 * (s.rpi + 2) + 2;
+    s.mirror = s.lgx == 3 ? 3 : 2;
+    // the 8 units a quarter-warp copies (2 groups x 4 voxels, or 4 x 2) in different banks
+    s.stride = (uint32_t)((1 << s.lgx) + 2) * 16 + (C == 16 ? 32 : 0);
+    const int cb = wg_block(C);
+    const int read = (s.ring - 1) * cb + 16 * wg_tiles(C) + (s.lgx == 3 ? cb : 0);   // the padding rows' reads end here
+    s.cols = (s.ring + s.mirror) * cb > read ? (s.ring + s.mirror) * cb : read;
+    s.iters = (nvox >> (2 * lg)) << (lge - s.lgx + s.lipc);
+    return s;
+}
+static uint32_t wgrad_smem(int C, int N, const WgradShape &s) { return 128 + (uint32_t)s.cols * s.stride + 4 * wg_dz_slot(N) + 64; }
+
+int wgrad_splits(int C, int N, int lg, int nvox) {
+    const WgradShape s = wgrad_shape(C, lg, nvox);
+    const int fit = 227 * 1024 / (int)(wgrad_smem(C, N, s) + 1024), tm = 512 / wg_cols(C, N);
+    const int most = 152 * (fit < tm ? (fit < 2 ? fit : 2) : (tm < 2 ? tm : 2));
+    const int n = (s.iters + 1) / 2;          // at least two iterations a CTA: each writes a slice of its own
+    return n < 1 ? 1 : n < most ? n : most;
 }
 
 template <int C, int N>
+__global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
+    pdl_enter();
+    constexpr int CG = C / 8, CB = wg_block(C), NM = wg_tiles(C), TC = wg_cols(C, N);
+    constexpr int NU = (3 * CG * 66 + 127) / 128, NZ = N / 16;
+    constexpr uint32_t ZS = wg_dz_slot(N), ZG = ZS / (N / 8);
+    extern __shared__ uint8_t raw[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 127) & ~(uintptr_t)127);
+    const uint32_t xbytes = (uint32_t)s.cols * s.stride, blk = (uint32_t)CB * s.stride;
+    // [0], [1]: an iteration's MMAs are done; [2], [3]: its rows are in shared memory
+    uint64_t *bar = reinterpret_cast<uint64_t *>(base + xbytes + 4 * ZS);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 4);
+    int *eflag = reinterpret_cast<int *>(tslot + 1);
+    const int r = threadIdx.x, warp = r >> 5;
+    const int i0 = (int)((long long)s.iters * blockIdx.x / gridDim.x);
+    const int n = (int)((long long)s.iters * (blockIdx.x + 1) / gridDim.x) - i0;   // >= 1: the grid is no larger than iters
+    const int ipm = (1 << s.lipc) - 1;
+
+    if (warp == 4) {
+        tmem_alloc(smem_u32(tslot), TC);
+        tmem_relinquish();
+    }
+    if (r == 0) {
+        mbar_init(smem_u32(&bar[0]), 1);
+        mbar_init(smem_u32(&bar[1]), 1);
+        mbar_init(smem_u32(&bar[2]), 128);
+        mbar_init(smem_u32(&bar[3]), 128);
+        *eflag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int e = r; e < (s.ring + s.mirror) << s.lgx; e += 160) {   // the ones: channel 0 of each unit
+        const int b = e >> s.lgx, x = e & ((1 << s.lgx) - 1);
+        uint8_t *p = base + (size_t)(b * CB + CB - 1) * s.stride + (size_t)x * 16;
+        *reinterpret_cast<uint4 *>(p) = make_uint4(0x3F80u, 0, 0, 0);
+        if (x < 2) *reinterpret_cast<uint4 *>(p + (16u << s.lgx)) = make_uint4(0x3F80u, 0, 0, 0);
+    }
+    fence_proxy_async_smem();
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = *tslot;
+    const uint32_t xb = smem_u32(base), zb = xb + xbytes;
+
+    if (warp == 4) {                          // ---- one thread issues every MMA
+        if (r == 128) {
+            const uint32_t idesc = idesc_bf16_f32(128, N) | (3u << 15);      // both operands MN-major
+            // MN-major without a swizzle: first stride along K (8 voxels), second along M or N
+            const uint64_t ad0 = sdesc_none(0, s.lgx == 3 ? blk : 128, s.stride), bd0 = sdesc_none(0, 128, ZG);
+            int f = 0;                        // sequence number of the iteration's first row
+            for (int it = 0; it < n; ++it) {
+                if (it > 0) f += s.rpi + (((i0 + it) & ipm) ? 0 : 2);
+                if (!mbar_wait_bounded(smem_u32(&bar[2 + (it & 1)]), (it >> 1) & 1, NN_WAIT)) *eflag = 1;
+                fence_after_sync();
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    const int row = (16 * ks) >> s.lgx, x = (16 * ks) & ((1 << s.lgx) - 1);
+                    const uint32_t sx = xb + (uint32_t)((f + row) % s.ring) * blk + (uint32_t)x * 16;
+                    const uint64_t bd = bd0 + ((zb + (uint32_t)(it & 3) * ZS + (uint32_t)ks * 256) >> 4);
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                        for (int j = 0; j < NM; ++j)
+                            mma_bf16(tmem + (uint32_t)((dx * NM + j) * N),
+                                     ad0 + ((sx + (uint32_t)dx * 16 + (uint32_t)j * 16 * s.stride) >> 4), bd, idesc,
+                                     (it > 0 || ks > 0) ? 1u : 0u);
+                }
+                mma_commit(smem_u32(&bar[it & 1]));
+            }
+        }
+    } else {                                  // ---- four warps copy
+        const int lg = a.lg, D = 1 << lg, up = a.up, lgi = lg - up;
+        const int lnx = lg > 6 ? lg - 6 : 0;  // x segments per row (log2)
+        const int TX = 1 << s.lgx, nub = 3 * CG * (TX + 2);
+        int off[NU];
+        uint32_t dst[NU];
+        const uint16_t *xcol = a.x, *zcol = a.dz;
+        int x0 = 0, rows = -1;                // rows: sequence number of the last row copied
+#pragma unroll
+        for (int j = 0; j < NU; ++j) {
+            const int u = r + 128 * j, cg = u % CG, v = u / CG;
+            dst[j] = xb + (uint32_t)((v / (TX + 2)) * CG + cg) * s.stride + (uint32_t)(v % (TX + 2)) * 16;
+        }
+        auto load_iter = [&](int k) {         // one copy group: the rows and gradients that iteration k adds
+            const int i = i0 + k, y0 = (i & ipm) * s.rpi;
+            const bool first = k == 0 || (i & ipm) == 0;
+            if (first) {
+                const int col = i >> s.lipc, z = (col >> lnx) & (D - 1), b = col >> (lnx + lg);
+                x0 = (col & ((1 << lnx) - 1)) << 6;
+                xcol = a.x + ((size_t)b << (3 * lgi)) * C;
+                zcol = a.dz + (((size_t)b << (3 * lg)) + ((size_t)z << (2 * lg))) * N;
+#pragma unroll
+                for (int j = 0; j < NU; ++j) {
+                    const int u = r + 128 * j, cg = u % CG, v = u / CG;
+                    const int x = x0 + v % (TX + 2) - 1, zz = z + v / (TX + 2) - 1;
+                    off[j] = (u < nub && (unsigned)x < (unsigned)D && (unsigned)zz < (unsigned)D)
+                                 ? (((zz >> up) << (2 * lgi)) + (x >> up)) * C + cg * 8
+                                 : -1;
+                }
+            }
+            for (int y = first ? y0 - 1 : y0 + 1; y <= y0 + s.rpi; ++y) {
+                ++rows;
+                const int slot = rows % s.ring;
+                const bool yin = (unsigned)y < (unsigned)D;
+                const uint16_t *xr = xcol + ((size_t)((yin ? y : 0) >> up) << lgi) * C;
+#pragma unroll
+                for (int j = 0; j < NU; ++j) {
+                    if (r + 128 * j < nub) {
+                        const bool in = yin && off[j] >= 0;
+                        cp_async16(dst[j] + (uint32_t)slot * blk, in ? xr + off[j] : a.x, in ? 16 : 0);
+                        if (slot < s.mirror)
+                            cp_async16(dst[j] + (uint32_t)(slot + s.ring) * blk, in ? xr + off[j] : a.x, in ? 16 : 0);
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < NZ; ++j) {    // 64 voxels x N / 8 units
+                const int u = r + 128 * j, v = u / (N / 8), ng = u % (N / 8);
+                const int y = y0 + (v >> s.lgx), x = x0 + (v & (TX - 1));
+                const bool in = y < D && x < D;
+                cp_async16(zb + (uint32_t)(k & 3) * ZS + (uint32_t)ng * ZG + (uint32_t)v * 16,
+                           in ? zcol + (((size_t)y << lg) + x) * N + ng * 8 : a.dz, in ? 16 : 0);
+            }
+            cp_async_commit();
+        };
+        int f = 0, fprev = 0, k = 0;          // k: iterations copied
+        for (int it = 0; it < n; ++it) {
+            if (it > 0) {
+                fprev = f;
+                f += s.rpi + (((i0 + it) & ipm) ? 0 : 2);
+            }
+            // the MMAs of iteration it - 2 are done: rows before fprev and its gradients are free
+            if (it >= 2 && !mbar_wait_bounded(smem_u32(&bar[it & 1]), ((it - 2) >> 1) & 1, NN_WAIT)) *eflag = 1;
+            while (k < n && k <= it + AHEAD &&
+                   rows + s.rpi + ((k == 0 || ((i0 + k) & ipm) == 0) ? 2 : 0) <= fprev + s.ring - 1)
+                load_iter(k++);
+            cp_async_wait_upto(k - 1 - it);
+            fence_proxy_async_smem();
+            mbar_arrive(smem_u32(&bar[2 + (it & 1)]));
+        }
+        // commits complete in order: the last iteration's covers every MMA
+        if (!mbar_wait_bounded(smem_u32(&bar[(n - 1) & 1]), ((n - 1) >> 1) & 1, NN_WAIT)) *eflag = 1;
+        fence_after_sync();
+        float *part = a.part + (size_t)blockIdx.x * ((NTAPS * C + 1) * N);
+        for (int q = 0; q < 3 * NM; ++q) {
+            float v[N];
+            const uint32_t acc = tmem + (uint32_t)(q * N) + ((uint32_t)(warp * 32) << 16);
+            tmem_ld16(acc, v);
+            if constexpr (N == 32) tmem_ld16(acc + 16, v + 16);
+            const int dx = q / NM, cm = 16 * (q % NM) + (r >> 3), dy = cm / CB, rem = cm % CB;
+            const int row = dy > 2 ? -1
+                            : rem < CB - 1 ? (9 * (rem / CG) + 3 * dy + dx) * C + 8 * (rem % CG) + (r & 7)
+                            : (dy == 0 && dx == 0 && (r & 7) == 0) ? NTAPS * C : -1;
+            if (row >= 0) {
+                float4 *o = reinterpret_cast<float4 *>(part + (size_t)row * N);
+#pragma unroll
+                for (int e = 0; e < N / 4; ++e) o[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            }
+        }
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (r == 0 && *eflag) atomicOr(a.err, 1);
+    if (warp == 4) tmem_dealloc(tmem, TC);
+}
+
+// gradients of every layer of the table from the CTAs' slices: [27 C + 1][N] summed over the
+// splits, written as w [N][27][C] then b [N].  32 elements x 8 groups of splits per block, the
+// groups added in order.
+__global__ void __launch_bounds__(256) k_wgrad_sum(WgradSums t) {
+    pdl_enter();
+    __shared__ float sm[8][32];
+    int l = 0;
+    while (l + 1 < t.layers && (int)blockIdx.x >= t.l[l + 1].block0) ++l;
+    const WgradSum &w = t.l[l];
+    const int elems = w.elems(), e = ((int)blockIdx.x - w.block0) * 32 + (threadIdx.x & 31), g = threadIdx.x >> 5;
+    float acc = 0.f;
+    if (e < elems)
+        for (int y = g; y < w.splits; y += 8) acc += w.part[(size_t)y * elems + e];
+    sm[g][threadIdx.x & 31] = acc;
+    __syncthreads();
+    if (g == 0 && e < elems) {
+#pragma unroll
+        for (int k = 1; k < 8; ++k) acc += sm[k][threadIdx.x];
+        const int k = e / w.N, nn = e % w.N;
+        if (w.C == 0) w.grad[e] = acc;
+        else w.grad[k < NTAPS * w.C ? nn * NTAPS * w.C + k : NTAPS * w.C * w.N + nn] = acc;
+    }
+    if (w.C == 0 && g == 1 && (int)blockIdx.x == w.block0) {   // the loss, its partials in a fixed order too
+        double d = 0.0;
+        for (int y = threadIdx.x & 31; y < w.splits; y += 32) d += t.loss_part[y];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+        if ((threadIdx.x & 31) == 0) *t.loss = d;
+    }
+}
+
+template <int C, int N, int EPI>
 static void set_conv() {
-    cudaFuncSetAttribute(k_conv_tc<C, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(C, N));
+    cudaFuncSetAttribute(k_conv_tc<C, N, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(C, N, EPI));
 }
 
-void init_conv() {
-    set_conv<16, 16>();
-    set_conv<16, 32>();
-    set_conv<32, 16>();
-    set_conv<32, 32>();
+void init_attributes() {
+    static bool done = false;
+    if (done) return;
+    set_conv<16, 16, CONV_PLAIN>();
+    set_conv<16, 32, CONV_PLAIN>();
+    set_conv<32, 16, CONV_PLAIN>();
+    set_conv<32, 32, CONV_PLAIN>();
+    set_conv<16, 16, CONV_POOL>();
+    set_conv<16, 32, CONV_POOL>();
+    set_conv<32, 32, CONV_POOL>();
+    set_conv<16, 16, CONV_PAIR>();
+    set_conv<32, 16, CONV_PAIR>();
+    set_conv<32, 16, CONV_EXPAND>();
+    set_conv<32, 32, CONV_EXPAND>();
+    set_conv<16, 16, CONV_HEAD>();
+    cudaFuncSetAttribute(k_wgrad_tc<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_wgrad_tc<16, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_wgrad_tc<32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_wgrad_tc<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    done = true;
 }
 
-template <int C, int N>
-static void launch_conv(const ConvArgs &a, cudaStream_t st) {
-    // as many CTAs as fit beside each other on an SM (227 KB shared memory, 4 of 128 threads at most)
-    constexpr int per_sm = 227 * 1024 / (int)(conv_smem(C, N) + 1024) < 4 ? 227 * 1024 / (int)(conv_smem(C, N) + 1024) : 4;
+template <int C, int N, int EPI>
+static int launch_conv(const ConvArgs &a, cudaStream_t st) {
+    // as many CTAs as fit beside each other on an SM (227 KB shared memory, 4 at most)
+    constexpr int fit = 227 * 1024 / (int)(conv_smem(C, N, EPI) + 1024);
+    constexpr int per_sm = fit < 4 ? fit : 4;
     const int ltx = a.lg > 3 ? a.lg - 3 : 0, lty = a.lg > 4 ? a.lg - 4 : 0;
     const int tiles = (a.nvox >> (2 * a.lg)) << (ltx + lty);
-    if (tiles > 0) launch_pdl(k_conv_tc<C, N>, tiles < 152 * per_sm ? tiles : 152 * per_sm, 128, conv_smem(C, N), st, a);
+    if (tiles > 0)
+        launch_pdl(k_conv_tc<C, N, EPI>, tiles < 152 * per_sm ? tiles : 152 * per_sm, 160, conv_smem(C, N, EPI), st, a);
+    return 0;
 }
 
 int conv(const ConvArgs &a, int C, int N, cudaStream_t st) {
-    if (C == 16 && N == 16) launch_conv<16, 16>(a, st);
-    else if (C == 16 && N == 32) launch_conv<16, 32>(a, st);
-    else if (C == 32 && N == 16) launch_conv<32, 16>(a, st);
-    else if (C == 32 && N == 32) launch_conv<32, 32>(a, st);
-    else return -1;
+    const int cn = C * 100 + N;
+    switch (a.epi) {
+        case CONV_HEAD: return cn == 1616 ? launch_conv<16, 16, CONV_HEAD>(a, st) : -1;
+        case CONV_POOL:
+            return cn == 1616   ? launch_conv<16, 16, CONV_POOL>(a, st)
+                   : cn == 1632 ? launch_conv<16, 32, CONV_POOL>(a, st)
+                   : cn == 3232 ? launch_conv<32, 32, CONV_POOL>(a, st)
+                                : -1;
+        case CONV_PAIR:
+            return cn == 1616 ? launch_conv<16, 16, CONV_PAIR>(a, st) : cn == 3216 ? launch_conv<32, 16, CONV_PAIR>(a, st) : -1;
+        case CONV_EXPAND:
+            return cn == 3216 ? launch_conv<32, 16, CONV_EXPAND>(a, st) : cn == 3232 ? launch_conv<32, 32, CONV_EXPAND>(a, st) : -1;
+        default:
+            return cn == 1616   ? launch_conv<16, 16, CONV_PLAIN>(a, st)
+                   : cn == 1632 ? launch_conv<16, 32, CONV_PLAIN>(a, st)
+                   : cn == 3216 ? launch_conv<32, 16, CONV_PLAIN>(a, st)
+                   : cn == 3232 ? launch_conv<32, 32, CONV_PLAIN>(a, st)
+                                : -1;
+    }
+}
+
+template <int C, int N>
+static int launch_wgrad(const WgradArgs &a, cudaStream_t st) {
+    const WgradShape s = wgrad_shape(C, a.lg, a.nvox);
+    if (s.iters > 0)
+        launch_pdl(k_wgrad_tc<C, N>, wgrad_splits(C, N, a.lg, a.nvox), 160, wgrad_smem(C, N, s), st, a, s);
     return 0;
+}
+
+int wgrad(const WgradArgs &a, int C, int N, cudaStream_t st) {
+    if (C == 16 && N == 16) return launch_wgrad<16, 16>(a, st);
+    if (C == 16 && N == 32) return launch_wgrad<16, 32>(a, st);
+    if (C == 32 && N == 16) return launch_wgrad<32, 16>(a, st);
+    if (C == 32 && N == 32) return launch_wgrad<32, 32>(a, st);
+    return -1;
+}
+
+void wgrad_sums(WgradSums &t, cudaStream_t st) {
+    int blocks = 0;
+    for (int l = 0; l < t.layers; ++l) {
+        t.l[l].block0 = blocks;
+        blocks += (t.l[l].elems() + 31) / 32;
+    }
+    launch_pdl(k_wgrad_sum, blocks, 256, 0, st, t);
 }
 
 }  // namespace nn

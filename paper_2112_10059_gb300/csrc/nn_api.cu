@@ -43,13 +43,12 @@ struct sph_nn {
     bool poisoned = false;
     int64_t P = 0;
     size_t p_off[NLAYER] = {}, head_off = 0;
-    size_t img_f_off[NLAYER] = {}, img_d_off[NLAYER] = {}, dw_off[NLAYER] = {};
-    float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr, *dw = nullptr;
-    size_t dw_total = 0;
-    float *wpart = nullptr;      // [WGRAD_MAX_SPLIT][rows][N] partial weight gradients (fixed-order sums)
-    float *hpart = nullptr;      // [HEAD_MAX_BLOCKS][34] partial head gradients
+    size_t img_f_off[NLAYER] = {}, img_d_off[NLAYER] = {}, part_off[NLAYER] = {};
+    float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
+    float *wpart = nullptr;      // every layer's partial weight gradients (fixed-order sums)
+    float *hpart = nullptr;      // [HEAD_BLOCKS][34] partial head gradients
     uint16_t *img = nullptr;
-    double *loss = nullptr;
+    double *loss = nullptr;      // the loss, then its HEAD_BLOCKS partials
     int *errflag = nullptr;
     unsigned *maxbits = nullptr;
     float *scratch = nullptr;       // pooled fields for input preparation
@@ -57,10 +56,9 @@ struct sph_nn {
     int step = 0;
     // activations and gradients (BF16), capacity cap samples
     std::vector<void *> allocs;
-    uint16_t *a00, *s0, *p0, *a10, *s1, *p1, *a20, *s2, *p2, *a30, *b3, *u2, *d2, *u1, *d1, *u0, *d0, *v0, *f;
-    uint16_t *g_f, *g_v0, *g_d0, *g_u0, *g_d1, *g_u1, *g_d2, *g_u2, *g_b3, *g_a30, *g_p2, *g_s2, *g_a20, *g_p1,
-        *g_s1, *g_a10, *g_p0, *g_s0, *g_a00;
-    float *y = nullptr;
+    uint16_t *a00, *s0, *p0, *a10, *s1, *p1, *a20, *s2, *p2, *a30, *b3, *u2, *d2, *u1, *d1, *d0, *v0, *f;
+    uint16_t *g_f, *g_v0, *g_d0, *g_d1, *g_u1, *g_d2, *g_u2, *g_b3, *g_a30, *g_s2, *g_a20,
+        *g_s1, *g_a10, *g_s0, *g_a00;
 };
 
 namespace {
@@ -107,35 +105,83 @@ int lg_of(int edge) {
 
 size_t vox(const sph_nn *n, int batch, int lvl) { return (size_t)batch << (3 * (n->lg0 - lvl)); }
 
-int conv_layer(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out, const uint16_t *add, bool dgrad,
-               const uint16_t *mask) {
+// the plain arguments of a layer's convolution (forward, or its data gradient), and its launch
+ConvArgs layer_args(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out, bool dgrad) {
     const LayerSpec &S = LAYERS[L];
-    ConvArgs a;
+    ConvArgs a{};
     a.x = in;
     a.w = n->img + (dgrad ? n->img_d_off[L] : n->img_f_off[L]);
     a.bias = dgrad ? nullptr : n->params + n->p_off[L] + (size_t)S.co * NTAPS * S.ci;
-    a.add = add;
-    a.mask = mask;
     a.out = out;
     a.relu = dgrad ? 0 : 1;
     a.nvox = (int)vox(n, batch, S.lvl);
     a.lg = n->lg0 - S.lvl;
     a.err = n->errflag;
+    return a;
+}
+
+int run_layer(sph_nn *n, int L, const ConvArgs &a, bool dgrad) {
+    const LayerSpec &S = LAYERS[L];
     int r = dgrad ? conv(a, S.co, S.ci, n->stream) : conv(a, S.ci, S.co, n->stream);
     return r ? fail(n, SPH_EINTERNAL, "unsupported layer shape") : SPH_OK;
 }
 
-int wgrad_layer(sph_nn *n, int L, int batch, const uint16_t *x, const uint16_t *dz) {
+int conv_layer(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out) {
+    return run_layer(n, L, layer_args(n, L, batch, in, out, false), false);
+}
+// forward, and the mean over each 2^3 block into pooled
+int conv_pool(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out, uint16_t *pooled) {
+    ConvArgs a = layer_args(n, L, batch, in, out, false);
+    a.epi = CONV_POOL;
+    a.out2 = pooled;
+    a.scale = 0.125f;
+    return run_layer(n, L, a, false);
+}
+// forward, and its nearest up-sampling plus the finer level's skip into sum
+int conv_up(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out, const uint16_t *skip, uint16_t *sum) {
+    ConvArgs a = layer_args(n, L, batch, in, out, false);
+    a.epi = CONV_EXPAND;
+    a.add2 = skip;
+    a.out2 = sum;
+    return run_layer(n, L, a, false);
+}
+// data gradient, zero where mask <= 0
+int dgrad_mask(sph_nn *n, int L, int batch, const uint16_t *g, uint16_t *out, const uint16_t *mask) {
+    ConvArgs a = layer_args(n, L, batch, g, out, true);
+    a.mask = mask;
+    return run_layer(n, L, a, true);
+}
+// data gradient (kept in full where out is given) summed over each 2^3 block: the gradient through
+// the up-sampling, zero where mask <= 0
+int dgrad_up(sph_nn *n, int L, int batch, const uint16_t *g, uint16_t *out, uint16_t *coarse, const uint16_t *mask) {
+    ConvArgs a = layer_args(n, L, batch, g, out, true);
+    a.epi = CONV_POOL;
+    a.out2 = coarse;
+    a.mask2 = mask;
+    return run_layer(n, L, a, true);
+}
+// data gradient through the pooling: (skip gradient + 1/8 of it) at each child, zero where mask <= 0
+int dgrad_pool(sph_nn *n, int L, int batch, const uint16_t *g, const uint16_t *skip, uint16_t *fine, const uint16_t *mask) {
+    ConvArgs a = layer_args(n, L, batch, g, nullptr, true);
+    a.epi = CONV_EXPAND;
+    a.add2 = skip;
+    a.mask2 = mask;
+    a.out2 = fine;
+    return run_layer(n, L, a, true);
+}
+
+// the layer's partial weight gradients, and its entry in the sums that end the backward pass
+int wgrad_layer(sph_nn *n, WgradSums &sums, int L, int batch, const uint16_t *x, const uint16_t *dz, int up = 0) {
     const LayerSpec &S = LAYERS[L];
     WgradArgs a;
     a.x = x;
     a.dz = dz;
-    a.dw = n->dw + n->dw_off[L];
+    a.part = n->wpart + n->part_off[L];
     a.nvox = (int)vox(n, batch, S.lvl);
     a.lg = n->lg0 - S.lvl;
-    a.chunks_per_cta = 0;
     a.err = n->errflag;
-    a.part = n->wpart;
+    a.up = up;
+    sums.l[sums.layers++] = {a.part, n->grads + n->p_off[L], S.ci, S.co, wgrad_splits(S.ci, S.co, a.lg, a.nvox), 0};
     return wgrad(a, S.ci, S.co, n->stream) ? fail(n, SPH_EINTERNAL, "unsupported layer shape") : SPH_OK;
 }
 
@@ -147,78 +193,77 @@ int refresh_images(sph_nn *n) {
     return SPH_OK;
 }
 
-int forward_pass(sph_nn *n, int B, const uint16_t *x) {
-    const int lg0 = n->lg0;
+// y: the head's output (null: none); train: also keep what only the backward pass reads
+int forward_pass(sph_nn *n, int B, const uint16_t *x, float *y, bool train) {
     int r = SPH_OK;
 #define RUN(expr)            \
     do {                     \
         r = (expr);          \
         if (r) return r;     \
     } while (0)
-    RUN(conv_layer(n, C00, B, x, n->a00, nullptr, false, nullptr));
-    RUN(conv_layer(n, C01, B, n->a00, n->s0, nullptr, false, nullptr));
-    pool2(n->s0, n->p0, B, lg0 - 1, 16, n->stream);
-    RUN(conv_layer(n, C10, B, n->p0, n->a10, nullptr, false, nullptr));
-    RUN(conv_layer(n, C11, B, n->a10, n->s1, nullptr, false, nullptr));
-    pool2(n->s1, n->p1, B, lg0 - 2, 32, n->stream);
-    RUN(conv_layer(n, C20, B, n->p1, n->a20, nullptr, false, nullptr));
-    RUN(conv_layer(n, C21, B, n->a20, n->s2, nullptr, false, nullptr));
-    pool2(n->s2, n->p2, B, lg0 - 3, 32, n->stream);
-    RUN(conv_layer(n, C30, B, n->p2, n->a30, nullptr, false, nullptr));
-    RUN(conv_layer(n, C31, B, n->a30, n->b3, nullptr, false, nullptr));
-    up_add(n->b3, n->s2, n->u2, B, lg0 - 2, 32, n->stream);
-    RUN(conv_layer(n, C22, B, n->u2, n->d2, nullptr, false, nullptr));
-    up_add(n->d2, n->s1, n->u1, B, lg0 - 1, 32, n->stream);
-    RUN(conv_layer(n, C12, B, n->u1, n->d1, nullptr, false, nullptr));
-    up_add(n->d1, nullptr, n->u0, B, lg0, 32, n->stream);
-    RUN(conv_layer(n, C02, B, n->u0, n->d0, nullptr, false, nullptr));
-    add(n->d0, n->s0, n->v0, vox(n, B, 0) * 16, n->stream);
-    RUN(conv_layer(n, C03, B, n->v0, n->f, nullptr, false, nullptr));
+    RUN(conv_layer(n, C00, B, x, n->a00));
+    RUN(conv_pool(n, C01, B, n->a00, n->s0, n->p0));
+    RUN(conv_layer(n, C10, B, n->p0, n->a10));
+    RUN(conv_pool(n, C11, B, n->a10, n->s1, n->p1));
+    RUN(conv_layer(n, C20, B, n->p1, n->a20));
+    RUN(conv_pool(n, C21, B, n->a20, n->s2, n->p2));
+    RUN(conv_layer(n, C30, B, n->p2, n->a30));
+    RUN(conv_up(n, C31, B, n->a30, train ? n->b3 : nullptr, n->s2, n->u2));
+    RUN(conv_up(n, C22, B, n->u2, train ? n->d2 : nullptr, n->s1, n->u1));
+    RUN(conv_layer(n, C12, B, n->u1, n->d1));
+    ConvArgs a = layer_args(n, C02, B, n->d1, train ? n->d0 : nullptr, false);
+    a.up = 1;                                   // reads d1 up-sampled
+    a.epi = CONV_PAIR;
+    a.add2 = n->s0;
+    a.out2 = n->v0;
+    RUN(run_layer(n, C02, a, false));
+    a = layer_args(n, C03, B, n->v0, train ? n->f : nullptr, false);
+    if (y) {
+        a.epi = CONV_HEAD;
+        a.hw = n->params + n->head_off;
+        a.y = y;
+    }
+    RUN(run_layer(n, C03, a, false));
     return SPH_OK;
 }
 
 int backward_pass(sph_nn *n, int B, const uint16_t *x, const float *t) {
-    const int lg0 = n->lg0;
     cudaStream_t st = n->stream;
     int r = SPH_OK;
-    NCK(cudaMemsetAsync(n->dw, 0, n->dw_total * sizeof(float), st));
-    NCK(cudaMemsetAsync(n->grads + n->head_off, 0, HEAD_N * sizeof(float), st));
-    NCK(cudaMemsetAsync(n->loss, 0, sizeof(double), st));
-    const float *hw = n->params + n->head_off;
-    head_loss_backward(n->f, hw, hw + HEAD_W, t, n->g_f, n->grads + n->head_off, n->loss, (int)vox(n, B, 0),
-                       LOSS_LAMBDA, LOSS_EPS, st, n->hpart);
-    RUN(wgrad_layer(n, C03, B, n->v0, n->g_f));
-    RUN(conv_layer(n, C03, B, n->g_f, n->g_v0, nullptr, true, nullptr));
-    mask_mul(n->g_v0, n->d0, n->g_d0, vox(n, B, 0) * 16, st);
-    RUN(wgrad_layer(n, C02, B, n->u0, n->g_d0));
-    RUN(conv_layer(n, C02, B, n->g_d0, n->g_u0, nullptr, true, nullptr));
-    up_back_mask(n->g_u0, n->d1, n->g_d1, B, lg0 - 1, 32, st);
-    RUN(wgrad_layer(n, C12, B, n->u1, n->g_d1));
-    RUN(conv_layer(n, C12, B, n->g_d1, n->g_u1, nullptr, true, nullptr));
-    up_back_mask(n->g_u1, n->d2, n->g_d2, B, lg0 - 2, 32, st);
-    RUN(wgrad_layer(n, C22, B, n->u2, n->g_d2));
-    RUN(conv_layer(n, C22, B, n->g_d2, n->g_u2, nullptr, true, nullptr));
-    up_back_mask(n->g_u2, n->b3, n->g_b3, B, lg0 - 3, 32, st);
-    RUN(wgrad_layer(n, C31, B, n->a30, n->g_b3));
-    RUN(conv_layer(n, C31, B, n->g_b3, n->g_a30, nullptr, true, n->a30));
-    RUN(wgrad_layer(n, C30, B, n->p2, n->g_a30));
-    RUN(conv_layer(n, C30, B, n->g_a30, n->g_p2, nullptr, true, nullptr));
-    pool_back_add_mask(n->g_p2, n->g_u2, n->s2, n->g_s2, B, lg0 - 2, 32, st);
-    RUN(wgrad_layer(n, C21, B, n->a20, n->g_s2));
-    RUN(conv_layer(n, C21, B, n->g_s2, n->g_a20, nullptr, true, n->a20));
-    RUN(wgrad_layer(n, C20, B, n->p1, n->g_a20));
-    RUN(conv_layer(n, C20, B, n->g_a20, n->g_p1, nullptr, true, nullptr));
-    pool_back_add_mask(n->g_p1, n->g_u1, n->s1, n->g_s1, B, lg0 - 1, 32, st);
-    RUN(wgrad_layer(n, C11, B, n->a10, n->g_s1));
-    RUN(conv_layer(n, C11, B, n->g_s1, n->g_a10, nullptr, true, n->a10));
-    RUN(wgrad_layer(n, C10, B, n->p0, n->g_a10));
-    RUN(conv_layer(n, C10, B, n->g_a10, n->g_p0, nullptr, true, nullptr));
-    pool_back_add_mask(n->g_p0, n->g_v0, n->s0, n->g_s0, B, lg0, 16, st);
-    RUN(wgrad_layer(n, C01, B, n->a00, n->g_s0));
-    RUN(conv_layer(n, C01, B, n->g_s0, n->g_a00, nullptr, true, n->a00));
-    RUN(wgrad_layer(n, C00, B, x, n->g_a00));
-    for (int L = 0; L < NLAYER; ++L)
-        collect_grads(n->dw + n->dw_off[L], LAYERS[L].ci, LAYERS[L].co, n->grads + n->p_off[L], st);
+    WgradSums sums;
+    const int nb = head_loss_backward(n->f, n->params + n->head_off, t, n->g_f, n->hpart, n->loss + 1,
+                                      (int)vox(n, B, 0), LOSS_LAMBDA, LOSS_EPS, st);
+    sums.loss = n->loss;
+    sums.loss_part = n->loss + 1;
+    sums.l[sums.layers++] = {n->hpart, n->grads + n->head_off, 0, HEAD_N, nb, 0};
+    RUN(wgrad_layer(n, sums, C03, B, n->v0, n->g_f));
+    ConvArgs a = layer_args(n, C03, B, n->g_f, n->g_v0, true);
+    a.epi = CONV_PAIR;
+    a.mask2 = n->d0;
+    a.out2 = n->g_d0;
+    RUN(run_layer(n, C03, a, true));
+    RUN(wgrad_layer(n, sums, C02, B, n->d1, n->g_d0, 1));
+    RUN(dgrad_up(n, C02, B, n->g_d0, nullptr, n->g_d1, n->d1));
+    RUN(wgrad_layer(n, sums, C12, B, n->u1, n->g_d1));
+    RUN(dgrad_up(n, C12, B, n->g_d1, n->g_u1, n->g_d2, n->d2));
+    RUN(wgrad_layer(n, sums, C22, B, n->u2, n->g_d2));
+    RUN(dgrad_up(n, C22, B, n->g_d2, n->g_u2, n->g_b3, n->b3));
+    RUN(wgrad_layer(n, sums, C31, B, n->a30, n->g_b3));
+    RUN(dgrad_mask(n, C31, B, n->g_b3, n->g_a30, n->a30));
+    RUN(wgrad_layer(n, sums, C30, B, n->p2, n->g_a30));
+    RUN(dgrad_pool(n, C30, B, n->g_a30, n->g_u2, n->g_s2, n->s2));
+    RUN(wgrad_layer(n, sums, C21, B, n->a20, n->g_s2));
+    RUN(dgrad_mask(n, C21, B, n->g_s2, n->g_a20, n->a20));
+    RUN(wgrad_layer(n, sums, C20, B, n->p1, n->g_a20));
+    RUN(dgrad_pool(n, C20, B, n->g_a20, n->g_u1, n->g_s1, n->s1));
+    RUN(wgrad_layer(n, sums, C11, B, n->a10, n->g_s1));
+    RUN(dgrad_mask(n, C11, B, n->g_s1, n->g_a10, n->a10));
+    RUN(wgrad_layer(n, sums, C10, B, n->p0, n->g_a10));
+    RUN(dgrad_pool(n, C10, B, n->g_a10, n->g_v0, n->g_s0, n->s0));
+    RUN(wgrad_layer(n, sums, C01, B, n->a00, n->g_s0));
+    RUN(dgrad_mask(n, C01, B, n->g_s0, n->g_a00, n->a00));
+    RUN(wgrad_layer(n, sums, C00, B, x, n->g_a00));
+    wgrad_sums(sums, st);
     NCK(cudaGetLastError());
     return SPH_OK;
 #undef RUN
@@ -284,7 +329,7 @@ int sph_nn_create(sph_nn **out, int device, void *stream, int edge, int max_batc
     n->lg0 = lg;
     n->cap = max_batch;
     init_attributes();
-    size_t po = 0, io = 0, dwo = 0;
+    size_t po = 0, io = 0, wo = 0;
     for (int L = 0; L < NLAYER; ++L) {
         const LayerSpec &S = LAYERS[L];
         n->p_off[L] = po;
@@ -293,12 +338,11 @@ int sph_nn_create(sph_nn **out, int device, void *stream, int edge, int max_batc
         io += (size_t)conv_chunks(S.ci) * S.co * 64;
         n->img_d_off[L] = io;
         io += (size_t)conv_chunks(S.co) * S.ci * 64;
-        n->dw_off[L] = dwo;
-        dwo += (size_t)wgrad_rows(S.ci) * S.co;
+        n->part_off[L] = wo;   // a smaller batch has no more slices
+        wo += (size_t)wgrad_splits(S.ci, S.co, lg - S.lvl, (int)vox(n, max_batch, S.lvl)) * (NTAPS * S.ci + 1) * S.co;
     }
     n->head_off = po;
     n->P = (int64_t)po + HEAD_N;
-    n->dw_total = dwo;
     int r = SPH_OK;
     auto A = [&](auto *&p, size_t cnt) {
         if (!r) r = alloc(n, p, cnt);
@@ -307,11 +351,10 @@ int sph_nn_create(sph_nn **out, int device, void *stream, int edge, int max_batc
     A(n->grads, n->P);
     A(n->m, n->P);
     A(n->v, n->P);
-    A(n->dw, dwo);
-    A(n->wpart, (size_t)WGRAD_MAX_SPLIT * wgrad_rows(32) * 32);
-    A(n->hpart, (size_t)HEAD_MAX_BLOCKS * 34);
+    A(n->wpart, wo);
+    A(n->hpart, (size_t)HEAD_BLOCKS * 34);
     A(n->img, io);
-    A(n->loss, 1);
+    A(n->loss, 1 + HEAD_BLOCKS);
     A(n->errflag, 1);
     A(n->maxbits, 4);
     const int B = max_batch;
@@ -319,11 +362,11 @@ int sph_nn_create(sph_nn **out, int device, void *stream, int edge, int max_batc
     A(n->a00, V0 * 16); A(n->s0, V0 * 16); A(n->p0, V1 * 16); A(n->a10, V1 * 32); A(n->s1, V1 * 32);
     A(n->p1, V2 * 32); A(n->a20, V2 * 32); A(n->s2, V2 * 32); A(n->p2, V3 * 32); A(n->a30, V3 * 32);
     A(n->b3, V3 * 32); A(n->u2, V2 * 32); A(n->d2, V2 * 32); A(n->u1, V1 * 32); A(n->d1, V1 * 32);
-    A(n->u0, V0 * 32); A(n->d0, V0 * 16); A(n->v0, V0 * 16); A(n->f, V0 * 16);
-    A(n->g_f, V0 * 16); A(n->g_v0, V0 * 16); A(n->g_d0, V0 * 16); A(n->g_u0, V0 * 32); A(n->g_d1, V1 * 32);
+    A(n->d0, V0 * 16); A(n->v0, V0 * 16); A(n->f, V0 * 16);
+    A(n->g_f, V0 * 16); A(n->g_v0, V0 * 16); A(n->g_d0, V0 * 16); A(n->g_d1, V1 * 32);
     A(n->g_u1, V1 * 32); A(n->g_d2, V2 * 32); A(n->g_u2, V2 * 32); A(n->g_b3, V3 * 32); A(n->g_a30, V3 * 32);
-    A(n->g_p2, V3 * 32); A(n->g_s2, V2 * 32); A(n->g_a20, V2 * 32); A(n->g_p1, V2 * 32); A(n->g_s1, V1 * 32);
-    A(n->g_a10, V1 * 32); A(n->g_p0, V1 * 16); A(n->g_s0, V0 * 16); A(n->g_a00, V0 * 16);
+    A(n->g_s2, V2 * 32); A(n->g_a20, V2 * 32); A(n->g_s1, V1 * 32);
+    A(n->g_a10, V1 * 32); A(n->g_s0, V0 * 16); A(n->g_a00, V0 * 16);
     if (!r) {
         n->scratch_n = 3 * (size_t)edge * edge * edge;
         A(n->scratch, n->scratch_n);
@@ -398,10 +441,8 @@ int sph_nn_forward(sph_nn *n, int B, const uint16_t *x, float *y) {
     if (!n || !x || !y || B < 1 || B > n->cap) return fail(n, SPH_EINVAL, "bad forward arguments");
     if (n->poisoned) return SPH_ECUDA;
     NCK(cudaSetDevice(n->device));
-    int r = forward_pass(n, B, x);
+    int r = forward_pass(n, B, x, y, false);
     if (r) return r;
-    const float *hw = n->params + n->head_off;
-    head_forward(n->f, hw, hw + HEAD_W, y, (int)vox(n, B, 0), n->stream);
     NCK(cudaGetLastError());
     return SPH_OK;
 }
@@ -410,7 +451,7 @@ int sph_nn_backward(sph_nn *n, int B, const uint16_t *x, const float *t, double 
     if (!n || !x || !t || B < 1 || B > n->cap) return fail(n, SPH_EINVAL, "bad backward arguments");
     if (n->poisoned) return SPH_ECUDA;
     NCK(cudaSetDevice(n->device));
-    int r = forward_pass(n, B, x);
+    int r = forward_pass(n, B, x, nullptr, true);
     if (!r) r = backward_pass(n, B, x, t);
     if (r) return r;
     if (loss_host) {
@@ -526,30 +567,31 @@ int sph_nn_conv3d_wgrad(int device, void *stream, int C, int N, int edge, int ba
     if (cudaSetDevice(device) != cudaSuccess) return SPH_ECUDA;
     init_attributes();
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    float *dw = nullptr;
+    const int nvox = batch << (3 * lg), splits = wgrad_splits(C, N, lg, nvox);
+    float *part = nullptr;
     int *err = nullptr;
-    const size_t rows = wgrad_rows(C);
-    if (cudaMalloc(&dw, rows * N * sizeof(float)) != cudaSuccess || cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&part, (size_t)splits * (NTAPS * C + 1) * N * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(dw);
+        cudaFree(part);
         return SPH_ENOMEM;
     }
-    cudaMemsetAsync(dw, 0, rows * N * sizeof(float), st);
     cudaMemsetAsync(err, 0, sizeof(int), st);
     WgradArgs a;
     a.x = x;
     a.dz = dz;
-    a.dw = dw;
-    a.nvox = batch << (3 * lg);
+    a.part = part;
+    a.nvox = nvox;
     a.lg = lg;
-    a.chunks_per_cta = 0;
     a.err = err;
     int r = wgrad(a, C, N, st);
-    collect_grads(dw, C, N, dwout, st);
+    WgradSums sums;
+    sums.l[sums.layers++] = {part, dwout, C, N, splits, 0};
+    wgrad_sums(sums, st);
     int e = 0;
     cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st);
     cudaError_t ce = cudaStreamSynchronize(st);
-    cudaFree(dw);
+    cudaFree(part);
     cudaFree(err);
     if (ce != cudaSuccess || cudaGetLastError() != cudaSuccess) return SPH_ECUDA;
     if (r) return SPH_EINTERNAL;

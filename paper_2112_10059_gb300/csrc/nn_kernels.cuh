@@ -20,9 +20,16 @@ namespace nn {
 constexpr int NTAPS = 27;
 // K chunks of 64 elements for C channels per tap (taps padded to 28 with zeros)
 __host__ __device__ constexpr int conv_chunks(int C) { return (NTAPS + 64 / C - 1) / (64 / C); }
-// rows of the weight-gradient accumulator [rows][N]: taps x C padded to whole 128-row tiles;
-// row 27 * C accumulates the bias gradient
-__host__ __device__ constexpr int wgrad_rows(int C) { return ((28 * C + 127) / 128) * 128; }
+// Epilogues of a convolution beside the plain one (bias, ReLU, residual, mask), each in place of
+// a pass over memory; all use the convolution's result as rounded to BF16.
+enum {
+    CONV_PLAIN = 0,
+    CONV_POOL,     // out2[parent] = scale * (sum of the 8 children), 0 where mask2 <= 0 (mask2 given); out optional
+    CONV_PAIR,     // out2 = out + add2 (add2 given), or out where mask2 > 0 and 0 elsewhere; out optional
+    CONV_EXPAND,   // out2[child] = out + add2[child], or (mask2 given) mask2[child] > 0 ? add2[child] + out / 8 : 0;
+                   // out optional
+    CONV_HEAD      // y = head weights . out + head bias (FP32); out optional
+};
 
 struct ConvArgs {
     const uint16_t *x;       // [nvox][C]
@@ -35,53 +42,56 @@ struct ConvArgs {
     int nvox, lg;
     int *err;                // bit 0: a bounded wait expired
     int up = 0;              // 1: x holds the grid of half the edge, read at each voxel's parent
+    int epi = CONV_PLAIN;
+    const uint16_t *add2 = nullptr, *mask2 = nullptr;
+    uint16_t *out2 = nullptr;
+    float scale = 1.f;
+    const float *hw = nullptr;   // [34] head weights and bias
+    float *y = nullptr;      // [nvox][2]
 };
 
 struct WgradArgs {
     const uint16_t *x;       // [nvox][C] layer input
     const uint16_t *dz;      // [nvox][N] gradient w.r.t. the layer's pre-activation
-    float *dw;               // [wgrad_rows(C)][N]: added into (reductions, or the fixed-order sum below)
+    float *part;             // [wgrad_splits][27 C + 1][N]: each CTA's sums, row 27 C the bias gradient's
     int nvox, lg;
-    int chunks_per_cta;      // chunks of 64 voxels per CTA
     int *err;
-    // optional [WGRAD_MAX_SPLIT][wgrad_rows(C)][N] scratch: each CTA stores its partial sum there
-    // and a second kernel adds the partials into dw in a fixed order (training is then
-    // reproducible bit for bit); nullptr: the CTAs add into dw with reductions
-    float *part = nullptr;
+    int up = 0;              // 1: x holds the grid of half the edge, read at each voxel's parent
 };
-constexpr int WGRAD_MAX_SPLIT = 160;   // voxel splits of one weight gradient (grid.y) at most
-constexpr int HEAD_MAX_BLOCKS = 8192;  // blocks of the head's loss / gradient kernel with partials
+// slices that one weight gradient writes (its CTAs)
+int wgrad_splits(int C, int N, int lg, int nvox);
+
+// Sums over the slices of several layers, each written as w [N][27][C] then b [N]; a layer with
+// C = 0 is the head (N = 34 elements as they are, and the loss).
+struct WgradSum {
+    const float *part;
+    float *grad;
+    int C, N, splits, block0;
+    __host__ __device__ int elems() const { return (NTAPS * C + 1) * N; }
+};
+struct WgradSums {
+    WgradSum l[13];
+    int layers = 0;
+    const double *loss_part = nullptr;
+    double *loss = nullptr;
+};
+void wgrad_sums(WgradSums &t, cudaStream_t st);
+constexpr int HEAD_BLOCKS = 608;       // blocks of the head's loss / gradient kernel at most
 
 // set the shared-memory limits of every instantiation (call once, outside graph capture)
 void init_attributes();
-void init_conv();   // the part of it in k_conv.cu
 // C, N in {16, 32}; returns 0, or -1 for an unsupported shape
 int conv(const ConvArgs &a, int C, int N, cudaStream_t st);
 int wgrad(const WgradArgs &a, int C, int N, cudaStream_t st);
 
-// element-wise and resampling (BF16 tensors, C a multiple of 8)
-void pool2(const uint16_t *in, uint16_t *out, int B, int lg_out, int C, cudaStream_t st);
-void up_add(const uint16_t *coarse, const uint16_t *skip, uint16_t *out, int B, int lg_out, int C,
-            cudaStream_t st);
-void add(const uint16_t *a, const uint16_t *b, uint16_t *out, size_t n, cudaStream_t st);
-void mask_mul(const uint16_t *g, const uint16_t *mask, uint16_t *out, size_t n, cudaStream_t st);
-void up_back_mask(const uint16_t *g_fine, const uint16_t *mask, uint16_t *out, int B, int lg_out, int C,
-                  cudaStream_t st);
-void pool_back_add_mask(const uint16_t *g_coarse, const uint16_t *add, const uint16_t *mask, uint16_t *out, int B,
-                        int lg_out, int C, cudaStream_t st);
-
-// head: y[m][j] = sum_c hw[j][c] f[m][c] + hb[j], j in {0, 1}; f has 16 channels
-void head_forward(const uint16_t *f, const float *hw, const float *hb, float *y, int nvox, cudaStream_t st);
-// loss of the residual r = y0 against t and of the error head e = y1 against log(|r - t| + eps);
-// writes the masked gradient of f (BF16), accumulates the head's gradient hg[34] and the loss sum
-// hpart (optional, [HEAD_MAX_BLOCKS][34] scratch, nvox <= 256 HEAD_MAX_BLOCKS): per-block partials of the
-// head gradient summed in a fixed order instead of reductions
-void head_loss_backward(const uint16_t *f, const float *hw, const float *hb, const float *t, uint16_t *g_f,
-                        float *hg, double *loss_sum, int nvox, float lambda, float eps, cudaStream_t st,
-                        float *hpart = nullptr);
+// loss of the residual r = y0 against t and of the error head e = y1 against log(|r - t| + eps)
+// (y[m][j] = sum_c hw[j][c] f[m][c] + hb[j]); writes the masked gradient of f (BF16) and each
+// block's part of the head's gradient (part [blocks][34]) and of the loss (loss_part [blocks]);
+// returns the number of blocks
+int head_loss_backward(const uint16_t *f, const float *hw, const float *t, uint16_t *g_f, float *part, double *loss_part,
+                       int nvox, float lambda, float eps, cudaStream_t st);
 
 // parameters: per layer w [N][27][C] then b [N] (FP32 master copy)
-void collect_grads(const float *dw, int C, int N, float *g, cudaStream_t st);
 void adam(float *p, const float *g, float *m, float *v, size_t n, float lr, float b1, float b2, float eps,
           float bc1, float bc2, cudaStream_t st);
 void make_images(const float *w, int C, int N, uint16_t *img_fwd, uint16_t *img_dgrad, cudaStream_t st);

@@ -1,11 +1,10 @@
 // Eight BF16 values (one 16-byte unit of a channels-last tensor) to and from FP32.
 #pragma once
-#include "tc_sm103.cuh"
+#include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace sph {
 namespace nn {
-
-using tc::f2bf;
 
 __device__ __forceinline__ void unpack8(const uint4 &q, float *f) {
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
@@ -18,7 +17,8 @@ __device__ __forceinline__ void unpack8(const uint4 &q, float *f) {
 __device__ __forceinline__ uint4 pack8(const float *f) {
     uint32_t w[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = (uint32_t)f2bf(f[2 * i]) | ((uint32_t)f2bf(f[2 * i + 1]) << 16);
+    for (int i = 0; i < 4; ++i)   // round to nearest even, the second operand in the low half
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[i]) : "f"(f[2 * i + 1]), "f"(f[2 * i]));
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 

@@ -108,6 +108,13 @@ __device__ __forceinline__ void mbar_init(uint32_t saddr, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t saddr, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr), "r"(bytes) : "memory");
 }
+// barrier `id` (1 .. 15) among `threads` threads of the CTA (whole warps)
+__device__ __forceinline__ void named_sync(uint32_t id, uint32_t threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t saddr) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr) : "memory");
+}
 __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t saddr, uint32_t parity) {
     uint32_t ok;
     asm volatile(
