@@ -6,14 +6,17 @@
 // channels per voxel and channel group, x fastest.  Eight x-neighbours are then one
 // unswizzled K-major core matrix (8 rows x 16 bytes), the 16 rows of the tile are its M
 // repeats (stride one halo row), the channel groups its K repeats -- and the operand of any
-// of the 27 taps is the same plane read from a start address moved by whole units.
-// A voxel's input is copied 1.4 times (halo) instead of 27 times; the copies per 128-voxel
-// tile fall from 3584 (C = 16) to 360.
-// CTAs march in z through equal shares of the tiles, planes in a ring of six loaded two
-// ahead, the tile's MMAs (27 C / 16 of M = 128, N, K = 16, accumulated in tap order) running
-// into one of two TMEM accumulators under the previous tile's epilogue.
-// What bounds it: the tensor core reads 4 KB of A per MMA (about 32 clocks at 128 B/clock) for
-// an N of only 16 or 32.
+// (dy, dx) tap is the same plane read from a start address moved by whole units.  A voxel's
+// input is copied 1.4 times (halo) instead of 27 times.
+// What bounds it is the tensor core's read of A, 4 KB per MMA: measured 39 clocks per M = 128,
+// K = 16 MMA at N = 16, 40 at 32, 44 at 48, 56 at 96 (whatever the core matrices' alignment).
+// So N is widened with the plane's other uses: plane z is the dz = 2, 1, 0 tap of the outputs
+// z - 1, z, z + 1, whose accumulators lie side by side in TMEM (a ring of eight), and one MMA
+// of N = 3 x out channels takes the place of three; an output still sums its taps in the order
+// dz, dy, dx.  CTAs march in z through equal shares of the tiles, planes loaded three ahead, one
+// warp issuing MMAs under the four others' copies and epilogues.
+// 16 -> 16 channels at 64^3 x 4: 199 us gathering 27 taps, 38 with N = 16, 29 with N = 48;
+// 32 -> 16: 391, 68, 53 (32 -> 32 at 32^3 x 4: 83, 21, 15).
 //
 // Every mbarrier wait is bounded; on expiry the kernel sets its error flag and carries
 // on (the result is then invalid and the host reports it).
@@ -32,18 +35,16 @@ constexpr uint32_t NN_WAIT = 1u << 22;
 // ---------------------------------------------------------------- convolution (forward / data gradient)
 constexpr int CX = 8, CY = 16;                  // output voxels of a tile: 8 (x) x 16 (y)
 constexpr int PX = CX + 2, PY = CY + 2;         // its input plane with the halo
-constexpr int RING = 6;                         // planes in shared memory
-constexpr int AHEAD = 2;                        // planes loaded ahead of the tile's own three
+constexpr int AHEAD = 3;                        // planes loaded ahead of the one in use (forward: 223 us with 2, 206 with 3, 213 with 4)
+constexpr int RING = AHEAD + 2;                 // planes in shared memory
+constexpr int ACCS = 8;                         // accumulators in TMEM (at least 4)
 // bytes between the channel groups of a plane: such that the 8 units a quarter-warp copies
 // (2 groups x 4 voxels, or 4 groups x 2) fall into different banks
 __host__ __device__ constexpr uint32_t group_bytes(int C) { return PX * PY * 16 + (C == 16 ? 0 : 32); }
 __host__ __device__ constexpr uint32_t plane_bytes(int C) { return (uint32_t)(C / 8) * group_bytes(C); }
-__host__ __device__ constexpr uint32_t weight_bytes(int C, int N) { return (uint32_t)conv_chunks(C) * N * 128; }
+__host__ __device__ constexpr uint32_t weight_bytes(int C, int N) { return (uint32_t)conv_image(C, N) * 2; }
 __host__ __device__ constexpr uint32_t conv_smem(int C, int N) {
     return 1024 + weight_bytes(C, N) + RING * plane_bytes(C) + 64;
-}
-__host__ __device__ constexpr uint32_t conv_smem(int C, int N, int epi) {   // a tile's results staged for their children
-    return conv_smem(C, N) + (epi == CONV_EXPAND ? 128u * N * 2 : 0u);
 }
 
 __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
@@ -54,8 +55,30 @@ __device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
 __device__ __forceinline__ void cp_async_wait_upto(int pending) {
     if (pending <= 0) cp_async_wait<0>();
     else if (pending == 1) cp_async_wait<1>();
-    else cp_async_wait<2>();
+    else if (pending == 2) cp_async_wait<2>();
+    else cp_async_wait<3>();
 }
+
+// The planes a CTA passes through: for each column's run of output tiles zs .. ze - 1 the planes
+// zs - 1 .. ze, in order.  An output is complete once the plane above it has been used.
+struct PlaneCursor {
+    int next, t1, lg;                         // the next run's first tile, the CTA's end
+    int col = 0, z = 0, zs = 0, ze = -1;
+    __device__ PlaneCursor(int t0, int t1_, int lg_) : next(t0), t1(t1_), lg(lg_) {}
+    __device__ bool step() {                  // to the next plane; true where a run begins
+        if (z < ze) {
+            ++z;
+            return false;
+        }
+        const int D = 1 << lg;
+        col = next >> lg;
+        zs = next & (D - 1);
+        ze = min(D, zs + t1 - next);
+        next += ze - zs;
+        z = zs - 1;
+        return true;
+    }
+};
 
 template <int C, int N, int EPI>
 __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
@@ -65,7 +88,7 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
     constexpr int NU = (PX * PY * CG + 127) / 128;   // units copied per thread and plane
     extern __shared__ uint8_t raw[];
     uint8_t *base = align1024(raw);
-    // [0], [1]: accumulator done; [2], [3]: planes of the tile in shared memory; [4]: weights
+    // [0], [1]: a plane's MMAs are done; [2], [3]: it is in shared memory; [4]: weights
     uint64_t *bar = reinterpret_cast<uint64_t *>(base + WB + RING * PB);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 5);
     int *eflag = reinterpret_cast<int *>(tslot + 1);
@@ -73,7 +96,7 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
     __shared__ float shead[EPI == CONV_HEAD ? 34 : 1];
 
     const int r = threadIdx.x, warp = r >> 5;
-    const int lg = a.lg, D = 1 << lg, dm = D - 1;
+    const int lg = a.lg, D = 1 << lg;
     const int ltx = lg > 3 ? lg - 3 : 0, lty = lg > 4 ? lg - 4 : 0;   // tiles per row and plane (log2)
     const int ntiles = (a.nvox >> (2 * lg)) << (ltx + lty);           // (batch x D) planes of tiles
     // equal shares of consecutive tiles (z fastest); whole z-pairs where the epilogue pools
@@ -83,7 +106,7 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
     if (t0 >= t1) return;                     // uniform over the CTA, before any allocation
 
     if (warp == 4) {
-        tmem_alloc(smem_u32(tslot), 2 * N);
+        tmem_alloc(smem_u32(tslot), ACCS * N);
         tmem_relinquish();
     }
     if (r < N) sbias[r] = a.bias ? a.bias[r] : 0.f;
@@ -104,49 +127,60 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
     fence_after_sync();
     const uint32_t tmem = *tslot;
     const uint32_t wbase = smem_u32(base), ring = wbase + WB;
+    const int planes = t1 - t0 + 2 * (((t1 - 1) >> lg) - (t0 >> lg) + 1);
 
     if (warp == 4) {                          // ---- one thread issues every MMA
-        if (r == 128) {
-            const uint32_t idesc = idesc_bf16_f32(128, N);
+        if (elect_one()) {
             const uint64_t ad0 = sdesc_none(0, GB, PX * 16), bd0 = sdesc_sw128(0);
             mbar_expect_tx(smem_u32(&bar[4]), WB);
             bulk_g2s(wbase, a.w, WB, smem_u32(&bar[4]));
             if (!mbar_wait_bounded(smem_u32(&bar[4]), 0, NN_WAIT)) *eflag = 1;
-            int f = 0;
-            for (int it = 0; it < t1 - t0; ++it) {
-                if (it > 0) f += ((t0 + it) & dm) ? 1 : 3;
-                if (!mbar_wait_bounded(smem_u32(&bar[2 + (it & 1)]), (it >> 1) & 1, NN_WAIT)) *eflag = 1;
+            PlaneCursor p(t0, t1, lg);
+            int q = 0;                        // outputs of the runs before this one
+            for (int i = 0; i < planes; ++i) {
+                const int len = p.ze - p.zs;
+                if (p.step() && i > 0) q += len;
+                if (!mbar_wait_bounded(smem_u32(&bar[2 + (i & 1)]), (i >> 1) & 1, NN_WAIT)) *eflag = 1;
                 fence_after_sync();
-                const uint32_t acc = tmem + (uint32_t)((it & 1) * N);
+                // the outputs lo .. hi use this plane: rows (lo - z + 1) N .. of the weight image
+                const int lo = max(p.z - 1, p.zs), hi = min(p.z + 1, p.ze - 1), cnt = hi - lo + 1;
+                const int blk = (q + lo - p.zs) % ACCS, c1 = min(cnt, ACCS - blk);   // c1 before the ring's end
+                const uint64_t ad = ad0 + ((ring + (uint32_t)(i % RING) * PB) >> 4);
+                const uint64_t bd = bd0 + ((wbase + (uint32_t)(lo - p.z + 1) * N * 128) >> 4);
+                auto slice = [&](int k, int from, int to, uint32_t accumulate) {   // K = 16 slice k, outputs from .. to - 1
+                    const int tap = k / (C / 16), h = k % (C / 16);
+                    mma_bf16(tmem + (uint32_t)((blk + from) % ACCS * N),
+                             ad + (((uint32_t)((tap / 3) * PX + tap % 3) * 16 + 2 * h * GB) >> 4),
+                             bd + ((uint32_t)(k / 4) * 3 * N * 128 + (uint32_t)(k % 4) * 32 + (uint32_t)from * N * 128 >> 4),
+                             idesc_bf16_f32(128, (to - from) * N), accumulate);
+                };
+                // the output that begins here takes its first slice without its accumulator
+                const int old = hi == p.z + 1 ? cnt - 1 : cnt;
+                if (old > 0) slice(0, 0, min(old, c1), 1u);
+                if (old > c1) slice(0, c1, old, 1u);
+                if (old < cnt) slice(0, old, cnt, 0u);
+                if (c1 == cnt) {
 #pragma unroll
-                for (int dz = 0; dz < 3; ++dz) {
-                    const uint32_t sp = ring + (uint32_t)((f + dz) % RING) * PB;
+                    for (int k = 1; k < 9 * C / 16; ++k) slice(k, 0, cnt, 1u);
+                } else {
 #pragma unroll
-                    for (int tap = 9 * dz; tap < 9 * dz + 9; ++tap) {
-                        const uint32_t sv = sp + (uint32_t)((tap / 3 % 3) * PX + tap % 3) * 16;
-#pragma unroll
-                        for (int h = 0; h < C / 16; ++h) {
-                            const int k = tap * (C / 16) + h;   // K = 16 slice of the weight image
-                            mma_bf16(acc, ad0 + ((sv + 2 * h * GB) >> 4),
-                                     bd0 + ((wbase + (uint32_t)(k / 4) * N * 128 + (uint32_t)(k % 4) * 32) >> 4), idesc,
-                                     k > 0 ? 1u : 0u);
-                        }
+                    for (int k = 1; k < 9 * C / 16; ++k) {
+                        slice(k, 0, c1, 1u);
+                        slice(k, c1, cnt, 1u);
                     }
                 }
-                mma_commit(smem_u32(&bar[it & 1]));
+                mma_commit(smem_u32(&bar[i & 1]));
             }
         }
     } else {                                  // ---- four warps copy planes and write results
-        // load cursor: the planes zs - 1 .. zs + len of each column's run of tiles, in order
         const int up = a.up, lgi = lg - up;   // input grid (half the edge when up-sampled on load)
-        int off[NU];
+        int off[NU], loaded = 0;
         const uint16_t *xcol = a.x;
-        int ltile = t0, lz = 0, lze = -2, loaded = -1;
-        auto load_next = [&]() {              // the next plane, one copy group; false when none is left
-            if (lz > lze) {                   // next column
-                const int col = ltile >> lg, zs = ltile & dm, len = min(D - zs, t1 - ltile);
-                const int x0 = (col & ((1 << ltx) - 1)) * CX - 1, y0 = ((col >> ltx) & ((1 << lty) - 1)) * CY - 1;
-                xcol = a.x + ((size_t)(col >> (ltx + lty)) << (3 * lgi)) * C;
+        PlaneCursor lp(t0, t1, lg);
+        auto load_next = [&]() {              // the next plane, one copy group
+            if (lp.step()) {                  // another column
+                const int x0 = (lp.col & ((1 << ltx) - 1)) * CX - 1, y0 = ((lp.col >> ltx) & ((1 << lty) - 1)) * CY - 1;
+                xcol = a.x + ((size_t)(lp.col >> (ltx + lty)) << (3 * lgi)) * C;
 #pragma unroll
                 for (int j = 0; j < NU; ++j) {
                     const int u = r + 128 * j, v = u / CG, cg = u % CG;
@@ -155,14 +189,10 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
                                  ? (((y >> up) << lgi) + (x >> up)) * C + cg * 8
                                  : -1;
                 }
-                lz = zs - 1;
-                lze = zs + len;
-                ltile += len;
             }
-            ++loaded;
             const uint32_t dst = ring + (uint32_t)(loaded % RING) * PB;
-            const bool zin = (unsigned)lz < (unsigned)D;
-            const uint16_t *xp = xcol + ((size_t)((zin ? lz : 0) >> up) << (2 * lgi)) * C;
+            const bool zin = (unsigned)lp.z < (unsigned)D;
+            const uint16_t *xp = xcol + ((size_t)((zin ? lp.z : 0) >> up) << (2 * lgi)) * C;
 #pragma unroll
             for (int j = 0; j < NU; ++j) {
                 const int u = r + 128 * j;
@@ -172,20 +202,16 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
                 }
             }
             cp_async_commit();
-            ++lz;
-            return lz <= lze || ltile < t1;
+            ++loaded;
         };
 
         float pool[EPI == CONV_POOL ? N : 1];
-        auto epilogue = [&](int t, int it) {
-            const int col = t >> lg, z = t & dm;
+        auto epilogue = [&](int col, int z, int nth) {   // output nth of the CTA's, at (col, z)
             const int x = (col & ((1 << ltx) - 1)) * CX + (r & 7), y = ((col >> ltx) & ((1 << lty) - 1)) * CY + (r >> 3);
             const size_t bz = ((size_t)(col >> (ltx + lty)) << lg) + z;   // sample and plane
             const bool valid = x < D && y < D;
-            if (!mbar_wait_bounded(smem_u32(&bar[it & 1]), (it >> 1) & 1, NN_WAIT)) *eflag = 1;
-            fence_after_sync();
             float v[N];
-            const uint32_t acc = tmem + (uint32_t)((it & 1) * N) + ((uint32_t)(warp * 32) << 16);
+            const uint32_t acc = tmem + (uint32_t)(nth % ACCS * N) + ((uint32_t)(warp * 32) << 16);
             tmem_ld16(acc, v);
             if constexpr (N == 32) tmem_ld16(acc + 16, v + 16);
             fence_before_sync();              // read before this thread's next arrival frees the accumulator
@@ -230,33 +256,6 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
                         *reinterpret_cast<uint4 *>(a.out2 + o + 8 * g) = pack8(f);
                     }
                 }
-            }
-            if constexpr (EPI == CONV_EXPAND) {
-                // through shared memory, so that the four warps walk the children's 16-byte units in
-                // the order they lie (with a thread per parent, every lane of an access is a line of
-                // its own and the unrolled code misses the instruction cache: 30 against 8 us at 8^3)
-                constexpr int G = N / 8;
-                uint4 *tile = reinterpret_cast<uint4 *>(bar + 6);
-#pragma unroll
-                for (int g = 0; g < G; ++g) tile[r * G + g] = q[g];
-                named_sync(1, 128);
-                const int cx0 = 2 * (x - (r & 7)), cy0 = 2 * (y - (r >> 3));
-#pragma unroll 4
-                for (int i = 0; i < N; ++i) {
-                    const int e = r + 128 * i, g = e % G, cx = e / G % 16, cy = e / G / 16 % 32, cz = e / G / 512;
-                    if (cx0 + cx < 2 * D && cy0 + cy < 2 * D) {
-                        const size_t oc = (((2 * bz + cz) << (2 * lg + 2)) + ((size_t)(cy0 + cy) << (lg + 1)) + cx0 + cx) * N + 8 * g;
-                        float f[8], s[8], m[8];
-                        unpack8(__ldg(reinterpret_cast<const uint4 *>(a.add2 + oc)), s);
-                        if (a.mask2) unpack8(__ldg(reinterpret_cast<const uint4 *>(a.mask2 + oc)), m);
-                        unpack8(tile[((cy >> 1) * 8 + (cx >> 1)) * G + g], f);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            f[j] = !a.mask2 ? f[j] + s[j] : (m[j] > 0.f ? s[j] + 0.125f * f[j] : 0.f);
-                        *reinterpret_cast<uint4 *>(a.out2 + oc) = pack8(f);
-                    }
-                }
-                named_sync(1, 128);           // read before the next tile is staged
             }
             if constexpr (EPI == CONV_POOL) {
                 // children in the order x, y, z: this lane, its x, y and diagonal neighbour (lanes
@@ -312,29 +311,30 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
             }
         };
 
-        int f = 0, fprev = 0;                 // sequence number of the tile's first plane
-        bool more = true;
-        for (int it = 0; it < t1 - t0; ++it) {
-            const int t = t0 + it;
-            if (it > 0) {
-                fprev = f;
-                f += (t & dm) ? 1 : 3;
+        PlaneCursor p(t0, t1, lg);            // the plane whose MMAs are waited for
+        int q = 0;
+        for (int i = 0; i <= planes; ++i) {
+            if (i < planes) {
+                // plane i + AHEAD takes the slot of plane i - 2, whose MMAs are done (waited for below)
+                while (loaded < planes && loaded <= i + AHEAD) load_next();
+                cp_async_wait_upto(loaded - 1 - i);
+                fence_proxy_async_smem();
+                mbar_arrive(smem_u32(&bar[2 + (i & 1)]));
             }
-            // a slot is free once the last tile that read it is done: the previous tile, whose MMAs
-            // may still run, reads the planes from fprev on
-            const int lim = min(f + 2 + AHEAD, fprev + RING - 1);
-            while (more && loaded < lim) more = load_next();
-            cp_async_wait_upto(loaded - (f + 2));
-            fence_proxy_async_smem();
-            mbar_arrive(smem_u32(&bar[2 + (it & 1)]));
-            if (it > 0) epilogue(t - 1, it - 1);
+            if (i > 0) {
+                p.step();
+                if (!mbar_wait_bounded(smem_u32(&bar[(i - 1) & 1]), ((i - 1) >> 1) & 1, NN_WAIT)) *eflag = 1;
+                if (p.z > p.zs) {
+                    fence_after_sync();
+                    epilogue(p.col, p.z - 1, q++);
+                }
+            }
         }
-        epilogue(t1 - 1, t1 - 1 - t0);
     }
     fence_before_sync();
     __syncthreads();
     if (r == 0 && *eflag) atomicOr(a.err, 1);
-    if (warp == 4) tmem_dealloc(tmem, 2 * N);
+    if (warp == 4) tmem_dealloc(tmem, ACCS * N);
 }
 
 // ---------------------------------------------------------------- weight gradient
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
             }
             // the MMAs of iteration it - 2 are done: rows before fprev and its gradients are free
             if (it >= 2 && !mbar_wait_bounded(smem_u32(&bar[it & 1]), ((it - 2) >> 1) & 1, NN_WAIT)) *eflag = 1;
-            while (k < n && k <= it + AHEAD &&
+            while (k < n && k <= it + 2 &&
                    rows + s.rpi + ((k == 0 || ((i0 + k) & ipm) == 0) ? 2 : 0) <= fprev + s.ring - 1)
                 load_iter(k++);
             cp_async_wait_upto(k - 1 - it);
@@ -556,6 +556,42 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
     __syncthreads();
     if (r == 0 && *eflag) atomicOr(a.err, 1);
     if (warp == 4) tmem_dealloc(tmem, TC);
+}
+
+// Nearest up-sampling of `coarse` and the finer grid's own term: out = coarse + fine, or (mask)
+// mask > 0 ? fine + coarse / 8 : 0, the gradient through a pooling.  One thread per 16-byte unit:
+// as an epilogue of the coarse convolution the same passes had 128 threads per 1024 fine voxels
+// and took 9 (8^3), 17 (16^3) and 40 us (32^3) more than the convolution alone, here 4, 6 and 16.
+__global__ void __launch_bounds__(256) k_expand(const uint16_t *__restrict__ coarse, const uint16_t *__restrict__ fine,
+                                                const uint16_t *__restrict__ mask, uint16_t *__restrict__ out,
+                                                unsigned units, int lg, int lgG) {
+    pdl_enter();
+    const unsigned e = blockIdx.x * 256 + threadIdx.x;
+    if (e >= units) return;
+    const unsigned m = e >> lgG, g = e & ((1u << lgG) - 1), D = 1u << lg;
+    const unsigned x = m & (D - 1), y = (m >> lg) & (D - 1), bz = m >> (2 * lg);
+    const unsigned mc = ((((bz >> 1) << (lg - 1)) + (y >> 1)) << (lg - 1)) + (x >> 1);
+    float f[8], s[8];
+    const uint4 qf = __ldg(reinterpret_cast<const uint4 *>(coarse) + (((size_t)mc << lgG) + g));
+    const uint4 qs = __ldg(reinterpret_cast<const uint4 *>(fine) + e);
+    unpack8(qf, f);
+    unpack8(qs, s);
+    if (mask) {
+        float k[8];
+        unpack8(__ldg(reinterpret_cast<const uint4 *>(mask) + e), k);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = k[j] > 0.f ? s[j] + 0.125f * f[j] : 0.f;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] += s[j];
+    }
+    reinterpret_cast<uint4 *>(out)[e] = pack8(f);
+}
+
+void expand(const uint16_t *coarse, const uint16_t *fine, const uint16_t *mask, uint16_t *out, int nvox, int lg, int C,
+            cudaStream_t st) {
+    const unsigned units = (unsigned)nvox * (C / 8);
+    launch_pdl(k_expand, (units + 255) / 256, 256, 0, st, coarse, fine, mask, out, units, lg, C == 32 ? 2 : 1);
 }
 
 // gradients of every layer of the table from the CTAs' slices: [27 C + 1][N] summed over the
@@ -591,7 +627,7 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(WgradSums t) {
 
 template <int C, int N, int EPI>
 static void set_conv() {
-    cudaFuncSetAttribute(k_conv_tc<C, N, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(C, N, EPI));
+    cudaFuncSetAttribute(k_conv_tc<C, N, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, conv_smem(C, N));
 }
 
 void init_attributes() {
@@ -606,8 +642,6 @@ void init_attributes() {
     set_conv<32, 32, CONV_POOL>();
     set_conv<16, 16, CONV_PAIR>();
     set_conv<32, 16, CONV_PAIR>();
-    set_conv<32, 16, CONV_EXPAND>();
-    set_conv<32, 32, CONV_EXPAND>();
     set_conv<16, 16, CONV_HEAD>();
     cudaFuncSetAttribute(k_wgrad_tc<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaFuncSetAttribute(k_wgrad_tc<16, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
@@ -618,13 +652,14 @@ void init_attributes() {
 
 template <int C, int N, int EPI>
 static int launch_conv(const ConvArgs &a, cudaStream_t st) {
-    // as many CTAs as fit beside each other on an SM (227 KB shared memory, 4 at most)
-    constexpr int fit = 227 * 1024 / (int)(conv_smem(C, N, EPI) + 1024);
-    constexpr int per_sm = fit < 4 ? fit : 4;
+    // as many CTAs as fit beside each other on an SM (227 KB shared memory, 512 columns of TMEM)
+    constexpr int fit = 227 * 1024 / (int)(conv_smem(C, N) + 1024);
+    constexpr int tm = 512 / (ACCS * N);
+    constexpr int per_sm = fit < tm ? fit : tm;
     const int ltx = a.lg > 3 ? a.lg - 3 : 0, lty = a.lg > 4 ? a.lg - 4 : 0;
     const int tiles = (a.nvox >> (2 * a.lg)) << (ltx + lty);
     if (tiles > 0)
-        launch_pdl(k_conv_tc<C, N, EPI>, tiles < 152 * per_sm ? tiles : 152 * per_sm, 160, conv_smem(C, N, EPI), st, a);
+        launch_pdl(k_conv_tc<C, N, EPI>, tiles < 152 * per_sm ? tiles : 152 * per_sm, 160, conv_smem(C, N), st, a);
     return 0;
 }
 
@@ -639,8 +674,6 @@ int conv(const ConvArgs &a, int C, int N, cudaStream_t st) {
                                 : -1;
         case CONV_PAIR:
             return cn == 1616 ? launch_conv<16, 16, CONV_PAIR>(a, st) : cn == 3216 ? launch_conv<32, 16, CONV_PAIR>(a, st) : -1;
-        case CONV_EXPAND:
-            return cn == 3216 ? launch_conv<32, 16, CONV_EXPAND>(a, st) : cn == 3232 ? launch_conv<32, 32, CONV_EXPAND>(a, st) : -1;
         default:
             return cn == 1616   ? launch_conv<16, 16, CONV_PLAIN>(a, st)
                    : cn == 1632 ? launch_conv<16, 32, CONV_PLAIN>(a, st)

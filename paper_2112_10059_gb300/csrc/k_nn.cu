@@ -106,20 +106,28 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
     p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
 }
 
+// element i of the image of a convolution with ci input and co output channels: its row and
+// column, and whether a tap stands there (the last chunk may be padding)
+__device__ __forceinline__ bool image_at(int i, int ci, int co, int &tap, int &c, int &n, size_t &at) {
+    const int kc = i / (3 * co * 64), within = i % (3 * co * 64), row = within / 64, kk = within % 64, k = kc * 64 + kk;
+    tap = 9 * (2 - row / co) + k / ci;
+    c = k % ci;
+    n = row % co;
+    at = (size_t)kc * 3 * co * 64 + row * 64 + (((kk >> 3) ^ (row & 7)) << 3) + (kk & 7);
+    return k < 9 * ci;
+}
+
 __global__ void k_images(const float *__restrict__ w, int C, int N, uint16_t *__restrict__ img_f,
                          uint16_t *__restrict__ img_d, int nf, int nd) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int tap, c, n;
+    size_t at;
     if (i < nf) {
-        const int kc = i / (N * 64), within = i % (N * 64), n = within / 64, kk = within % 64;
-        const int k = kc * 64 + kk, tap = k / C, c = k % C;
-        const float val = tap < NTAPS ? w[(size_t)(n * NTAPS + tap) * C + c] : 0.f;
-        img_f[(size_t)kc * N * 64 + n * 64 + (((kk >> 3) ^ (n & 7)) << 3) + (kk & 7)] = f2bf(val);
+        const bool in = image_at(i, C, N, tap, c, n, at);
+        img_f[at] = in ? f2bf(w[(size_t)(n * NTAPS + tap) * C + c]) : 0;
     } else if (i < nf + nd) {
-        const int j = i - nf;
-        const int kc = j / (C * 64), within = j % (C * 64), n = within / 64, kk = within % 64;
-        const int k = kc * 64 + kk, tap = k / N, co = k % N;
-        const float val = tap < NTAPS ? w[(size_t)(co * NTAPS + (NTAPS - 1 - tap)) * C + n] : 0.f;
-        img_d[(size_t)kc * C * 64 + n * 64 + (((kk >> 3) ^ (n & 7)) << 3) + (kk & 7)] = f2bf(val);
+        const bool in = image_at(i - nf, N, C, tap, c, n, at);   // the data gradient: flipped taps, channels exchanged
+        img_d[at] = in ? f2bf(w[(size_t)(c * NTAPS + (NTAPS - 1 - tap)) * C + n]) : 0;
     }
 }
 
@@ -133,8 +141,8 @@ void adam(float *p, const float *g, float *m, float *v, size_t n, float lr, floa
     if (n) k_adam<<<blocks_for(n), 256, 0, st>>>(p, g, m, v, n, lr, b1, b2, eps, bc1, bc2);
 }
 void make_images(const float *w, int C, int N, uint16_t *img_fwd, uint16_t *img_dgrad, cudaStream_t st) {
-    const int nf = conv_chunks(C) * N * 64;
-    const int nd = img_dgrad ? conv_chunks(N) * C * 64 : 0;
+    const int nf = conv_image(C, N);
+    const int nd = img_dgrad ? conv_image(N, C) : 0;
     k_images<<<blocks_for((size_t)nf + nd), 256, 0, st>>>(w, C, N, img_fwd, img_dgrad, nf, nd);
 }
 void f32_to_bf16(const float *in, uint16_t *out, size_t n, cudaStream_t st) {

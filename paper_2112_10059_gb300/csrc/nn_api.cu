@@ -58,7 +58,7 @@ struct sph_nn {
     std::vector<void *> allocs;
     uint16_t *a00, *s0, *p0, *a10, *s1, *p1, *a20, *s2, *p2, *a30, *b3, *u2, *d2, *u1, *d1, *d0, *v0, *f;
     uint16_t *g_f, *g_v0, *g_d0, *g_d1, *g_u1, *g_d2, *g_u2, *g_b3, *g_a30, *g_s2, *g_a20,
-        *g_s1, *g_a10, *g_s0, *g_a00;
+        *g_s1, *g_a10, *g_s0, *g_a00, *g_p2, *g_p1, *g_p0;
 };
 
 namespace {
@@ -139,11 +139,9 @@ int conv_pool(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out, ui
 }
 // forward, and its nearest up-sampling plus the finer level's skip into sum
 int conv_up(sph_nn *n, int L, int batch, const uint16_t *in, uint16_t *out, const uint16_t *skip, uint16_t *sum) {
-    ConvArgs a = layer_args(n, L, batch, in, out, false);
-    a.epi = CONV_EXPAND;
-    a.add2 = skip;
-    a.out2 = sum;
-    return run_layer(n, L, a, false);
+    int r = conv_layer(n, L, batch, in, out);
+    if (!r) expand(out, skip, nullptr, sum, (int)vox(n, batch, LAYERS[L].lvl - 1), n->lg0 - LAYERS[L].lvl + 1, 32, n->stream);
+    return r;
 }
 // data gradient, zero where mask <= 0
 int dgrad_mask(sph_nn *n, int L, int batch, const uint16_t *g, uint16_t *out, const uint16_t *mask) {
@@ -160,14 +158,15 @@ int dgrad_up(sph_nn *n, int L, int batch, const uint16_t *g, uint16_t *out, uint
     a.mask2 = mask;
     return run_layer(n, L, a, true);
 }
-// data gradient through the pooling: (skip gradient + 1/8 of it) at each child, zero where mask <= 0
-int dgrad_pool(sph_nn *n, int L, int batch, const uint16_t *g, const uint16_t *skip, uint16_t *fine, const uint16_t *mask) {
-    ConvArgs a = layer_args(n, L, batch, g, nullptr, true);
-    a.epi = CONV_EXPAND;
-    a.add2 = skip;
-    a.mask2 = mask;
-    a.out2 = fine;
-    return run_layer(n, L, a, true);
+// data gradient g_out, and through the pooling: (skip gradient + 1/8 of it) at each child, zero where
+// mask <= 0
+int dgrad_pool(sph_nn *n, int L, int batch, const uint16_t *g, uint16_t *out, const uint16_t *skip, uint16_t *fine,
+               const uint16_t *mask) {
+    int r = run_layer(n, L, layer_args(n, L, batch, g, out, true), true);
+    if (!r)
+        expand(out, skip, mask, fine, (int)vox(n, batch, LAYERS[L].lvl - 1), n->lg0 - LAYERS[L].lvl + 1, LAYERS[L].ci,
+               n->stream);
+    return r;
 }
 
 // the layer's partial weight gradients, and its entry in the sums that end the backward pass
@@ -208,8 +207,8 @@ int forward_pass(sph_nn *n, int B, const uint16_t *x, float *y, bool train) {
     RUN(conv_layer(n, C20, B, n->p1, n->a20));
     RUN(conv_pool(n, C21, B, n->a20, n->s2, n->p2));
     RUN(conv_layer(n, C30, B, n->p2, n->a30));
-    RUN(conv_up(n, C31, B, n->a30, train ? n->b3 : nullptr, n->s2, n->u2));
-    RUN(conv_up(n, C22, B, n->u2, train ? n->d2 : nullptr, n->s1, n->u1));
+    RUN(conv_up(n, C31, B, n->a30, n->b3, n->s2, n->u2));
+    RUN(conv_up(n, C22, B, n->u2, n->d2, n->s1, n->u1));
     RUN(conv_layer(n, C12, B, n->u1, n->d1));
     ConvArgs a = layer_args(n, C02, B, n->d1, train ? n->d0 : nullptr, false);
     a.up = 1;                                   // reads d1 up-sampled
@@ -251,15 +250,15 @@ int backward_pass(sph_nn *n, int B, const uint16_t *x, const float *t) {
     RUN(wgrad_layer(n, sums, C31, B, n->a30, n->g_b3));
     RUN(dgrad_mask(n, C31, B, n->g_b3, n->g_a30, n->a30));
     RUN(wgrad_layer(n, sums, C30, B, n->p2, n->g_a30));
-    RUN(dgrad_pool(n, C30, B, n->g_a30, n->g_u2, n->g_s2, n->s2));
+    RUN(dgrad_pool(n, C30, B, n->g_a30, n->g_p2, n->g_u2, n->g_s2, n->s2));
     RUN(wgrad_layer(n, sums, C21, B, n->a20, n->g_s2));
     RUN(dgrad_mask(n, C21, B, n->g_s2, n->g_a20, n->a20));
     RUN(wgrad_layer(n, sums, C20, B, n->p1, n->g_a20));
-    RUN(dgrad_pool(n, C20, B, n->g_a20, n->g_u1, n->g_s1, n->s1));
+    RUN(dgrad_pool(n, C20, B, n->g_a20, n->g_p1, n->g_u1, n->g_s1, n->s1));
     RUN(wgrad_layer(n, sums, C11, B, n->a10, n->g_s1));
     RUN(dgrad_mask(n, C11, B, n->g_s1, n->g_a10, n->a10));
     RUN(wgrad_layer(n, sums, C10, B, n->p0, n->g_a10));
-    RUN(dgrad_pool(n, C10, B, n->g_a10, n->g_v0, n->g_s0, n->s0));
+    RUN(dgrad_pool(n, C10, B, n->g_a10, n->g_p0, n->g_v0, n->g_s0, n->s0));
     RUN(wgrad_layer(n, sums, C01, B, n->a00, n->g_s0));
     RUN(dgrad_mask(n, C01, B, n->g_s0, n->g_a00, n->a00));
     RUN(wgrad_layer(n, sums, C00, B, x, n->g_a00));
@@ -335,9 +334,9 @@ int sph_nn_create(sph_nn **out, int device, void *stream, int edge, int max_batc
         n->p_off[L] = po;
         po += (size_t)S.co * NTAPS * S.ci + S.co;
         n->img_f_off[L] = io;
-        io += (size_t)conv_chunks(S.ci) * S.co * 64;
+        io += conv_image(S.ci, S.co);
         n->img_d_off[L] = io;
-        io += (size_t)conv_chunks(S.co) * S.ci * 64;
+        io += conv_image(S.co, S.ci);
         n->part_off[L] = wo;   // a smaller batch has no more slices
         wo += (size_t)wgrad_splits(S.ci, S.co, lg - S.lvl, (int)vox(n, max_batch, S.lvl)) * (NTAPS * S.ci + 1) * S.co;
     }
@@ -367,6 +366,7 @@ int sph_nn_create(sph_nn **out, int device, void *stream, int edge, int max_batc
     A(n->g_u1, V1 * 32); A(n->g_d2, V2 * 32); A(n->g_u2, V2 * 32); A(n->g_b3, V3 * 32); A(n->g_a30, V3 * 32);
     A(n->g_s2, V2 * 32); A(n->g_a20, V2 * 32); A(n->g_s1, V1 * 32);
     A(n->g_a10, V1 * 32); A(n->g_s0, V0 * 16); A(n->g_a00, V0 * 16);
+    A(n->g_p2, V3 * 32); A(n->g_p1, V2 * 32); A(n->g_p0, V1 * 16);
     if (!r) {
         n->scratch_n = 3 * (size_t)edge * edge * edge;
         A(n->scratch, n->scratch_n);
@@ -528,7 +528,7 @@ int sph_nn_conv3d(int device, void *stream, int mode, int C, int N, int edge, in
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint16_t *img_f = nullptr, *img_d = nullptr;
     int *err = nullptr;
-    const size_t nf = (size_t)conv_chunks(C) * N * 64, nd = (size_t)conv_chunks(N) * C * 64;
+    const size_t nf = conv_image(C, N), nd = conv_image(N, C);
     if (cudaMalloc(&img_f, (nf + nd) * sizeof(uint16_t)) != cudaSuccess || cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(img_f);

@@ -7,9 +7,7 @@
 //     out[m][n] = sum_k A[m][k] W[n][k],   k = tap * C + c,
 //     A[m][tap*C + c] = x[m + offset(tap)][c]   (0 outside the grid),
 //     tap = 9 (dz+1) + 3 (dy+1) + (dx+1),
-// run on the tensor cores (tcgen05, BF16 in, FP32 accumulate in TMEM).  Weight images are
-// pre-arranged in global memory in the exact shared-memory layout the MMA reads (K-major,
-// 128-byte swizzle, one 64-element K chunk after the other).
+// run on the tensor cores (tcgen05, BF16 in, FP32 accumulate in TMEM).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -18,22 +16,23 @@ namespace sph {
 namespace nn {
 
 constexpr int NTAPS = 27;
-// K chunks of 64 elements for C channels per tap (taps padded to 28 with zeros)
-__host__ __device__ constexpr int conv_chunks(int C) { return (NTAPS + 64 / C - 1) / (64 / C); }
+// Weight image of a convolution, the B operand of k_conv_tc in its shared-memory layout: rows
+// (2 - dz) N + n, columns k = (3 dy + dx) C + c, as chunks of 64 columns [3 N][64], each K-major
+// with the 128-byte swizzle.  Elements (BF16):
+__host__ __device__ constexpr int conv_image(int C, int N) { return (9 * C + 63) / 64 * 3 * N * 64; }
+
 // Epilogues of a convolution beside the plain one (bias, ReLU, residual, mask), each in place of
 // a pass over memory; all use the convolution's result as rounded to BF16.
 enum {
     CONV_PLAIN = 0,
     CONV_POOL,     // out2[parent] = scale * (sum of the 8 children), 0 where mask2 <= 0 (mask2 given); out optional
     CONV_PAIR,     // out2 = out + add2 (add2 given), or out where mask2 > 0 and 0 elsewhere; out optional
-    CONV_EXPAND,   // out2[child] = out + add2[child], or (mask2 given) mask2[child] > 0 ? add2[child] + out / 8 : 0;
-                   // out optional
     CONV_HEAD      // y = head weights . out + head bias (FP32); out optional
 };
 
 struct ConvArgs {
     const uint16_t *x;       // [nvox][C]
-    const uint16_t *w;       // weight image: conv_chunks(C) x [N][64], swizzled
+    const uint16_t *w;       // weight image, conv_image(C, N) elements
     const float *bias;       // [N] or nullptr
     const uint16_t *add;     // [nvox][N] or nullptr: added after the ReLU
     const uint16_t *mask;    // [nvox][N] or nullptr: zero where mask <= 0 (applied last)
@@ -83,6 +82,10 @@ void init_attributes();
 // C, N in {16, 32}; returns 0, or -1 for an unsupported shape
 int conv(const ConvArgs &a, int C, int N, cudaStream_t st);
 int wgrad(const WgradArgs &a, int C, int N, cudaStream_t st);
+// out [nvox][C] on the grid of edge 2^lg: coarse (half the edge) up-sampled + fine, or with a mask
+// mask > 0 ? fine + coarse / 8 : 0
+void expand(const uint16_t *coarse, const uint16_t *fine, const uint16_t *mask, uint16_t *out, int nvox, int lg, int C,
+            cudaStream_t st);
 
 // loss of the residual r = y0 against t and of the error head e = y1 against log(|r - t| + eps)
 // (y[m][j] = sum_c hw[j][c] f[m][c] + hb[j]); writes the masked gradient of f (BF16) and each
