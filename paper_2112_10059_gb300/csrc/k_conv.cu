@@ -174,48 +174,57 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
         }
     } else {                                  // ---- four warps copy planes and write results
         const int up = a.up, lgi = lg - up;   // input grid (half the edge when up-sampled on load)
-        int off[NU], loaded = 0;
+        int off[NU], loaded = 0, slot = 0;    // off: a unit's place in its plane, and whether it is in the grid
+        uint32_t in = 0, dst[NU];
         const uint16_t *xcol = a.x;
         PlaneCursor lp(t0, t1, lg);
+#pragma unroll
+        for (int j = 0; j < NU; ++j) {
+            const int u = r + 128 * j;
+            dst[j] = ring + (uint32_t)(u % CG) * GB + (uint32_t)(u / CG) * 16;
+        }
         auto load_next = [&]() {              // the next plane, one copy group
             if (lp.step()) {                  // another column
                 const int x0 = (lp.col & ((1 << ltx) - 1)) * CX - 1, y0 = ((lp.col >> ltx) & ((1 << lty) - 1)) * CY - 1;
                 xcol = a.x + ((size_t)(lp.col >> (ltx + lty)) << (3 * lgi)) * C;
+                in = 0;
 #pragma unroll
                 for (int j = 0; j < NU; ++j) {
                     const int u = r + 128 * j, v = u / CG, cg = u % CG;
                     const int x = x0 + v % PX, y = y0 + v / PX;
-                    off[j] = ((unsigned)x < (unsigned)D && (unsigned)y < (unsigned)D)
-                                 ? (((y >> up) << lgi) + (x >> up)) * C + cg * 8
-                                 : -1;
+                    const bool ok = (unsigned)x < (unsigned)D && (unsigned)y < (unsigned)D;
+                    off[j] = ok ? (((y >> up) << lgi) + (x >> up)) * C + cg * 8 : 0;
+                    in |= (ok ? 16u : 0u) << j;
                 }
             }
-            const uint32_t dst = ring + (uint32_t)(loaded % RING) * PB;
             const bool zin = (unsigned)lp.z < (unsigned)D;
+            const uint32_t zmask = zin ? in : 0u;
             const uint16_t *xp = xcol + ((size_t)((zin ? lp.z : 0) >> up) << (2 * lgi)) * C;
 #pragma unroll
-            for (int j = 0; j < NU; ++j) {
-                const int u = r + 128 * j;
-                if (u < PX * PY * CG) {
-                    const bool in = zin && off[j] >= 0;
-                    cp_async16(dst + (uint32_t)(u % CG) * GB + (uint32_t)(u / CG) * 16, in ? xp + off[j] : a.x, in ? 16 : 0);
-                }
-            }
+            for (int j = 0; j < NU; ++j)
+                if (r + 128 * j < PX * PY * CG) cp_async16(dst[j] + (uint32_t)slot * PB, xp + off[j], zmask >> j & 16u);
+            slot = slot == RING - 1 ? 0 : slot + 1;
             cp_async_commit();
             ++loaded;
         };
 
         float pool[EPI == CONV_POOL ? N : 1];
-        auto epilogue = [&](int col, int z, int nth) {   // output nth of the CTA's, at (col, z)
+        bool valid = false;                   // this thread's voxel of the run's tiles
+        size_t at = 0, atp = 0;               // its place at z = 0, and its parent's
+        auto place = [&](int col) {
             const int x = (col & ((1 << ltx) - 1)) * CX + (r & 7), y = ((col >> ltx) & ((1 << lty) - 1)) * CY + (r >> 3);
-            const size_t bz = ((size_t)(col >> (ltx + lty)) << lg) + z;   // sample and plane
-            const bool valid = x < D && y < D;
+            const size_t b = (size_t)(col >> (ltx + lty));
+            valid = x < D && y < D;
+            at = (b << (3 * lg)) + ((size_t)y << lg) + x;
+            if (EPI == CONV_POOL) atp = (b << (3 * lg - 3)) + ((size_t)(y >> 1) << (lg - 1)) + (x >> 1);
+        };
+        auto epilogue = [&](int z, int nth) { // output nth of the CTA's, at plane z of its run
             float v[N];
             const uint32_t acc = tmem + (uint32_t)(nth % ACCS * N) + ((uint32_t)(warp * 32) << 16);
             tmem_ld16(acc, v);
             if constexpr (N == 32) tmem_ld16(acc + 16, v + 16);
             fence_before_sync();              // read before this thread's next arrival frees the accumulator
-            const size_t o = ((bz << (2 * lg)) + ((size_t)y << lg) + x) * N;
+            const size_t o = (at + ((size_t)z << (2 * lg))) * N;
             uint4 q[N / 8];
 #pragma unroll
             for (int g = 0; g < N / 8; ++g) {
@@ -282,7 +291,7 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
                     }
                 }
                 if ((z & 1) && valid && !(r & 1) && !(r & 8)) {
-                    const size_t op = ((((bz >> 1) << (2 * lg - 2)) + ((size_t)(y >> 1) << (lg - 1))) + (x >> 1)) * N;
+                    const size_t op = (atp + ((size_t)(z >> 1) << (2 * lg - 2))) * N;
 #pragma unroll
                     for (int g = 0; g < N / 8; ++g) {
                         float f[8];
@@ -322,11 +331,11 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
                 mbar_arrive(smem_u32(&bar[2 + (i & 1)]));
             }
             if (i > 0) {
-                p.step();
+                if (p.step()) place(p.col);
                 if (!mbar_wait_bounded(smem_u32(&bar[(i - 1) & 1]), ((i - 1) >> 1) & 1, NN_WAIT)) *eflag = 1;
                 if (p.z > p.zs) {
                     fence_after_sync();
-                    epilogue(p.col, p.z - 1, q++);
+                    epilogue(p.z - 1, q++);
                 }
             }
         }
@@ -344,20 +353,23 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
 // units as above, so nothing is transposed or repeated.  Shared memory holds, per y row, the
 // units of [z - 1, z, z + 1][channel group][x] at one stride; the core matrices of three
 // neighbouring rows then follow each other at that stride in the order (dy, dz, group), which
-// makes M tiles of 128 rows that cover the nine (dy, dz) taps (a tenth of the rows is padding),
-// and the three dx are start addresses one unit apart.  A constant plane of ones behind the
-// three z gives the bias gradient as one more row.
-// CTAs march in y through equal shares of the (sample, z, x segment) columns, 64 voxels an
+// makes M tiles of 128 rows that cover the nine (dy, dz) taps (a tenth of the rows is padding).
+// The three dx are dz at three x shifts, side by side as N = 3 x out channels: an MMA is bound by
+// reading its 4 KB of x, whatever its N (16 -> 16 at 64^3 x 4: 289 us with both operands
+// transposed in registers, 78 with the dx as three MMAs on shifted x, 40 so; 32 -> 16: 606,
+// 187, 66).  A constant plane of ones behind the three z gives the bias gradient as one more
+// row.  CTAs march in y through equal shares of the (sample, z, x segment) columns, 64 voxels an
 // iteration, rows in a ring whose first slots are mirrored behind its last so that three rows
 // always follow each other.  Each CTA's sums go to its own slice of `part`; k_wgrad_sum adds
 // the slices in order (training is reproducible bit for bit).
-// What bounds it: 4 KB of x read from shared memory per MMA, as above.
 __host__ __device__ constexpr int wg_block(int C) { return 3 * (C / 8) + 1; }               // core-matrix columns per row
 __host__ __device__ constexpr int wg_tiles(int C) { return (3 * wg_block(C) + 15) / 16; }   // M tiles per dx
 __host__ __device__ constexpr int wg_cols(int C, int N) {                                   // TMEM columns (power of 2)
     return 3 * wg_tiles(C) * N <= 128 ? 128 : 3 * wg_tiles(C) * N <= 256 ? 256 : 512;
 }
-constexpr uint32_t wg_dz_slot(int N) { return (uint32_t)(N / 8) * 1024 + 128; }
+// 64 voxels of one channel group of dz, padded as the x stride below; a slot holds three shifts
+__host__ __device__ constexpr uint32_t wg_dz_group(int N) { return 1024 + (N == 16 ? 64 : 32); }
+__host__ __device__ constexpr uint32_t wg_dz_slot(int N) { return 3 * (uint32_t)(N / 8) * wg_dz_group(N); }
 
 struct WgradShape {      // how a layer's voxels are cut, from its edge alone
     int lgx;             // x segment of a row: 2^lgx voxels, 8 .. 64
@@ -373,10 +385,10 @@ static WgradShape wgrad_shape(int C, int lg, int nvox) {
     s.lgx = lge > 6 ? 6 : lge;
     s.rpi = 64 >> s.lgx;
     s.lipc = lge - (6 - s.lgx);
-    s.ring = 2 * (s.rpi + 2) + 2;
+    s.ring = 2 * (s.rpi + 2) + 1;
     s.mirror = s.lgx == 3 ? 3 : 2;
     // the 8 units a quarter-warp copies (2 groups x 4 voxels, or 4 x 2) in different banks
-    s.stride = (uint32_t)((1 << s.lgx) + 2) * 16 + (C == 16 ? 32 : 0);
+    s.stride = (16u << s.lgx) + (C == 16 ? 64 : 32);
     const int cb = wg_block(C);
     const int read = (s.ring - 1) * cb + 16 * wg_tiles(C) + (s.lgx == 3 ? cb : 0);   // the padding rows' reads end here
     s.cols = (s.ring + s.mirror) * cb > read ? (s.ring + s.mirror) * cb : read;
@@ -389,16 +401,19 @@ int wgrad_splits(int C, int N, int lg, int nvox) {
     const WgradShape s = wgrad_shape(C, lg, nvox);
     const int fit = 227 * 1024 / (int)(wgrad_smem(C, N, s) + 1024), tm = 512 / wg_cols(C, N);
     const int most = 152 * (fit < tm ? (fit < 2 ? fit : 2) : (tm < 2 ? tm : 2));
-    const int n = (s.iters + 1) / 2;          // at least two iterations a CTA: each writes a slice of its own
+    const int n = (s.iters + 3) / 4;          // at least four iterations a CTA: each writes a slice of its own
     return n < 1 ? 1 : n < most ? n : most;
 }
 
+constexpr int WGT = 160;     // four warps copy, one issues the MMAs (eight copying: 29 us more per backward pass)
+
 template <int C, int N>
-__global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
+__global__ void __launch_bounds__(WGT) k_wgrad_tc(WgradArgs a, WgradShape s) {
     pdl_enter();
     constexpr int CG = C / 8, CB = wg_block(C), NM = wg_tiles(C), TC = wg_cols(C, N);
-    constexpr int NU = (3 * CG * 66 + 127) / 128, NZ = N / 16;
-    constexpr uint32_t ZS = wg_dz_slot(N), ZG = ZS / (N / 8);
+    constexpr int LT = WGT - 32;              // copying threads
+    constexpr int NU = (3 * CG * 64 + LT - 1) / LT, NZ = (3 * 64 * (N / 8) + LT - 1) / LT;
+    constexpr uint32_t ZS = wg_dz_slot(N), ZG = wg_dz_group(N);
     extern __shared__ uint8_t raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 127) & ~(uintptr_t)127);
     const uint32_t xbytes = (uint32_t)s.cols * s.stride, blk = (uint32_t)CB * s.stride;
@@ -411,23 +426,22 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
     const int n = (int)((long long)s.iters * (blockIdx.x + 1) / gridDim.x) - i0;   // >= 1: the grid is no larger than iters
     const int ipm = (1 << s.lipc) - 1;
 
-    if (warp == 4) {
+    if (warp == LT / 32) {
         tmem_alloc(smem_u32(tslot), TC);
         tmem_relinquish();
     }
     if (r == 0) {
         mbar_init(smem_u32(&bar[0]), 1);
         mbar_init(smem_u32(&bar[1]), 1);
-        mbar_init(smem_u32(&bar[2]), 128);
-        mbar_init(smem_u32(&bar[3]), 128);
+        mbar_init(smem_u32(&bar[2]), LT);
+        mbar_init(smem_u32(&bar[3]), LT);
         *eflag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int e = r; e < (s.ring + s.mirror) << s.lgx; e += 160) {   // the ones: channel 0 of each unit
+    for (int e = r; e < (s.ring + s.mirror) << s.lgx; e += WGT) {   // the ones: channel 0 of each unit
         const int b = e >> s.lgx, x = e & ((1 << s.lgx) - 1);
         uint8_t *p = base + (size_t)(b * CB + CB - 1) * s.stride + (size_t)x * 16;
         *reinterpret_cast<uint4 *>(p) = make_uint4(0x3F80u, 0, 0, 0);
-        if (x < 2) *reinterpret_cast<uint4 *>(p + (16u << s.lgx)) = make_uint4(0x3F80u, 0, 0, 0);
     }
     fence_proxy_async_smem();
     fence_before_sync();
@@ -436,9 +450,9 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
     const uint32_t tmem = *tslot;
     const uint32_t xb = smem_u32(base), zb = xb + xbytes;
 
-    if (warp == 4) {                          // ---- one thread issues every MMA
-        if (r == 128) {
-            const uint32_t idesc = idesc_bf16_f32(128, N) | (3u << 15);      // both operands MN-major
+    if (warp == LT / 32) {                          // ---- one thread issues every MMA
+        if (elect_one()) {
+            const uint32_t idesc = idesc_bf16_f32(128, 3 * N) | (3u << 15);  // both operands MN-major
             // MN-major without a swizzle: first stride along K (8 voxels), second along M or N
             const uint64_t ad0 = sdesc_none(0, s.lgx == 3 ? blk : 128, s.stride), bd0 = sdesc_none(0, 128, ZG);
             int f = 0;                        // sequence number of the iteration's first row
@@ -452,28 +466,31 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
                     const uint32_t sx = xb + (uint32_t)((f + row) % s.ring) * blk + (uint32_t)x * 16;
                     const uint64_t bd = bd0 + ((zb + (uint32_t)(it & 3) * ZS + (uint32_t)ks * 256) >> 4);
 #pragma unroll
-                    for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                        for (int j = 0; j < NM; ++j)
-                            mma_bf16(tmem + (uint32_t)((dx * NM + j) * N),
-                                     ad0 + ((sx + (uint32_t)dx * 16 + (uint32_t)j * 16 * s.stride) >> 4), bd, idesc,
-                                     (it > 0 || ks > 0) ? 1u : 0u);
+                    for (int j = 0; j < NM; ++j)
+                        mma_bf16(tmem + (uint32_t)(j * 3 * N), ad0 + ((sx + (uint32_t)j * 16 * s.stride) >> 4), bd, idesc,
+                                 (it > 0 || ks > 0) ? 1u : 0u);
                 }
                 mma_commit(smem_u32(&bar[it & 1]));
             }
         }
-    } else {                                  // ---- four warps copy
+    } else {                                  // ---- the other warps copy
         const int lg = a.lg, D = 1 << lg, up = a.up, lgi = lg - up;
         const int lnx = lg > 6 ? lg - 6 : 0;  // x segments per row (log2)
-        const int TX = 1 << s.lgx, nub = 3 * CG * (TX + 2);
-        int off[NU];
-        uint32_t dst[NU];
+        const int TX = 1 << s.lgx, nub = 3 * CG * TX;
+        int off[NU], zoff[NZ];                // places in a row, and whether they are in the grid
+        uint32_t in = 0, zin = 0, dst[NU], zdst[NZ];
+        int slot = 0;
         const uint16_t *xcol = a.x, *zcol = a.dz;
         int x0 = 0, rows = -1;                // rows: sequence number of the last row copied
 #pragma unroll
         for (int j = 0; j < NU; ++j) {
-            const int u = r + 128 * j, cg = u % CG, v = u / CG;
-            dst[j] = xb + (uint32_t)((v / (TX + 2)) * CG + cg) * s.stride + (uint32_t)(v % (TX + 2)) * 16;
+            const int u = r + LT * j, cg = u % CG, v = u / CG;
+            dst[j] = xb + (uint32_t)((v >> s.lgx) * CG + cg) * s.stride + (uint32_t)(v & (TX - 1)) * 16;
+        }
+#pragma unroll
+        for (int j = 0; j < NZ; ++j) {        // 3 shifts x 64 voxels x N / 8 units
+            const int u = r + LT * j, ng = u % (N / 8), v = u / (N / 8) % 64, dx = u / (N / 8) / 64;
+            zdst[j] = zb + (uint32_t)(dx * (N / 8) + ng) * ZG + (uint32_t)v * 16;
         }
         auto load_iter = [&](int k) {         // one copy group: the rows and gradients that iteration k adds
             const int i = i0 + k, y0 = (i & ipm) * s.rpi;
@@ -482,39 +499,44 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
                 const int col = i >> s.lipc, z = (col >> lnx) & (D - 1), b = col >> (lnx + lg);
                 x0 = (col & ((1 << lnx) - 1)) << 6;
                 xcol = a.x + ((size_t)b << (3 * lgi)) * C;
+                in = zin = 0;
                 zcol = a.dz + (((size_t)b << (3 * lg)) + ((size_t)z << (2 * lg))) * N;
 #pragma unroll
                 for (int j = 0; j < NU; ++j) {
-                    const int u = r + 128 * j, cg = u % CG, v = u / CG;
-                    const int x = x0 + v % (TX + 2) - 1, zz = z + v / (TX + 2) - 1;
-                    off[j] = (u < nub && (unsigned)x < (unsigned)D && (unsigned)zz < (unsigned)D)
-                                 ? (((zz >> up) << (2 * lgi)) + (x >> up)) * C + cg * 8
-                                 : -1;
+                    const int u = r + LT * j, cg = u % CG, v = u / CG;
+                    const int x = x0 + (v & (TX - 1)), zz = z + (v >> s.lgx) - 1;
+                    const bool ok = u < nub && (unsigned)x < (unsigned)D && (unsigned)zz < (unsigned)D;
+                    off[j] = ok ? (((zz >> up) << (2 * lgi)) + (x >> up)) * C + cg * 8 : 0;
+                    in |= (ok ? 16u : 0u) << j;
+                }
+#pragma unroll
+                for (int j = 0; j < NZ; ++j) {
+                    const int u = r + LT * j, ng = u % (N / 8), v = u / (N / 8) % 64, dx = u / (N / 8) / 64;
+                    const int y = v >> s.lgx, x = x0 + (v & (TX - 1)) - (dx - 1);   // y: below the iteration's first
+                    const bool ok = y < D && (unsigned)x < (unsigned)D;
+                    zoff[j] = ok ? ((y << lg) + x) * N + ng * 8 : 0;
+                    zin |= (ok ? 16u : 0u) << j;
                 }
             }
             for (int y = first ? y0 - 1 : y0 + 1; y <= y0 + s.rpi; ++y) {
                 ++rows;
-                const int slot = rows % s.ring;
                 const bool yin = (unsigned)y < (unsigned)D;
+                const uint32_t ymask = yin ? in : 0u, at = (uint32_t)slot * blk;
                 const uint16_t *xr = xcol + ((size_t)((yin ? y : 0) >> up) << lgi) * C;
 #pragma unroll
-                for (int j = 0; j < NU; ++j) {
-                    if (r + 128 * j < nub) {
-                        const bool in = yin && off[j] >= 0;
-                        cp_async16(dst[j] + (uint32_t)slot * blk, in ? xr + off[j] : a.x, in ? 16 : 0);
-                        if (slot < s.mirror)
-                            cp_async16(dst[j] + (uint32_t)(slot + s.ring) * blk, in ? xr + off[j] : a.x, in ? 16 : 0);
-                    }
-                }
-            }
+                for (int j = 0; j < NU; ++j)
+                    if (r + LT * j < nub) cp_async16(dst[j] + at, xr + off[j], ymask >> j & 16u);
+                if (slot < s.mirror) {
 #pragma unroll
-            for (int j = 0; j < NZ; ++j) {    // 64 voxels x N / 8 units
-                const int u = r + 128 * j, v = u / (N / 8), ng = u % (N / 8);
-                const int y = y0 + (v >> s.lgx), x = x0 + (v & (TX - 1));
-                const bool in = y < D && x < D;
-                cp_async16(zb + (uint32_t)(k & 3) * ZS + (uint32_t)ng * ZG + (uint32_t)v * 16,
-                           in ? zcol + (((size_t)y << lg) + x) * N + ng * 8 : a.dz, in ? 16 : 0);
+                    for (int j = 0; j < NU; ++j)
+                        if (r + LT * j < nub) cp_async16(dst[j] + at + (uint32_t)s.ring * blk, xr + off[j], ymask >> j & 16u);
+                }
+                slot = slot == s.ring - 1 ? 0 : slot + 1;
             }
+            const uint16_t *zr = zcol + ((size_t)y0 << lg) * N;
+#pragma unroll
+            for (int j = 0; j < NZ; ++j)
+                if (r + LT * j < 3 * 64 * (N / 8)) cp_async16(zdst[j] + (uint32_t)(k & 3) * ZS, zr + zoff[j], zin >> j & 16u);
             cp_async_commit();
         };
         int f = 0, fprev = 0, k = 0;          // k: iterations copied
@@ -536,15 +558,16 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
         if (!mbar_wait_bounded(smem_u32(&bar[(n - 1) & 1]), ((n - 1) >> 1) & 1, NN_WAIT)) *eflag = 1;
         fence_after_sync();
         float *part = a.part + (size_t)blockIdx.x * ((NTAPS * C + 1) * N);
-        for (int q = 0; q < 3 * NM; ++q) {
+        if (warp < 4) for (int q = 0; q < 3 * NM; ++q) {
+            const int j = q / 3, dx = q % 3;
             float v[N];
             const uint32_t acc = tmem + (uint32_t)(q * N) + ((uint32_t)(warp * 32) << 16);
             tmem_ld16(acc, v);
             if constexpr (N == 32) tmem_ld16(acc + 16, v + 16);
-            const int dx = q / NM, cm = 16 * (q % NM) + (r >> 3), dy = cm / CB, rem = cm % CB;
+            const int cm = 16 * j + (r >> 3), dy = cm / CB, rem = cm % CB;
             const int row = dy > 2 ? -1
                             : rem < CB - 1 ? (9 * (rem / CG) + 3 * dy + dx) * C + 8 * (rem % CG) + (r & 7)
-                            : (dy == 0 && dx == 0 && (r & 7) == 0) ? NTAPS * C : -1;
+                            : (dy == 0 && dx == 1 && (r & 7) == 0) ? NTAPS * C : -1;
             if (row >= 0) {
                 float4 *o = reinterpret_cast<float4 *>(part + (size_t)row * N);
 #pragma unroll
@@ -555,7 +578,7 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(WgradArgs a, WgradShape s) {
     fence_before_sync();
     __syncthreads();
     if (r == 0 && *eflag) atomicOr(a.err, 1);
-    if (warp == 4) tmem_dealloc(tmem, TC);
+    if (warp == LT / 32) tmem_dealloc(tmem, TC);
 }
 
 // Nearest up-sampling of `coarse` and the finer grid's own term: out = coarse + fine, or (mask)
@@ -687,7 +710,7 @@ template <int C, int N>
 static int launch_wgrad(const WgradArgs &a, cudaStream_t st) {
     const WgradShape s = wgrad_shape(C, a.lg, a.nvox);
     if (s.iters > 0)
-        launch_pdl(k_wgrad_tc<C, N>, wgrad_splits(C, N, a.lg, a.nvox), 160, wgrad_smem(C, N, s), st, a, s);
+        launch_pdl(k_wgrad_tc<C, N>, wgrad_splits(C, N, a.lg, a.nvox), WGT, wgrad_smem(C, N, s), st, a, s);
     return 0;
 }
 

@@ -118,6 +118,25 @@ def test_conv_weight_gradient(sur, C, N, edge, batch):
         C, N, edge, np.max(np.abs(out - ref)))
 
 
+@pytest.mark.parametrize("C,N,edge,batch", [(c, n, e, b) for c, n in SHAPES for e, b in [(2, 2), (16, 3), (64, 1)]] +
+                         [(16, 16, 128, 1)])
+def test_conv_weight_gradient_columns(sur, C, N, edge, batch):
+    """Marches that cross columns with the ring of rows wrapping, rows shorter than an iteration (2,
+    16) and rows of several x segments (128).  Each of the CTAs' sums is at most steps = ceil(voxels
+    / 64 / 152) * 4 accumulations of 16 products, each rounded towards zero (2^-23 of a partial sum
+    of at most 5 sigma = 5 sqrt(voxels) for unit normals)."""
+    rng = np.random.default_rng(1300 + C + 5 * N + edge)
+    x = _bf(rng.standard_normal((batch, edge, edge, edge, C)))
+    dz = _bf(rng.standard_normal((batch, edge, edge, edge, N)))
+    out = _host(sur.conv3d_wgrad(C, N, edge, batch, _to_dev_bf16(x), _to_dev_bf16(dz)))
+    dw, db = nn.conv3d_wgrad(x, dz)
+    ref = np.concatenate([dw.ravel(), db])
+    n = batch * edge ** 3
+    steps = 4 * max(4, -(-n // (64 * 152)))
+    tol = max(4e-5, steps * 2.0 ** -23 * 5) * np.sqrt(n)
+    assert np.max(np.abs(out - ref)) <= tol, "wgrad C%d N%d e%d: %.3e (%.3e)" % (C, N, edge, np.max(np.abs(out - ref)), tol)
+
+
 def _net_inputs(edge, batch, seed):
     rng = np.random.default_rng(seed)
     x = np.zeros((batch, edge, edge, edge, nn.IN_CH))
