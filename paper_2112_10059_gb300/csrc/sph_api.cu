@@ -114,7 +114,7 @@ struct sph_ctx {
     double r_s = 0.0;                 // strategy 3 ratio (0: off)
     DevBuf b_skip;
     bool near_table = false;          // resolved for the current evaluation
-    DevBuf b_gtab;
+    DevBuf b_gtab, b_dtab;            // near-field table; FP64 pair weights of the direct sum
     // buffers
     DevBuf b_maxes, b_cnt, b_off, b_tot, b_skey, b_spc, b_sq, b_tkey, b_tpc, b_bstat;
     DevBuf b_boxat, b_flag, b_pos, b_rng, b_scan, b_lvl;
@@ -1914,7 +1914,7 @@ void sph_destroy(sph_ctx *c) {
                      &c->b_lcnt, &c->b_loff, &c->b_usrc, &c->b_vsrc, &c->b_vocs, &c->b_vtrg, &c->b_wsrc, &c->b_xsrc, &c->b_pkeys, &c->b_ppairs, &c->b_heavy,
                      &c->b_ueq, &c->b_dchk, &c->o_work, &c->o_etab, &c->o_m2m, &c->o_l2l,
                      &c->o_m2l, &c->o_m2lbf, &c->o_l2lbf, &c->o_m2mbf, &c->b_err, &c->b_work, &c->b_mtg, &c->b_nearbuf, &c->o_slot, &c->o_surf, &c->o_cheb, &c->o_self, &c->h_q, &c->h_e, &c->h_m,
-                     &c->h_s, &c->b_tmask, &c->b_near, &c->b_gtab, &c->b_skip, &c->o_l2pimg, &c->s_qc, &c->s_Sc, &c->s_y, &c->s_Sp, &c->s_x, &c->s_Sf,
+                     &c->h_s, &c->b_tmask, &c->b_near, &c->b_gtab, &c->b_dtab, &c->b_skip, &c->o_l2pimg, &c->s_qc, &c->s_Sc, &c->s_y, &c->s_Sp, &c->s_x, &c->s_Sf,
                      &c->s_mask, &c->s_svox, &c->s_err, &c->s_pe, &c->s_flags, &c->s_counts};
     for (DevBuf *b : all)
         if (b->p) cudaFree(b->p);
@@ -2086,7 +2086,6 @@ int eval_direct(sph_ctx *c, int fp64, void *s_dev) {
     DirectArgs A;
     A.src_pc = P<uint32_t>(c->b_spc);
     A.src_q = P<float>(c->b_sq);
-    A.wscale = (float)(c->source_scale * c->h * c->h * c->h);
     A.ns = (int)c->ns;
     A.trg_key = P<uint32_t>(c->b_tkey);
     A.nt = (int)c->nt;
@@ -2097,6 +2096,11 @@ int eval_direct(sph_ctx *c, int fp64, void *s_dev) {
     A.kp64.self_int = c->self_int;
     A.self_mode = c->self_mode; A.nx = c->nx; A.ny = c->ny; A.fp64 = fp64;
     A.out = s_dev;
+    if (fp64) {   // without room for the table the pairs are summed without it
+        A.table_entries = direct_table_entries(c->ns, c->nt, c->nx, c->ny, c->nz);
+        if (A.table_entries && ensure(c, c->b_dtab, A.table_entries * sizeof(double)) == SPH_OK) A.table = P<double>(c->b_dtab);
+        if (c->poisoned) return SPH_ECUDA;
+    }
     if (direct_launch(A, c->stream) != 0) CK(cudaGetLastError());
     return SPH_OK;
 }

@@ -51,7 +51,6 @@ int select_launch(const SelectArgs &A, cudaStream_t st);
 struct DirectArgs {
     const uint32_t *src_pc;
     const float *src_q;
-    float wscale;
     int ns;
     const uint32_t *trg_key;         // Morton keys of the targets (cells by key_pc)
     int nt;
@@ -59,7 +58,11 @@ struct DirectArgs {
     KParams64 kp64;
     int self_mode, nx, ny, fp64;
     void *out;
+    double *table = nullptr;         // FP64: room for table_entries pair weights (none: G per pair)
+    int64_t table_entries = 0;
 };
+// entries of the FP64 pair-weight table for these sets, 0 where it does not pay
+int64_t direct_table_entries(int64_t ns, int64_t nt, int nx, int ny, int nz);
 int direct_launch(const DirectArgs &A, cudaStream_t st);
 
 // ---------------------------------------------------------------- tree

@@ -1,0 +1,66 @@
+"""The direct sums where their forms change: FP64 with the pair weights in shared memory, in global
+memory or formed pair by pair; FP32 with chunks of sources that are far, near or meet the targets,
+with and without the series form, one and four warps a CTA, and counts that fill no tile."""
+import numpy as np
+import pytest
+
+import oracle
+import sph_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sph():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2112_10059_gb300 as m
+    return m
+
+
+# nx, ny, nz, h (cm), pressure (Torr), share of the cells that are sources, targets (share of a random mask)
+CASES = [(24, 24, 24, 0.2 / 24, 760.0, 1.0, 1.0),        # all pairs, weights in shared memory
+         (40, 24, 33, 1e-3, 76.0, 0.02, 0.3),            # R small enough for the series form
+         (40, 24, 33, 1e-2, 760.0, 0.02, 0.3),
+         (200, 9, 7, 5e-3, 760.0, 0.03, 0.5),            # 39,702 weights: global memory
+         (64, 50, 41, 1.0 / 64, 760.0, 3.5 / 131200, 3.5 / 131200),   # a few pairs: no table
+         (96, 96, 96, 1.0 / 96, 380.0, 3e-4, 1.0),       # four warps a CTA, mostly far chunks
+         (1, 1, 1, 0.01, 760.0, 1.0, 1.0)]
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_direct_forms(sph, case):
+    import torch
+    nx, ny, nz, h, p, fs, ft = case
+    n = nx * ny * nz
+    u = si.uniform01(77, n)
+    q = np.where(u <= fs, 0.5 + 0.5 * si.uniform01(78, n), 0.0).astype(np.float32)
+    q[np.argmin(u)] = 1.0
+    mask = (si.uniform01(79, n) <= ft).astype(np.uint8)
+    mask[n // 2] = 1
+    ctx = sph.Context(0)
+    pO2 = si.pO2_of(p)
+    sph.set_grid(ctx, nx, ny, nz, h, pO2)
+    qd, md = torch.from_numpy(q).cuda(), torch.from_numpy(mask).cuda()
+    sph.set_sources(ctx, qd, 0.01)
+    sph.set_targets(ctx, mask=md)
+    sph.set_criteria(ctx, 0.25)
+    J = np.nonzero(q >= 0.25)[0].astype(np.int32)
+    T = np.nonzero(mask)[0].astype(np.int32)
+    if T.size * J.size > 2e8:                # a sample of the targets is checked
+        S = T[:: max(1, int(T.size * J.size / 2e8) + 1)]
+    else:
+        S = T
+    alpha, beta = oracle.alpha_beta(pO2, 0.035, 2.0)
+    ref = oracle.sph(nx, ny, nz, h, alpha, beta, q, 0.01, J, S)
+    d64 = sph.eval_direct(ctx, fp64=True).cpu().numpy()
+    assert np.max(np.abs(d64[S] / ref - 1)) < 1e-13
+    off = np.ones(n, bool)
+    off[T] = False
+    assert np.all(d64[off] == 0)
+    d32 = sph.eval_direct(ctx, fp64=False).cpu().numpy().astype(np.float64)
+    # positive terms added one after another in FP32, each within a few ulp of the approximate
+    # exponentials and root (arguments up to 40 in log2 units: 2^-24 of them)
+    tol = J.size * 2.0 ** -24 + 8e-6
+    assert np.max(np.abs(d32[S] / ref - 1)) < tol
+    assert np.all(d32[off] == 0)
