@@ -153,8 +153,9 @@ int set_criteria(sph_ctx *ctx, double i_frac, double e_frac, double e_applied,
  * Default: SPH_FAR_CHEBYSHEV, 5.  Takes effect at the next eval. */
 int sph_set_far_field(sph_ctx *ctx, int method, int order);
 
-/* Near field (Eq. nearfar, the exact part): SPH_NEAR_EXP evaluates the kernel with its
- * exponentials for every source-target pair (default); SPH_NEAR_TABLE reads G for the integer
+/* Near field (Eq. nearfar, the exact part): SPH_NEAR_EXP (default) uses the kernel's
+ * exponential form: once per cell offset and block between leaves of edge 4 or less, whose offsets
+ * are few, per source-target pair elsewhere; SPH_NEAR_TABLE reads G for the integer
  * squared cell offsets below 4096 from a table built per evaluation with the same arithmetic
  * (uniform grids make every offset an integer); SPH_NEAR_AUTO times both on the first eval
  * of each problem class and keeps the faster.  Takes effect at the next eval. */

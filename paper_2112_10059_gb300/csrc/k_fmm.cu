@@ -1146,6 +1146,209 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p(FmmDev F, const int *__r
     }
 }
 
+static P2PConst p2p_const(const FmmDev &F) {
+    P2PConst K;
+    const float h = F.kp.h;
+    K.k1 = F.kp.a2 * h;                       // a2 = alpha log2(e)
+    K.k2 = F.kp.b2 * h;                       // b2 = (beta - alpha) log2(e)
+    K.bma_h = F.kp.bma * h;
+    K.k12 = K.k1 + K.k2;
+    // the self weight multiplies the scaled weight w' = w C / h^3: g_self w = (g_self h^3 / C) w'
+    K.wself = F.self_mode ? F.kp.gself * h * h * h / F.kp.C : 0.f;
+    return K;
+}
+
+// ---------------------------------------------------------------- near field (U lists) by offset table
+// Between leaves of edge 4 or less (the deepest level at leaf sizes up to 511) every offset lies
+// in [-7, 7]^3, so the scaled kernel of the whole near field is a table of 15^3 values, formed by
+// the exp form itself once per CTA.  A point's cell is one integer lin = x + 20 y + 304 z and a
+// pair's entry lin_s - lin_t + centre; with these pitches the 32 targets of a full half leaf
+// (4 x 4 x 2 cells) fall into 32 different banks for any source, so a pair costs one conflict-free
+// shared load and one FMA: bound by shared-memory wavefronts (1.25 per 32 pairs with the broadcast
+// of the source; 25 pairs per SM and clock) instead of three special-function results (8).  Four
+// warps share a leaf's sources, each lane sums two targets, and the warps' sums are added in
+// order.  Entries of larger leaves take the exp form (the staged points and p2p_sum below).
+// Uniform 128^3 (3.4e9 pairs): 2290 us by the exp form alone, 670 us so; wide streamer 192^3:
+// 996, 290.
+constexpr int NG_PY = 20, NG_PZ = 304, NG_CENTRE = 7 * (1 + NG_PY + NG_PZ), NG_N = 2 * NG_CENTRE + 1;
+constexpr int NG_CAP = 2048;         // staged points per round (16 KiB; 1024 in the exp form)
+
+__device__ __forceinline__ int near_lin(uint32_t pc) { return pc_i(pc) + NG_PY * pc_j(pc) + NG_PZ * pc_k(pc); }
+
+// sums of sources [lo, hi) (even, in pairs) for the targets at byte offsets b0 and b1 of the table
+template <bool TWO>
+__device__ __forceinline__ void near_grid_sum(const int2 *__restrict__ pts, int lo, int hi, const char *__restrict__ b0,
+                                              const char *__restrict__ b1, float &a0, float &a1) {
+#pragma unroll 4
+    for (int j = lo; j < hi; j += 2) {
+        const int4 v = *reinterpret_cast<const int4 *>(pts + j);
+        a0 = fmaf(*reinterpret_cast<const float *>(b0 + v.x), __int_as_float(v.y), a0);
+        if (TWO) a1 = fmaf(*reinterpret_cast<const float *>(b1 + v.x), __int_as_float(v.y), a1);
+        a0 = fmaf(*reinterpret_cast<const float *>(b0 + v.z), __int_as_float(v.w), a0);
+        if (TWO) a1 = fmaf(*reinterpret_cast<const float *>(b1 + v.z), __int_as_float(v.w), a1);
+    }
+}
+
+template <bool TAYLOR>
+__global__ void __launch_bounds__(P2P_WARPS * 32) k_near_grid(FmmDev F, const int *__restrict__ list,
+                                                              const int *__restrict__ count, int stride, P2PConst K) {
+    pdl_enter();
+    __shared__ float tab[NG_N + 1];
+    __shared__ __align__(16) int2 stage[NG_CAP];
+    __shared__ int eb[P2P_MAXU], en[P2P_MAXU], eo[P2P_MAXU];   // entries: first source, count (negative: exp form), place
+    __shared__ int wsum[P2P_WARPS][2];
+    __shared__ int own_lo;                 // place of the leaf's own sources in the exp form's list, or -1
+    __shared__ float red[P2P_WARPS][64];
+    float4 *stage4 = reinterpret_cast<float4 *>(stage);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ int ccnt[P2P_CLASSES];
+    if (tid < P2P_CLASSES) ccnt[tid] = count[tid];
+    __syncthreads();
+    int nitems = 0;
+#pragma unroll
+    for (int c = 0; c < P2P_CLASSES; ++c) nitems += ccnt[c];
+    if ((int)blockIdx.x >= nitems) return;
+    for (int e = tid; e < NG_N; e += P2P_WARPS * 32) {
+        const int dz = e / NG_PZ - 7, dy = e % NG_PZ / NG_PY - 7, dx = e % NG_PZ % NG_PY - 7;
+        const float d2 = (float)(dx * dx + dy * dy + dz * dz);
+        tab[e] = e == NG_CENTRE ? K.wself : p2p_g<TAYLOR>(fmaxf(d2, 1.f), K);
+    }
+    const TreeDev &T = F.T;
+    const float h = F.kp.h;
+    const float wsc = F.wscale * F.kp.C / (h * h * h);          // source weight -> scaled weight
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        int c = 0, j = it;
+        while (c < P2P_CLASSES - 1 && j >= ccnt[c]) j -= ccnt[c++];
+        const int b = list[(size_t)c * stride + j];
+        const int tb = T.b_tb[b], nt = T.b_te[b] - tb, lv = T.b_level[b];
+        const int l0 = F.L.u_off[b], l1 = F.L.u_off[b + 1];
+        float *nslot = F.near_buf + (size_t)it * F.near_s;
+        const bool small_b = F.D - lv <= 2;
+        const bool full = F.D - lv == 2 && nt == 64;
+        uint32_t bx, by, bz;
+        demorton3(T.b_key[b], bx, by, bz);
+        const int corner = ((int)bx + NG_PY * (int)by + NG_PZ * (int)bz) << (F.D - lv);   // lin of the leaf's lowest cell
+        for (int c0 = 0; c0 < nt; c0 += 64) {                   // 64 targets at a time
+            const bool two = c0 + 32 < nt;
+            // lanes past the end repeat the last target (their sums are not written)
+            const uint32_t p0 = key_pc(F.trg_key[tb + min(c0 + lane, nt - 1)]);
+            const uint32_t p1 = key_pc(F.trg_key[tb + min(c0 + 32 + lane, nt - 1)]);
+            const char *b0 = reinterpret_cast<const char *>(tab + (NG_CENTRE - (small_b ? near_lin(p0) - corner : 0)));
+            const char *b1 = reinterpret_cast<const char *>(tab + (NG_CENTRE - (small_b ? near_lin(p1) - corner : 0)));
+            float a0 = 0.f, a1 = 0.f;
+            for (int ub0 = l0; ub0 < l1; ub0 += P2P_MAXU) {
+                // the entries' places in the list of their form (one entry per thread)
+                __syncthreads();
+                const int nu = min(P2P_MAXU, l1 - ub0);
+                int A = -1, sb = 0, cnt = 0;
+                if (tid < nu) {
+                    A = F.L.u_src[ub0 + tid];
+                    sb = T.b_sb[A];
+                    cnt = T.b_se[A] - sb;
+                }
+                const bool grid = small_b && A >= 0 && F.D - T.b_level[max(A, 0)] <= 2;
+                int s0 = grid ? cnt : 0, s1 = grid ? 0 : cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int q0 = __shfl_up_sync(0xffffffffu, s0, o), q1 = __shfl_up_sync(0xffffffffu, s1, o);
+                    if (lane >= o) {
+                        s0 += q0;
+                        s1 += q1;
+                    }
+                }
+                if (lane == 31) {
+                    wsum[warp][0] = s0;
+                    wsum[warp][1] = s1;
+                }
+                if (tid == 0) own_lo = -1;
+                __syncthreads();
+                int n0 = 0, n1 = 0, w0 = 0, w1 = 0;
+#pragma unroll
+                for (int w = 0; w < P2P_WARPS; ++w) {
+                    if (w == warp) {
+                        w0 = n0;
+                        w1 = n1;
+                    }
+                    n0 += wsum[w][0];
+                    n1 += wsum[w][1];
+                }
+                if (tid < nu) {
+                    eb[tid] = sb;
+                    en[tid] = grid ? cnt : -cnt;
+                    eo[tid] = grid ? w0 + s0 - cnt : w1 + s1 - cnt;
+                    if (!grid && A == b) own_lo = w1 + s1 - cnt;
+                }
+                for (int r0 = 0; r0 < n0; r0 += NG_CAP) {       // table form
+                    __syncthreads();
+                    const int rn = min(NG_CAP, n0 - r0), rp = (rn + 1) & ~1;
+#pragma unroll 2
+                    for (int e = warp; e < nu; e += P2P_WARPS) {
+                        const int m = en[e], at = eo[e] - r0, first = eb[e];
+#pragma unroll 2
+                        for (int q = lane; q < m; q += 32)
+                            if ((unsigned)(at + q) < (unsigned)NG_CAP)
+                                stage[at + q] = make_int2(4 * (near_lin(__ldg(F.src_pc + first + q)) - corner),
+                                                          __float_as_int(__ldg(F.src_q + first + q) * wsc));
+                    }
+                    // the odd one out: no weight, at the leaf's own first target (inside the table)
+                    if (tid == 0 && rp > rn) stage[rn] = make_int2(4 * (near_lin(p0) - corner), 0);
+                    __syncthreads();
+                    const int per = ((rp + 2 * P2P_WARPS - 1) / (2 * P2P_WARPS)) * 2;
+                    const int lo = min(rp, warp * per), hi = min(rp, lo + per);
+                    if (full) near_grid_sum<true>(stage, lo, hi, b0, b0 - 8 * NG_PZ, a0, a1);
+                    else if (two) near_grid_sum<true>(stage, lo, hi, b0, b1, a0, a1);
+                    else near_grid_sum<false>(stage, lo, hi, b0, b1, a0, a1);
+                }
+                for (int r0 = 0; r0 < n1; r0 += NG_CAP / 2) {   // exp form
+                    __syncthreads();
+                    const int rn = min(NG_CAP / 2, n1 - r0);
+                    for (int e = warp; e < nu; e += P2P_WARPS) {
+                        const int m = -en[e], at = eo[e] - r0, first = eb[e];
+                        for (int q = lane; q < m; q += 32)
+                            if ((unsigned)(at + q) < (unsigned)(NG_CAP / 2)) {
+                                const uint32_t pc = __ldg(F.src_pc + first + q);
+                                stage4[at + q] = make_float4((float)pc_i(pc), (float)pc_j(pc), (float)pc_k(pc),
+                                                             __ldg(F.src_q + first + q) * wsc);
+                            }
+                    }
+                    __syncthreads();
+                    const int per = (rn + P2P_WARPS - 1) / P2P_WARPS;
+                    const int lo = min(rn, warp * per), hi = min(rn, lo + per);
+                    // only the leaf's own cells can be the target's cell
+                    const int own = own_lo, own_n = T.b_se[b] - T.b_sb[b];
+                    const int olo = own >= 0 ? min(max(own - r0, lo), hi) : hi;
+                    const int ohi = own >= 0 ? min(max(own + own_n - r0, olo), hi) : hi;
+                    for (int k = 0; k < (two ? 2 : 1); ++k) {
+                        const uint32_t tp = k ? p1 : p0;
+                        const float fx = (float)pc_i(tp), fy = (float)pc_j(tp), fz = (float)pc_k(tp);
+                        float a = p2p_sum<TAYLOR, false>(stage4, lo, olo, fx, fy, fz, K, nullptr);
+                        if (olo < ohi) a += p2p_sum<TAYLOR, false, true>(stage4, olo, ohi, fx, fy, fz, K, nullptr);
+                        a += p2p_sum<TAYLOR, false>(stage4, ohi, hi, fx, fy, fz, K, nullptr);
+                        if (k) a1 += a;
+                        else a0 += a;
+                    }
+                }
+            }
+            red[warp][lane] = a0;
+            red[warp][32 + lane] = a1;
+            __syncthreads();
+            if (tid < 64 && c0 + tid < nt) nslot[c0 + tid] = (red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid]);
+            __syncthreads();
+        }
+    }
+}
+
+void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, cudaStream_t st,
+                   int per_sm) {
+    if (nboxes <= 0) return;
+    const int grid = std::min(nboxes, 152 * per_sm);
+    const P2PConst K = p2p_const(F);
+    if (K.bma_h >= 0.5f)
+        launch_pdl(k_near_grid<false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K);
+    else
+        launch_pdl(k_near_grid<true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K);
+}
+
 // out[cell of t] += near_buf[slot of t]: one warp per leaf of the class lists (the items in the
 // near field's order); every target belongs to one leaf, so plain read-modify-writes suffice
 __global__ void __launch_bounds__(256) k_near_add(FmmDev F, const int *__restrict__ list,
@@ -1173,18 +1376,6 @@ __global__ void __launch_bounds__(256) k_near_add(FmmDev F, const int *__restric
             out[(int64_t)pc_i(tp) + (int64_t)F.nx * ((int64_t)pc_j(tp) + (int64_t)F.ny * pc_k(tp))] += ns[t - tb];
         }
     }
-}
-
-static P2PConst p2p_const(const FmmDev &F) {
-    P2PConst K;
-    const float h = F.kp.h;
-    K.k1 = F.kp.a2 * h;                       // a2 = alpha log2(e)
-    K.k2 = F.kp.b2 * h;                       // b2 = (beta - alpha) log2(e)
-    K.bma_h = F.kp.bma * h;
-    K.k12 = K.k1 + K.k2;
-    // the self weight multiplies the scaled weight w' = w C / h^3: g_self w = (g_self h^3 / C) w'
-    K.wself = F.self_mode ? F.kp.gself * h * h * h / F.kp.C : 0.f;
-    return K;
 }
 
 void fmm_near_table(const FmmDev &F, float *gtab, cudaStream_t st) {

@@ -770,18 +770,19 @@ bool m2l_target_tiles(const sph_ctx *c, const PassState &S) {
                     (c->m2l_tiles == 2 && (c->m2l_form >= 0 ? c->m2l_form == 1 : nV >= 32 * nb)));
 }
 
-// CTAs per SM of the overlapped near field's U-list launch.  Where the far-field chain is the
-// longer of the two, 6 (measured best at the 256^3 headline) leave slots to its kernels; where
-// the near field is the longer one (every cell a source: the uniform 128^3 tree), it gets the
-// whole machine (16; measured best there).  Estimates from the list totals: near-field
-// evaluations at most U entries x leaf size^2 at 1.6e12/s; far field a fixed 150 us plus the
-// M2L at its measured cost per V pair (0.45 ns in pair tiles, 0.19 ns in target tiles).
+// CTAs per SM of the overlapped near field's U-list launch.  Five fit beside each other (37 KB of
+// shared memory each); where the far-field chain is the longer of the two, four leave slots to its
+// kernels (256^3 headline: 458 us with 4, 464 with 5, 467 with 6; uniform 128^3: 2830, 2813, 2811).
+// Estimates from the list totals: near-field pairs at most U entries x leaf size^2 at 5e12/s; far
+// field a fixed 150 us plus the M2L at its measured cost per V pair (0.45 ns in pair tiles, 0.19 ns
+// in target tiles).  The tabulated near field keeps its own figures (1.6e12/s, 16 and 6).
 int near_cap(const sph_ctx *c, const PassState &S) {
     if (c->near_per_sm > 0) return c->near_per_sm;
     const double s = c->leaf_eff;
-    const double near_us = (double)c->list_tot[0] * s * s / 1.6e6;
+    const bool table = S.F.gtab != nullptr;
+    const double near_us = (double)c->list_tot[0] * s * s / (table ? 1.6e6 : 5e6);
     const double far_us = 150.0 + (double)c->list_tot[1] * (m2l_target_tiles(c, S) ? 0.19e-3 : 0.45e-3);
-    return near_us > far_us ? 16 : 6;
+    return near_us > far_us ? (table ? 16 : 5) : (table ? 6 : 4);
 }
 
 // Queue the passes on c->stream: memsets and kernels only (no allocation, no sync).
@@ -820,7 +821,10 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
             ++c->launches;
         }
         if (tm) tm->mark_at(12, c->near_stream);
-        fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, S));
+        if (F.gtab)
+            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, S));
+        else
+            fmm_near_grid(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), c->near_stream, near_cap(c, S));
         ++c->launches;
         if (tm) tm->mark_at(14, c->near_stream);
     }

@@ -297,6 +297,9 @@ void fmm_work_lists(const FmmDev &F, int nboxes, int *src_list, int *src_cnt, in
 void fmm_p2p(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,
              cudaStream_t st, int pass_lo = 0, int pass_hi = 2, int per_sm = 16, const int *w_list = nullptr,
              const int *w_cnt = nullptr, int max_w = 0);
+// the U-list part into the leaves' slots of F.near_buf by the offset table, for the same lists
+void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, cudaStream_t st,
+                   int per_sm);
 // out[cell of t] += F.near_buf[slot of t] for every target of every leaf of those lists
 // flags / flags_host (optional): flags[0..2) copied to the mapped host address flags_host once
 // every earlier kernel of the stream has completed

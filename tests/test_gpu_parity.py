@@ -261,6 +261,29 @@ def test_graph_reuse_follows_the_arguments(sph):
         assert oracle.rel_l2(o, ref) < 1e-6
 
 
+@pytest.mark.parametrize("p_torr", [76.0, 760.0])
+@pytest.mark.parametrize("leaf", [8, 32, 64, 128, 600])
+def test_near_field_offset_table(sph, monkeypatch, leaf, p_torr):
+    """The near field by the offset table between small leaves (edges 2 and 4, full and partly
+    selected ones, lists of both forms, leaves of several 64-target chunks) against the exp form of
+    every pair (SPH_NEAR_OVERLAP=0): the same kernel values, added in another order.  Per target at
+    most 27 x 64 + 600 positive FP32 terms whose partial sums round by 2^-24: 1e-6 is 4 sigma."""
+    p = si.streamer(n=40, box=0.35, p_torr=p_torr, chan_len=0.15, i_frac=1e-3, targets_all=True, leaf_size=leaf,
+                    sigma_head=0.03, chan_radius=0.03, seed=31)
+    mask = si.random_mask(p.ncell, 0.6, 32)
+    mask.reshape(40, 40, 40)[:20, :20] = 1          # whole leaves beside partly selected ones
+    outs = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("SPH_NEAR_OVERLAP", flag)
+        c = sph.Context(0)
+        _, out, _ = sph.solve(p, c, m2l_precision=sph.M2L_F32, mask=mask)
+        outs.append(out.cpu().numpy().astype(np.float64))
+        c.close()
+    T = np.nonzero(mask)[0]
+    assert oracle.rel_l2(outs[0][T], outs[1][T]) < 1e-6
+    assert np.array_equal(outs[0] == 0, outs[1] == 0)
+
+
 def test_direct_fp64_and_fp32_c0(sph, ctx):
     p = si.plain_24()
     sph.solve(p, ctx)
