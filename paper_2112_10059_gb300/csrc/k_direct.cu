@@ -20,10 +20,10 @@ namespace sph {
 //   - far: e^{-(beta - alpha) R} < 2^-25, so that 1 - it is 1 in FP32 and its ex2 is left out;
 //   - near: both exponentials;
 //   - general: the boxes meet (a source may be the target's own cell) or R is small enough for
-//     the series form of 1 - e^{-x} (g_of_cells, pair by pair).
+//     the series form of 1 - e^{-x} (general_g, pair by pair).
 // 160^3 cells, 7,072 sources (2.9e10 pairs): 28.2 ms pair by pair with integer offsets (their
 // conversion is a fourth result of the same unit), 10.5 ms so.
-constexpr int DS = 512;    // sources per shared-memory tile
+constexpr int DS = 256;    // sources per shared-memory tile
 constexpr int DC = 32;     // sources per chunk
 
 struct F2 {
@@ -61,19 +61,37 @@ struct DirectK {
     float wscale;       // source_scale C (the 1 / h^3 of G and the cell volume cancel)
     float self;         // ball integral / C, or 0
     float far2, near2;  // squared distances (cells) from which a chunk is far / near
-    KParams kp;         // general form: g_of_cells h^3 / C
-    float general;      // h^3 / C
+    float bma_h;        // (beta - alpha) h
 };
 
-__global__ void __launch_bounds__(128) k_direct_f32(const uint32_t *__restrict__ src_pc,
+// G h^3 / C at squared distance d2 >= 1 (cells), for any R: both forms of 1 - e^{-x} and a selection,
+// so that the pairs of a chunk overlap (one_minus_exp_neg branches)
+__device__ __forceinline__ float general_g(float d2, const DirectK &k) {
+    const float ir = rsqrt_approx(d2), R = d2 * ir, x = k.bma_h * R;
+    float p = -2.4801587301587302e-05f;            // x (1 - x/2! + x^2/3! - ... - x^7/8!)
+    p = fmaf(p, x, 1.9841269841269841e-04f);
+    p = fmaf(p, x, -1.3888888888888889e-03f);
+    p = fmaf(p, x, 8.3333333333333333e-03f);
+    p = fmaf(p, x, -4.1666666666666667e-02f);
+    p = fmaf(p, x, 1.6666666666666667e-01f);
+    p = fmaf(p, x, -0.5f);
+    p = fmaf(p, x, 1.0f) * x;
+    const float em = x < 0.5f ? p : 1.f - ex2_approx(-k.b2 * R);
+    return ex2_approx(-k.a2 * R) * em * (ir * ir * ir);
+}
+
+constexpr int WARPS = 4;
+
+__global__ void __launch_bounds__(32 * WARPS) k_direct_f32(const uint32_t *__restrict__ src_pc,
                                                     const float *__restrict__ src_q, int ns,
                                                     const uint32_t *__restrict__ trg_key, int nt, DirectK k, int nx,
                                                     int ny, float *__restrict__ out_dense) {
     __shared__ float4 sxy[DS], szs[DS];   // {x, x, y, y}, {z, z, x^2 + y^2 + z^2 twice}
     __shared__ float2 sw[DS];
     __shared__ int box[DS / DC][6];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int t0 = (blockIdx.x * nwarps + warp) * 64 + lane;
+    constexpr int Q = DS / DC / WARPS;     // chunks a warp stages
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t0 = (blockIdx.x * WARPS + warp) * 64 + lane;
     // targets past the end repeat the last one (their sums are not written)
     const uint32_t pa = key_pc(trg_key[min(t0, nt - 1)]), pb = key_pc(trg_key[min(t0 + 32, nt - 1)]);
     const int ax = pc_i(pa), ay = pc_j(pa), az = pc_k(pa), bx = pc_i(pb), by = pc_j(pb), bz = pc_k(pb);
@@ -84,24 +102,34 @@ __global__ void __launch_bounds__(128) k_direct_f32(const uint32_t *__restrict__
     const F2 tt = f2((float)(ax * ax + ay * ay + az * az), (float)(bx * bx + by * by + bz * bz));
     const F2 a2 = f2(-k.a2, -k.a2), b2 = f2(-k.b2, -k.b2);
     F2 acc = f2(0.f, 0.f);
+    uint32_t np[Q];                        // the next tile's sources, loaded under this one's pairs
+    float nq[Q];
+    auto fetch = [&](int s0) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int s = min(s0 + (warp + i * WARPS) * DC + lane, ns - 1);
+            np[i] = src_pc[s];
+            nq[i] = src_q[s];
+        }
+    };
+    if (ns > 0) fetch(0);
     for (int s0 = 0; s0 < ns; s0 += DS) {
         const int m = min(DS, ns - s0);
         __syncthreads();
-        for (int u = warp * DC; u < m; u += nwarps * DC) {   // a warp stages a chunk and its box
-            const int s = min(u + lane, m - 1);
-            const uint32_t p = src_pc[s0 + s];
-            const int x = pc_i(p), y = pc_j(p), z = pc_k(p);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {          // a warp stages a chunk and its box (past the end: the last source)
+            const int u = (warp + i * WARPS) * DC + lane;
+            const int x = pc_i(np[i]), y = pc_j(np[i]), z = pc_k(np[i]);
             const float fx = (float)x, fy = (float)y, fz = (float)z, ss = (float)(x * x + y * y + z * z);
-            const float w = src_q[s0 + s] * k.wscale;
-            if (u + lane < m) {
-                sxy[u + lane] = make_float4(fx, fx, fy, fy);
-                szs[u + lane] = make_float4(fz, fz, ss, ss);
-                sw[u + lane] = make_float2(w, w);
-            }
+            const float w = nq[i] * k.wscale;
+            sxy[u] = make_float4(fx, fx, fy, fy);
+            szs[u] = make_float4(fz, fz, ss, ss);
+            sw[u] = make_float2(w, w);
             const int b0 = __reduce_min_sync(~0u, x), b1 = __reduce_max_sync(~0u, x), b2_ = __reduce_min_sync(~0u, y);
             const int b3 = __reduce_max_sync(~0u, y), b4 = __reduce_min_sync(~0u, z), b5 = __reduce_max_sync(~0u, z);
             if (lane < 6) box[u / DC][lane] = lane == 0 ? b0 : lane == 1 ? b1 : lane == 2 ? b2_ : lane == 3 ? b3 : lane == 4 ? b4 : b5;
         }
+        if (s0 + DS < ns) fetch(s0 + DS);
         __syncthreads();
         for (int c = 0; c < m; c += DC) {
             const int *b = box[c / DC];
@@ -139,10 +167,11 @@ __global__ void __launch_bounds__(128) k_direct_f32(const uint32_t *__restrict__
                     acc = f2_fma(g, f2(sw[u].x, sw[u].y), acc);
                 }
             } else {
+#pragma unroll 4
                 for (int u = c; u < end; ++u) {
                     const float2 dd = f2_get(dist2(u));
-                    const float ga = dd.x > 0.f ? g_of_cells((int)dd.x, k.kp) * k.general : k.self;
-                    const float gb = dd.y > 0.f ? g_of_cells((int)dd.y, k.kp) * k.general : k.self;
+                    const float ga = dd.x > 0.f ? general_g(fmaxf(dd.x, 1.f), k) : k.self;
+                    const float gb = dd.y > 0.f ? general_g(fmaxf(dd.y, 1.f), k) : k.self;
                     acc = f2_fma(f2(ga, gb), f2(sw[u].x, sw[u].y), acc);
                 }
             }
@@ -151,6 +180,36 @@ __global__ void __launch_bounds__(128) k_direct_f32(const uint32_t *__restrict__
     const float2 r = f2_get(acc);
     if (t0 < nt) out_dense[(int64_t)ax + (int64_t)nx * ((int64_t)ay + (int64_t)ny * az)] = r.x;
     if (t0 + 32 < nt) out_dense[(int64_t)bx + (int64_t)nx * ((int64_t)by + (int64_t)ny * bz)] = r.y;
+}
+
+// The same sums with one target a thread and the general form throughout: where the targets are
+// too few to fill the chip the longest warp counts, and a warp of 64 targets is long where its
+// chunks are not far (37,692 targets x 218 sources: 62 us a call against 74 in pairs).
+__global__ void __launch_bounds__(128) k_direct_f32_few(const uint32_t *__restrict__ src_pc,
+                                                        const float *__restrict__ src_q, int ns,
+                                                        const uint32_t *__restrict__ trg_key, int nt, DirectK k, int nx,
+                                                        int ny, float *__restrict__ out_dense) {
+    __shared__ float4 sp[512];
+    const int t = blockIdx.x * 128 + threadIdx.x;
+    const uint32_t tp = key_pc(trg_key[min(t, nt - 1)]);
+    const float tx = (float)pc_i(tp), ty = (float)pc_j(tp), tz = (float)pc_k(tp);
+    float acc = 0.f;
+    for (int s0 = 0; s0 < ns; s0 += 512) {
+        const int m = min(512, ns - s0);
+        __syncthreads();
+        for (int u = threadIdx.x; u < m; u += 128) {
+            const uint32_t p = src_pc[s0 + u];
+            sp[u] = make_float4((float)pc_i(p), (float)pc_j(p), (float)pc_k(p), src_q[s0 + u] * k.wscale);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int u = 0; u < m; ++u) {
+            const float4 p = sp[u];
+            const float dx = tx - p.x, dy = ty - p.y, dz = tz - p.z, d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            acc = fmaf(d2 > 0.f ? general_g(fmaxf(d2, 1.f), k) : k.self, p.w, acc);
+        }
+    }
+    if (t < nt) out_dense[(int64_t)pc_i(tp) + (int64_t)nx * ((int64_t)pc_j(tp) + (int64_t)ny * pc_k(tp))] = acc;
 }
 
 // ---------------------------------------------------------------- FP64
@@ -302,15 +361,18 @@ int direct_launch(const DirectArgs &A, cudaStream_t st) {
         k.b2 = (float)(d.bma * d.h * log2e);
         k.wscale = (float)(d.scale * d.C);
         k.self = A.self_mode ? (float)(d.self_int / d.C) : 0.f;
-        k.kp = A.kp;
-        k.general = (float)(d.vol / d.C);
+        k.bma_h = (float)(d.bma * d.h);
         const double far = 25.5 / (d.bma * d.h * log2e), near = std::max(1.0, 0.5 / (d.bma * d.h));
         k.far2 = (float)std::max(far * far, near * near);
         k.near2 = (float)(near * near);
         // 64 targets a warp: four warps a CTA share the staged tile where that still fills the chip
-        const int warps = A.nt >= 256 * 152 * 4 ? 4 : 1;
-        k_direct_f32<<<(A.nt + 64 * warps - 1) / (64 * warps), 32 * warps, 0, st>>>(A.src_pc, A.src_q, A.ns, A.trg_key, A.nt, k,
-                                                                                    A.nx, A.ny, (float *)A.out);
+        // pairs of targets from three CTAs of 256 targets an SM on
+        if (A.nt >= 256 * 152 * 3)
+            k_direct_f32<<<(A.nt + 255) / 256, 32 * WARPS, 0, st>>>(A.src_pc, A.src_q, A.ns, A.trg_key, A.nt, k, A.nx, A.ny,
+                                                                    (float *)A.out);
+        else
+            k_direct_f32_few<<<(A.nt + 127) / 128, 128, 0, st>>>(A.src_pc, A.src_q, A.ns, A.trg_key, A.nt, k, A.nx, A.ny,
+                                                                 (float *)A.out);
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

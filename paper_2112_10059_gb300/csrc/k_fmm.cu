@@ -171,25 +171,122 @@ __device__ __forceinline__ void upward_box(const FmmDev &F, int level, int b) {
 }
 
 // CTAs walk the compact list of this level's boxes that hold sources.
-// leaves_only: the split boxes' M2M runs on the tensor cores (k_m2m_tc)
+// kinds: 0 every box, 1 the leaves alone (the split boxes' M2M runs on the tensor cores, k_m2m_tc),
+// 2 the split boxes alone (the leaves' P2M runs in k_p2m_small)
 __global__ void __launch_bounds__(2 * MAXPAD) k_upward(FmmDev F, int level, const int *__restrict__ list,
-                                                       const int *__restrict__ count, int leaves_only) {
+                                                       const int *__restrict__ count, int kinds) {
     pdl_enter();
     const int cnt = *count;
     for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
         const int b = list[i];
-        if (leaves_only && !F.T.b_leaf[b]) continue;   // uniform across the CTA
+        if (kinds != 0 && (kinds == 1) != (F.T.b_leaf[b] != 0)) continue;   // uniform across the CTA
         upward_box(F, level, b);
         __syncthreads();
     }
 }
 
-int fmm_upward_level(const FmmDev &F, int level, int box_count, const int *list, const int *count, bool leaves_only,
-                     cudaStream_t st) {
+// P2M of the leaves of edge 4 or less (Chebyshev): one warp per leaf.  The leaf's weights are laid
+// out on its 4^3 cells and anterpolated one axis after the other, 4 (16 p + 4 p^2 + p^3) FMAs
+// whatever the number of sources, from one basis of p x 4 values per level -- box by box, each source's
+// 3 p basis values and p^3 products were formed anew by a CTA (253 us for the 32,768 full leaves
+// of a uniform 128^3 tree, P2MFIG so).
+constexpr int P2M_WARPS = 8;
+
+template <int P>
+__global__ void __launch_bounds__(P2M_WARPS * 32) k_p2m_small(FmmDev F, int level, const int *__restrict__ list,
+                                                              const int *__restrict__ count) {
+    pdl_enter();
+    __shared__ float basis[P][4];
+    __shared__ __align__(16) float cells[P2M_WARPS][64], t1[P2M_WARPS][16 * P], t2[P2M_WARPS][4 * P * P];
+    __shared__ float tc[8], wc[8];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int size = 1 << (F.D - level);
+    if (tid < P) {
+        const float tk = F.O.cheb_t[tid];
+        float w = 1.f;
+        for (int j = 0; j < P; ++j)
+            if (j != tid) w *= tk - F.O.cheb_t[j];
+        tc[tid] = tk;
+        wc[tid] = 1.f / w;
+    }
+    __syncthreads();
+    if (tid < 4) {                            // cell i of the box at (2 i + 1) / size - 1
+        float S[8];
+        cheb_basis_w(P, tc, wc, (float)(2 * tid + 1 - size) / (float)size, S);
+        for (int k = 0; k < P; ++k) basis[k][tid] = tid < size ? S[k] : 0.f;
+    }
+    __syncthreads();
+    const TreeDev &T = F.T;
+    const int cnt = *count, np = F.O.npad;
+    for (int i = blockIdx.x * P2M_WARPS + warp; i < cnt; i += gridDim.x * P2M_WARPS) {
+        const int b = list[i];
+        const int sb = T.b_sb[b], ns = T.b_se[b] - sb;
+        if (!T.b_leaf[b]) continue;
+        float *cl = cells[warp], *x1 = t1[warp], *x2 = t2[warp];
+        __syncwarp();
+        cl[lane] = 0.f;
+        cl[32 + lane] = 0.f;
+        __syncwarp();
+        for (int s = lane; s < ns; s += 32) {
+            const uint32_t pc = __ldg(F.src_pc + sb + s);
+            cl[(pc_i(pc) & (size - 1)) + 4 * (pc_j(pc) & (size - 1)) + 16 * (pc_k(pc) & (size - 1))] =
+                __ldg(F.src_q + sb + s) * F.wscale;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = lane; o < 16 * P; o += 32) {         // [y + 4 z][a]
+            const int a = o % P;
+            const float4 v = *reinterpret_cast<const float4 *>(cl + 4 * (o / P));
+            x1[o] = fmaf(basis[a][3], v.w, fmaf(basis[a][2], v.z, fmaf(basis[a][1], v.y, basis[a][0] * v.x)));
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = lane; o < 4 * P * P; o += 32) {      // [z][b][a]
+            const int a = o % P, c = o / P % P;
+            const float *v = x1 + 4 * P * (o / (P * P)) + a;
+            x2[o] = fmaf(basis[c][3], v[3 * P], fmaf(basis[c][2], v[2 * P], fmaf(basis[c][1], v[P], basis[c][0] * v[0])));
+        }
+        __syncwarp();
+        float *u = F.ueq + (size_t)b * np;
+#pragma unroll
+        for (int o = lane; o < P * P * P; o += 32) {      // [c][b][a]
+            const int c = o / (P * P);
+            const float *v = x2 + o % (P * P);
+            u[o] = fmaf(basis[c][3], v[3 * P * P], fmaf(basis[c][2], v[2 * P * P], fmaf(basis[c][1], v[P * P], basis[c][0] * v[0])));
+        }
+        for (int o = P * P * P + lane; o < np; o += 32) u[o] = 0.f;
+    }
+}
+
+static void p2m_small_launch(const FmmDev &F, int level, int boxes, const int *list, const int *count, cudaStream_t st) {
+    const int grid = std::min((boxes + P2M_WARPS - 1) / P2M_WARPS, 152 * 8);
+    const int threads = P2M_WARPS * 32;
+    switch (F.O.order) {
+        case 2: launch_pdl(k_p2m_small<2>, grid, threads, 0, st, F, level, list, count); break;
+        case 3: launch_pdl(k_p2m_small<3>, grid, threads, 0, st, F, level, list, count); break;
+        case 4: launch_pdl(k_p2m_small<4>, grid, threads, 0, st, F, level, list, count); break;
+        case 5: launch_pdl(k_p2m_small<5>, grid, threads, 0, st, F, level, list, count); break;
+        case 6: launch_pdl(k_p2m_small<6>, grid, threads, 0, st, F, level, list, count); break;
+        case 7: launch_pdl(k_p2m_small<7>, grid, threads, 0, st, F, level, list, count); break;
+        default: launch_pdl(k_p2m_small<8>, grid, threads, 0, st, F, level, list, count); break;
+    }
+}
+
+int fmm_upward_level(const FmmDev &F, int level, int box_count, int leaf_count, const int *list, const int *count,
+                     bool leaves_only, cudaStream_t st) {
     if (box_count <= 0 || level < 2) return 0;
+    int kinds = leaves_only ? 1 : 0, launches = 0;
+    if (F.O.method == FAR_CHEB && F.D - level <= 2) {
+        if (leaf_count > 0) {
+            p2m_small_launch(F, level, box_count, list, count, st);
+            ++launches;
+        }
+        if (leaves_only || leaf_count == box_count) return launches;
+        kinds = 2;
+    }
     int grid = box_count < 152 * 8 ? box_count : 152 * 8;
-    launch_pdl(k_upward, grid, 2 * F.O.npad, 0, st, F, level, list, count, leaves_only ? 1 : 0);
-    return 1;
+    launch_pdl(k_upward, grid, 2 * F.O.npad, 0, st, F, level, list, count, kinds);
+    return launches + 1;
 }
 
 // Compact work lists: per level the boxes with sources (stored in the level's box range),

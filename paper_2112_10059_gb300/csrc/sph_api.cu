@@ -837,7 +837,8 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
         // with the tensor-core M2M the box-by-box kernel takes the leaves alone (P2M), and
         // neither kernel is launched on a level without its kind of box
         if (!m2m_tc || c->lvl_sleaf[l] > 0)
-            c->launches += fmm_upward_level(F, l, c->lvl_src[l], S.w_src + c->lvl_base[l], S.w_cnt + l, m2m_tc,
+            c->launches += fmm_upward_level(F, l, c->lvl_src[l], c->lvl_sleaf[l], S.w_src + c->lvl_base[l],
+                                            S.w_cnt + l, m2m_tc,
                                             c->stream);
         if (m2m_tc && l < c->Lmax && c->lvl_src[l] > c->lvl_sleaf[l]) {
             fmm_m2m_tc_level(F, l, c->lvl_src[l], S.w_src + c->lvl_base[l], S.w_cnt + l, F.O.m2m_img, S.err,

@@ -274,7 +274,7 @@ struct FmmDev {
     int near_s = 0;
 };
 // returns the number of kernels launched
-int fmm_upward_level(const FmmDev &F, int level, int box_count, const int *list, const int *count, bool leaves_only,
+int fmm_upward_level(const FmmDev &F, int level, int box_count, int leaf_count, const int *list, const int *count, bool leaves_only,
                      cudaStream_t st);
 // near-field leaves in classes by their number of kernel evaluations w: class c holds
 // P2P_CLASS0 >> c <= w < P2P_CLASS0 >> (c - 1) (class 0: w >= P2P_CLASS0, the last: the rest)
