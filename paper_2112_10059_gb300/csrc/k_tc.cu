@@ -297,84 +297,145 @@ __global__ void __launch_bounds__(256) k_m2l_tc(FmmDev F, PairsDev Pd, const uin
 }
 
 // ---------------------------------------------------------------- M2L, persistent tile loop
-// Two CTAs per SM, each taking tile blockIdx.x first and then the tiles gridDim.x + ticket (a
-// counter, cleared before the passes, so that CTAs that start late beside other kernels take
-// fewer), with the tensor memory and barriers set up once.  Per tile: (1) the previous tile's bulk reductions
-// have read the staged rows (the B tiles), (2) gather and split the 64 source rows, (3) MMAs
-// once the operator image has landed, (4) the next tile's pair indices while they run, (5) the
-// MMAs complete, (6) the next tile's operator image streams into the A tile, (7) the results
-// are staged in the B tiles and added into the targets by bulk reductions that complete under
-// the next tile's steps (1)-(2).  The same sums as k_m2l_tc.
-__global__ void __launch_bounds__(256) k_m2l_tc_loop(FmmDev F, PairsDev Pd, const uint16_t *__restrict__ images,
-                                                     int *err, int *ticket) {
+// Two CTAs per SM, each taking runs of `run` consecutive tiles (run blockIdx.x first, then
+// gridDim.x + ticket: a counter, cleared before the passes, so that CTAs that start late beside
+// other kernels take fewer), with the tensor memory and barriers set up once.  A tile's work is a
+// chain (gather, split, MMAs, staging, reductions), so everything that can be is taken out of it:
+//   - the 64 source rows of the next tile are loaded into registers while this tile's MMAs and
+//     epilogue run, and the pair indices of the tile after that, from one record per tile;
+//   - the operator image stays while the run's tiles share it (it was half of the 128 KB that a
+//     tile moved) and otherwise streams in under the epilogue;
+//   - the bulk reductions complete under the next tile's steps.
+// Per tile: (1) the previous tile's staged rows have been read, (2) the rows are split into the B
+// tiles, (3) MMAs once the image has landed, next loads issued, (4) the MMAs complete, (5) the
+// next image if it is another, (6) the results are staged in the B tiles and added into the
+// targets' rows.  The same sums as k_m2l_tc.
+// Wide streamer 192^3 (2.9 M pairs, 45 k tiles): 727 us with one tile a ticket, its rows and
+// indices loaded in the chain and an image a tile; M2LFIG so.
+__global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, const uint16_t *__restrict__ images,
+                                                        int *err, int *ticket, int run) {
     // prologue (the V pairs, their tiles and the operator images were written before the passes)
     extern __shared__ uint8_t smem_raw[];
     const int ntile = Pd.tile_off[Pd.nkeys];
-    if ((int)blockIdx.x >= ntile) return;                // uniform, before any allocation
+    if ((int)blockIdx.x * run >= ntile) return;          // uniform, before any allocation
     TcSmem s = carve(smem_raw);
-    __shared__ int s_src[2][TCN], s_dst[2][TCN];
-    __shared__ int s_ok, s_next;
+    __shared__ int s_src[3][TCN], s_dst[3][TCN], s_key[3];   // pair indices and key of tile j of this CTA, slot j % 3
+    __shared__ int s_tile[4];                            // the CTA's tile j, slot j % 4 (>= ntile: none)
+    __shared__ int s_ok;
     const int tid = threadIdx.x;
-    // pair indices of `tile` into slot `slot` (threads < TCN; each finds the tile's key itself)
-    auto tile_meta = [&](int tile, int slot) {
-        const int key = Pd.tile_key[tile];
-        const int p0 = Pd.off[key] + (tile - Pd.tile_off[key]) * TCN;
-        const int p1 = min(p0 + TCN, Pd.off[key + 1]);
-        const int q = p0 + tid;
-        s_src[slot][tid] = q < p1 ? Pd.src[q] : -1;
-        s_dst[slot][tid] = q < p1 ? Pd.trg[q] : -1;
-        return key;
-    };
     auto issue_image = [&](int key) {
         const uint16_t *img = images + (size_t)key * (2 * A_BYTES / 2);
         tc::mbar_expect_tx(tc::smem_u32(s.bar_a), 2 * A_BYTES);
         tc::bulk_g2s(tc::smem_u32(s.a_hi), img, A_BYTES, tc::smem_u32(s.bar_a));
         tc::bulk_g2s(tc::smem_u32(s.a_lo), img + A_BYTES / 2, A_BYTES, tc::smem_u32(s.bar_a));
     };
+    // record of a tile: {first pair, key << 7 | pairs}
+    auto record = [&](int tile) { return tile < ntile ? Pd.tile_rec[tile] : make_int2(0, 0); };
+    auto put_meta = [&](int slot, const int2 &rec, int src, int dst) {
+        s_src[slot][tid] = tid < (rec.y & 127) ? src : -1;
+        s_dst[slot][tid] = tid < (rec.y & 127) ? dst : -1;
+        if (tid == 0) s_key[slot] = rec.y >> 7;
+    };
     tile_setup(s);
+    int images_issued = 0, images_waited = 0;            // thread 0's
     if (tid < TCN) {
-        const int key0 = tile_meta(blockIdx.x, 0);
-        if (tid == 0) issue_image(key0);
+        const int2 r0 = record(blockIdx.x * run);
+        const int q = tid < (r0.y & 127) ? r0.x + tid : 0;
+        put_meta(0, r0, Pd.src[q], Pd.trg[q]);
+        if (tid == 0) {
+            issue_image(r0.y >> 7);
+            ++images_issued;
+        }
     }
     pdl_enter();
+    // thread 0 deals the tiles: the rest of a run, then the run of a ticket drawn a run ahead
+    int next = blockIdx.x * run + 1, end = min(blockIdx.x * run + run, ntile), drawn = 0;
+    auto deal = [&]() {
+        if (next >= end) {
+            const int r = drawn;
+            drawn = (int)gridDim.x + atomicAdd(ticket, 1);
+            next = min(r, ntile) * run;                  // r * run < 2^31: at most ntile + one run per CTA
+            end = min(next + run, ntile);
+            if (next >= ntile) {
+                next = end = ntile;
+                return ntile;
+            }
+        }
+        return next++;
+    };
+    if (tid == 0) {
+        drawn = (int)gridDim.x + atomicAdd(ticket, 1);
+        s_tile[0] = blockIdx.x * run;
+        s_tile[1] = deal();
+        s_tile[2] = deal();
+    }
+    __syncthreads();
     const uint32_t tmem = *s.tmem_base;
     const int np = F.O.npad, n = F.O.n;
     const int warp = tid >> 5, lane = tid & 31;
     const int q = warp & 3, i = q * 32 + lane;           // TMEM lane = operator row
     const int cbeg = (warp >> 2) * (TCN / 2);
     float *stage = reinterpret_cast<float *>(s.b_hi);    // TCN rows of TCK FP32 (the two B tiles)
-    int it = 0, flag = 0;
-    bool image_pending = true;                            // an image copy not yet waited for
-    for (int tile = blockIdx.x; tile < ntile; ++it) {
-        const int slot = it & 1;
-        if (tid == 0) s_next = (int)gridDim.x + atomicAdd(ticket, 1);
-        // (1) the previous tile's staged rows have been read (and slot's indices are visible)
+    float4 rows[8];                                      // rows warp, warp + 8, ... of the next tile, 16 bytes a lane
+    auto load_rows = [&](int slot) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int src = s_src[slot][warp + 8 * u];
+            rows[u] = src >= 0 ? __ldg(reinterpret_cast<const float4 *>(F.ueq + (size_t)src * np) + lane)
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    load_rows(0);
+    int2 rec = make_int2(0, 0);                          // record of the tile after the next (threads < TCN)
+    if (tid < TCN) {
+        const int2 r1 = record(s_tile[1]);
+        const int p = tid < (r1.y & 127) ? r1.x + tid : 0;
+        put_meta(1, r1, Pd.src[p], Pd.trg[p]);
+        rec = record(s_tile[2]);
+    }
+    int flag = 0, s3 = 0;                                // s3: it % 3
+    for (int it = 0;; ++it) {
+        if (s_tile[it & 3] >= ntile) break;              // uniform: written before a barrier all have passed
+        // (1) the previous tile's staged rows have been read
         if (tid < TCN) tc::bulk_wait_read_all();
+        if (tid == 0) s_tile[(it + 3) & 3] = deal();
         __syncthreads();
-        const int nt = s_next;
-        // (2) the source rows into the B tiles
-        gather_rows_split(s.b_hi, s.b_lo, s_src[slot], TCN, F.ueq, np);
+        const int n3 = s3 == 2 ? 0 : s3 + 1, nn3 = n3 == 2 ? 0 : n3 + 1;
+        const bool more = s_tile[(it + 1) & 3] < ntile;
+        // (2) this tile's rows into the B tiles
+#pragma unroll
+        for (int u = 0; u < 8; ++u) put_split4(s.b_hi, s.b_lo, warp + 8 * u, 4 * lane, TCN, rows[u]);
         tc::fence_proxy_async_smem();
         __syncthreads();
         // (3) MMAs once the image has landed
         if (tid == 0) {
-            int ok = tc::mbar_wait_bounded(tc::smem_u32(s.bar_a), it & 1, WAIT_LIMIT);
+            int ok = 1;
+            if (images_waited < images_issued) {
+                ok = tc::mbar_wait_bounded(tc::smem_u32(s.bar_a), images_waited & 1, WAIT_LIMIT);
+                images_waited += ok;
+            }
             if (ok) {
-                image_pending = false;
                 tc::fence_after_sync();
                 issue_mmas(s, tmem);
             }
             s_ok = ok;
         }
-        // (4) the next tile's pair indices while the MMAs run
-        int nkey = 0;
-        if (nt < ntile && tid < TCN) nkey = tile_meta(nt, slot ^ 1);
+        // the next tile's rows and the indices of the one after it, in flight under the MMAs
+        if (more) load_rows(n3);
+        int m_src = -1, m_dst = -1;
+        const int2 m_rec = rec;
+        if (tid < TCN) {
+            const int p = tid < (m_rec.y & 127) ? m_rec.x + tid : 0;
+            m_src = Pd.src[p];
+            m_dst = Pd.trg[p];
+            rec = record(s_tile[(it + 3) & 3]);
+        }
         __syncthreads();
         if (!s_ok) {
             flag = 1;
             break;
         }
-        // (5) the MMAs complete (uniform outcome)
+        // (4) the MMAs complete (uniform outcome)
         const bool mma_ok = tc::mbar_wait_bounded(tc::smem_u32(s.bar_mma), it & 1, WAIT_LIMIT);
         if (__syncthreads_or(!mma_ok)) {
             flag = 2;
@@ -382,12 +443,12 @@ __global__ void __launch_bounds__(256) k_m2l_tc_loop(FmmDev F, PairsDev Pd, cons
             break;
         }
         tc::fence_after_sync();
-        // (6) the next tile's image into the A tile (its readers, the MMAs, have completed)
-        if (tid == 0 && nt < ntile) {
-            issue_image(nkey);
-            image_pending = true;
+        // (5) the next tile's image, if it is another one (its readers, the MMAs, have completed)
+        if (tid == 0 && more && s_key[n3] != s_key[s3]) {
+            issue_image(s_key[n3]);
+            ++images_issued;
         }
-        // (7) results staged as one FP32 row per pair in the B tiles, then one bulk reduction per
+        // (6) results staged as one FP32 row per pair in the B tiles, then one bulk reduction per
         // pair into its target's row (padding rows add zeros)
         for (int c0 = cbeg; c0 < cbeg + TCN / 2; c0 += 16) {
             float v[16];
@@ -399,18 +460,19 @@ __global__ void __launch_bounds__(256) k_m2l_tc_loop(FmmDev F, PairsDev Pd, cons
         tc::fence_before_sync();                         // the TMEM reads before the next tile's MMAs
         __syncthreads();
         if (tid < TCN) {
-            const int d = s_dst[slot][tid];
+            const int d = s_dst[s3][tid];
             if (d >= 0) {
                 tc::bulk_reduce_add_f32(F.dchk + (size_t)d * np, tc::smem_u32(stage + tid * TCK), (uint32_t)np * 4u);
                 tc::bulk_commit();
             }
+            put_meta(nn3, m_rec, m_src, m_dst);          // slot of tile it - 1: all are past it
         }
-        tile = nt;
+        s3 = n3;
     }
-    if (tid == 0 && flag) {
-        atomicOr(err, flag);
+    if (tid == 0) {
+        if (flag) atomicOr(err, flag);
         // an image copy in flight lands before this CTA's memory is released
-        if (image_pending) tc::mbar_wait_bounded(tc::smem_u32(s.bar_a), it & 1, WAIT_LIMIT);
+        if (images_waited < images_issued) tc::mbar_wait_bounded(tc::smem_u32(s.bar_a), images_waited & 1, WAIT_LIMIT);
     }
     if (tid < TCN) tc::bulk_wait_read_all();
     tile_teardown(s);
@@ -1744,7 +1806,9 @@ void fmm_m2l_tc(const FmmDev &F, const PairsDev &Pd, int nV, const uint16_t *ima
     if (tile_loop && ticket) {
         const int upper = (nV + TCN - 1) / TCN + Pd.nkeys;   // tiles at most
         const int ctas = loop_ctas > 0 ? loop_ctas : 2 * sm_count();
-        launch_pdl(k_m2l_tc_loop, std::min(upper, ctas), 256, TC_SMEM, st, F, Pd, images, err, ticket);
+        // runs as long as every CTA still takes about eight of them
+        const int run = std::min(8, std::max(1, nV / TCN / (8 * ctas)));
+        launch_pdl(k_m2l_tc_loop, std::min((upper + run - 1) / run, ctas), 256, TC_SMEM, st, F, Pd, images, err, ticket, run);
         return;
     }
     int grid = (nV + TCN - 1) / TCN + Pd.nkeys;

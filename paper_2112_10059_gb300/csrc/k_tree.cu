@@ -718,10 +718,13 @@ template <bool FILL>
 __global__ void __launch_bounds__(256) k_lists_warp(TreeDev T, ListDev L, PairsDev Pd, int D) {
     pdl_enter();
     if (FILL) {
-        // the key of every V-pair tile (k_lists_layout laid the tiles out)
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Pd.nkeys; k += gridDim.x * blockDim.x) {
-            const int x = Pd.tile_off[k], t1 = Pd.tile_cnt[k];
-            for (int t = 0; t < t1; ++t) Pd.tile_key[x + t] = k;
+        // the key and record of every V-pair tile (k_lists_layout laid the tiles out), a warp per key
+        for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < Pd.nkeys; k += (int)(gridDim.x * blockDim.x) >> 5) {
+            const int x = Pd.tile_off[k], t1 = Pd.tile_cnt[k], p0 = Pd.off[k], p1 = Pd.off[k + 1];
+            for (int t = threadIdx.x & 31; t < t1; t += 32) {
+                Pd.tile_key[x + t] = k;
+                Pd.tile_rec[x + t] = make_int2(p0 + t * VPAIR_TILE, (k << 7) | min(VPAIR_TILE, p1 - p0 - t * VPAIR_TILE));
+            }
         }
     }
     const int lane = threadIdx.x & 31;

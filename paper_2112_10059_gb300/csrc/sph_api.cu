@@ -352,6 +352,8 @@ PairsDev pairs_dev(sph_ctx *c) {
     int *pp = P<int>(c->b_ppairs);
     Pd.trg = pp; Pd.src = pp ? pp + nV : nullptr;
     Pd.tile_key = pp ? pp + 2 * (size_t)nV : nullptr;
+    const size_t tiles = (size_t)nV / VPAIR_TILE + nkeys + 1;
+    Pd.tile_rec = pp ? reinterpret_cast<int2 *>(pp + ((2 * (size_t)nV + tiles + 1) & ~(size_t)1)) : nullptr;
     return Pd;
 }
 
@@ -534,7 +536,7 @@ int lists_fill(sph_ctx *c) {
     ENS(c->b_xsrc, std::max(1, c->list_tot[3]) * sizeof(int));
     {
         const size_t nV = std::max(1, c->list_tot[1]), nkeys = (size_t)(c->Lmax + 1) * NSLOT;
-        ENS(c->b_ppairs, (2 * nV + nV / 64 + nkeys + 1) * sizeof(int));
+        ENS(c->b_ppairs, (2 * nV + 3 * (nV / VPAIR_TILE + nkeys + 1) + 1) * sizeof(int));
     }
     ListDev L = list_dev(c);
     int *ltot = P<int>(c->b_tot) + 4;

@@ -346,6 +346,7 @@ struct PairsDev {
     int *trg, *src;       // [nV]
     int *total_tiles;     // [1]
     int *tile_key;        // [nV / 64 + nkeys]: key of every tile (one load instead of a search per CTA)
+    int2 *tile_rec;       // [nV / 64 + nkeys]: {first pair, key << 7 | pairs}
 };
 constexpr int VPAIR_TILE = 64;   // V pairs per M2L tile (the tensor-core tile's N)
 void fmm_m2l_pairs(const FmmDev &F, const PairsDev &Pd, int nV, int m2l_prec, cudaStream_t st);
