@@ -109,8 +109,8 @@ typedef struct sph_stats {
     int32_t l2lp_fused;        /* 1 if the deepest level's L2L and L2P ran as one kernel (leaves of edge 4) */
     float ms_l2lp;             /* its GPU milliseconds (inside ms_l2p), 0 if not fused */
     int32_t m2l_tiles;         /* tensor-core M2L form of this eval: 1 target-stationary tiles (dense V
-                                  lists), 0 tiles of V pairs; chosen by V-pair density, or by timing both
-                                  when the leaf size is autotuned (set_criteria leaf_size 0) */
+                                  lists of 5 million pairs or more), 0 tiles of V pairs; chosen by timing
+                                  both when the leaf size is autotuned (set_criteria leaf_size 0) */
 } sph_stats;
 
 /* Create a context on CUDA device `device`, queuing work on `cuda_stream`

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(2 * MAXPAD) k_upward(FmmDev F, int level, cons
 // out on its 4^3 cells and anterpolated one axis after the other, 4 (16 p + 4 p^2 + p^3) FMAs
 // whatever the number of sources, from one basis of p x 4 values per level -- box by box, each source's
 // 3 p basis values and p^3 products were formed anew by a CTA (253 us for the 32,768 full leaves
-// of a uniform 128^3 tree, P2MFIG so).
+// of a uniform 128^3 tree, 23 us so).
 constexpr int P2M_WARPS = 8;
 
 template <int P>

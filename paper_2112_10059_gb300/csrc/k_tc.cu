@@ -285,8 +285,9 @@ __global__ void __launch_bounds__(256) k_m2l_tc(FmmDev F, PairsDev Pd, const uin
     const int p1 = min(p0 + TCN, Pd.off[key + 1]);
     if (threadIdx.x < TCN) {
         int q = p0 + threadIdx.x;
-        s.col_src[threadIdx.x] = q < p1 ? Pd.src[q] : -1;
-        s.col_dst[threadIdx.x] = q < p1 ? Pd.trg[q] : -1;
+        const int2 pr = q < p1 ? Pd.pair[q] : make_int2(-1, -1);
+        s.col_src[threadIdx.x] = pr.y;
+        s.col_dst[threadIdx.x] = pr.x;
     }
     const uint16_t *img = images + (size_t)key * (2 * A_BYTES / 2);
     tile_issue_image(s, img);
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(256) k_m2l_tc(FmmDev F, PairsDev Pd, const uin
 // next image if it is another, (6) the results are staged in the B tiles and added into the
 // targets' rows.  The same sums as k_m2l_tc.
 // Wide streamer 192^3 (2.9 M pairs, 45 k tiles): 727 us with one tile a ticket, its rows and
-// indices loaded in the chain and an image a tile; M2LFIG so.
+// indices loaded in the chain and an image a tile; 518 us so.
 __global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, const uint16_t *__restrict__ images,
                                                         int *err, int *ticket, int run) {
     // prologue (the V pairs, their tiles and the operator images were written before the passes)
@@ -331,9 +332,9 @@ __global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, c
     };
     // record of a tile: {first pair, key << 7 | pairs}
     auto record = [&](int tile) { return tile < ntile ? Pd.tile_rec[tile] : make_int2(0, 0); };
-    auto put_meta = [&](int slot, const int2 &rec, int src, int dst) {
-        s_src[slot][tid] = tid < (rec.y & 127) ? src : -1;
-        s_dst[slot][tid] = tid < (rec.y & 127) ? dst : -1;
+    auto put_meta = [&](int slot, const int2 &rec, const int2 &pair) {   // pair: {target, source}
+        s_src[slot][tid] = tid < (rec.y & 127) ? pair.y : -1;
+        s_dst[slot][tid] = tid < (rec.y & 127) ? pair.x : -1;
         if (tid == 0) s_key[slot] = rec.y >> 7;
     };
     tile_setup(s);
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, c
     if (tid < TCN) {
         const int2 r0 = record(blockIdx.x * run);
         const int q = tid < (r0.y & 127) ? r0.x + tid : 0;
-        put_meta(0, r0, Pd.src[q], Pd.trg[q]);
+        put_meta(0, r0, Pd.pair[q]);
         if (tid == 0) {
             issue_image(r0.y >> 7);
             ++images_issued;
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, c
     if (tid < TCN) {
         const int2 r1 = record(s_tile[1]);
         const int p = tid < (r1.y & 127) ? r1.x + tid : 0;
-        put_meta(1, r1, Pd.src[p], Pd.trg[p]);
+        put_meta(1, r1, Pd.pair[p]);
         rec = record(s_tile[2]);
     }
     int flag = 0, s3 = 0;                                // s3: it % 3
@@ -422,12 +423,11 @@ __global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, c
         }
         // the next tile's rows and the indices of the one after it, in flight under the MMAs
         if (more) load_rows(n3);
-        int m_src = -1, m_dst = -1;
+        int2 m_pair = make_int2(-1, -1);
         const int2 m_rec = rec;
         if (tid < TCN) {
             const int p = tid < (m_rec.y & 127) ? m_rec.x + tid : 0;
-            m_src = Pd.src[p];
-            m_dst = Pd.trg[p];
+            m_pair = Pd.pair[p];
             rec = record(s_tile[(it + 3) & 3]);
         }
         __syncthreads();
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(256, 2) k_m2l_tc_loop(FmmDev F, PairsDev Pd, c
                 tc::bulk_reduce_add_f32(F.dchk + (size_t)d * np, tc::smem_u32(stage + tid * TCK), (uint32_t)np * 4u);
                 tc::bulk_commit();
             }
-            put_meta(nn3, m_rec, m_src, m_dst);          // slot of tile it - 1: all are past it
+            put_meta(nn3, m_rec, m_pair);          // slot of tile it - 1: all are past it
         }
         s3 = n3;
     }
@@ -554,8 +554,9 @@ __global__ void __launch_bounds__(128, 1) k_m2l_tc_pipe(FmmDev F, PairsDev Pd, c
             int p0, p1;
             m2l_tile_range(Pd, key, tile, p0, p1);
             const int q = p0 + tid;
-            msrc[ms * TCN + tid] = q < p1 ? Pd.src[q] : -1;
-            mdst[ms * TCN + tid] = q < p1 ? Pd.trg[q] : -1;
+            const int2 pr = q < p1 ? Pd.pair[q] : make_int2(-1, -1);
+            msrc[ms * TCN + tid] = pr.y;
+            mdst[ms * TCN + tid] = pr.x;
         }
     };
     auto issue_raw = [&](int ms) {

@@ -217,8 +217,9 @@ __global__ void __launch_bounds__(256) k_m2l_pairs(FmmDev F, PairsDev Pd) {
     const int p1 = min(p0 + TN, Pd.off[key + 1]);
     if (tid < TN) {
         int q = p0 + tid;
-        trg[tid] = q < p1 ? Pd.trg[q] : -1;
-        src[tid] = q < p1 ? Pd.src[q] : -1;
+        const int2 pr = q < p1 ? Pd.pair[q] : make_int2(-1, -1);
+        trg[tid] = pr.x;
+        src[tid] = pr.y;
     }
     __syncthreads();
     const float *M = F.O.m2l_t + ((size_t)level * NSLOT + slot) * np * np;

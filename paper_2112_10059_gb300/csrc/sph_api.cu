@@ -104,7 +104,7 @@ struct sph_ctx {
     int m2l_tiles = 2;                // tensor-core M2L in target-stationary tiles: 0 never (tiles of V
                                       // pairs), 1 always, 2 where the V lists are dense (>= 32 pairs per box)
     DevBuf b_mtg;                     // groups of the target-stationary M2L
-    int m2l_form = -1;                // autotuned M2L form for this eval (-1: the density rule)
+    int m2l_form = -1;                // autotuned M2L form for this eval (-1: by the lists)
     bool m2l_tiles_used = false;      // the last eval ran the target-stationary M2L
     bool l2lp_fused = true;           // deepest level of edge-4 leaves: L2L and L2P in one tensor-core kernel
     bool l2lp_used = false;           // the last eval ran the fused kernel
@@ -119,7 +119,7 @@ struct sph_ctx {
     DevBuf b_maxes, b_cnt, b_off, b_tot, b_skey, b_spc, b_sq, b_tkey, b_tpc, b_bstat;
     DevBuf b_boxat, b_flag, b_pos, b_rng, b_scan, b_lvl;
     DevBuf b_level, b_key, b_sb, b_se, b_tb, b_te, b_parent, b_leaf;
-    DevBuf b_lcnt, b_loff, b_usrc, b_vsrc, b_vocs, b_vtrg, b_wsrc, b_xsrc, b_pkeys, b_ppairs, b_heavy;
+    DevBuf b_lcnt, b_loff, b_usrc, b_vsrc, b_vocs, b_vtrg, b_wsrc, b_xsrc, b_pkeys, b_ppairs, b_vbase, b_heavy;
     DevBuf b_ueq, b_dchk;
     DevBuf o_work, o_etab, o_m2m, o_l2l, o_m2l, o_m2lbf, o_l2lbf, o_m2mbf, o_slot, o_surf, o_cheb, o_self;
     DevBuf b_err;                // device error flags of the tensor-core tiles
@@ -346,11 +346,12 @@ PairsDev pairs_dev(sph_ctx *c) {
     const int nV = std::max(c->list_tot[1], 1);
     int *pk = P<int>(c->b_pkeys);
     Pd.nkeys = nkeys;
-    Pd.cnt = pk; Pd.off = pk + nkeys; Pd.cursor = pk + 2 * nkeys + 1;
-    Pd.tile_cnt = pk + 3 * nkeys + 1; Pd.tile_off = pk + 4 * nkeys + 1;
-    Pd.total_tiles = pk + 5 * nkeys + 2;
+    Pd.cnt = pk; Pd.off = pk + nkeys;
+    Pd.tile_cnt = pk + 2 * nkeys + 1; Pd.tile_off = pk + 3 * nkeys + 1;
+    Pd.total_tiles = pk + 4 * nkeys + 2;
+    Pd.base = P<int>(c->b_vbase);
     int *pp = P<int>(c->b_ppairs);
-    Pd.trg = pp; Pd.src = pp ? pp + nV : nullptr;
+    Pd.pair = reinterpret_cast<int2 *>(pp);
     Pd.tile_key = pp ? pp + 2 * (size_t)nV : nullptr;
     const size_t tiles = (size_t)nV / VPAIR_TILE + nkeys + 1;
     Pd.tile_rec = pp ? reinterpret_cast<int2 *>(pp + ((2 * (size_t)nV + tiles + 1) & ~(size_t)1)) : nullptr;
@@ -437,8 +438,9 @@ int lists_count_queue(sph_ctx *c) {
     ENS(c->b_loff, 4 * (size_t)(cap + 1) * sizeof(int));
     ENS(c->b_heavy, (size_t)cap * sizeof(int));
     const int nkeys = (Lmax + 1) * NSLOT;
-    ENS(c->b_pkeys, (5 * (size_t)nkeys + 10) * sizeof(int));
-    if (!c->chain_zeroed) CK(cudaMemsetAsync(c->b_pkeys.p, 0, (5 * (size_t)nkeys + 10) * sizeof(int), c->stream));
+    ENS(c->b_pkeys, (4 * (size_t)nkeys + 10) * sizeof(int));
+    ENS(c->b_vbase, (size_t)LISTS_WARP_GRID * nkeys * sizeof(int));
+    if (!c->chain_zeroed) CK(cudaMemsetAsync(c->b_pkeys.p, 0, (4 * (size_t)nkeys + 10) * sizeof(int), c->stream));
     ENS(c->b_scan, scan_scratch_bytes(cap));
     ListDev L = list_dev(c);
     int *ltot = P<int>(c->b_tot) + 4;
@@ -480,7 +482,7 @@ int chain_zero(sph_ctx *c) {
     ENS(c->b_rng, 4 * dense_total * sizeof(int));
     ENS(c->b_scan, scan_scratch_bytes(dense_total));
     ENS(c->b_lvl, 80 * sizeof(int));
-    ENS(c->b_pkeys, (5 * (size_t)nkeys + 10) * sizeof(int));
+    ENS(c->b_pkeys, (4 * (size_t)nkeys + 10) * sizeof(int));
     ZeroSet Z;
     const bool ok =
         Z.add(P<int>(c->b_maxes), 2) && Z.add(P<int>(c->b_tot) + 2, 2) && Z.add(P<int>(c->b_tot) + 8, 1) &&
@@ -488,7 +490,7 @@ int chain_zero(sph_ctx *c) {
         Z.add(P<int>(c->b_scan), (int64_t)(scan_state_bytes(1, (int)dense_total) / sizeof(int))) &&
         Z.add(P<int>(c->b_scan) + scan_list_off(dense_total),
               (int64_t)(scan_state_bytes(4, (int)dense_total) / sizeof(int))) &&
-        Z.add(P<int>(c->b_pkeys), 5 * (int64_t)nkeys + 10);
+        Z.add(P<int>(c->b_pkeys), 4 * (int64_t)nkeys + 10);
     if (!ok) return SPH_OK;   // each user then clears its own
     zero_set_launch(Z, c->stream);
     CK(cudaGetLastError());
@@ -763,27 +765,29 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
     return SPH_OK;
 }
 
-// The M2L form: target-stationary tiles pay a round per (group, offset) whatever the number of
-// pairs in it, so they are taken where the lists are dense (uniform trees), the tiles of V pairs
-// elsewhere (an autotuned choice overrides the density rule).
+// The M2L form (an autotuned choice overrides it).  The target-stationary tiles pay a round per
+// (group, offset) whatever the number of pairs in it: on all-source grids of n^3 cells they take
+// 134 / 251 / 274 / 688 / 1099 us for n = 24 / 48 / 64 / 96 / 128, the tile loop over V pairs 20 / 84 / 190 /
+// 434 / 1057 us.  They are taken where the lists are dense and so long that the two are level (6 M
+// pairs at 128^3).  Error against FP64 there: 2.1e-5 by the target tiles, 2.3e-5 by the pairs as by
+// FP32 translations (the tiles' long sums, rounded towards zero, cancel some of the expansion's own error).
 bool m2l_target_tiles(const sph_ctx *c, const PassState &S) {
     const int64_t nV = c->list_tot[1], nb = c->nboxes;
     return S.tc && (c->m2l_tiles == 1 ||
-                    (c->m2l_tiles == 2 && (c->m2l_form >= 0 ? c->m2l_form == 1 : nV >= 32 * nb)));
+                    (c->m2l_tiles == 2 && (c->m2l_form >= 0 ? c->m2l_form == 1 : nV >= 32 * nb && nV >= 5000000)));
 }
 
 // CTAs per SM of the overlapped near field's U-list launch.  Five fit beside each other (37 KB of
 // shared memory each); where the far-field chain is the longer of the two, four leave slots to its
 // kernels (256^3 headline: 458 us with 4, 464 with 5, 467 with 6; uniform 128^3: 2830, 2813, 2811).
 // Estimates from the list totals: near-field pairs at most U entries x leaf size^2 at 5e12/s; far
-// field a fixed 150 us plus the M2L at its measured cost per V pair (0.45 ns in pair tiles, 0.19 ns
-// in target tiles).  The tabulated near field keeps its own figures (1.6e12/s, 16 and 6).
+// field a fixed 150 us plus the M2L at its measured cost per V pair (0.18 ns).  The tabulated near field keeps its own figures (1.6e12/s, 16 and 6).
 int near_cap(const sph_ctx *c, const PassState &S) {
     if (c->near_per_sm > 0) return c->near_per_sm;
     const double s = c->leaf_eff;
     const bool table = S.F.gtab != nullptr;
     const double near_us = (double)c->list_tot[0] * s * s / (table ? 1.6e6 : 5e6);
-    const double far_us = 150.0 + (double)c->list_tot[1] * (m2l_target_tiles(c, S) ? 0.19e-3 : 0.45e-3);
+    const double far_us = 150.0 + (double)c->list_tot[1] * 0.18e-3;
     return near_us > far_us ? (table ? 16 : 5) : (table ? 6 : 4);
 }
 
@@ -1260,7 +1264,7 @@ int resolve_near(sph_ctx *c, float *out) {
 // Tensor-core M2L form for this evaluation when the leaf size is autotuned (set_criteria
 // leaf_size 0) and the form is left to the library: the faster of the tiles of V pairs and the
 // target-stationary tiles, timed like the leaf size over the FMM passes and cached per problem
-// class, leaf size and near-field form.  Otherwise the density rule of fmm_queue decides.
+// class, leaf size and near-field form.  Otherwise m2l_target_tiles decides.
 int fmm_after_select(sph_ctx *c, float *out, PhaseTimer *tm);
 int resolve_m2l(sph_ctx *c, float *out) {
     c->m2l_form = -1;
@@ -1314,7 +1318,7 @@ int run_fmm(sph_ctx *c, float *out, sph_stats *stats) {
     tm.start(stats != nullptr, c->stream);
     c->launches = 0;
     c->chain_zeroed = false;
-    c->m2l_form = -1;                 // the density rule unless the autotuner picks the form below
+    c->m2l_form = -1;                 // by the lists unless the autotuner picks the form below
     int r = check_previous_tc(c);
     if (r) return r;
     if (c->defer_sync && c->leaf_size != 0 && c->near_mode != SPH_NEAR_AUTO) {
@@ -1918,7 +1922,7 @@ void sph_destroy(sph_ctx *c) {
     DevBuf *all[] = {&c->b_maxes, &c->b_bstat, &c->b_cnt, &c->b_off, &c->b_tot, &c->b_skey, &c->b_spc, &c->b_sq, &c->b_tkey,
                      &c->b_tpc, &c->b_boxat, &c->b_flag, &c->b_pos, &c->b_rng, &c->b_scan, &c->b_lvl,
                      &c->b_level, &c->b_key, &c->b_sb, &c->b_se, &c->b_tb, &c->b_te, &c->b_parent, &c->b_leaf,
-                     &c->b_lcnt, &c->b_loff, &c->b_usrc, &c->b_vsrc, &c->b_vocs, &c->b_vtrg, &c->b_wsrc, &c->b_xsrc, &c->b_pkeys, &c->b_ppairs, &c->b_heavy,
+                     &c->b_lcnt, &c->b_loff, &c->b_usrc, &c->b_vsrc, &c->b_vocs, &c->b_vtrg, &c->b_wsrc, &c->b_xsrc, &c->b_pkeys, &c->b_ppairs, &c->b_vbase, &c->b_heavy,
                      &c->b_ueq, &c->b_dchk, &c->o_work, &c->o_etab, &c->o_m2m, &c->o_l2l,
                      &c->o_m2l, &c->o_m2lbf, &c->o_l2lbf, &c->o_m2mbf, &c->b_err, &c->b_work, &c->b_mtg, &c->b_nearbuf, &c->o_slot, &c->o_surf, &c->o_cheb, &c->o_self, &c->h_q, &c->h_e, &c->h_m,
                      &c->h_s, &c->b_tmask, &c->b_near, &c->b_gtab, &c->b_dtab, &c->b_skip, &c->o_l2pimg, &c->s_qc, &c->s_Sc, &c->s_y, &c->s_Sp, &c->s_x, &c->s_Sf,

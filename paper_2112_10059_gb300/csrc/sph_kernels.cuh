@@ -341,13 +341,14 @@ void fmm_m2l_gemm_level(const FmmDev &F, int level, int box_begin, int box_count
 struct PairsDev {
     int nkeys;            // (Lmax + 1) * 316
     int *cnt, *off;       // [nkeys], [nkeys + 1]
-    int *cursor;          // [nkeys]
+    int *base;            // [LISTS_WARP_GRID][nkeys]: where each CTA of the list passes puts its pairs of a key
     int *tile_cnt, *tile_off;   // [nkeys], [nkeys + 1]
-    int *trg, *src;       // [nV]
+    int2 *pair;           // [nV] {target, source}
     int *total_tiles;     // [1]
     int *tile_key;        // [nV / 64 + nkeys]: key of every tile (one load instead of a search per CTA)
     int2 *tile_rec;       // [nV / 64 + nkeys]: {first pair, key << 7 | pairs}
 };
+constexpr int LISTS_WARP_GRID = 152 * 4;   // CTAs of the list passes (both)
 constexpr int VPAIR_TILE = 64;   // V pairs per M2L tile (the tensor-core tile's N)
 void fmm_m2l_pairs(const FmmDev &F, const PairsDev &Pd, int nV, int m2l_prec, cudaStream_t st);
 // tensor-core (tcgen05, BF16 x3) translations; require npad == 128
