@@ -1407,10 +1407,11 @@ __global__ void __launch_bounds__(LP_T, 1) k_l2lp_tc(FmmDev F, int level, int pa
 }
 
 // S += E d_own at the targets of the deepest-level leaves (edge 4) in `list` (count[0] of them:
-// the leaves with V or X entries, whose own local terms the fused kernel leaves out), FP32
-// from the level's interpolation table E ([n][64], cells in local Morton order), staged in
-// shared memory once per CTA.  One warp per leaf: lane k takes the cells of local index k and
-// k + 32; every cell belongs to one leaf, so plain read-modify-writes suffice.  The next
+// the leaves with V or X entries, whose own local terms the fused kernel leaves out), FP32, axis
+// by axis from the 5 x 4 values of the one-dimensional basis: 1,220 FMAs a leaf instead of the 8,000
+// of the table E, whose shared-memory reads bounded the kernel (32,768 leaves of the uniform 128^3
+// tree: 57 us by the table, 22 us so).  One warp per leaf: lane k takes the cells of local index
+// k and k + 32; every cell belongs to one leaf, so plain read-modify-writes suffice.  The next
 // leaf's index and expansion are fetched while the current one is evaluated, and the current
 // leaf's cell values (and mask bytes) are read before its contraction, so that a warp's
 // loads overlap its arithmetic instead of following it.
@@ -1420,12 +1421,23 @@ __global__ void __launch_bounds__(OWN_W * 32) k_l2p_own(FmmDev F, int level, con
     pdl_enter();
     const int cnt = *count;
     if ((int)blockIdx.x * OWN_W >= cnt) return;            // uniform, before the table is staged
-    __shared__ float Es[TCK * 64];                          // [n][64]
+    constexpr int P = 5;                                    // the tensor-core path's order (P^3 <= TCK)
+    __shared__ float basis[P][4];                           // value of node k's polynomial at cell i
     __shared__ __align__(16) float sd[OWN_W][TCK];
+    __shared__ float tz[OWN_W][4 * P * P], ty[OWN_W][16 * P];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n = F.O.n, np = F.O.npad;
-    const float4 *E4 = reinterpret_cast<const float4 *>(F.O.e_tab + F.O.e_off[level]);
-    for (int j = threadIdx.x; j < n * 16; j += blockDim.x) reinterpret_cast<float4 *>(Es)[j] = __ldg(E4 + j);
+    const int np = F.O.npad;
+    if (threadIdx.x < 4 * P) {
+        const int k = threadIdx.x / 4;
+        const float x = (float)(2 * (int)(threadIdx.x & 3) - 3) * 0.25f, tk = F.O.cheb_t[k];
+        float num = 1.f, den = 1.f;
+        for (int j = 0; j < P; ++j)
+            if (j != k) {
+                num *= x - F.O.cheb_t[j];
+                den *= tk - F.O.cheb_t[j];
+            }
+        basis[k][threadIdx.x & 3] = num / den;
+    }
     const TreeDev &T = F.T;
     const int stride = gridDim.x * OWN_W;
     int i = blockIdx.x * OWN_W + warp;
@@ -1461,13 +1473,38 @@ __global__ void __launch_bounds__(OWN_W * 32) k_l2p_own(FmmDev F, int level, con
             old[h] = keep[h] ? out[o[h]] : 0.f;
         }
         __syncwarp();
-        float a0 = 0.f, a1 = 0.f;
-#pragma unroll 5
-        for (int k = 0; k < n; ++k) {
-            const float dk = sd[warp][k];
-            a0 = fmaf(Es[k * 64 + lane], dk, a0);
-            a1 = fmaf(Es[k * 64 + lane + 32], dk, a1);
+        const float *d = sd[warp];
+        float *dz = tz[warp], *dy = ty[warp];
+#pragma unroll
+        for (int e = lane; e < 4 * P * P; e += 32) {        // [z][b][a]
+            const int z = e / (P * P), ba = e % (P * P);
+            float a = basis[0][z] * d[ba];
+#pragma unroll
+            for (int k = 1; k < P; ++k) a = fmaf(basis[k][z], d[k * P * P + ba], a);
+            dz[e] = a;
         }
+        __syncwarp();
+#pragma unroll
+        for (int e = lane; e < 16 * P; e += 32) {           // [z][y][a]
+            const int z = e / (4 * P), y = e / P & 3, x = e % P;
+            float a = basis[0][y] * dz[z * P * P + x];
+#pragma unroll
+            for (int k = 1; k < P; ++k) a = fmaf(basis[k][y], dz[z * P * P + k * P + x], a);
+            dy[e] = a;
+        }
+        __syncwarp();
+        float acc[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t lx, ly, lz;
+            demorton3((uint32_t)(lane + 32 * h), lx, ly, lz);
+            const float *v = dy + (lz * 4 + ly) * P;
+            float a = basis[0][lx] * v[0];
+#pragma unroll
+            for (int k = 1; k < P; ++k) a = fmaf(basis[k][lx], v[k], a);
+            acc[h] = a;
+        }
+        const float a0 = acc[0], a1 = acc[1];
         if (keep[0]) out[o[0]] = old[0] + a0;
         if (keep[1]) out[o[1]] = old[1] + a1;
         __syncwarp();
@@ -1501,7 +1538,7 @@ void fmm_l2lp_tc_level(const FmmDev &F, int level, int parent_begin, int parent_
 void fmm_l2p_own(const FmmDev &F, int level, const int *list, const int *count, int max_count, float *out,
                  cudaStream_t st) {
     if (max_count <= 0 || F.O.e_off[level] < 0 || F.O.npad > TCK || (1 << (F.D - level)) != 4) return;
-    const int grid = std::max(1, std::min((max_count + OWN_W - 1) / OWN_W, 4 * sm_count()));
+    const int grid = std::max(1, std::min((max_count + OWN_W - 1) / OWN_W, 8 * sm_count()));
     launch_pdl(k_l2p_own, grid, OWN_W * 32, 0, st, F, level, list, count, out);
 }
 
