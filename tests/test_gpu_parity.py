@@ -161,6 +161,37 @@ def test_selection_whole_bricks(sph, monkeypatch, dims):
             _check_fmm(out.cpu().numpy(), ref, To, p.name)
 
 
+@pytest.mark.parametrize("dims,shift", [((64, 48, 48), 0), ((64, 48, 48), 1), ((56, 40, 33), 0), ((50, 37, 40), 3)])
+def test_selection_whole_bricks_of_a_mask(sph, monkeypatch, dims, shift):
+    """Bricks wholly inside or outside a target mask are decided by the statistics pass; one cell
+    more or less, bricks past the grid, row pitches that are no multiple of 4 and a mask whose
+    first byte is not aligned give the oracle's sets in all three selection forms."""
+    import torch
+    nx, ny, nz = dims
+    p = si.brick_structured(nx, ny, nz)
+    m = np.zeros((nz, ny, nx), np.uint8)
+    m[:, :32, :32] = 7                       # any non-zero byte is a target
+    m[3, 5, 7] = 0                           # one cell out of a full brick
+    m[20, 34, 20] = 1                        # one cell into an empty one
+    Jo, To = oracle.select(p.q, None, m.ravel(), p.i_frac)
+    buf = torch.zeros(m.size + 16, dtype=torch.uint8, device="cuda")
+    md = buf[shift:shift + m.size]
+    md.copy_(torch.from_numpy(m.ravel()))
+    q = torch.from_numpy(p.q).cuda()
+    for two, lb in SELECT_FORMS:
+        monkeypatch.setenv("SPH_SELECT_TWO_PASS", two)
+        monkeypatch.setenv("SPH_SELECT_LOOKBACK", lb)
+        c = sph.Context(0)
+        sph.set_grid(c, nx, ny, nz, p.h, p.pO2_torr)
+        sph.set_sources(c, q, p.source_scale)
+        sph.set_targets(c, mask=md)
+        sph.set_criteria(c, p.i_frac)
+        sph.eval_sph(c)
+        J, T = sph.get_selection(c)
+        c.close()
+        assert np.array_equal(J, Jo) and np.array_equal(T, To), (two, lb)
+
+
 @pytest.mark.parametrize("case", [(16, 16, 16, 0.05, 0.3, 8, 2), (12, 9, 7, 0.2, 0.1, 4, 3),
                                   (20, 10, 13, 0.5, 0.02, 6, 5), (32, 32, 32, 0.02, 0.5, 16, 9)])
 def test_tree_bit_exact(sph, ctx, case):
