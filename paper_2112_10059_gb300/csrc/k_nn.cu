@@ -150,32 +150,36 @@ void f32_to_bf16(const float *in, uint16_t *out, size_t n, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------- coarse inputs
-__global__ void k_pool_avg_f32(const float *__restrict__ fine, int nf, int f, float *__restrict__ coarse) {
-    const int nc = nf / f;
-    const size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (p >= (size_t)nc * nc * nc) return;
-    const int x = (int)(p % nc), y = (int)((p / nc) % nc), z = (int)(p / ((size_t)nc * nc));
-    float s = 0.f;
-    for (int k = 0; k < f; ++k)
-        for (int j = 0; j < f; ++j) {
-            const float *row = fine + ((size_t)(z * f + k) * nf + (y * f + j)) * nf + x * f;
-            for (int i = 0; i < f; ++i) s += row[i];
+// Mean and largest value over f^3 blocks (either output may be null), one thread per block, its
+// cells in the order x, y, z.  Bound by memory: rows in 16-byte loads where the block edge and the
+// pitch allow it (256^3 by 4: 16 us a field and output before, 17 for both outputs).
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_pool(const float *__restrict__ fine, int nf, int f, float *__restrict__ avg,
+                                              float *__restrict__ mx) {
+    const int nc = nf / f, x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
+    if (x >= nc || y >= nc) return;
+    float s = 0.f, m = 0.f;
+    for (int k = 0; k < f; ++k) {
+        const float *row = fine + ((size_t)(z * f + k) * nf + (size_t)y * f) * nf + (size_t)x * f;
+#pragma unroll 4
+        for (int j = 0; j < f; ++j, row += nf) {
+            if (VEC) {
+                for (int i = 0; i < f; i += 4) {
+                    const float4 v = __ldg(reinterpret_cast<const float4 *>(row + i));
+                    s += v.x; s += v.y; s += v.z; s += v.w;
+                    m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
+                }
+            } else {
+                for (int i = 0; i < f; ++i) {
+                    s += row[i];
+                    m = fmaxf(m, row[i]);
+                }
+            }
         }
-    coarse[p] = s / (float)(f * f * f);
-}
-
-__global__ void k_pool_max_f32(const float *__restrict__ fine, int nf, int f, float *__restrict__ coarse) {
-    const int nc = nf / f;
-    const size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (p >= (size_t)nc * nc * nc) return;
-    const int x = (int)(p % nc), y = (int)((p / nc) % nc), z = (int)(p / ((size_t)nc * nc));
-    float s = 0.f;
-    for (int k = 0; k < f; ++k)
-        for (int j = 0; j < f; ++j) {
-            const float *row = fine + ((size_t)(z * f + k) * nf + (y * f + j)) * nf + x * f;
-            for (int i = 0; i < f; ++i) s = fmaxf(s, row[i]);
-        }
-    coarse[p] = s;
+    }
+    const size_t p = ((size_t)z * nc + y) * nc + x;
+    if (avg) avg[p] = s / (float)(f * f * f);
+    if (mx) mx[p] = m;
 }
 
 // maxima of up to four non-negative fields (b, d may be null) as float bits
@@ -227,13 +231,12 @@ __global__ void k_make_target(const float *__restrict__ St, const float *__restr
     t[i] = (a > 0.f && b > 0.f) ? logf(a / b) : 0.f;
 }
 
-void pool_avg_f32(const float *fine, int n_fine, int f, float *coarse, cudaStream_t st) {
-    const size_t nc = (size_t)(n_fine / f);
-    if (nc) k_pool_avg_f32<<<blocks_for(nc * nc * nc), 256, 0, st>>>(fine, n_fine, f, coarse);
-}
-void pool_max_f32(const float *fine, int n_fine, int f, float *coarse, cudaStream_t st) {
-    const size_t nc = (size_t)(n_fine / f);
-    if (nc) k_pool_max_f32<<<blocks_for(nc * nc * nc), 256, 0, st>>>(fine, n_fine, f, coarse);
+void pool_f32(const float *fine, int n_fine, int f, float *avg, float *mx, cudaStream_t st) {
+    const int nc = n_fine / f;
+    if (nc == 0) return;
+    const dim3 grid((nc + 31) / 32, (nc + 7) / 8, nc), block(32, 8);
+    if (f % 4 == 0 && (reinterpret_cast<uintptr_t>(fine) & 15) == 0) k_pool<true><<<grid, block, 0, st>>>(fine, n_fine, f, avg, mx);
+    else k_pool<false><<<grid, block, 0, st>>>(fine, n_fine, f, avg, mx);
 }
 void max4(const float *a, const float *b, const float *c, const float *d, size_t n, unsigned *maxbits,
           cudaStream_t st) {
@@ -284,42 +287,54 @@ __global__ void k_apply_residual(const float *__restrict__ Sc, const float *__re
     if (i < n) Sp[i] = use_net ? Sc[i] * expf(y[2 * i]) : Sc[i];
 }
 
-__global__ void k_block_pred_err(const float *__restrict__ y, int lgD, float *__restrict__ pe, int nblocks) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nblocks) return;
+__global__ void __launch_bounds__(128) k_block_pred_err(const float *__restrict__ y, int lgD, float *__restrict__ pe) {
+    const int b = blockIdx.x;                  // one CTA per block, four voxels a thread
     float m = 0.f;
-    for (int j = 0; j < JUDGE_BLOCK * JUDGE_BLOCK * JUDGE_BLOCK; ++j)
+#pragma unroll
+    for (int j = threadIdx.x; j < JUDGE_BLOCK * JUDGE_BLOCK * JUDGE_BLOCK; j += 128)
         m = fmaxf(m, expf(y[2 * (size_t)voxel_in_block(b, j, lgD) + 1]));
-    pe[b] = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    __shared__ float w[4];
+    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) pe[b] = fmaxf(fmaxf(w[0], w[1]), fmaxf(w[2], w[3]));
 }
 
 __global__ void k_judge_pick(int lgD, int f, uint64_t seed, int samples, uint8_t *__restrict__ mask,
                              int *__restrict__ sample_vox, int nblocks) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // a row of f fine cells of a sample
+    const int e = i / (f * f), row = i % (f * f);
     if (e >= nblocks * samples) return;
-    const int b = e / samples, s = e % samples;
     const int j = (int)(mix64(seed ^ ((uint64_t)e * 0xD1B54A32D192ED03ull)) & 511u);
-    const int v = voxel_in_block(b, j, lgD);
-    sample_vox[e] = v;
-    for (int a = 0; a < f * f * f; ++a) mask[fine_cell(v, lgD, f, a)] = 1;
-    (void)s;
+    const int v = voxel_in_block(e / samples, j, lgD);
+    if (row == 0) sample_vox[e] = v;
+    const size_t c = fine_cell(v, lgD, f, row * f);
+    for (int a = 0; a < f; ++a) mask[c + a] = 1;
 }
 
-__global__ void k_judge_err(const float *__restrict__ Sf, const float *__restrict__ Sp,
-                            const int *__restrict__ sample_vox, int lgD, int f, int samples, float *__restrict__ err,
-                            int nblocks) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per block, a lane per sample (its cells added in the order x, y, z).
+__global__ void __launch_bounds__(128) k_judge_err(const float *__restrict__ Sf, const float *__restrict__ Sp,
+                                                   const int *__restrict__ sample_vox, int lgD, int f, int samples,
+                                                   float *__restrict__ err, int nblocks) {
+    const int b = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (b >= nblocks) return;
     float m = 0.f;
-    for (int s = 0; s < samples; ++s) {
+    for (int s = lane; s < samples; s += 32) {
         const int v = sample_vox[b * samples + s];
         float acc = 0.f;
-        for (int a = 0; a < f * f * f; ++a) acc += Sf[fine_cell(v, lgD, f, a)];
+#pragma unroll 4
+        for (int r = 0; r < f * f; ++r) {
+            const float *row = Sf + fine_cell(v, lgD, f, r * f);
+            for (int a = 0; a < f; ++a) acc += row[a];
+        }
         acc /= (float)(f * f * f);
         const float rel = acc > 0.f ? fabsf(Sp[v] - acc) / acc : (Sp[v] != 0.f ? INFINITY : 0.f);
         m = fmaxf(m, rel);
     }
-    err[b] = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) err[b] = m;
 }
 
 __global__ void k_fallback_flags(const float *__restrict__ err, const float *__restrict__ pe, int use_pred,
@@ -335,26 +350,56 @@ __global__ void k_fallback_flags(const float *__restrict__ err, const float *__r
     atomicMax(counts + 3, __float_as_uint(fminf(err[b], 3.0e38f)));
 }
 
-__global__ void k_fallback_mask(const int *__restrict__ flags, int lgD, int f, uint8_t *__restrict__ mask) {
-    const int D = 1 << lgD, n = D * f;
-    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= (size_t)n * n * n) return;
-    const int x = (int)(i % n), y = (int)((i / n) % n), z = (int)(i / ((size_t)n * n));
-    const int v = ((z / f) * D + y / f) * D + x / f;
-    mask[i] = (uint8_t)flags[block_of(v, lgD)];
+// 16 fine cells of a row per thread (the edge f D is a multiple of 8): one store where they are whole
+__global__ void __launch_bounds__(256) k_fallback_mask(const int *__restrict__ flags, int lgD, int f, uint8_t *__restrict__ mask) {
+    const int D = 1 << lgD, n = D * f, nb = D / JUDGE_BLOCK, edge = f * JUDGE_BLOCK;
+    const int per_row = (n + 15) / 16, i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= per_row * n) return;
+    const int y = i / per_row, x0 = (i % per_row) * 16, z = blockIdx.y;
+    const int *fl = flags + ((z / edge) * nb + y / edge) * nb;
+    uint8_t *o = mask + ((size_t)z * n + y) * n + x0;
+    uint32_t w[4] = {0, 0, 0, 0};
+    int bx = x0 / edge, left = (bx + 1) * edge - x0;      // cells left in the block
+#pragma unroll
+    for (int a = 0; a < 16; ++a) {
+        if (x0 + a < n) w[a / 4] |= (uint32_t)(fl[bx] != 0) << (8 * (a % 4));
+        if (--left == 0) {
+            bx = min(bx + 1, nb - 1);
+            left = edge;
+        }
+    }
+    if ((n & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0) *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+    else
+        for (int a = 0; a < 16 && x0 + a < n; ++a) o[a] = (uint8_t)(w[a / 4] >> (8 * (a % 4)));
 }
 
-__global__ void k_combine(const float *__restrict__ Sp, const float *__restrict__ Sf, const int *__restrict__ flags,
-                          int lgD, int f, float *__restrict__ out) {
-    const int D = 1 << lgD;
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+// Sp in passing blocks, the mean of the fine cells (in the order x, y, z) in failing ones
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_combine(const float *__restrict__ Sp, const float *__restrict__ Sf,
+                                                 const int *__restrict__ flags, int lgD, int f, float *__restrict__ out) {
+    const int D = 1 << lgD, n = D * f;
+    const int v = blockIdx.x * 256 + threadIdx.x;
     if (v >= D * D * D) return;
     if (!flags[block_of(v, lgD)]) {
         out[v] = Sp[v];
         return;
     }
     float acc = 0.f;
-    for (int a = 0; a < f * f * f; ++a) acc += Sf[fine_cell(v, lgD, f, a)];
+    const float *plane = Sf + fine_cell(v, lgD, f, 0);
+    for (int k = 0; k < f; ++k, plane += (size_t)n * n) {
+        const float *row = plane;
+#pragma unroll 4
+        for (int j = 0; j < f; ++j, row += n) {
+            if (VEC) {
+                for (int i = 0; i < f; i += 4) {
+                    const float4 q = __ldg(reinterpret_cast<const float4 *>(row + i));
+                    acc += q.x; acc += q.y; acc += q.z; acc += q.w;
+                }
+            } else {
+                for (int i = 0; i < f; ++i) acc += row[i];
+            }
+        }
+    }
     out[v] = acc / (float)(f * f * f);
 }
 
@@ -367,20 +412,19 @@ void apply_residual(const float *Sc, const float *y, int use_net, float *Sp, siz
     if (n) k_apply_residual<<<blocks_for(n), 256, 0, st>>>(Sc, y, use_net, Sp, n);
 }
 void block_pred_err(const float *y, int lgD, float *pe, cudaStream_t st) {
-    const int nb = nblocks_of(lgD);
-    k_block_pred_err<<<blocks_for(nb, 128), 128, 0, st>>>(y, lgD, pe, nb);
+    k_block_pred_err<<<nblocks_of(lgD), 128, 0, st>>>(y, lgD, pe);
 }
 void judge_mask(int lgD, int factor, uint64_t seed, int samples, uint8_t *mask, int *sample_vox, cudaStream_t st) {
     const size_t n = (size_t)(factor << lgD);
     cudaMemsetAsync(mask, 0, n * n * n, st);
     const int nb = nblocks_of(lgD);
-    k_judge_pick<<<blocks_for((size_t)nb * samples, 128), 128, 0, st>>>(lgD, factor, seed, samples, mask, sample_vox,
-                                                                      nb);
+    k_judge_pick<<<blocks_for((size_t)nb * samples * factor * factor, 128), 128, 0, st>>>(lgD, factor, seed, samples, mask,
+                                                                                        sample_vox, nb);
 }
 void judge_err(const float *Sf, const float *Sp, const int *sample_vox, int lgD, int factor, int samples, float *err,
                cudaStream_t st) {
     const int nb = nblocks_of(lgD);
-    k_judge_err<<<blocks_for(nb, 128), 128, 0, st>>>(Sf, Sp, sample_vox, lgD, factor, samples, err, nb);
+    k_judge_err<<<blocks_for(nb, 4), 128, 0, st>>>(Sf, Sp, sample_vox, lgD, factor, samples, err, nb);
 }
 void fallback_flags(const float *err, const float *pe, int use_pred, float tol, int nblocks, int *flags,
                     unsigned *counts, cudaStream_t st) {
@@ -388,12 +432,15 @@ void fallback_flags(const float *err, const float *pe, int use_pred, float tol, 
     k_fallback_flags<<<blocks_for(nblocks, 128), 128, 0, st>>>(err, pe, use_pred, tol, nblocks, flags, counts);
 }
 void fallback_mask(const int *flags, int lgD, int factor, uint8_t *mask, cudaStream_t st) {
-    const size_t n = (size_t)(factor << lgD);
-    k_fallback_mask<<<blocks_for(n * n * n), 256, 0, st>>>(flags, lgD, factor, mask);
+    const int n = factor << lgD;
+    k_fallback_mask<<<dim3(blocks_for((size_t)((n + 15) / 16) * n), n), 256, 0, st>>>(flags, lgD, factor, mask);
 }
 void combine(const float *Sp, const float *Sf, const int *flags, int lgD, int factor, float *out, cudaStream_t st) {
     const size_t n = (size_t)1 << (3 * lgD);
-    k_combine<<<blocks_for(n), 256, 0, st>>>(Sp, Sf, flags, lgD, factor, out);
+    if (factor % 4 == 0 && (reinterpret_cast<uintptr_t>(Sf) & 15) == 0)
+        k_combine<true><<<blocks_for(n), 256, 0, st>>>(Sp, Sf, flags, lgD, factor, out);
+    else
+        k_combine<false><<<blocks_for(n), 256, 0, st>>>(Sp, Sf, flags, lgD, factor, out);
 }
 
 }  // namespace nn

@@ -489,9 +489,8 @@ int sph_nn_make_inputs(sph_nn *n, int nf, int factor, const float *I, const floa
     NCK(cudaSetDevice(n->device));
     const size_t nc = (size_t)n->edge * n->edge * n->edge;
     float *Ic = n->scratch, *Im = n->scratch + nc, *Ec = E ? n->scratch + 2 * nc : nullptr;
-    pool_avg_f32(I, nf, factor, Ic, n->stream);
-    pool_max_f32(I, nf, factor, Im, n->stream);
-    if (E) pool_avg_f32(E, nf, factor, Ec, n->stream);
+    pool_f32(I, nf, factor, Ic, Im, n->stream);
+    if (E) pool_f32(E, nf, factor, Ec, nullptr, n->stream);
     max4(Ic, Ec, S, Im, nc, n->maxbits, n->stream);
     make_inputs(Ic, Ec, S, Im, n->maxbits, x, nc, n->stream);
     NCK(cudaGetLastError());
@@ -504,7 +503,7 @@ int sph_nn_make_target(sph_nn *n, int nf, int factor, const float *Sf, const flo
     if (n->poisoned) return SPH_ECUDA;
     NCK(cudaSetDevice(n->device));
     const size_t nc = (size_t)n->edge * n->edge * n->edge;
-    pool_avg_f32(Sf, nf, factor, n->scratch, n->stream);
+    pool_f32(Sf, nf, factor, n->scratch, nullptr, n->stream);
     make_target(n->scratch, Sc, t, nc, n->stream);
     NCK(cudaGetLastError());
     return SPH_OK;
@@ -513,7 +512,7 @@ int sph_nn_make_target(sph_nn *n, int nf, int factor, const float *Sf, const flo
 int sph_pool_avg(int device, void *stream, int nf, int factor, const float *fine, float *coarse) {
     if (!fine || !coarse || factor < 1 || nf < factor || nf % factor) return SPH_EINVAL;
     if (cudaSetDevice(device) != cudaSuccess) return SPH_ECUDA;
-    pool_avg_f32(fine, nf, factor, coarse, static_cast<cudaStream_t>(stream));
+    pool_f32(fine, nf, factor, coarse, nullptr, static_cast<cudaStream_t>(stream));
     return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ECUDA;
 }
 

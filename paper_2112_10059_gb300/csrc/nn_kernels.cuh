@@ -101,8 +101,8 @@ void make_images(const float *w, int C, int N, uint16_t *img_fwd, uint16_t *img_
 void f32_to_bf16(const float *in, uint16_t *out, size_t n, cudaStream_t st);
 
 // coarse inputs of the network from pooled fields
-void pool_avg_f32(const float *fine, int n_fine, int f, float *coarse, cudaStream_t st);
-void pool_max_f32(const float *fine, int n_fine, int f, float *coarse, cudaStream_t st);
+// mean and largest value over f^3 blocks of an n_fine^3 field (avg or mx may be null)
+void pool_f32(const float *fine, int n_fine, int f, float *avg, float *mx, cudaStream_t st);
 void max4(const float *a, const float *b, const float *c, const float *d, size_t n, unsigned *maxbits,
           cudaStream_t st);
 void make_inputs(const float *I, const float *E, const float *S, const float *Imax, const unsigned *maxbits,

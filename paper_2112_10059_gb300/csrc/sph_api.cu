@@ -859,8 +859,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
         if (tm) tm->mark_at(15, c->near_stream);
         if (c->list_tot[2] > 0 && F.O.method == FAR_CHEB) {
             // only the leaves with W entries (at most one per W entry)
-            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), out, c->near_stream, 1, 2, 16, S.w_wl,
-                    S.w_cnt + 39, c->list_tot[2]);
+            fmm_near_w(F, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), S.w_wl, S.w_cnt + 39, c->list_tot[2], c->near_stream);
             ++c->launches;
         }
         if (tm) tm->mark_at(13, c->near_stream);
@@ -1717,7 +1716,7 @@ int run_surrogate(sph_ctx *c, sph_nn *net, int factor, double tol, int samples, 
     } guard{ev};
     CK(cudaEventRecord(ev[0], s));
     // 1. coarse FMM on the pooled source
-    nn::pool_avg_f32(c->q, n, factor, P<float>(c->s_qc), s);
+    nn::pool_f32(c->q, n, factor, P<float>(c->s_qc), nullptr, s);
     sph_problem pc;
     pc.nx = pc.ny = pc.nz = D;
     pc.h_cm = c->h * factor; pc.pO2_torr = c->pO2; pc.chi_min = c->chi_min; pc.chi_max = c->chi_max;

@@ -292,14 +292,14 @@ void fmm_work_lists(const FmmDev &F, int nboxes, int *src_list, int *src_cnt, in
 // p2p_list, passes [pass_lo, pass_hi); adds into out, or into F.near_buf where it is set (pass 0
 // clears the leaf's slots; a launch of pass 1 alone must follow the one of pass 0).  At most
 // per_sm CTAs per SM (grid-stride over the leaves).
-// w_list / w_cnt (a launch of pass 1 alone): walk only those leaves (fmm_work_lists), with a
-// grid of at most max_w CTAs
 void fmm_p2p(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,
-             cudaStream_t st, int pass_lo = 0, int pass_hi = 2, int per_sm = 16, const int *w_list = nullptr,
-             const int *w_cnt = nullptr, int max_w = 0);
+             cudaStream_t st, int pass_lo = 0, int pass_hi = 2, int per_sm = 16);
 // the U-list part into the leaves' slots of F.near_buf by the offset table, for the same lists
 void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, cudaStream_t st,
                    int per_sm);
+// the W-list part (Chebyshev far field) of the leaves in w_list (fmm_work_lists; at most max_w), added to the slots
+void fmm_near_w(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, const int *w_list, const int *w_cnt,
+                int max_w, cudaStream_t st);
 // out[cell of t] += F.near_buf[slot of t] for every target of every leaf of those lists
 // flags / flags_host (optional): flags[0..2) copied to the mapped host address flags_host once
 // every earlier kernel of the stream has completed
