@@ -1,13 +1,9 @@
 // Far-field translations as batched, gathered GEMMs (FP32 SIMT, register tiled).
 //
-// M2L (paper Section 2.4, far interactions through the hierarchy): for a tile
-// of 64 consecutive target boxes B of one level and every one of the 316
-// offsets o, the rows u_A of the source boxes A = B + o that lie in V(B) are
-// gathered (zero where there is none) and multiplied by the level's M2L_o:
-//     d_B += sum_o M2L_o u_{B+o}
-// so each operator is read once per tile instead of once per box pair.  V(B)
-// membership is recomputed from the dense level array: A exists, holds
-// sources, and the parents of A and B are adjacent (|o|_inf >= 2 always).
+// M2L (paper Section 2.4, far interactions through the hierarchy): for a tile of 64 V pairs (target
+// box B, source box A) of one level and offset o,
+//     d_B += M2L_o u_A,
+// so that an operator is read once per tile instead of once per box pair.
 //
 // L2L: for a tile of 64 parent boxes P of level l-1 and one child slot c,
 //     d_{child c of P} += L2L_c d_P.
@@ -18,6 +14,7 @@
 // are stored transposed ([k][i], row stride npad), so an operator K-slab is a
 // contiguous, coalesced read.
 #include "sph_kernels.cuh"
+#include "tc_sm103.cuh"
 
 namespace sph {
 
@@ -40,129 +37,104 @@ __device__ __forceinline__ void mma_tile(const float (*As)[TM], const float (*Bs
     }
 }
 
-// acc += Op[i0.., :] * X[:, cols]: Op transposed [k][i] with row stride ldA and M valid rows,
-// K = np; X columns = state rows src[col] (row stride np).
+// shared memory of a tile: two K slabs of each operand, then the staged results
+constexpr int TS = TM + 4;                                  // row stride of a staged column
+constexpr int TILE_FLOATS = TN * TS > 2 * TK * (TM + TN) ? TN * TS : 2 * TK * (TM + TN);
+
+// acc += Op[i0.., :] * X[:, cols]: Op transposed [k][i] with row stride ldA and M valid rows (VEC:
+// multiples of 4, 16-byte aligned), K = np; X columns = state rows src[col] (row stride np).  The
+// next slab is loaded into registers under this slab's FMAs and stored into the other buffer:
+// these launches have few CTAs, so a slab whose loads were waited for took three times its FMAs
+// (L2L of the four levels of a 90 x 61 x 117 grid 125 us with the loads waited for and 32 scalar
+// reductions a thread, 71 us so; M2L of its 32,013 pairs 116, 89).
+template <bool VEC>
 __device__ __forceinline__ void gemm_slab_g(const float *__restrict__ opT, int ldA, int M, int np, int i0,
-                                            const float *__restrict__ state, const int *src, float (*As)[TM],
-                                            float (*Bs)[TN], float acc[8][4]) {
+                                            const float *__restrict__ state, const int *src, float *smem, float acc[8][4]) {
+    float (*As)[TK][TM] = reinterpret_cast<float (*)[TK][TM]>(smem);
+    float (*Bs)[TK][TN] = reinterpret_cast<float (*)[TK][TN]>(smem + 2 * TK * TM);
     const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-    for (int k0 = 0; k0 < np; k0 += TK) {
-        for (int e = tid; e < TK * TM; e += 256) {
-            int kk = e / TM, ii = e % TM;
-            int i = i0 + ii;
-            As[kk][ii] = i < M ? __ldg(opT + (size_t)(k0 + kk) * ldA + i) : 0.f;
+    const int bc = tid % TN, bq = tid / TN, s = src[bc];    // this thread's column and quarter of a slab
+    float a[8];
+    float4 b;
+    auto load = [&](int k0) {
+        if (VEC) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int e = tid + 256 * j, i = i0 + e % 32 * 4;
+                const float4 v = i < M ? __ldg(reinterpret_cast<const float4 *>(opT + (size_t)(k0 + e / 32) * ldA + i))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+                a[4 * j] = v.x; a[4 * j + 1] = v.y; a[4 * j + 2] = v.z; a[4 * j + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int e = tid + 256 * j, i = i0 + e % TM;
+                a[j] = i < M ? __ldg(opT + (size_t)(k0 + e / TM) * ldA + i) : 0.f;
+            }
         }
-        for (int e = tid; e < TK * TN; e += 256) {
-            int c = e / TK, kk = e % TK;
-            int s = src[c];
-            Bs[kk][c] = s >= 0 ? state[(size_t)s * np + k0 + kk] : 0.f;
+        b = s >= 0 ? *reinterpret_cast<const float4 *>(state + (size_t)s * np + k0 + 4 * bq) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto store = [&](int buf) {
+        if (VEC) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int e = tid + 256 * j;
+                *reinterpret_cast<float4 *>(&As[buf][e / 32][e % 32 * 4]) = make_float4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) As[buf][(tid + 256 * j) / TM][(tid + 256 * j) % TM] = a[j];
         }
-        __syncthreads();
-        mma_tile(As, Bs, ty, tx, acc);
+        Bs[buf][4 * bq][bc] = b.x;
+        Bs[buf][4 * bq + 1][bc] = b.y;
+        Bs[buf][4 * bq + 2][bc] = b.z;
+        Bs[buf][4 * bq + 3][bc] = b.w;
+    };
+    load(0);
+    store(0);
+    __syncthreads();
+    for (int k0 = 0, buf = 0; k0 < np; k0 += TK, buf ^= 1) {
+        if (k0 + TK < np) load(k0 + TK);
+        mma_tile(As[buf], Bs[buf], ty, tx, acc);
+        if (k0 + TK < np) store(buf ^ 1);
         __syncthreads();
     }
 }
 
 __device__ __forceinline__ void gemm_slab(const float *__restrict__ opT, int np, int i0,
-                                          const float *__restrict__ state, const int *src, float (*As)[TM],
-                                          float (*Bs)[TN], float acc[8][4]) {
-    gemm_slab_g(opT, np, np, np, i0, state, src, As, Bs, acc);
+                                          const float *__restrict__ state, const int *src, float *smem, float acc[8][4]) {
+    gemm_slab_g<true>(opT, np, np, np, i0, state, src, smem, acc);
 }
 
-__device__ __forceinline__ void scatter_atomic(float *__restrict__ out, int np, int n, int i0, const int *dst,
-                                               const float acc[8][4]) {
-    const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-#pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-        int d = dst[tx * 4 + cc];
-        if (d < 0) continue;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            int i = i0 + ty * 8 + r;
-            if (i < n) atomicAdd(out + (size_t)d * np + i, acc[r][cc]);
-        }
-    }
-}
-
+// out[dst[c]][i0 ..] += the tile's column c, a row of up to 128 values each by one bulk reduction
+// (32 scalar reductions a thread, each warp's to 32 different rows, took as long as the FMAs).
+// Ends with the staged columns read.
 __device__ __forceinline__ void scatter_add(float *__restrict__ out, int np, int n, int i0, const int *dst,
-                                            const float acc[8][4]) {
+                                            float *smem, const float acc[8][4]) {
     const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-        int d = dst[tx * 4 + cc];
-        if (d < 0) continue;
+    for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            int i = i0 + ty * 8 + r;
-            if (i < n) atomicAdd(out + (size_t)d * np + i, acc[r][cc]);   // reduction: no dependent load
+        for (int h = 0; h < 2; ++h) {
+            float v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) v[r] = i0 + ty * 8 + 4 * h + r < n ? acc[4 * h + r][cc] : 0.f;
+            *reinterpret_cast<float4 *>(smem + (tx * 4 + cc) * TS + ty * 8 + 4 * h) = make_float4(v[0], v[1], v[2], v[3]);
         }
-    }
-}
-
-// ---------------------------------------------------------------- M2L
-__global__ void __launch_bounds__(256) k_m2l_gemm(FmmDev F, int level, int box_begin, int box_count) {
-    pdl_enter();
-    __shared__ __align__(16) float As[TK][TM];
-    __shared__ __align__(16) float Bs[TK][TN];
-    __shared__ int trg[TN], src[TN];
-    __shared__ int tco[TN][3];
-    const int tid = threadIdx.x;
-    const int np = F.O.npad, n = F.O.n;
-    const int t0 = blockIdx.x * TN;
-    const int i0 = blockIdx.y * TM;
-    const TreeDev &T = F.T;
-    // early exit when no box of the tile has a V list
-    int first = box_begin + t0, last = box_begin + min(t0 + TN, box_count);
-    if (F.L.v_off[first] == F.L.v_off[last]) return;
-    if (tid < TN) {
-        int b = box_begin + t0 + tid;
-        int ok = (t0 + tid < box_count) && (T.b_te[b] > T.b_tb[b]);
-        trg[tid] = ok ? b : -1;
-        uint32_t x = 0, y = 0, z = 0;
-        if (ok) demorton3(T.b_key[b], x, y, z);
-        tco[tid][0] = x; tco[tid][1] = y; tco[tid][2] = z;
+    tc::fence_proxy_async_smem();
+    __syncthreads();
+    if (tid < TN && dst[tid] >= 0) {
+        tc::bulk_reduce_add_f32(out + (size_t)dst[tid] * np + i0, tc::smem_u32(smem + tid * TS), (uint32_t)min(TM, np - i0) * 4u);
+        tc::bulk_commit();
+        tc::bulk_wait_read_all();
     }
     __syncthreads();
-    const int nside = 1 << level;
-    const int *bat = T.box_at + dense_off(level);
-    const float *Mlev = F.O.m2l_t + (size_t)level * NSLOT * np * np;
-    float acc[8][4];
-#pragma unroll
-    for (int r = 0; r < 8; ++r)
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) acc[r][cc] = 0.f;
-    int slot = 0;
-    for (int code = 0; code < SPH_NOFF; ++code) {
-        const int ox = code % 7 - 3, oy = (code / 7) % 7 - 3, oz = code / 49 - 3;
-        if (abs(ox) <= 1 && abs(oy) <= 1 && abs(oz) <= 1) continue;   // uniform: same for all threads
-        int found = 0;
-        if (tid < TN) {
-            int a = -1;
-            if (trg[tid] >= 0) {
-                int bx = tco[tid][0], by = tco[tid][1], bz = tco[tid][2];
-                int ax = bx + ox, ay = by + oy, az = bz + oz;
-                bool in = ax >= 0 && ay >= 0 && az >= 0 && ax < nside && ay < nside && az < nside;
-                bool padj = abs((ax >> 1) - (bx >> 1)) <= 1 && abs((ay >> 1) - (by >> 1)) <= 1 &&
-                            abs((az >> 1) - (bz >> 1)) <= 1;
-                if (in && padj) {
-                    int A = bat[morton3(ax, ay, az)];
-                    if (A >= 0 && T.b_se[A] > T.b_sb[A]) a = A;
-                }
-            }
-            src[tid] = a;
-            found = a >= 0;
-        }
-        if (__syncthreads_or(found)) gemm_slab(Mlev + (size_t)slot * np * np, np, i0, F.ueq, src, As, Bs, acc);
-        ++slot;
-    }
-    scatter_add(F.dchk, np, n, i0, trg, acc);
 }
 
 // ---------------------------------------------------------------- L2L
 __global__ void __launch_bounds__(256) k_l2l_gemm(FmmDev F, int level, int parent_begin, int parent_count) {
     pdl_enter();
-    __shared__ __align__(16) float As[TK][TM];
-    __shared__ __align__(16) float Bs[TK][TN];
+    __shared__ __align__(16) float tile_s[TILE_FLOATS];
     __shared__ int par[TN], dst[TN];
     const int tid = threadIdx.x;
     const int np = F.O.npad, n = F.O.n;
@@ -188,8 +160,8 @@ __global__ void __launch_bounds__(256) k_l2l_gemm(FmmDev F, int level, int paren
     for (int r = 0; r < 8; ++r)
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) acc[r][cc] = 0.f;
-    gemm_slab(F.O.l2l_t + ((size_t)level * 8 + c) * np * np, np, i0, F.dchk, par, As, Bs, acc);
-    scatter_add(F.dchk, np, n, i0, dst, acc);
+    gemm_slab(F.O.l2l_t + ((size_t)level * 8 + c) * np * np, np, i0, F.dchk, par, tile_s, acc);
+    scatter_add(F.dchk, np, n, i0, dst, tile_s, acc);
 }
 
 // ---------------------------------------------------------------- V pairs grouped by offset
@@ -201,8 +173,7 @@ __global__ void __launch_bounds__(256) k_l2l_gemm(FmmDev F, int level, int paren
 // One CTA per tile of up to 64 V pairs sharing (level, offset): d_B += M2L_{l,o} u_A, scatter-added.
 __global__ void __launch_bounds__(256) k_m2l_pairs(FmmDev F, PairsDev Pd) {
     pdl_enter();
-    __shared__ __align__(16) float As[TK][TM];
-    __shared__ __align__(16) float Bs[TK][TN];
+    __shared__ __align__(16) float tile_s[TILE_FLOATS];
     __shared__ int trg[TN], src[TN];
     __shared__ int s_key;
     const int tid = threadIdx.x;
@@ -229,8 +200,8 @@ __global__ void __launch_bounds__(256) k_m2l_pairs(FmmDev F, PairsDev Pd) {
         for (int r = 0; r < 8; ++r)
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) acc[r][cc] = 0.f;
-        gemm_slab(M, np, i0, F.ueq, src, As, Bs, acc);
-        scatter_atomic(F.dchk, np, n, i0, trg, acc);
+        gemm_slab(M, np, i0, F.ueq, src, tile_s, acc);
+        scatter_add(F.dchk, np, n, i0, trg, tile_s, acc);
     }
 }
 
@@ -251,9 +222,9 @@ void fmm_m2l_pairs(const FmmDev &F, const PairsDev &Pd, int nV, int m2l_prec, cu
 __global__ void __launch_bounds__(256) k_l2p_gemm(FmmDev F, int level, int box_begin, int box_count,
                                                   float *__restrict__ out) {
     pdl_enter();
-    __shared__ __align__(16) float As[TK][TM];
-    __shared__ __align__(16) float Bs[TK][TN];
-    __shared__ float Cs[TM][TN + 1];
+    __shared__ __align__(16) float tile[TM * (TN + 1)];     // the operands' slabs, then the results
+    float (*Cs)[TN + 1] = reinterpret_cast<float (*)[TN + 1]>(tile);
+    static_assert(TM * (TN + 1) >= 2 * TK * (TM + TN), "tile");
     __shared__ int col[TN];
     const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
     const int np = F.O.npad;
@@ -275,7 +246,7 @@ __global__ void __launch_bounds__(256) k_l2p_gemm(FmmDev F, int level, int box_b
     for (int r = 0; r < 8; ++r)
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) acc[r][cc] = 0.f;
-    gemm_slab_g(F.O.e_tab + F.O.e_off[level], rows, rows, np, i0, F.dchk, col, As, Bs, acc);
+    gemm_slab_g<false>(F.O.e_tab + F.O.e_off[level], rows, rows, np, i0, F.dchk, col, tile, acc);
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -301,12 +272,6 @@ void fmm_l2p_gemm_level(const FmmDev &F, int level, int box_begin, int box_count
     int e = 1 << (F.D - level);
     dim3 grid((box_count + TN - 1) / TN, (e * e * e + TM - 1) / TM);
     launch_pdl(k_l2p_gemm, grid, 256, 0, st, F, level, box_begin, box_count, out);
-}
-
-void fmm_m2l_gemm_level(const FmmDev &F, int level, int box_begin, int box_count, cudaStream_t st) {
-    if (box_count <= 0 || level < 2) return;
-    dim3 grid((box_count + TN - 1) / TN, (F.O.npad + TM - 1) / TM);
-    launch_pdl(k_m2l_gemm, grid, 256, 0, st, F, level, box_begin, box_count);
 }
 
 void fmm_l2l_gemm_level(const FmmDev &F, int level, int parent_begin, int parent_count, cudaStream_t st) {
