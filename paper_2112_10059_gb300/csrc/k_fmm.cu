@@ -5,10 +5,10 @@
 // Every box carries two state vectors of n values (rows padded to npad): u_B
 // from the sources inside B and d_B from the sources far from B (see OpsDev for
 // their meaning under FAR_CHEB / FAR_SURFACE).
-//   k_upward     level l, boxes with sources:
-//                  leaf  -> P2M: FAR_CHEB    u_B[m] = sum_s S_m(y_s) w_s  (anterpolation)
+//   k_upward, k_p2m_small   level l, leaves with sources:
+//                  P2M: FAR_CHEB    u_B[m] = sum_s S_m(y_s) w_s  (anterpolation)
 //                                FAR_SURFACE u_B[i] = sum_s G(|x_i - y_s|) w_s (check potential)
-//                  other -> M2M: u_B = sum over children c of M2M_c u_c.
+//   k_m2m_simt   level l, split boxes with sources: u_B = sum over children c of M2M_c u_c.
 //   k_m2l_simt   level l, target boxes with a V list: d_B += M2L_o u_A (FP32 SIMT).
 //   k_p2l        X list: d_B[i] += sum over the coarser leaf's sources of G(|x_i - y_s|) w_s.
 //   k_down       level l >= 3: d_B += L2L_c d_parent.
@@ -79,7 +79,6 @@ __device__ __forceinline__ void upward_box(const FmmDev &F, int level, int b) {
     int sb = T.b_sb[b], se = T.b_se[b];
     if (se <= sb) return;
     const int n = F.O.n, np = F.O.npad;
-    __shared__ float vec[MAXPAD];
     __shared__ float part[2][MAXPAD];
     __shared__ uint32_t spc[UT];
     __shared__ float sw[UT];
@@ -150,36 +149,65 @@ __device__ __forceinline__ void upward_box(const FmmDev &F, int level, int b) {
         part[half][pt] = acc;
         __syncthreads();
         if (tid < np) u[tid] = tid < n ? part[0][tid] + part[1][tid] : 0.f;
-    } else {
-        // M2M from the children (level + 1)
-        float acc = 0.f;
-        uint32_t ck = T.b_key[b] << 3;
-        const int *bat = T.box_at + dense_off(level + 1);
+    }
+}
+
+// FP32 M2M of the split boxes of a level: u = sum over the children c of M2M_c u_c.  The threads
+// are groups of npad, as many as fit a CTA (8 at order 5: a child each), thread t of a group owning
+// row t; the operators' columns are read 8 at a time.  Few boxes have this work and a box's
+// operators are 512 KB from L2, so it is bound by latency: one CTA of two groups taking the
+// children in turn took 48 / 34 / 27 / 16 us for 116 / 32 / 10 / 6 boxes, 15 so.
+__global__ void __launch_bounds__(1024, 1) k_m2m_simt(FmmDev F, int level, const int *__restrict__ list,
+                                                   const int *__restrict__ count) {
+    pdl_enter();
+    __shared__ float vec[8][MAXPAD];
+    __shared__ float part[1024];
+    const TreeDev &T = F.T;
+    const int n = F.O.n, np = F.O.npad, tid = threadIdx.x, groups = blockDim.x / np;
+    const int pt = tid % np, g = tid / np;
+    const int *bat = T.box_at + dense_off(level + 1);
+    const int cnt = *count;
+    for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
+        const int b = list[i];
+        if (T.b_leaf[b]) continue;                           // uniform across the CTA
+        const uint32_t ck = T.b_key[b] << 3;
+        unsigned have = 0;
+#pragma unroll
         for (int c = 0; c < 8; ++c) {
-            int C = bat[ck + c];
-            if (C < 0 || T.b_se[C] <= T.b_sb[C]) continue;   // uniform across the CTA
-            __syncthreads();
-            if (tid < np) vec[tid] = F.ueq[(size_t)C * np + tid];
-            __syncthreads();
-            const float *M = F.O.m2m_t + ((size_t)level * 8 + c) * np * np;
-            for (int j = half; j < n; j += 2) acc = fmaf(M[(size_t)j * np + pt], vec[j], acc);
+            const int C = bat[ck + c];
+            have |= (C >= 0 && T.b_se[C] > T.b_sb[C] ? 1u : 0u) << c;
         }
-        part[half][pt] = acc;
         __syncthreads();
-        if (tid < np) u[tid] = tid < n ? part[0][tid] + part[1][tid] : 0.f;
+        for (int e = tid; e < 8 * np; e += blockDim.x) {
+            const int c = e / np;
+            if (have >> c & 1) vec[c][e % np] = F.ueq[(size_t)bat[ck + c] * np + e % np];
+        }
+        __syncthreads();
+        float acc = 0.f;
+        for (int c = g; c < 8; c += groups) {
+            if (!(have >> c & 1)) continue;
+            const float *M = F.O.m2m_t + ((size_t)level * 8 + c) * np * np + pt;
+#pragma unroll 8
+            for (int j = 0; j < n; ++j) acc = fmaf(__ldg(M + (size_t)j * np), vec[c][j], acc);
+        }
+        part[tid] = acc;
+        __syncthreads();
+        if (tid < np) {
+            for (int k = 1; k < groups; ++k) acc += part[k * np + tid];
+            F.ueq[(size_t)b * np + tid] = tid < n ? acc : 0.f;
+        }
     }
 }
 
 // CTAs walk the compact list of this level's boxes that hold sources.
-// kinds: 0 every box, 1 the leaves alone (the split boxes' M2M runs on the tensor cores, k_m2m_tc),
-// 2 the split boxes alone (the leaves' P2M runs in k_p2m_small)
+// P2M of its leaves (the split boxes' M2M: k_m2m_simt, or k_m2m_tc on the tensor cores).
 __global__ void __launch_bounds__(2 * MAXPAD) k_upward(FmmDev F, int level, const int *__restrict__ list,
-                                                       const int *__restrict__ count, int kinds) {
+                                                       const int *__restrict__ count) {
     pdl_enter();
     const int cnt = *count;
     for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
         const int b = list[i];
-        if (kinds != 0 && (kinds == 1) != (F.T.b_leaf[b] != 0)) continue;   // uniform across the CTA
+        if (!F.T.b_leaf[b]) continue;        // uniform across the CTA
         upward_box(F, level, b);
         __syncthreads();
     }
@@ -275,18 +303,20 @@ static void p2m_small_launch(const FmmDev &F, int level, int boxes, const int *l
 int fmm_upward_level(const FmmDev &F, int level, int box_count, int leaf_count, const int *list, const int *count,
                      bool leaves_only, cudaStream_t st) {
     if (box_count <= 0 || level < 2) return 0;
-    int kinds = leaves_only ? 1 : 0, launches = 0;
-    if (F.O.method == FAR_CHEB && F.D - level <= 2) {
-        if (leaf_count > 0) {
+    int launches = 0;
+    if (leaf_count > 0) {
+        if (F.O.method == FAR_CHEB && F.D - level <= 2)
             p2m_small_launch(F, level, box_count, list, count, st);
-            ++launches;
-        }
-        if (leaves_only || leaf_count == box_count) return launches;
-        kinds = 2;
+        else
+            launch_pdl(k_upward, std::min(box_count, 152 * 8), 2 * F.O.npad, 0, st, F, level, list, count);
+        ++launches;
     }
-    int grid = box_count < 152 * 8 ? box_count : 152 * 8;
-    launch_pdl(k_upward, grid, 2 * F.O.npad, 0, st, F, level, list, count, kinds);
-    return launches + 1;
+    if (!leaves_only && box_count > leaf_count) {
+        const int groups = std::min(8, 1024 / F.O.npad);
+        launch_pdl(k_m2m_simt, std::min(box_count, 152 * 2), groups * F.O.npad, 0, st, F, level, list, count);
+        ++launches;
+    }
+    return launches;
 }
 
 // Compact work lists: per level the boxes with sources (stored in the level's box range),
@@ -308,7 +338,8 @@ __device__ __forceinline__ int warp_append(unsigned act, bool pred, int *counter
 __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, int *__restrict__ src_cnt,
                              int *__restrict__ leaf_list, int *__restrict__ leaf_cnt, int *__restrict__ p2p_list,
                              int *__restrict__ p2p_cnt, int p2p_stride, int *__restrict__ own_list,
-                             int *__restrict__ own_cnt, int *__restrict__ w_list, int *__restrict__ w_cnt) {
+                             int *__restrict__ own_cnt, int *__restrict__ w_list, int *__restrict__ w_cnt,
+                             int *__restrict__ x_list, int *__restrict__ x_cnt) {
     pdl_enter();
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nboxes) return;
@@ -344,6 +375,9 @@ __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, i
     }
     i = warp_append(act, own && leaf_t, own_cnt);
     if (own && leaf_t) own_list[i] = b;
+    const bool has_x = l >= 2 && F.L.x_off[b + 1] != F.L.x_off[b];
+    i = warp_append(act, has_x, x_cnt);
+    if (has_x) x_list[i] = b;
     // per level, the leaves with targets (the separable L2P walks these only; the fused deepest
     // level, whose boxes start at d_sparse_from, needs no list)
     const bool l2p = leaf_t && l >= 2 && F.l2p_list != nullptr && !(F.d_sparse_from >= 0 && b >= F.d_sparse_from);
@@ -384,10 +418,10 @@ __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, i
 
 void fmm_work_lists(const FmmDev &F, int nboxes, int *src_list, int *src_cnt, int *leaf_list, int *leaf_cnt,
                     int *p2p_list, int *p2p_cnt, int p2p_stride, int *own_list, int *own_cnt, cudaStream_t st,
-                    int *w_list, int *w_cnt) {
+                    int *w_list, int *w_cnt, int *x_list, int *x_cnt) {
     if (nboxes <= 0) return;
     launch_pdl(k_work_lists, (nboxes + 255) / 256, 256, 0, st, F, nboxes, src_list, src_cnt, leaf_list, leaf_cnt, p2p_list,
-                                                       p2p_cnt, p2p_stride, own_list, own_cnt, w_list, w_cnt);
+                                                       p2p_cnt, p2p_stride, own_list, own_cnt, w_list, w_cnt, x_list, x_cnt);
 }
 
 // ------------------------------------------------------------------ M2L (FP32 SIMT)
@@ -421,63 +455,6 @@ void fmm_m2l_level(const FmmDev &F, int level, int box_begin, int box_count, int
     if (box_count <= 0 || level < 2) return;
     (void)m2l_prec;
     launch_pdl(k_m2l_simt, box_count, 2 * F.O.npad, 0, st, F, level, box_begin, box_count);
-}
-
-// ------------------------------------------------------------------ P2L (X list)
-__global__ void __launch_bounds__(2 * MAXPAD) k_p2l(FmmDev F, int level, int box_begin, int box_count) {
-    pdl_enter();
-    int b = box_begin + blockIdx.x;
-    if (blockIdx.x >= box_count) return;
-    int x0 = F.L.x_off[b], x1 = F.L.x_off[b + 1];
-    if (x1 <= x0) return;
-    const int n = F.O.n, np = F.O.npad;
-    __shared__ uint32_t spc[UT];
-    __shared__ float sw[UT];
-    __shared__ float part[2][MAXPAD];
-    const int tid = threadIdx.x, pt = tid % np, half = tid / np;
-    const int size = 1 << (F.D - level);
-    const float w = F.kp.h * size * 0.5f;
-    const float hh = 0.5f * F.kp.h;
-    const float rad = F.O.method == FAR_CHEB ? w : (float)F.O.r.dc * w;
-    int bx, by, bz;
-    box_coords(F.T, b, bx, by, bz);
-    float cx = 0, cy = 0, cz = 0;
-    if (pt < n) {
-        cx = rad * F.O.nodes[4 * pt + 0];
-        cy = rad * F.O.nodes[4 * pt + 1];
-        cz = rad * F.O.nodes[4 * pt + 2];
-    }
-    float acc = 0.f;
-    for (int x = x0; x < x1; ++x) {
-        int A = F.L.x_src[x];
-        int sb = F.T.b_sb[A], se = F.T.b_se[A];
-        for (int s0 = sb; s0 < se; s0 += UT) {
-            int m = min(UT, se - s0);
-            __syncthreads();
-            for (int v = tid; v < m; v += blockDim.x) {
-                spc[v] = F.src_pc[s0 + v];
-                sw[v] = F.src_q[s0 + v] * F.wscale;
-            }
-            __syncthreads();
-            if (pt < n) {
-                for (int v = half; v < m; v += 2) {
-                    uint32_t pc = spc[v];
-                    float sx, sy, sz;
-                    rel_cell(pc_i(pc), pc_j(pc), pc_k(pc), bx, by, bz, size, hh, sx, sy, sz);
-                    float dx = cx - sx, dy = cy - sy, dz = cz - sz;
-                    acc = fmaf(g_of_r2(dx * dx + dy * dy + dz * dz, F.kp), sw[v], acc);
-                }
-            }
-        }
-    }
-    part[half][pt] = acc;
-    __syncthreads();
-    if (tid < n) F.dchk[(size_t)b * np + tid] += part[0][tid] + part[1][tid];
-}
-
-void fmm_p2l_level(const FmmDev &F, int level, int box_begin, int box_count, cudaStream_t st) {
-    if (box_count <= 0 || level < 2) return;
-    launch_pdl(k_p2l, box_count, 2 * F.O.npad, 0, st, F, level, box_begin, box_count);
 }
 
 // ------------------------------------------------------------------ downward: L2L
@@ -1240,6 +1217,84 @@ static P2PConst p2p_const(const FmmDev &F) {
     // the self weight multiplies the scaled weight w' = w C / h^3: g_self w = (g_self h^3 / C) w'
     K.wself = F.self_mode ? F.kp.gself * h * h * h / F.kp.C : 0.f;
     return K;
+}
+
+// ---------------------------------------------------------------- P2L (X lists)
+// d_B += the field of the X-list leaves' sources at B's nodes, for the boxes in x_list (those
+// with X entries, of every level: one launch).  The sources of 32 entries at a time are staged in
+// cell units, a warp an entry; thread t sums node t % npad over one half of them in the near
+// field's scaled form.  A launch per level with a CTA for every box, an entry at a time, its cells
+// converted for every node and pair, took 161 us for the 157,431 boxes of one level of a snapshot
+// and 46 us on a ragged 90 x 61 x 117 grid, 15 there so.
+constexpr int PX_CAP = 1024;
+
+template <bool TAYLOR>
+__global__ void __launch_bounds__(2 * MAXPAD, 1) k_p2l(FmmDev F, P2PConst K, const int *__restrict__ list,
+                                                    const int *__restrict__ count) {
+    pdl_enter();
+    __shared__ float4 stage[PX_CAP];
+    __shared__ float part[MAXPAD];
+    const TreeDev &T = F.T;
+    const int n = F.O.n, np = F.O.npad, tid = threadIdx.x, pt = tid % np, half = tid / np;
+    const int warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+    const float h = F.kp.h, wsc = F.wscale * F.kp.C / (h * h * h);
+    const float4 node = __ldg(reinterpret_cast<const float4 *>(F.O.nodes) + pt);   // padded to np rows
+    const int cnt = *count;
+    for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
+        const int b = list[i], size = 1 << (F.D - T.b_level[b]);
+        uint32_t ux, uy, uz;
+        demorton3(T.b_key[b], ux, uy, uz);
+        const float r = 0.5f * (float)size, rad = F.O.method == FAR_CHEB ? r : (float)F.O.r.dc * r;
+        const float cx = (float)ux * size + r - 0.5f + rad * node.x, cy = (float)uy * size + r - 0.5f + rad * node.y,
+                    cz = (float)uz * size + r - 0.5f + rad * node.z;
+        float acc = 0.f;
+        const int x1 = F.L.x_off[b + 1];
+        for (int x0 = F.L.x_off[b]; x0 < x1; x0 += 32) {     // lane k of every warp: entry x0 + k
+            int sb = 0, m = 0;
+            if (x0 + lane < x1) {
+                const int A = F.L.x_src[x0 + lane];
+                sb = T.b_sb[A];
+                m = T.b_se[A] - sb;
+            }
+            int off = m;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int q = __shfl_up_sync(0xffffffffu, off, o);
+                if (lane >= o) off += q;
+            }
+            const int total = __shfl_sync(0xffffffffu, off, 31);
+            off -= m;
+            for (int r0 = 0; r0 < total; r0 += PX_CAP) {
+                __syncthreads();
+                for (int e = warp; e < 32; e += nw) {
+                    const int me = __shfl_sync(0xffffffffu, m, e), at = __shfl_sync(0xffffffffu, off, e) - r0;
+                    const int first = __shfl_sync(0xffffffffu, sb, e);
+                    for (int q = lane; q < me; q += 32)
+                        if ((unsigned)(at + q) < (unsigned)PX_CAP) {
+                            const uint32_t pc = __ldg(F.src_pc + first + q);
+                            stage[at + q] = make_float4((float)pc_i(pc), (float)pc_j(pc), (float)pc_k(pc),
+                                                        __ldg(F.src_q + first + q) * wsc);
+                        }
+                }
+                __syncthreads();
+                const int rn = min(PX_CAP, total - r0), mid = rn / 2;
+                acc += p2p_sum<TAYLOR, false>(stage, half ? mid : 0, half ? rn : mid, cx, cy, cz, K, nullptr);
+            }
+        }
+        if (half) part[pt] = acc;
+        __syncthreads();
+        if (!half && pt < n) F.dchk[(size_t)b * np + pt] += acc + part[pt];
+        __syncthreads();
+    }
+}
+
+int fmm_p2l(const FmmDev &F, const int *list, const int *count, int max_boxes, cudaStream_t st) {
+    if (max_boxes <= 0) return 0;
+    const P2PConst K = p2p_const(F);
+    const int grid = std::min(max_boxes, 152 * 4);
+    if (K.bma_h >= 0.5f) launch_pdl(k_p2l<false>, grid, 2 * F.O.npad, 0, st, F, K, list, count);
+    else launch_pdl(k_p2l<true>, grid, 2 * F.O.npad, 0, st, F, K, list, count);
+    return 1;
 }
 
 // ---------------------------------------------------------------- near field (U lists) by offset table

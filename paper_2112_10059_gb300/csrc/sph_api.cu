@@ -676,7 +676,7 @@ struct PhaseTimer {
 // ------------------------------------------------------------------ FMM passes
 struct PassState {
     FmmDev F;
-    int *w_src = nullptr, *w_leaf = nullptr, *w_p2p = nullptr, *w_cnt = nullptr, *w_own = nullptr, *w_wl = nullptr;
+    int *w_src = nullptr, *w_leaf = nullptr, *w_p2p = nullptr, *w_cnt = nullptr, *w_own = nullptr, *w_wl = nullptr, *w_xl = nullptr;
     PairsDev Pd;
     int *err = nullptr;
     bool tc = false;
@@ -698,7 +698,7 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
     const size_t vb = (size_t)std::max(nb, 1) * c->npad() * sizeof(float);
     ENS(c->b_ueq, vb);
     ENS(c->b_dchk, vb);
-    ENS(c->b_work, ((5 + P2P_CLASSES) * (size_t)std::max(nb, 1) + 64) * sizeof(int));
+    ENS(c->b_work, ((6 + P2P_CLASSES) * (size_t)std::max(nb, 1) + 64) * sizeof(int));
     ENS(c->b_err, 16 * sizeof(int));
     FmmDev &F = S.F;
     F.T = tree_dev(c);
@@ -731,6 +731,7 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
     F.l2p_list = S.w_cnt + 64;                  // [nb], per level at lvl_base[l]
     S.w_own = F.l2p_list + std::max(nb, 1);     // [nb]: deepest-level leaves with V / X entries, count w_cnt[62]
     S.w_wl = S.w_own + std::max(nb, 1);         // [nb]: near-field leaves with W entries, count w_cnt[39]
+    S.w_xl = S.w_wl + std::max(nb, 1);          // [nb]: boxes with X entries, count w_cnt[63]
     F.l2p_cnt = S.w_cnt + 40;                   // [16]
     S.Pd = pairs_dev(c);
     S.err = P<int>(c->b_err);
@@ -812,7 +813,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
     // the mapped read-back buffer, where that kernel runs; else by copies
     const bool err_mapped = c->pinned_dev && F.near_buf && nb > 0;
     fmm_work_lists(F, nb, S.w_src, S.w_cnt, S.w_leaf, S.w_cnt + 32, S.w_p2p, S.w_cnt + 56, std::max(nb, 1),
-                   S.w_own, S.w_cnt + 62, c->stream, S.w_wl, S.w_cnt + 39);
+                   S.w_own, S.w_cnt + 62, c->stream, S.w_wl, S.w_cnt + 39, S.w_xl, S.w_cnt + 63);
     c->launches += nb > 0;
     const bool near_fork = F.near_buf && nb > 0;
     if (near_fork) {
@@ -868,13 +869,10 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
     c->l2lp_used = fused && c->lvl_count[c->Lmax - 1] > 0;
     if (c->translate_per_box) {
         if (tm) { tm->mark_at(5, c->stream); tm->mark_at(6, c->stream); }
+        c->launches += fmm_p2l(F, S.w_xl, S.w_cnt + 63, c->list_tot[3], c->stream);
         for (int l = 2; l <= c->Lmax; ++l) {
             fmm_m2l_level(F, l, c->lvl_base[l], c->lvl_count[l], c->m2l_prec, c->stream);
             c->launches += c->lvl_count[l] > 0;
-            if (c->list_tot[3] > 0) {
-                fmm_p2l_level(F, l, c->lvl_base[l], c->lvl_count[l], c->stream);
-                c->launches += c->lvl_count[l] > 0;
-            }
             fmm_down_level(F, l, c->lvl_base[l], c->lvl_count[l], c->stream);
             c->launches += l >= 3 && c->lvl_count[l] > 0;
         }
@@ -901,11 +899,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
             c->launches += nV > 0;
         }
         if (tm) tm->mark_at(6, c->stream);
-        for (int l = 2; l <= c->Lmax; ++l)
-            if (c->list_tot[3] > 0) {
-                fmm_p2l_level(F, l, c->lvl_base[l], c->lvl_count[l], c->stream);
-                c->launches += c->lvl_count[l] > 0;
-            }
+        c->launches += fmm_p2l(F, S.w_xl, S.w_cnt + 63, c->list_tot[3], c->stream);
         for (int l = 3; l <= c->Lmax - (fused ? 1 : 0); ++l) {
             // 8 children per CTA where that still gives every SM a CTA; one child per CTA (8x the
             // CTAs, 1/8 of the serial work each) for the small upper levels

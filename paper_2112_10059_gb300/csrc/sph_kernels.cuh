@@ -283,11 +283,11 @@ constexpr int64_t P2P_CLASS0 = 1 << 16;
 // p2p_list: P2P_CLASSES lists of p2p_stride slots, p2p_cnt: their P2P_CLASSES counts
 // own_list / own_cnt: the deepest-level leaves with targets and V or X entries (where
 // F.d_sparse_from >= 0), for fmm_l2p_own
-// w_list / w_cnt (optional): the near-field leaves with W entries, each as its slot in the class
-// lists (class x p2p_stride + index in the class), for a launch of the W-list pass alone
+// w_list / w_cnt: the near-field leaves with W entries, each as its slot in the class lists (class x
+// p2p_stride + index in the class); x_list / x_cnt: the boxes with X entries
 void fmm_work_lists(const FmmDev &F, int nboxes, int *src_list, int *src_cnt, int *leaf_list, int *leaf_cnt,
                     int *p2p_list, int *p2p_cnt, int p2p_stride, int *own_list, int *own_cnt, cudaStream_t st,
-                    int *w_list = nullptr, int *w_cnt = nullptr);
+                    int *w_list, int *w_cnt, int *x_list, int *x_cnt);
 // near field over the U lists (pass 0) and W lists (pass 1) of the leaves in the class lists of
 // p2p_list, passes [pass_lo, pass_hi); adds into out, or into F.near_buf where it is set (pass 0
 // clears the leaf's slots; a launch of pass 1 alone must follow the one of pass 0).  At most
@@ -307,7 +307,7 @@ void fmm_near_add(const FmmDev &F, int nboxes, const int *p2p_list, const int *p
                   cudaStream_t st,
                   const int *flags = nullptr, int *flags_host = nullptr);
 void fmm_m2l_level(const FmmDev &F, int level, int box_begin, int box_count, int m2l_prec, cudaStream_t st);
-void fmm_p2l_level(const FmmDev &F, int level, int box_begin, int box_count, cudaStream_t st);
+int fmm_p2l(const FmmDev &F, const int *list, const int *count, int max_boxes, cudaStream_t st);   // kernels launched
 void fmm_down_level(const FmmDev &F, int level, int box_begin, int box_count, cudaStream_t st);
 void fmm_leaf(const FmmDev &F, int nboxes, const int *list, const int *count, float *out_dense, cudaStream_t st);
 // tensor-core L2P (FAR_CHEB, images present): writes S at the targets of the level's leaves
@@ -336,7 +336,6 @@ constexpr int GTAB_N = 4096;           // table of the scaled kernel for squared
 void fmm_near_table(const FmmDev &F, float *gtab, cudaStream_t st);
 size_t l2p_image_elems(int edge);
 void make_l2p_images(const float *etab, int edge, int n, uint16_t *img, cudaStream_t st);
-void fmm_m2l_gemm_level(const FmmDev &F, int level, int box_begin, int box_count, cudaStream_t st);
 // V pairs grouped by (level, offset slot): built once per tree, then one M2L launch for all levels.
 struct PairsDev {
     int nkeys;            // (Lmax + 1) * 316
