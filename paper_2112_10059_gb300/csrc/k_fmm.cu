@@ -325,6 +325,7 @@ int fmm_upward_level(const FmmDev &F, int level, int box_count, int leaf_count, 
 // Append with one atomic per (warp, counter): lanes with `pred` that share a counter get
 // consecutive slots from the group's leader.  Every lane of `act` must call it.
 __device__ __forceinline__ int warp_append(unsigned act, bool pred, int *counter) {
+    if (!__any_sync(act, pred)) return 0;     // most warps append to few of the lists
     const int lane = threadIdx.x & 31;
     const unsigned long long key = pred ? reinterpret_cast<unsigned long long>(counter) : 0ull;
     const unsigned grp = __match_any_sync(act, key);

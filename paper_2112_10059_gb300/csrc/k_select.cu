@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
     uint32_t bx, by, bz;
     demorton3(brick, bx, by, bz);
     const int x0 = (int)bx << 4, y0 = (int)by << 4, z0 = (int)bz << 4;
+    if (x0 >= r.nx || y0 >= r.ny || z0 >= r.nz) return;      // outside the grid: never looked at
     const int tid = threadIdx.x, seg = tid & 3;
     float mq = -INFINITY, lo = INFINITY, hi = -INFINITY;
     bool nan_e = false;
@@ -340,12 +341,29 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
             }
         }
     } else {
-        for (int i = tid; i < 4096; i += STAT_T) {
-            const int x = x0 + (i & 15), y = y0 + ((i >> 4) & 15), z = z0 + (i >> 8);
-            const bool in = x < r.nx && y < r.ny && z < r.nz;
-            const int64_t lin = in ? (int64_t)x + (int64_t)r.nx * ((int64_t)y + (int64_t)r.ny * z) : 0;
-            take(in && q ? __ldg(q + lin) : 0.f, in && e ? __ldg(e + lin) : 0.f, in);
-            if (in && mk) take_mask(__ldg(mk + lin));
+        // an odd pitch: cell by cell, eight planes' loads in flight at a time (48 us on
+        // 222^3 one after another, 33 so)
+        const int x = x0 + (tid & 15), y = y0 + (tid >> 4);
+        const bool col = x < r.nx && y < r.ny;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float a[8], c[8];
+            uint32_t m[8];
+            bool in[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int z = z0 + 8 * h + k;
+                in[k] = col && z < r.nz;
+                const int64_t lin = in[k] ? (int64_t)x + (int64_t)r.nx * ((int64_t)y + (int64_t)r.ny * z) : 0;
+                a[k] = in[k] && q ? __ldg(q + lin) : 0.f;
+                c[k] = in[k] && e ? __ldg(e + lin) : 0.f;
+                m[k] = in[k] && mk ? __ldg(mk + lin) : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                take(a[k], c[k], in[k]);
+                if (in[k] && mk) take_mask(m[k]);
+            }
         }
     }
 #pragma unroll
@@ -375,21 +393,29 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
     }
 }
 
-// Status of brick `brick` from its statistics (st, as k_brick_stats): 1 if no cell is a source
-// and every cell a target, 2 if no cell is selected at all, 0 if the cells must be read.  Only a
-// brick of 16^3 cells wholly inside the grid is decided this way; the comparisons are those of
-// the per-cell rules (v >= threshold in FP32, NaN never selected).
+// Status of brick `brick` of 16^3 cells from its statistics (st, as k_brick_stats): 1 if none of
+// its cells inside the grid is a source and each of them a target, 2 if none is selected (a brick
+// outside the grid has none), 0 if the cells must be read.  The comparisons are those of the
+// per-cell rules (v >= threshold in FP32, NaN never selected).  Bricks that reach past the grid,
+// and those of the enclosing power-of-two cube that lie outside it (1352 of 4096 on 222^3, where
+// another 547 reach past it), are decided as well: reading them took the count pass there 35 us
+// and the emit pass 58, now 8 and 38.
 __device__ __forceinline__ int brick_mode(const SelRule &r, uint32_t brick, float4 st, float thr_q, float thr_e,
                                           bool qpos) {
     uint32_t bx, by, bz;
     demorton3(brick, bx, by, bz);
-    if (((int)bx << 4) + 16 > r.nx || ((int)by << 4) + 16 > r.ny || ((int)bz << 4) + 16 > r.nz) return 0;
+    if (((int)bx << 4) >= r.nx || ((int)by << 4) >= r.ny || ((int)bz << 4) >= r.nz) return 2;
     if (r.src_all || (qpos && st.x >= thr_q)) return 0;       // a source in the brick
     if (r.trg_mode == 0) return 1;
     if (r.trg_mode == 2) return st.y >= 0.5f ? 1 : (st.z < 0.5f ? 2 : 0);   // wholly inside or outside the mask
     if (st.w == 0.f && st.y >= thr_e) return 1;               // every |E| at or above the threshold
     if (!(st.z >= thr_e)) return 2;                           // none
     return 0;
+}
+
+// cells inside the grid of the brick of 16^3 at (x0, y0, z0)
+__device__ __forceinline__ int brick_cells(const SelRule &r, int x0, int y0, int z0) {
+    return max(0, min(16, r.nx - x0)) * max(0, min(16, r.ny - y0)) * max(0, min(16, r.nz - z0));
 }
 
 // Decoupled look-back by the whole block: 512 predecessor states per round (every brick in
@@ -478,11 +504,12 @@ constexpr int SEL_T = 512;
 // Cell u sits at (mx + (u & 1), my + ((u >> 1) & 1), mz + (u >> 2)): the pairs (u, u + 1), u
 // even, are x-neighbours at an even x, read as one float2 when the row pitch and the arrays
 // allow it.  The target mask is written if `tmask` (two cells per 2-byte store where aligned).
+// `given`: the brick is known to hold no source and only targets, nothing is read.
 __device__ __forceinline__ void cube_rules(const SelRule &r, const float *__restrict__ q, const float *__restrict__ e,
                                            const uint8_t *__restrict__ mask, int tid, int x0, int y0, int z0,
                                            int ncell, float thr_q, float thr_e, bool qpos,
                                            uint8_t *__restrict__ tmask, int (&my_bits)[8], float (&my_q)[8],
-                                           uint32_t &mx, uint32_t &my, uint32_t &mz) {
+                                           uint32_t &mx, uint32_t &my, uint32_t &mz, bool given = false) {
     demorton3((uint32_t)(8 * tid), mx, my, mz);
     const bool vec2 = (r.nx & 1) == 0 && (reinterpret_cast<uintptr_t>(q) & 7) == 0 &&
                       (r.trg_mode != 1 || (reinterpret_cast<uintptr_t>(e) & 7) == 0);
@@ -499,7 +526,9 @@ __device__ __forceinline__ void cube_rules(const SelRule &r, const float *__rest
         const uint32_t l0 = row ? (uint32_t)x + (uint32_t)r.nx * ((uint32_t)y + (uint32_t)r.ny * (uint32_t)z) : 0u;
         lin[u0] = l0;
         lin[u0 + 1] = l0 + 1;
-        if (vec2 && in[u0 + 1] && r.trg_mode != 2) {
+        if (given) {
+            my_q[u0] = my_q[u0 + 1] = ev[u0] = ev[u0 + 1] = 0.f;
+        } else if (vec2 && in[u0 + 1] && r.trg_mode != 2) {
             const float2 a = __ldg(reinterpret_cast<const float2 *>(q + l0));
             my_q[u0] = a.x;
             my_q[u0 + 1] = a.y;
@@ -520,7 +549,9 @@ __device__ __forceinline__ void cube_rules(const SelRule &r, const float *__rest
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         int bits = 0;
-        if (in[u]) {
+        if (given) {
+            bits = in[u] ? 2 : 0;
+        } else if (in[u]) {
             if (r.src_all || (qpos && my_q[u] >= thr_q)) bits |= 1;
             if (r.trg_mode == 0) bits |= 2;
             else if (r.trg_mode == 1) { if (ev[u] >= thr_e) bits |= 2; }
@@ -610,15 +641,16 @@ __device__ __forceinline__ void cube_emit(uint32_t brick, int b, int tid, int x0
     }
 }
 
-// A brick of 16^3 cells decided by its statistics (mode 1: every cell a target, mode 2: none;
-// no source either way): its target mask, and for mode 1 its 4096 targets from trg_key[pt0]
-// in Morton order (keys brick << 12 | i).
+// A brick of 16^3 cells decided by its statistics (mode 1: every cell a target, the brick wholly
+// inside the grid; mode 2: none; no source either way): its target mask, and for mode 1 its 4096
+// targets from trg_key[pt0] in Morton order (keys brick << 12 | i).
 __device__ __forceinline__ void brick_emit_decided(const SelRule &r, uint32_t brick, int mode, int tid, int x0,
                                                    int y0, int z0, unsigned pt0, uint32_t *__restrict__ trg_key,
                                                    uint32_t *__restrict__ trg_pc, uint8_t *__restrict__ tmask) {
     if (tmask) {
         const uint8_t m = mode == 1 ? 1 : 0;
-        if ((r.nx & 15) == 0 && (reinterpret_cast<uintptr_t>(tmask) & 15) == 0) {
+        if ((r.nx & 15) == 0 && (reinterpret_cast<uintptr_t>(tmask) & 15) == 0 &&
+            brick_cells(r, x0, y0, z0) == 4096) {
             for (int row = tid; row < 256; row += blockDim.x) {   // one 16-byte store per row
                 const int64_t o = (int64_t)x0 + (int64_t)r.nx * ((int64_t)(y0 + (row & 15)) +
                                                                  (int64_t)r.ny * (z0 + (row >> 4)));
@@ -626,12 +658,21 @@ __device__ __forceinline__ void brick_emit_decided(const SelRule &r, uint32_t br
                 *reinterpret_cast<uint4 *>(tmask + o) = make_uint4(m4, m4, m4, m4);
             }
         } else {
-            for (int i = tid; i < 4096; i += blockDim.x)
-                tmask[(int64_t)(x0 + (i & 15)) +
-                      (int64_t)r.nx * ((int64_t)(y0 + ((i >> 4) & 15)) + (int64_t)r.ny * (z0 + (i >> 8)))] = m;
+            for (int i = tid; i < 4096; i += blockDim.x) {
+                const int x = x0 + (i & 15), y = y0 + ((i >> 4) & 15), z = z0 + (i >> 8);
+                if (x < r.nx && y < r.ny && z < r.nz)
+                    tmask[(int64_t)x + (int64_t)r.nx * ((int64_t)y + (int64_t)r.ny * z)] = m;
+            }
         }
     }
     if (mode != 1) return;
+    if (!trg_pc && ((reinterpret_cast<uintptr_t>(trg_key + pt0)) & 15) == 0) {   // four keys a store
+        for (int i = 4 * tid; i < 4096; i += 4 * (int)blockDim.x) {
+            const uint32_t k = (brick << 12) | (uint32_t)i;
+            *reinterpret_cast<uint4 *>(trg_key + pt0 + i) = make_uint4(k, k + 1, k + 2, k + 3);
+        }
+        return;
+    }
     for (int i = tid; i < 4096; i += blockDim.x) {
         trg_key[pt0 + i] = (brick << 12) | (uint32_t)i;
         if (trg_pc) {
@@ -677,6 +718,11 @@ __global__ void __launch_bounds__(SEL_T) k_select_onepass(
         s_brick = (int)atomicAdd(ticket, 1u);
         block_thresholds(r, maxes, &s_thr_q, &s_thr_e, &s_qpos);
         s_mode = bstat ? brick_mode(r, (uint32_t)s_brick, bstat[s_brick], s_thr_q, s_thr_e, s_qpos) : 0;
+        if (s_mode == 1) {                         // targets of a brick that reaches past the grid: ranked below
+            uint32_t ux, uy, uz;
+            demorton3((uint32_t)s_brick, ux, uy, uz);
+            if (brick_cells(r, (int)ux << 4, (int)uy << 4, (int)uz << 4) != 4096) s_mode = 0;
+        }
     }
     __syncthreads();
     const int brick = s_brick;
@@ -747,7 +793,9 @@ __global__ void __launch_bounds__(SEL_T) k_select_count(SelRule r, const float *
             const int m = brick_mode(r, (uint32_t)bk, bstat[bk], s_thr_q, s_thr_e, s_qpos);
             if (m != 0) {
                 cnt_s[bk] = 0;
-                cnt_t[bk] = m == 1 ? ncell : 0;
+                uint32_t ux, uy, uz;
+                demorton3((uint32_t)bk, ux, uy, uz);
+                cnt_t[bk] = m == 1 ? brick_cells(r, (int)ux << b, (int)uy << b, (int)uz << b) : 0;
             } else {
                 s_und[atomicAdd(&s_nund, 1)] = (int)bk;
             }
@@ -817,7 +865,7 @@ __global__ void __launch_bounds__(SEL_T) k_select_emit(
             demorton3(brick, bx, by, bz);
             const int x0 = bx << b, y0 = by << b, z0 = bz << b;
             const int mode = s_mode[j];
-            if (mode != 0) {
+            if (mode == 2 || (mode == 1 && brick_cells(r, x0, y0, z0) == 4096)) {
                 brick_emit_decided(r, brick, mode, tid, x0, y0, z0, (unsigned)s_ot[j], trg_key, trg_pc, tmask);
                 continue;
             }
@@ -825,7 +873,7 @@ __global__ void __launch_bounds__(SEL_T) k_select_emit(
             float my_q[8];
             uint32_t mx, my, mz;
             cube_rules(r, q, e, mask, tid, x0, y0, z0, ncell, s_thr_q, s_thr_e, s_qpos, tmask, my_bits, my_q, mx,
-                       my, mz);
+                       my, mz, mode == 1);
             int ns = 0, nt = 0;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {

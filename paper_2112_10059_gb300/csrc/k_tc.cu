@@ -1238,6 +1238,10 @@ __global__ void __launch_bounds__(LP_T, 1) k_l2lp_tc(FmmDev F, int level, int pa
     const uint32_t idesc = tc::idesc_bf16_f32(TCM, 64);
     const int q = warp & 3, r = q * 32 + lane;              // TMEM lane quadrant, parent row
     const bool vec_ok = (F.nx % 4) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    const int64_t ncell = (int64_t)F.nx * F.ny * F.nz;
+    __shared__ float4 s_row[LP_T / 32][32];
+    __shared__ int64_t s_base[LP_T / 32][32];
+    __shared__ uint32_t s_keep[LP_T / 32][32];
     // child c's cells: warps w and w + 4 share TMEM lanes 32 (w % 4) .. and take half of
     // the 64 columns each
     auto epilogue = [&](int c) {
@@ -1253,9 +1257,10 @@ __global__ void __launch_bounds__(LP_T, 1) k_l2lp_tc(FmmDev F, int level, int pa
 #pragma unroll
         for (int h = 0; h < 2; ++h)
             tc::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(64 * c + 32 * (warp >> 2) + 16 * h), w[h]);
-        if (C < 0) return;
-        const bool inside = bx + 4 <= F.nx && by + 4 <= F.ny && bz + 4 <= F.nz;
-        if (vec_ok && inside) {
+        // in a warp whose boxes all lie inside the grid (or are none)
+        const bool inside = C < 0 || (bx + 4 <= F.nx && by + 4 <= F.ny && bz + 4 <= F.nz);
+        if (vec_ok && __all_sync(0xffffffffu, inside)) {
+            if (C < 0) return;
             // one 16-byte store per row of 4 cells; in a partly selected box the non-target
             // cells of a row get their zero in the same store (never a partial 32-byte sector,
             // which the memory system would have to merge), the row's 4 mask bytes read as one
@@ -1284,27 +1289,53 @@ __global__ void __launch_bounds__(LP_T, 1) k_l2lp_tc(FmmDev F, int level, int pa
                 }
             return;
         }
-        // partly selected or overhanging box: every mask byte is fetched before the first
-        // store (a byte load placed after a float store would wait for it)
-        bool keep[2][16];
+        // a row pitch or box that 16-byte rows do not fit: each row of 4 cells goes through shared
+        // memory to the 4 lanes of its cells, so that a store covers 8 rows of 16 bytes and not
+        // one cell of 32 rows.  A row's 4 mask bytes come out of the one or two aligned words that
+        // hold them, all words in flight at once and before the first store (222^3 cells: 127 us
+        // in all with 32 byte loads one after another, 79 so).
+        uint32_t keep = full ? 0xffffffffu : 0u;
+        if (__any_sync(0xffffffffu, C >= 0 && !full)) {
+            uint32_t m0[8], m1[8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int cell = 32 * (warp >> 2) + 16 * h + j;
-                const int x = bx + (cell & 3), y = by + ((cell >> 2) & 3), z = bz + (cell >> 4);
-                const bool inb = full || (x < F.nx && y < F.ny && z < F.nz);   // box overhangs the grid
-                const int64_t o = (int64_t)x + (int64_t)F.nx * ((int64_t)y + (int64_t)F.ny * z);
-                keep[h][j] = inb && (full || __ldg(F.tmask + o) != 0);
+            for (int row = 0; row < 8; ++row) {
+                const int cell = 32 * (warp >> 2) + 4 * row;
+                const int y = by + ((cell >> 2) & 3), z = bz + (cell >> 4);
+                const int64_t o = (int64_t)bx + (int64_t)F.nx * ((int64_t)y + (int64_t)F.ny * z);
+                const uint32_t *pm = reinterpret_cast<const uint32_t *>(F.tmask) + (o >> 2);
+                const bool rd = C >= 0 && !full && y < F.ny && z < F.nz;
+                m0[row] = m1[row] = 0;
+                if (rd) m0[row] = __ldg(pm);
+                if (rd && (o & 3) != 0 && (o | 3) + 1 < ncell) m1[row] = __ldg(pm + 1);
             }
+            const uint32_t xin = bx + 4 <= F.nx ? 15u : (1u << max(0, F.nx - bx)) - 1u;   // box overhangs the grid
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int cell = 32 * (warp >> 2) + 16 * h + j;
-                const int x = bx + (cell & 3), y = by + ((cell >> 2) & 3), z = bz + (cell >> 4);
-                if (keep[h][j]) out[(int64_t)x + (int64_t)F.nx * ((int64_t)y + (int64_t)F.ny * z)] = w[h][j];
+            for (int row = 0; row < 8; ++row) {
+                const int cell = 32 * (warp >> 2) + 4 * row;
+                const int y = by + ((cell >> 2) & 3), z = bz + (cell >> 4);
+                const int64_t o = (int64_t)bx + (int64_t)F.nx * ((int64_t)y + (int64_t)F.ny * z);
+                const uint32_t m = __funnelshift_r(m0[row], m1[row], 8 * (int)(o & 3));
+                keep |= (((m & 1u) | (m >> 7 & 2u) | (m >> 14 & 4u) | (m >> 21 & 8u)) & xin) << (4 * row);
             }
+        }
+        __syncwarp();                              // the previous child's words have been read
+        s_keep[warp][lane] = keep;
+        s_base[warp][lane] = (int64_t)bx + (int64_t)F.nx * ((int64_t)by + (int64_t)F.ny * bz);
+#pragma unroll
+        for (int row = 0; row < 8; ++row) {
+            __syncwarp();
+            s_row[warp][lane] = make_float4(w[row >> 2][4 * (row & 3)], w[row >> 2][4 * (row & 3) + 1],
+                                            w[row >> 2][4 * (row & 3) + 2], w[row >> 2][4 * (row & 3) + 3]);
+            __syncwarp();
+            const int cell = 32 * (warp >> 2) + 4 * row;
+            const int64_t ro = (int64_t)F.nx * ((int64_t)((cell >> 2) & 3) + (int64_t)F.ny * (cell >> 4)) + (lane & 3);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int L = 8 * i + (lane >> 2);
+                if (s_keep[warp][L] >> (4 * row + (lane & 3)) & 1u)
+                    out[s_base[warp][L] + ro] = reinterpret_cast<const float *>(&s_row[warp][L])[lane & 3];
+            }
+        }
     };
     int g = 0;                                              // rounds of this CTA so far
     bool waited = false;

@@ -259,7 +259,7 @@ int select_queue(sph_ctx *c, bool copy = true) {
     ENS(c->b_spc, ncell * sizeof(uint32_t));
     ENS(c->b_sq, ncell * sizeof(float));
     ENS(c->b_tkey, ncell * sizeof(uint32_t));
-    ENS(c->b_tmask, ncell);
+    ENS(c->b_tmask, (ncell + 3) & ~(int64_t)3);      // read in 4-byte words
     ENS(c->b_bstat, nbr * 4 * sizeof(float));
     SelectArgs A;
     A.nx = c->nx; A.ny = c->ny; A.nz = c->nz; A.D = D; A.brick_log2 = b;

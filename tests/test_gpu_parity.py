@@ -5,6 +5,8 @@
 * adaptive FMM: rel-L2 <= 1e-3 over the targets and max-rel <= 1e-2 on targets
   with S > 1e-3 max S (the accuracy gate), 0 at every non-target cell.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -190,6 +192,27 @@ def test_selection_whole_bricks_of_a_mask(sph, monkeypatch, dims, shift):
         J, T = sph.get_selection(c)
         c.close()
         assert np.array_equal(J, Jo) and np.array_equal(T, To), (two, lb)
+
+
+@pytest.mark.parametrize("rule", ["emag", "all"])
+@pytest.mark.parametrize("dims", [(51, 38, 45), (33, 49, 31), (66, 35, 32)])
+def test_selection_bricks_past_the_grid(sph, monkeypatch, dims, rule):
+    """Grids with bricks that reach past them and bricks of the enclosing cube outside them, both
+    decided by the statistics pass: the oracle's sets in all three selection forms, and the
+    FMM's results on a row pitch that no 16-byte store fits (odd, and twice an odd number)."""
+    p = si.brick_structured(*dims)
+    if rule == "all":
+        p = dataclasses.replace(p, targets_all=True)
+    ref, Jo, To = oracle.sph_problem(p)
+    for two, lb in SELECT_FORMS:
+        monkeypatch.setenv("SPH_SELECT_TWO_PASS", two)
+        monkeypatch.setenv("SPH_SELECT_LOOKBACK", lb)
+        c = sph.Context(0)
+        _, out, _ = sph.solve(p, c, m2l_precision=sph.M2L_BF16X3)
+        J, T = sph.get_selection(c)
+        c.close()
+        assert np.array_equal(J, Jo) and np.array_equal(T, To), (two, lb)
+        _check_fmm(out.cpu().numpy(), ref, To, p.name)
 
 
 @pytest.mark.parametrize("case", [(16, 16, 16, 0.05, 0.3, 8, 2), (12, 9, 7, 0.2, 0.1, 4, 3),
