@@ -20,9 +20,12 @@
 //                       FAR_SURFACE FP64 equivalent density of A, then FP64 kernel sums.
 // CTAs of the box kernels have 2 * npad threads: thread t owns state row t % npad
 // and half (t / npad) of the reduction, so each matrix column is read coalesced.
+#include <cuda_bf16.h>
+
 #include <algorithm>
 
 #include "sph_kernels.cuh"
+#include "tc_sm103.cuh"
 
 namespace sph {
 
@@ -336,6 +339,11 @@ __device__ __forceinline__ int warp_append(unsigned act, bool pred, int *counter
     return base + __popc(grp & ((1u << lane) - 1u));
 }
 
+// A leaf's near field costs the matrix form (k_near_mma) 2.5 ns of the whole chip whatever its
+// sources, the table form (k_near_grid) 12.6 ps a source (both measured on the uniform 128^3 tree): they are
+// level at 200 of the 1728 cells, more where tiles are few.
+constexpr int NEAR_MMA_MIN = 384;
+
 __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, int *__restrict__ src_cnt,
                              int *__restrict__ leaf_list, int *__restrict__ leaf_cnt, int *__restrict__ p2p_list,
                              int *__restrict__ p2p_cnt, int p2p_stride, int *__restrict__ own_list,
@@ -389,17 +397,21 @@ __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, i
     // near-field leaves by their number of kernel evaluations (targets x U-list sources and
     // W-list nodes), in classes of halving size, so that the near field can start the heaviest
     // first and end on light ones
-    int cls = P2P_CLASSES - 1;
+    int cls = P2P_MMA - 1;
     if (p2p) {
         int64_t ns = 0;
+        bool same = l == F.near_mma_level && T.b_te[b] - T.b_tb[b] == NM_CELLS;
         for (int u = F.L.u_off[b]; u < F.L.u_off[b + 1]; ++u) {
             const int A = F.L.u_src[u];
             ns += T.b_se[A] - T.b_sb[A];
+            if (same) same = T.b_level[A] == l;
         }
+        const bool dense = same && ns >= NEAR_MMA_MIN;
         if (F.O.method == FAR_CHEB) ns += (int64_t)(F.L.w_off[b + 1] - F.L.w_off[b]) * F.O.n;   // W nodes
         const int64_t w = ns * (T.b_te[b] - T.b_tb[b]);
         cls = 0;
-        while (cls < P2P_CLASSES - 1 && w < (P2P_CLASS0 >> cls)) ++cls;
+        while (cls < P2P_MMA - 1 && w < (P2P_CLASS0 >> cls)) ++cls;
+        if (dense) cls = P2P_MMA;
     }
     int my_idx = 0;
     for (int c = 0; c < P2P_CLASSES; ++c) {
@@ -1331,7 +1343,8 @@ __device__ __forceinline__ void near_grid_sum(const int2 *__restrict__ pts, int 
 
 template <bool TAYLOR>
 __global__ void __launch_bounds__(P2P_WARPS * 32) k_near_grid(FmmDev F, const int *__restrict__ list,
-                                                              const int *__restrict__ count, int stride, P2PConst K) {
+                                                              const int *__restrict__ count, int stride,
+                                                              const int *__restrict__ near_max, P2PConst K) {
     pdl_enter();
     __shared__ float tab[NG_N + 1];
     __shared__ __align__(16) int2 stage[NG_CAP];
@@ -1346,7 +1359,8 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_near_grid(FmmDev F, const in
     __syncthreads();
     int nitems = 0;
 #pragma unroll
-    for (int c = 0; c < P2P_CLASSES; ++c) nitems += ccnt[c];
+    for (int c = 0; c < P2P_MMA; ++c) nitems += ccnt[c];
+    if (F.near_mma_level >= 0 && !near_mma_range(*near_max)) nitems += ccnt[P2P_MMA];
     if ((int)blockIdx.x >= nitems) return;
     for (int e = tid; e < NG_N; e += P2P_WARPS * 32) {
         const int dz = e / NG_PZ - 7, dy = e % NG_PZ / NG_PY - 7, dx = e % NG_PZ % NG_PY - 7;
@@ -1559,15 +1573,94 @@ void fmm_near_w(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int st
         launch_pdl(k_near_w<true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K, w_list, w_cnt);
 }
 
-void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, cudaStream_t st,
-                   int per_sm) {
+// ---------------------------------------------------------------- operands of the matrix near field
+__device__ __forceinline__ void split3(float x, uint32_t (&s)[NM_SPLIT]) {
+#pragma unroll
+    for (int k = 0; k < NM_SPLIT; ++k) {             // each rest is exact
+        const __nv_bfloat16 b = __float2bfloat16_rn(x);
+        s[k] = __bfloat16_as_ushort(b);
+        x -= __bfloat162float(b);
+    }
+}
+
+// Blocks below NP_G: the kernel's values of an offset between two leaves, [split][target][source]
+// (cells in local Morton order, K-major with the 128-byte swizzle); the others a warp per source
+// leaf: its weights on its 64 cells.  Weights and kernel values as the sums of three BF16 parts.
+constexpr int NP_G = NM_OFFS * NM_CELLS * NM_CELLS / 2 / 256, NP_WARPS = 8;
+
+template <bool TAYLOR>
+__global__ void __launch_bounds__(NP_WARPS * 32) k_near_pack(FmmDev F, P2PConst K, const int *__restrict__ list,
+                                                             const int *__restrict__ count, int row0,
+                                                             uint16_t *__restrict__ rows, uint16_t *__restrict__ matrices,
+                                                             int *__restrict__ near_max) {
+    pdl_enter();
+    __shared__ float cells[NP_WARPS][NM_CELLS];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if ((int)blockIdx.x < NP_G) {
+        const int e = 2 * (blockIdx.x * 256 + tid);
+        const int o = e / (NM_CELLS * NM_CELLS), t = e / NM_CELLS % NM_CELLS, s0 = e % NM_CELLS;
+        uint32_t tx, ty, tz, part[2][NM_SPLIT];
+        demorton3((uint32_t)t, tx, ty, tz);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            uint32_t sx, sy, sz;
+            demorton3((uint32_t)(s0 + j), sx, sy, sz);
+            const int dx = 4 * (o % 3 - 1) + (int)sx - (int)tx, dy = 4 * (o / 3 % 3 - 1) + (int)sy - (int)ty,
+                      dz = 4 * (o / 9 - 1) + (int)sz - (int)tz;
+            const int d2 = dx * dx + dy * dy + dz * dz;
+            split3(d2 ? p2p_g<TAYLOR>((float)d2, K) : K.wself, part[j]);
+        }
+        uint8_t *m = reinterpret_cast<uint8_t *>(matrices + (size_t)o * NM_MATRIX) + tc::sw128_offset(t, s0, NM_CELLS);
+#pragma unroll
+        for (int k = 0; k < NM_SPLIT; ++k)
+            *reinterpret_cast<uint32_t *>(m + (size_t)k * NM_CELLS * NM_CELLS * 2) = part[0][k] | part[1][k] << 16;
+        return;
+    }
+    const float wsc = F.wscale * F.kp.C / (F.kp.h * F.kp.h * F.kp.h);
+    const int n = *count, nw = ((int)gridDim.x - NP_G) * NP_WARPS;
+    uint32_t most = 0;
+    for (int i = ((int)blockIdx.x - NP_G) * NP_WARPS + warp; i < n; i += nw) {
+        const int b = list[i], sb = F.T.b_sb[b], ns = F.T.b_se[b] - sb;
+        __syncwarp();
+        cells[warp][lane] = cells[warp][32 + lane] = 0.f;
+        __syncwarp();
+        for (int s = lane; s < ns; s += 32) {
+            const uint32_t pc = __ldg(F.src_pc + sb + s);
+            const float w = __ldg(F.src_q + sb + s) * wsc;
+            cells[warp][morton3((uint32_t)pc_i(pc) & 3u, (uint32_t)pc_j(pc) & 3u, (uint32_t)pc_k(pc) & 3u)] = w;
+            most = max(most, __float_as_uint(w) & 0x7FFFFFFFu);       // NaN above infinity above all else
+        }
+        __syncwarp();
+        uint32_t a[NM_SPLIT], c[NM_SPLIT];
+        split3(cells[warp][2 * lane], a);
+        split3(cells[warp][2 * lane + 1], c);
+        uint32_t *row = reinterpret_cast<uint32_t *>(rows + (size_t)(b - row0) * NM_ROW) + lane;
+#pragma unroll
+        for (int k = 0; k < NM_SPLIT; ++k) row[k * 32] = a[k] | c[k] << 16;
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0 && most) atomicMax(near_max, (int)most);
+}
+
+void fmm_near_pack(const FmmDev &F, const int *src_list, const int *src_count, int max_src, int row0, uint16_t *rows,
+                   uint16_t *matrices, int *near_max, cudaStream_t st) {
+    const P2PConst K = p2p_const(F);
+    const int grid = NP_G + std::min((max_src + NP_WARPS - 1) / NP_WARPS, 152 * 8);
+    if (K.bma_h >= 0.5f)
+        launch_pdl(k_near_pack<false>, grid, NP_WARPS * 32, 0, st, F, K, src_list, src_count, row0, rows, matrices, near_max);
+    else
+        launch_pdl(k_near_pack<true>, grid, NP_WARPS * 32, 0, st, F, K, src_list, src_count, row0, rows, matrices, near_max);
+}
+
+void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, const int *near_max,
+                   cudaStream_t st, int per_sm) {
     if (nboxes <= 0) return;
     const int grid = std::min(nboxes, 152 * per_sm);
     const P2PConst K = p2p_const(F);
     if (K.bma_h >= 0.5f)
-        launch_pdl(k_near_grid<false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K);
+        launch_pdl(k_near_grid<false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, near_max, K);
     else
-        launch_pdl(k_near_grid<true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, K);
+        launch_pdl(k_near_grid<true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, near_max, K);
 }
 
 // out[cell of t] += near_buf[slot of t]: one warp per leaf of the class lists (the items in the

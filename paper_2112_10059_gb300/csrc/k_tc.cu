@@ -46,6 +46,18 @@ __global__ void __launch_bounds__(256, 1) k_m2l_tiles(FmmDev F, const int *__res
                                                       const int *__restrict__ ngroups, int *__restrict__ counter,
                                                       const uint16_t *__restrict__ images, int *err);
 
+// matrix near field (below)
+constexpr uint32_t NM_A = TCM * NM_CELLS * 2, NM_B = NM_CELLS * NM_CELLS * 2;   // one part of a step's operands
+constexpr uint32_t NM_STAGE = NM_SPLIT * (NM_A + NM_B);
+constexpr int NM_RING = 3, NM_ACCS = 6;          // steps in shared memory; accumulators of hi hi
+constexpr uint32_t NM_SMEM = 1024 + NM_RING * NM_STAGE + 4 * TCM * 4 + 128;
+constexpr int NM_COPY = 256;                     // copying threads
+__global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const int *__restrict__ p2p_list,
+                                                             const int *__restrict__ p2p_cnt, int stride, int row0,
+                                                             const uint16_t *__restrict__ rows,
+                                                             const uint16_t *__restrict__ matrices,
+                                                             const int *__restrict__ near_max, int *err);
+
 // Operator (FP32, transposed [k][i], stride np) -> BF16 hi / lo images, K-major SW128.
 __global__ void k_make_image(const float *__restrict__ opT, int np, uint16_t *__restrict__ img) {
     pdl_enter();
@@ -1588,6 +1600,7 @@ void tc_init_attributes() {
     cudaFuncSetAttribute(k_l2p_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L2P_SMEM);
     cudaFuncSetAttribute(k_l2lp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LP_SMEM);
     cudaFuncSetAttribute(k_m2l_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MT_SMEM);
+    cudaFuncSetAttribute(k_near_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NM_SMEM);
     cudaFuncSetAttribute(k_m2l_tc_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PIPE_SMEM);
     done = true;
 }
@@ -1840,6 +1853,212 @@ __global__ void __launch_bounds__(256, 1) k_m2l_tiles(FmmDev F, const int *__res
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem, TCM);
+}
+
+// ---------------------------------------------------------------- near field of dense leaves
+// Between leaves of edge 4 of one level, the near field of an offset o is one 64 x 64 matrix of
+// kernel values for every pair of leaves, so the near field of 128 leaves is
+//     S[leaf][target] = sum over o, source cells of q[leaf + o][cell] G_o[target][cell]:
+// M = 128 leaves, N = 64 targets, K = 27 x 64 cells.  FP32 factors as sums of three BF16 parts
+// (24 bits); the products hi hi, hi mid, mid hi, hi lo, lo hi and mid mid are formed, the largest
+// left out is 2^-24 of the sum.  The tensor core's additions round towards zero (one accumulator for
+// everything: 8.5e-6 of a sum lost), so they are kept few: an offset's hi hi are a sum of four MMAs of
+// their own, in a ring of six accumulators, added up in FP32 registers; the parts below have two more
+// accumulators for the whole tile (8 x 64 columns of TMEM).
+// A step is an offset: 48 KB of rows gathered by 16-byte copies, 24 KB of matrices by a bulk copy,
+// 24 MMAs; three steps in shared memory.  A step takes 1.4 us, bound by the copies (51 bytes a
+// ns and SM; the MMAs alone take 0.6).  Eight warps look the leaves up an offset ahead, copy, add up and
+// write results, one thread issues MMAs.
+// Uniform 128^3 (32,768 full leaves, 3.4e9 pairs): 712 us by the offset table, 82 so and 14 for its
+// operands; wide streamer 192^3 303, and 44 + 12 + 39 for the other leaves by the table.
+__global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const int *__restrict__ p2p_list,
+                                                             const int *__restrict__ p2p_cnt, int stride, int row0,
+                                                             const uint16_t *__restrict__ rows,
+                                                             const uint16_t *__restrict__ matrices,
+                                                             const int *__restrict__ near_max, int *err) {
+    pdl_enter();
+    const int cnt = p2p_cnt[P2P_MMA], tiles = (cnt + TCM - 1) / TCM;
+    if ((int)blockIdx.x >= tiles || !near_mma_range(*near_max)) return;   // uniform, before any allocation
+    const int *list = p2p_list + (size_t)P2P_MMA * stride;
+    int first = 0;                                // the class's first slot
+    for (int c = 0; c < P2P_MMA; ++c) first += p2p_cnt[c];
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    int (*tab)[TCM] = reinterpret_cast<int (*)[TCM]>(base + NM_RING * NM_STAGE);   // rows of an offset, or -1
+    uint64_t *bar_a = reinterpret_cast<uint64_t *>(tab + 4);   // [3] a step's rows are there
+    uint64_t *bar_b = bar_a + NM_RING;            // [3] its matrices
+    uint64_t *bar_e = bar_b + NM_RING;            // [3] its MMAs are done
+    uint64_t *bar_d = bar_e + NM_RING;            // [2] a tile's MMAs are done; its accumulators are read
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar_d + 2);
+    volatile int *failed = reinterpret_cast<volatile int *>(tslot + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp == NM_COPY / 32) {
+        tc::tmem_alloc(tc::smem_u32(tslot), 512);
+        tc::tmem_relinquish();
+    }
+    if (tid == 0) {
+        for (int k = 0; k < NM_RING; ++k) {
+            tc::mbar_init(tc::smem_u32(bar_a + k), NM_COPY);
+            tc::mbar_init(tc::smem_u32(bar_b + k), 1);
+            tc::mbar_init(tc::smem_u32(bar_e + k), 1);
+        }
+        tc::mbar_init(tc::smem_u32(bar_d), 1);
+        tc::mbar_init(tc::smem_u32(bar_d + 1), NM_COPY);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *failed = 0;
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tslot, ring = tc::smem_u32(base);
+    // a wait that runs out ends every later one at once (the result is then invalid, the host told)
+    auto wait = [&](uint64_t *bar, int use) {
+        if (*failed) return;
+        if (!tc::mbar_wait_bounded(tc::smem_u32(bar), use & 1, WAIT_LIMIT)) *failed = 1;
+    };
+    if (warp == NM_COPY / 32) {                   // ---- one thread issues every MMA
+        if (tc::elect_one()) {
+            const uint32_t idesc = tc::idesc_bf16_f32(TCM, NM_CELLS);
+            int step = 0, turn = 0;
+            for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++turn) {
+                if (turn > 0) wait(bar_d + 1, turn - 1);
+                for (int o = 0; o < NM_OFFS; ++o, ++step) {
+                    const int st = step % NM_RING, use = step / NM_RING;
+                    wait(bar_b + st, use);
+                    wait(bar_a + st, use);
+                    tc::fence_after_sync();
+                    const uint64_t a = tc::sdesc_sw128(ring + st * NM_STAGE), b = tc::sdesc_sw128(ring + st * NM_STAGE + NM_SPLIT * NM_A);
+                    const uint32_t big = tmem + (uint32_t)(o % NM_ACCS) * NM_CELLS;
+                    const uint32_t mid = tmem + NM_ACCS * NM_CELLS, low = mid + NM_CELLS;
+#pragma unroll
+                    for (int ks = 0; ks < NM_CELLS / 16; ++ks) {
+                        const uint64_t ah = a + ((32 * ks) >> 4), am = ah + (NM_A >> 4), al = am + (NM_A >> 4);
+                        const uint64_t bh = b + ((32 * ks) >> 4), bm = bh + (NM_B >> 4), bl = bm + (NM_B >> 4);
+                        tc::mma_bf16(big, ah, bh, idesc, ks > 0);
+                        tc::mma_bf16(mid, ah, bm, idesc, o > 0 || ks > 0);
+                        tc::mma_bf16(mid, am, bh, idesc, 1);
+                        tc::mma_bf16(low, ah, bl, idesc, o > 0 || ks > 0);
+                        tc::mma_bf16(low, al, bh, idesc, 1);
+                        tc::mma_bf16(low, am, bm, idesc, 1);
+                    }
+                    tc::mma_commit(tc::smem_u32(bar_e + st));
+                }
+                tc::mma_commit(tc::smem_u32(bar_d));
+            }
+            // after a failure: every MMA issued has completed before the memory is released
+            if (*failed && turn > 0) tc::mbar_wait_bounded(tc::smem_u32(bar_d), (turn - 1) & 1, WAIT_LIMIT);
+        }
+        __syncwarp();
+    } else {                                      // ---- eight warps copy operands and write results
+        const TreeDev &T = F.T;
+        const int l = F.near_mma_level, edge = 1 << l;
+        const uint8_t *vs = T.vsrc + dense_off(l);
+        const int *ba = T.box_at + dense_off(l);
+        // results: warps w and w + 4 take TMEM lanes 32 (w % 4) .. (leaves) and 32 targets each
+        const int q = warp & 3, c0 = (warp >> 2) * 32;
+        const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+        float sum[32];
+        auto add = [&](int k) {                   // accumulator k to the sums
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float v[16];
+                tc::tmem_ld16(acc + (uint32_t)k * NM_CELLS + 16 * h, v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) sum[16 * h + j] += v[j];
+            }
+        };
+        int step = 0, turn = 0;
+        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++turn) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) sum[j] = 0.f;
+            // threads below 128: the row of leaf `tid`'s neighbour at offset o
+            const int member = tile * TCM + tid;
+            uint32_t bx = 0, by = 0, bz = 0;
+            const bool have = tid < TCM && member < cnt;
+            if (have) demorton3(T.b_key[list[member]], bx, by, bz);
+            auto lookup = [&](int o) {
+                const int x = (int)bx + o % 3 - 1, y = (int)by + o / 3 % 3 - 1, z = (int)bz + o / 9 - 1;
+                if (!have || o >= NM_OFFS || (unsigned)x >= (unsigned)edge || (unsigned)y >= (unsigned)edge ||
+                    (unsigned)z >= (unsigned)edge)
+                    return -1;
+                const uint32_t slot = morton3((uint32_t)x, (uint32_t)y, (uint32_t)z);
+                const int box = __ldg(ba + slot);
+                return __ldg(vs + slot) ? box - row0 : -1;
+            };
+            if (tid < TCM) tab[0][tid] = lookup(0);
+            int next = lookup(1);
+            asm volatile("bar.sync 1, %0;" ::"n"(NM_COPY) : "memory");
+            for (int o = 0; o < NM_OFFS; ++o, ++step) {
+                const int st = step % NM_RING, use = step / NM_RING;
+                if (tid < TCM) tab[(o + 1) & 3][tid] = next;
+                next = lookup(o + 2);
+                if (use > 0) wait(bar_e + st, use - 1);
+                const uint32_t at = ring + st * NM_STAGE;
+                if (tid == 0) {
+                    tc::mbar_expect_tx(tc::smem_u32(bar_b + st), NM_SPLIT * NM_B);
+                    tc::bulk_g2s(at + NM_SPLIT * NM_A, matrices + (size_t)o * NM_MATRIX, NM_SPLIT * NM_B, tc::smem_u32(bar_b + st));
+                }
+#pragma unroll
+                for (int u = 0; u < TCM * NM_SPLIT * 8 / NM_COPY; ++u) {
+                    const int e = tid + NM_COPY * u, j = e / (NM_SPLIT * 8), g = e % (NM_SPLIT * 8);   // leaf, 16-byte unit
+                    const int r = tab[o & 3][j];
+                    tc::cp_async16(at + (uint32_t)(g >> 3) * NM_A + (uint32_t)j * 128 + (uint32_t)(((g & 7) ^ (j & 7)) << 4),
+                                   rows + (size_t)max(r, 0) * NM_ROW + 8 * g, r >= 0 ? 16u : 0u);
+                }
+                tc::cp_async_commit();
+                if (o >= NM_RING) {               // the MMAs of offset o - NM_RING are done (waited for above)
+                    tc::fence_after_sync();
+                    add((o - NM_RING) % NM_ACCS);
+                    tc::fence_before_sync();      // read before this thread's arrivals let its next MMAs begin
+                }
+                if (o > 0) {                      // the step before has landed
+                    tc::cp_async_wait<1>();
+                    tc::fence_proxy_async_smem();
+                    tc::mbar_arrive(tc::smem_u32(bar_a + (step - 1) % NM_RING));
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(NM_COPY) : "memory");   // the next offset's rows are in tab
+            }
+            tc::cp_async_wait<0>();
+            tc::fence_proxy_async_smem();
+            tc::mbar_arrive(tc::smem_u32(bar_a + (step - 1) % NM_RING));
+            wait(bar_d, turn);
+            tc::fence_after_sync();
+#pragma unroll
+            for (int o = NM_OFFS - NM_RING; o < NM_OFFS; ++o) add(o % NM_ACCS);
+            add(NM_ACCS);
+            add(NM_ACCS + 1);
+            const int m = tile * TCM + 32 * q + lane;
+            if (m < cnt) {
+                float *slot = F.near_buf + (size_t)(first + m) * F.near_s + c0;
+                if ((F.near_s & 3) == 0) {
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        *reinterpret_cast<float4 *>(slot + j) = make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) slot[j] = sum[j];
+                }
+            }
+            tc::fence_before_sync();
+            tc::mbar_arrive(tc::smem_u32(bar_d + 1));
+        }
+        // after a failure: this CTA's matrices have landed before its memory is released
+        if (tid == 0 && *failed)
+            for (int k = 0; k < NM_RING; ++k)
+                if (step > k) tc::mbar_wait_bounded(tc::smem_u32(bar_b + k), ((step - 1 - k) / NM_RING) & 1, WAIT_LIMIT);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (tid == 0 && *failed) atomicOr(err, 64);
+    if (warp == NM_COPY / 32) tc::tmem_dealloc(tmem, 512);
+}
+
+void fmm_near_mma(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, int max_leaves, int row0,
+                  const uint16_t *rows, const uint16_t *matrices, const int *near_max, int *err, cudaStream_t st) {
+    if (max_leaves <= 0) return;
+    tc_init_attributes();
+    launch_pdl(k_near_mma, std::min((max_leaves + TCM - 1) / TCM, sm_count()), NM_COPY + 32, NM_SMEM, st, F, p2p_list, p2p_cnt,
+               stride, row0, rows, matrices, near_max, err);
 }
 
 MtLevels m2l_tile_levels(int Lmax) {

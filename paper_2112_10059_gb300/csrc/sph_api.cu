@@ -103,6 +103,7 @@ struct sph_ctx {
     int fault_alloc = 0;              // > 0: the fault_alloc-th allocation fails (SPH_FAULT=alloc[:k])
     int m2l_tiles = 2;                // tensor-core M2L in target-stationary tiles: 0 never (tiles of V
                                       // pairs), 1 always, 2 where the V lists are dense (>= 32 pairs per box)
+    int near_mma = 2;                 // near field of dense leaves as a matrix product: 0 never, 1 always, 2 where it pays
     DevBuf b_mtg;                     // groups of the target-stationary M2L
     int m2l_form = -1;                // autotuned M2L form for this eval (-1: by the lists)
     bool m2l_tiles_used = false;      // the last eval ran the target-stationary M2L
@@ -115,6 +116,7 @@ struct sph_ctx {
     DevBuf b_skip;
     bool near_table = false;          // resolved for the current evaluation
     DevBuf b_gtab, b_dtab;            // near-field table; FP64 pair weights of the direct sum
+    DevBuf b_nrows, b_nmat;           // operands of the matrix near field
     // buffers
     DevBuf b_maxes, b_cnt, b_off, b_tot, b_skey, b_spc, b_sq, b_tkey, b_tpc, b_bstat;
     DevBuf b_boxat, b_flag, b_pos, b_rng, b_scan, b_lvl;
@@ -692,6 +694,20 @@ bool l2lp_fusable(const sph_ctx *c, const PassState &S) {
            F.O.l2pc_off >= 0 && c->Lmax >= 3 && c->Lmax == c->D - 2 && F.O.l2p_off[c->Lmax] >= 0;
 }
 
+// Whether dense leaves take their near field as a matrix product (k_near_mma).  A tile of 128
+// leaves takes 40 us, however few tiles there are, and its operands 12; the offset table is level
+// with it at 2e8 pairs (40 us at 5e12/s, 60 beside the far field).  Below 16 sources a source leaf
+// hardly a leaf has the sources that it takes (k_work_lists).
+bool near_mma_pays(const sph_ctx *c, const PassState &S) {
+    const FmmDev &F = S.F;
+    if (!S.tc || !F.near_buf || F.gtab || c->near_mma == 0 || c->Lmax != c->D - 2 || c->Lmax < 2) return false;
+    if (c->near_mma == 1) return true;
+    int64_t leaves = 0;
+    for (int l = 0; l <= c->Lmax; ++l) leaves += c->lvl_sleaf[l];
+    const double mean = (double)c->ns / (double)std::max<int64_t>(leaves, 1);
+    return mean >= 16.0 && (double)c->list_tot[0] * mean * 64.0 >= 2e8;
+}
+
 // Every buffer the passes need (so that fmm_queue allocates nothing and can be captured).
 int fmm_prepare(sph_ctx *c, PassState &S) {
     const int nb = c->nboxes;
@@ -726,13 +742,15 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
     }
     S.w_src = P<int>(c->b_work);
     S.w_leaf = S.w_src + std::max(nb, 1);
+    // w_cnt: [0] boxes with sources per level, [32] leaves, [33] the near field's largest weight, [36] .. [39] see
+    // below, [40] leaves per level for the L2P, [55] .. [61] near-field classes, [62] own terms, [63] X entries
     S.w_p2p = S.w_leaf + std::max(nb, 1);                   // P2P_CLASSES lists of max(nb, 1) slots
     S.w_cnt = S.w_p2p + P2P_CLASSES * std::max(nb, 1);
     F.l2p_list = S.w_cnt + 64;                  // [nb], per level at lvl_base[l]
     S.w_own = F.l2p_list + std::max(nb, 1);     // [nb]: deepest-level leaves with V / X entries, count w_cnt[62]
     S.w_wl = S.w_own + std::max(nb, 1);         // [nb]: near-field leaves with W entries, count w_cnt[39]
     S.w_xl = S.w_wl + std::max(nb, 1);          // [nb]: boxes with X entries, count w_cnt[63]
-    F.l2p_cnt = S.w_cnt + 40;                   // [16]
+    F.l2p_cnt = S.w_cnt + 40;                   // [15]
     S.Pd = pairs_dev(c);
     S.err = P<int>(c->b_err);
     S.tc = c->m2l_prec == SPH_M2L_BF16X3 && F.O.m2l_img != nullptr && !c->translate_per_box;
@@ -751,6 +769,14 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
         if (!c->near_join) CK(cudaEventCreateWithFlags(&c->near_join, cudaEventDisableTiming));
         if (!c->near_up) CK(cudaEventCreateWithFlags(&c->near_up, cudaEventDisableTiming));
         if (!c->near_l2l) CK(cudaEventCreateWithFlags(&c->near_l2l, cudaEventDisableTiming));
+    }
+    F.near_mma_level = -1;                      // the state was cleared to zeros
+    if (near_mma_pays(c, S)) {
+        const int L = c->Lmax;
+        const int r = ensure(c, c->b_nrows, std::max<size_t>(c->lvl_count[L], 1) * NM_ROW * sizeof(uint16_t));
+        const int r2 = r == SPH_OK ? ensure(c, c->b_nmat, NM_OFFS * NM_MATRIX * sizeof(uint16_t)) : r;
+        if (c->poisoned) return SPH_ECUDA;
+        if (r2 == SPH_OK) F.near_mma_level = L;       // without room the other near-field form takes every leaf
     }
     // the fused deepest level reads only the d rows of leaves with V or X entries: the rows of
     // that level are then cleared one by one by the work lists, the levels above by a memset
@@ -812,7 +838,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
     // the tiles' flags reach the host through the near-field add (the last kernel), written into
     // the mapped read-back buffer, where that kernel runs; else by copies
     const bool err_mapped = c->pinned_dev && F.near_buf && nb > 0;
-    fmm_work_lists(F, nb, S.w_src, S.w_cnt, S.w_leaf, S.w_cnt + 32, S.w_p2p, S.w_cnt + 56, std::max(nb, 1),
+    fmm_work_lists(F, nb, S.w_src, S.w_cnt, S.w_leaf, S.w_cnt + 32, S.w_p2p, S.w_cnt + 55, std::max(nb, 1),
                    S.w_own, S.w_cnt + 62, c->stream, S.w_wl, S.w_cnt + 39, S.w_xl, S.w_cnt + 63);
     c->launches += nb > 0;
     const bool near_fork = F.near_buf && nb > 0;
@@ -829,9 +855,19 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
         }
         if (tm) tm->mark_at(12, c->near_stream);
         if (F.gtab)
-            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, S));
-        else
-            fmm_near_grid(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), c->near_stream, near_cap(c, S));
+            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, S));
+        else {
+            const int L = F.near_mma_level, row0 = L >= 0 ? c->lvl_base[L] : 0;
+            int *near_max = S.w_cnt + 33;
+            if (L >= 0) {
+                uint16_t *rows = P<uint16_t>(c->b_nrows), *mat = P<uint16_t>(c->b_nmat);
+                fmm_near_pack(F, S.w_src + row0, S.w_cnt + L, c->lvl_src[L], row0, rows, mat, near_max, c->near_stream);
+                fmm_near_mma(F, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), c->lvl_leaf[L], row0, rows, mat, near_max, S.err,
+                             c->near_stream);
+                c->launches += 1 + (c->lvl_leaf[L] > 0);
+            }
+            fmm_near_grid(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), near_max, c->near_stream, near_cap(c, S));
+        }
         ++c->launches;
         if (tm) tm->mark_at(14, c->near_stream);
     }
@@ -860,7 +896,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
         if (tm) tm->mark_at(15, c->near_stream);
         if (c->list_tot[2] > 0 && F.O.method == FAR_CHEB) {
             // only the leaves with W entries (at most one per W entry)
-            fmm_near_w(F, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), S.w_wl, S.w_cnt + 39, c->list_tot[2], c->near_stream);
+            fmm_near_w(F, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), S.w_wl, S.w_cnt + 39, c->list_tot[2], c->near_stream);
             ++c->launches;
         }
         if (tm) tm->mark_at(13, c->near_stream);
@@ -978,7 +1014,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
     if (F.near_buf) {
         if (nb > 0) {
             CK(cudaStreamWaitEvent(c->stream, c->near_join, 0));
-            fmm_near_add(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), out, c->stream,
+            fmm_near_add(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->stream,
                          err_mapped ? S.err : nullptr, err_mapped ? c->pinned_dev + 48 : nullptr);
             ++c->launches;
         }
@@ -988,7 +1024,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
             fmm_near_table(F, const_cast<float *>(F.gtab), c->stream);
             ++c->launches;
         }
-        fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 56, std::max(nb, 1), out, c->stream);
+        fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->stream);
         c->launches += nb > 0;
     }
     if (tm) tm->mark_at(9, c->stream);
@@ -1077,6 +1113,7 @@ std::vector<uint8_t> graph_signature(const sph_ctx *c, const PassState &S, const
     put(c->list_tot, sizeof c->list_tot);
     const int64_t sc[] = {c->nboxes, c->Lmax, c->D, c->m2l_prec, c->translate_per_box, c->l2l_eight, c->l2p_simt,
                           c->l2p_tc_tables, c->m2l_pipe, c->m2l_loop, c->m2l_loop_ctas, c->l2lp_fused, c->m2l_tiles, c->m2l_form,
+                          (int64_t)reinterpret_cast<uintptr_t>(c->b_nrows.p), (int64_t)reinterpret_cast<uintptr_t>(c->b_nmat.p),
                           (int64_t)reinterpret_cast<uintptr_t>(out)};
     put(sc, sizeof sc);
     return v;
@@ -1486,6 +1523,7 @@ int configure_sub(sph_ctx *sub, const sph_ctx *parent, const sph_problem &p) {
     sub->near_per_sm = parent->near_per_sm;
     sub->l2lp_fused = parent->l2lp_fused;
     sub->m2l_tiles = parent->m2l_tiles;
+    sub->near_mma = parent->near_mma;
     sub->defer_sync = parent->defer_sync;
     sub->near_mode = parent->near_mode;
     sub->r_s = parent->r_s;
@@ -1869,6 +1907,7 @@ int sph_create(sph_ctx **out, int device, void *cuda_stream) {
     if (const char *e = getenv("SPH_NEAR_OVERLAP")) c->near_overlap = atoi(e) != 0;
     if (const char *e = getenv("SPH_NEAR_PER_SM")) c->near_per_sm = std::max(1, atoi(e));
     if (const char *e = getenv("SPH_L2LP_FUSED")) c->l2lp_fused = atoi(e) != 0;
+    if (const char *e = getenv("SPH_NEAR_MMA")) c->near_mma = atoi(e);
     if (const char *e = getenv("SPH_M2L_TILES")) c->m2l_tiles = atoi(e);
     c->select_wait = env_limit("SPH_WAIT_LIMIT_SELECT", SELECT_WAIT_LIMIT);
     if (const char *e = getenv("SPH_FAULT")) {
@@ -1918,7 +1957,7 @@ void sph_destroy(sph_ctx *c) {
                      &c->b_lcnt, &c->b_loff, &c->b_usrc, &c->b_vsrc, &c->b_vocs, &c->b_vtrg, &c->b_wsrc, &c->b_xsrc, &c->b_pkeys, &c->b_ppairs, &c->b_vbase, &c->b_heavy,
                      &c->b_ueq, &c->b_dchk, &c->o_work, &c->o_etab, &c->o_m2m, &c->o_l2l,
                      &c->o_m2l, &c->o_m2lbf, &c->o_l2lbf, &c->o_m2mbf, &c->b_err, &c->b_work, &c->b_mtg, &c->b_nearbuf, &c->o_slot, &c->o_surf, &c->o_cheb, &c->o_self, &c->h_q, &c->h_e, &c->h_m,
-                     &c->h_s, &c->b_tmask, &c->b_near, &c->b_gtab, &c->b_dtab, &c->b_skip, &c->o_l2pimg, &c->s_qc, &c->s_Sc, &c->s_y, &c->s_Sp, &c->s_x, &c->s_Sf,
+                     &c->h_s, &c->b_tmask, &c->b_near, &c->b_gtab, &c->b_dtab, &c->b_nrows, &c->b_nmat, &c->b_skip, &c->o_l2pimg, &c->s_qc, &c->s_Sc, &c->s_y, &c->s_Sp, &c->s_x, &c->s_Sf,
                      &c->s_mask, &c->s_svox, &c->s_err, &c->s_pe, &c->s_flags, &c->s_counts};
     for (DevBuf *b : all)
         if (b->p) cudaFree(b->p);

@@ -257,7 +257,7 @@ struct FmmDev {
     const float *gtab;      // optional near-field table: g(d2) for integer squared offsets d2 < GTAB_N
     float r_s;              // strategy 3 (skip W boxes whose bounded share is below r_s S_est); 0 = off
     unsigned long long *skip_count;   // (target, W box) pairs skipped by strategy 3
-    int *l2p_list = nullptr, *l2p_cnt = nullptr;   // per level (at lvl_base[l]): leaves with targets, [16] counts
+    int *l2p_list = nullptr, *l2p_cnt = nullptr;   // per level (at lvl_base[l]): leaves with targets, [15] counts
     float wscale;
     KParams kp;
     double alpha, beta, C64;   // FP64 kernel constants for the FP64 evaluation paths
@@ -272,13 +272,16 @@ struct FmmDev {
     // far-field passes; fmm_near_add adds the slots into the output afterwards
     float *near_buf = nullptr;
     int near_s = 0;
+    // >= 0: the level of edge-4 leaves whose dense near fields are taken by fmm_near_mma
+    int near_mma_level = -1;
 };
 // returns the number of kernels launched
 int fmm_upward_level(const FmmDev &F, int level, int box_count, int leaf_count, const int *list, const int *count, bool leaves_only,
                      cudaStream_t st);
 // near-field leaves in classes by their number of kernel evaluations w: class c holds
-// P2P_CLASS0 >> c <= w < P2P_CLASS0 >> (c - 1) (class 0: w >= P2P_CLASS0, the last: the rest)
-constexpr int P2P_CLASSES = 6;
+// P2P_CLASS0 >> c <= w < P2P_CLASS0 >> (c - 1) (class 0: w >= P2P_CLASS0, the last but one: the
+// rest); class P2P_MMA: the leaves taken by fmm_near_mma
+constexpr int P2P_CLASSES = 7, P2P_MMA = P2P_CLASSES - 1;
 constexpr int64_t P2P_CLASS0 = 1 << 16;
 // p2p_list: P2P_CLASSES lists of p2p_stride slots, p2p_cnt: their P2P_CLASSES counts
 // own_list / own_cnt: the deepest-level leaves with targets and V or X entries (where
@@ -295,8 +298,24 @@ void fmm_work_lists(const FmmDev &F, int nboxes, int *src_list, int *src_cnt, in
 void fmm_p2p(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,
              cudaStream_t st, int pass_lo = 0, int pass_hi = 2, int per_sm = 16);
 // the U-list part into the leaves' slots of F.near_buf by the offset table, for the same lists
-void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, cudaStream_t st,
-                   int per_sm);
+// (class P2P_MMA is left out unless the weights' maximum near_max is outside fmm_near_mma's range)
+void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, const int *near_max,
+                   cudaStream_t st, int per_sm);
+// the same for the leaves of class P2P_MMA as a matrix product; fmm_near_pack first lays out the
+// weights of the source leaves of level F.near_mma_level (src_list; rows by box - row0) and the
+// kernel's matrices, and leaves the bits of the largest |weight| in near_max (zeroed before)
+constexpr int NM_OFFS = 27, NM_CELLS = 64, NM_SPLIT = 3;
+constexpr size_t NM_ROW = NM_SPLIT * NM_CELLS;                            // BF16 values of a leaf's row
+constexpr size_t NM_MATRIX = (size_t)NM_SPLIT * NM_CELLS * NM_CELLS;      // and of an offset's matrix
+// the weights' range: above, a BF16 rounding could overflow; below, a third part would underflow
+__device__ __forceinline__ bool near_mma_range(int max_bits) {
+    const float w = __int_as_float(max_bits);
+    return w >= 0x1p-80f && w <= 0x1p120f;                               // false for NaN
+}
+void fmm_near_pack(const FmmDev &F, const int *src_list, const int *src_count, int max_src, int row0, uint16_t *rows,
+                   uint16_t *matrices, int *near_max, cudaStream_t st);
+void fmm_near_mma(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, int max_leaves, int row0,
+                  const uint16_t *rows, const uint16_t *matrices, const int *near_max, int *err, cudaStream_t st);
 // the W-list part (Chebyshev far field) of the leaves in w_list (fmm_work_lists; at most max_w), added to the slots
 void fmm_near_w(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, const int *w_list, const int *w_cnt,
                 int max_w, cudaStream_t st);

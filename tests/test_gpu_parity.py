@@ -861,3 +861,51 @@ def test_m2l_target_tiles_uniform_tree(sph, monkeypatch):
     assert oracle.rel_l2(outs["1"], outs["0"]) < 1e-5
     assert oracle.rel_l2(outs["1"][samp], ref) <= REL_L2
     assert oracle.max_rel(outs["1"][samp], ref, 1e-3) <= MAX_REL
+
+
+def _box_of(p, nx, ny, nz):
+    """The corner box nx x ny x nz of a cubic problem."""
+    n = p.nx
+    cut = lambda a: None if a is None else np.ascontiguousarray(a.reshape(n, n, n)[:nz, :ny, :nx]).reshape(-1)
+    return dataclasses.replace(p, nx=nx, ny=ny, nz=nz, q=cut(p.q), emag=cut(p.emag), name="%dx%dx%d" % (nx, ny, nz))
+
+
+@pytest.mark.parametrize("case", ["one_tile", "ragged_tiles", "odd_edges", "holes", "leaf_65", "small_weights"])
+def test_matrix_near_field_equals_table(sph, monkeypatch, case):
+    """Dense leaves' near field as a matrix product (SPH_NEAR_MMA=1: wherever a leaf qualifies)
+    against the offset table: fewer leaves than a tile's 128 rows, a partly filled last tile and
+    rows without a neighbour at the box's faces, leaves that overhang the grid (left to the table
+    beside the others), source leaves with empty cells, slots of a size that 16-byte stores do not fit,
+    and weights below the BF16 parts' range (the table takes every leaf).  All terms of a sum are
+    positive; a hi hi accumulator takes 4 additions rounded towards zero, the lower parts' 324 at 2^-8
+    of their size: 1e-6 and less, and the FP32 sums of the other form lose 2^-24 a term at random."""
+    full = lambda n: si.streamer(n=n, box=n / 128, chan_len=n / 256, i_frac=0.0, targets_all=True, sigma_head=0.1 * n / 128,
+                                 chan_radius=0.1 * n / 128, seed=60 + n, with_efield=False)
+    leaf = 64
+    if case == "one_tile":
+        p = full(16)
+    elif case in ("ragged_tiles", "leaf_65"):
+        p, leaf = full(24), 64 if case == "ragged_tiles" else 65
+    elif case == "odd_edges":
+        p = _box_of(full(48), 46, 33, 27)
+    elif case == "holes":
+        p = full(32)
+        q = p.q.copy()
+        q[np.random.default_rng(5).random(q.size) < 0.4] = 0.0
+        p = dataclasses.replace(p, q=q, i_frac=1e-30)
+    else:
+        p = full(16)
+        p = dataclasses.replace(p, q=(p.q * np.float32(1e-24 / p.q.max())).astype(np.float32))
+    outs = []
+    for flag in ("1", "0", "0", "0", "0"):
+        monkeypatch.setenv("SPH_NEAR_MMA", flag)
+        c = sph.Context(0)
+        _, out, st = sph.solve(p, c, m2l_precision=sph.M2L_BF16X3, leaf_size=leaf, stats=True)
+        outs.append(out.cpu().numpy().astype(np.float64))
+        c.close()
+    new, old = outs[0], outs[1]
+    assert np.all(np.isfinite(new)) and np.count_nonzero(new) == p.ncell
+    # the far field's reductions add in another order each time: what the table form's runs differ by themselves
+    own = np.max([np.abs(o - old) for o in outs[2:]], axis=0)
+    assert np.max(np.abs(new - old) / np.abs(old)) <= 8e-6 + 2 * np.max(own / np.abs(old))
+    assert oracle.rel_l2(new, old) <= 4e-6
