@@ -202,8 +202,9 @@ def rooflines(tree, step_stats, args, nt, ns, ncell, peaks, pipes, traffic_ok=Tr
                   have V or X entries read (npad x 4 B each) with S read and written at their
                   targets (8 B per target), and the other levels' leaves (npad x 4 B per leaf
                   with targets + 4 B per target written) -- only where such leaves exist;
-      near (MUFU, k_p2p): P2P pairs + M2P evaluations, 2 ex2 + 1 rsqrt each, against the measured
-                  ex2 and rsqrt rates;
+      near (k_near_grid, k_near_mma, k_near_w): P2P pairs + M2P evaluations against the measured
+                  ex2 and rsqrt rates at 2 ex2 + 1 rsqrt each; an offset table and matrix products
+                  stand for most pairs' evaluations, so the fraction may pass 1;
       select (HBM, k_brick_stats + k_select_onepass): 8 B per cell (q and |E| read once) + 4 B
                   per selected index (sources and targets) -- the minimum of the operation: the
                   maxima pass reads every cell, the rules re-read only the bricks that the
@@ -275,7 +276,7 @@ def rooflines(tree, step_stats, args, nt, ns, ncell, peaks, pipes, traffic_ok=Tr
             "k_l2p_sep_small + k_l2p_sep", False, "hbm",
             4.0 * npad * (n_leaf_t + n_deep) + 4.0 * nt_other + 8.0 * nt_own, "bytes", med("ms_l2p") - ms_lp, hbm,
             "GB/s", hbm_basis)
-    add("near", "k_p2p", True, "alu", float(p2p + m2p), "kernel-evals", med("ms_near"), mufu_evals, "evals/s",
+    add("near", "k_near_grid + k_near_mma + k_near_w", False, "alu", float(p2p + m2p), "kernel-evals", med("ms_near"), mufu_evals, "evals/s",
         "MUFU: 2 ex2 + 1 rsqrt per evaluation at the measured %.3g ex2/s and %.3g rsqrt/s (%s)"
         % (pipes["ex2_per_s"], pipes["rsqrt_per_s"], pipes["source"]))
     add("select", "k_brick_stats + k_select_onepass", False, "hbm", 8.0 * ncell + 4.0 * (nt + ns),

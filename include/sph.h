@@ -154,8 +154,9 @@ int set_criteria(sph_ctx *ctx, double i_frac, double e_frac, double e_applied,
 int sph_set_far_field(sph_ctx *ctx, int method, int order);
 
 /* Near field (Eq. nearfar, the exact part): SPH_NEAR_EXP (default) uses the kernel's
- * exponential form: once per cell offset and block between leaves of edge 4 or less, whose offsets
- * are few, per source-target pair elsewhere; SPH_NEAR_TABLE reads G for the integer
+ * exponential form: once per cell offset between leaves of edge 4 or less, whose offsets are few
+ * (dense ones then sum on the tensor cores, values and weights as three BF16 parts), per
+ * source-target pair elsewhere; SPH_NEAR_TABLE reads G for the integer
  * squared cell offsets below 4096 from a table built per evaluation with the same arithmetic
  * (uniform grids make every offset an integer); SPH_NEAR_AUTO times both on the first eval
  * of each problem class and keeps the faster.  Takes effect at the next eval. */
