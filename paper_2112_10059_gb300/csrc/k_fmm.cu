@@ -414,7 +414,8 @@ __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, i
         if (dense) cls = P2P_MMA;
     }
     int my_idx = 0;
-    for (int c = 0; c < P2P_CLASSES; ++c) {
+    const int classes = F.near_mma_level >= 0 ? P2P_CLASSES : P2P_MMA;   // the last is empty otherwise
+    for (int c = 0; c < classes; ++c) {
         const bool in = p2p && cls == c;
         i = warp_append(act, in, p2p_cnt + c);
         if (in) {

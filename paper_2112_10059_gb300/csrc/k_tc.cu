@@ -1866,9 +1866,9 @@ __global__ void __launch_bounds__(256, 1) k_m2l_tiles(FmmDev F, const int *__res
 // their own, in a ring of six accumulators, added up in FP32 registers; the parts below have two more
 // accumulators for the whole tile (8 x 64 columns of TMEM).
 // A step is an offset: 48 KB of rows gathered by 16-byte copies, 24 KB of matrices by a bulk copy,
-// 24 MMAs; three steps in shared memory.  A step takes 1.4 us, bound by the copies (51 bytes a
-// ns and SM; the MMAs alone take 0.6).  Eight warps look the leaves up an offset ahead, copy, add up and
-// write results, one thread issues MMAs.
+// 24 MMAs; three steps in shared memory.  A step takes 1.4 us against 0.6 us of MMAs, bound by the
+// latency of its copies (tensor pipe 27% active, L2 at 22%).  Eight warps look the leaves up an
+// offset ahead, copy, add up and write results, one thread issues MMAs.
 // Uniform 128^3 (32,768 full leaves, 3.4e9 pairs): 712 us by the offset table, 82 so and 14 for its
 // operands; wide streamer 192^3 303, and 44 + 12 + 39 for the other leaves by the table.
 __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const int *__restrict__ p2p_list,

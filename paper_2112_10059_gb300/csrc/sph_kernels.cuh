@@ -307,11 +307,13 @@ void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *
 constexpr int NM_OFFS = 27, NM_CELLS = 64, NM_SPLIT = 3;
 constexpr size_t NM_ROW = NM_SPLIT * NM_CELLS;                            // BF16 values of a leaf's row
 constexpr size_t NM_MATRIX = (size_t)NM_SPLIT * NM_CELLS * NM_CELLS;      // and of an offset's matrix
+#ifdef __CUDACC__
 // the weights' range: above, a BF16 rounding could overflow; below, a third part would underflow
 __device__ __forceinline__ bool near_mma_range(int max_bits) {
     const float w = __int_as_float(max_bits);
     return w >= 0x1p-80f && w <= 0x1p120f;                               // false for NaN
 }
+#endif
 void fmm_near_pack(const FmmDev &F, const int *src_list, const int *src_count, int max_src, int row0, uint16_t *rows,
                    uint16_t *matrices, int *near_max, cudaStream_t st);
 void fmm_near_mma(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, int max_leaves, int row0,
