@@ -1322,7 +1322,7 @@ int fmm_p2l(const FmmDev &F, const int *list, const int *count, int max_boxes, c
 // warps share a leaf's sources, each lane sums two targets, and the warps' sums are added in
 // order.  Entries of larger leaves take the exp form (the staged points and p2p_sum below).
 // Uniform 128^3 (3.4e9 pairs): 2290 us by the exp form alone, 670 us so; wide streamer 192^3:
-// 996, 290.
+// 996, 290 (39 since its dense leaves are k_near_mma's; all of the uniform tree's are).
 constexpr int NG_PY = 20, NG_PZ = 304, NG_CENTRE = 7 * (1 + NG_PY + NG_PZ), NG_N = 2 * NG_CENTRE + 1;
 constexpr int NG_CAP = 2048;         // staged points per round (16 KiB; 1024 in the exp form)
 
