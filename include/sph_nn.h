@@ -63,7 +63,8 @@ int sph_nn_get_params(sph_nn *net, float *params_host, int64_t n);
 /* Gradient of the last sph_nn_backward, flat, same layout (synchronises the stream). */
 int sph_nn_get_grads(sph_nn *net, float *grads_host, int64_t n);
 
-/* Forward pass: x_dev BF16 [batch][D^3][16] -> y_dev FP32 [batch][D^3][2]. */
+/* Forward pass: x_dev BF16 [batch][D^3][16] -> y_dev FP32 [batch][D^3][2].  Here and below x_dev is
+ * read in 16-byte units and must be 16-byte aligned; the FP32 arrays need the 4 bytes of a float. */
 int sph_nn_forward(sph_nn *net, int batch, const uint16_t *x_dev, float *y_dev);
 /* Forward + backward against t_dev; the gradient stays on the device; *loss_host (optional)
  * receives L (synchronises the stream). */

@@ -316,7 +316,15 @@ __global__ void __launch_bounds__(160) k_conv_tc(ConvArgs a) {
                     r0 = fmaf(shead[c], f[c], r0);
                     e0 = fmaf(shead[16 + c], f[c], e0);
                 }
-                if (valid) *reinterpret_cast<float2 *>(a.y + o / N * 2) = make_float2(r0, e0);
+                if (valid) {                  // y is the caller's: its two floats need not be 8-byte aligned
+                    float *y = a.y + o / N * 2;
+                    if ((reinterpret_cast<uintptr_t>(a.y) & 7) == 0) {
+                        *reinterpret_cast<float2 *>(y) = make_float2(r0, e0);
+                    } else {
+                        y[0] = r0;
+                        y[1] = e0;
+                    }
+                }
             }
         };
 

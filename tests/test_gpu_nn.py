@@ -236,3 +236,21 @@ def test_bad_arguments(sur):
     x = torch.zeros(2 * 8 ** 3 * 16, dtype=torch.bfloat16, device="cuda")
     with pytest.raises(Exception):
         net.forward(x, 2)         # above max_batch
+
+
+@pytest.mark.parametrize("edge,batch", [(8, 3), (32, 1)])
+def test_forward_output_off_eight_bytes(sur, edge, batch):
+    """y is the caller's array of floats: one that starts 4 bytes past an 8-byte boundary gets the
+    same values, and nothing beside it is written."""
+    import torch
+    net = sur.Net(edge=edge, max_batch=batch, seed=12)
+    n = batch * edge ** 3 * 2
+    x = torch.rand(batch * edge ** 3 * 16, device="cuda").to(torch.bfloat16)
+    buf = torch.full((n + 2,), -7.0, device="cuda")
+    assert buf.data_ptr() % 8 == 0
+    y = net.forward(x, batch)
+    net.forward(x, batch, y=buf[1:n + 1])
+    torch.cuda.synchronize()
+    net.close()
+    assert torch.equal(buf[1:n + 1], y)
+    assert buf[0] == -7.0 and buf[n + 1] == -7.0
