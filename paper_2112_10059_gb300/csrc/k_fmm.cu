@@ -1325,21 +1325,36 @@ int fmm_p2l(const FmmDev &F, const int *list, const int *count, int max_boxes, c
 // 996, 290 (39 since its dense leaves are k_near_mma's; all of the uniform tree's are).
 constexpr int NG_PY = 20, NG_PZ = 304, NG_CENTRE = 7 * (1 + NG_PY + NG_PZ), NG_N = 2 * NG_CENTRE + 1;
 constexpr int NG_CAP = 2048;         // staged points per round (16 KiB; 1024 in the exp form)
+constexpr int NG_GROUP = 16;         // sources summed by themselves
 
 __device__ __forceinline__ int near_lin(uint32_t pc) { return pc_i(pc) + NG_PY * pc_j(pc) + NG_PZ * pc_k(pc); }
 
-// sums of sources [lo, hi) (even, in pairs) for the targets at byte offsets b0 and b1 of the table
+// sums of sources [lo, hi) (even, in pairs) for the targets at byte offsets b0 and b1 of the table.
+// Sixteen sources are summed by themselves before they join the warp's sum: in one chain the terms
+// behind a target's own cell, the largest, all round at its last place (432 terms a warp: rms error
+// 2.4e-7 to 1.3e-6 of a sum, pair by pair in k_p2p 1.9e-7 to 4.7e-7, here 1.2e-7 to 2.8e-7).
 template <bool TWO>
 __device__ __forceinline__ void near_grid_sum(const int2 *__restrict__ pts, int lo, int hi, const char *__restrict__ b0,
                                               const char *__restrict__ b1, float &a0, float &a1) {
-#pragma unroll 4
-    for (int j = lo; j < hi; j += 2) {
+    auto pair = [&](int j, float &p0, float &p1) {
         const int4 v = *reinterpret_cast<const int4 *>(pts + j);
-        a0 = fmaf(*reinterpret_cast<const float *>(b0 + v.x), __int_as_float(v.y), a0);
-        if (TWO) a1 = fmaf(*reinterpret_cast<const float *>(b1 + v.x), __int_as_float(v.y), a1);
-        a0 = fmaf(*reinterpret_cast<const float *>(b0 + v.z), __int_as_float(v.w), a0);
-        if (TWO) a1 = fmaf(*reinterpret_cast<const float *>(b1 + v.z), __int_as_float(v.w), a1);
+        p0 = fmaf(*reinterpret_cast<const float *>(b0 + v.x), __int_as_float(v.y), p0);
+        if (TWO) p1 = fmaf(*reinterpret_cast<const float *>(b1 + v.x), __int_as_float(v.y), p1);
+        p0 = fmaf(*reinterpret_cast<const float *>(b0 + v.z), __int_as_float(v.w), p0);
+        if (TWO) p1 = fmaf(*reinterpret_cast<const float *>(b1 + v.z), __int_as_float(v.w), p1);
+    };
+    int j = lo;
+    for (; j + NG_GROUP <= hi; j += NG_GROUP) {
+        float p0 = 0.f, p1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < NG_GROUP; k += 2) pair(j + k, p0, p1);
+        a0 += p0;
+        if (TWO) a1 += p1;
     }
+    float p0 = 0.f, p1 = 0.f;
+    for (; j < hi; j += 2) pair(j, p0, p1);
+    a0 += p0;
+    if (TWO) a1 += p1;
 }
 
 template <bool TAYLOR>

@@ -1,0 +1,79 @@
+"""The near-field forms alone, against the FP64 oracle.
+
+Every cell of a 16^3 grid is a source (i_frac 0), the weights are zero outside the first 12^3 cells
+and the targets are the leaf of cells 4 .. 7 of each axis: all weights lie in the leaf and in its
+neighbours, every source box beyond them sums to exactly zero, and S is the near field and nothing
+else.  Its sums are taken in a fixed order, so a form's result is the same bits at every call.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+N, LO, HI = 16, 4, 8
+PAIRS, TABLE, MATRIX = {"SPH_NEAR_OVERLAP": "0"}, {"SPH_NEAR_MMA": "0"}, {"SPH_NEAR_MMA": "1"}
+
+
+@pytest.fixture(scope="module")
+def sph():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2112_10059_gb300 as m
+    return m
+
+
+def _targets():
+    m = np.zeros((N, N, N), np.uint8)
+    m[LO:HI, LO:HI, LO:HI] = 1
+    return m.reshape(-1)
+
+
+def _weights(kind, seed):
+    u = np.random.default_rng(seed).random((N, N, N))
+    q = {"uniform": 0.5 + 0.5 * u, "const": np.ones_like(u), "noise": u, "wide": 10.0 ** (-6.0 * u)}[kind]
+    q[12:] = q[:, 12:] = q[:, :, 12:] = 0.0
+    return q.astype(np.float32).reshape(-1)
+
+
+def _near(sph, monkeypatch, form, q, h, pO2, scale=1.0):
+    import torch
+    for k in ("SPH_NEAR_OVERLAP", "SPH_NEAR_MMA"):
+        monkeypatch.delenv(k, raising=False)
+    for k, v in form.items():
+        monkeypatch.setenv(k, v)
+    c = sph.Context(0)
+    sph.set_grid(c, N, N, N, h, pO2)
+    sph.set_sources(c, torch.from_numpy(q).cuda(), scale)
+    sph.set_targets(c, mask=torch.from_numpy(_targets()).cuda())
+    sph.set_criteria(c, 0.0, leaf_size=64)
+    out, _ = sph.eval_sph(c)
+    S = out.cpu().numpy()[_targets() != 0]
+    c.close()
+    return S
+
+
+def _exact(q, h, pO2, scale=1.0):
+    a, b = oracle.alpha_beta(pO2, 0.035, 2.0)
+    return oracle.sph(N, N, N, h, a, b, q, scale, np.nonzero(q)[0].astype(np.int32),
+                      np.nonzero(_targets())[0].astype(np.int32))
+
+
+# cell edge (cm) and pO2 (Torr): both sides of the series form, and a coarse grid
+GRIDS = [(1.0 / 128, 150.0), (1e-3, 15.0), (1.0 / 24, 150.0)]
+
+
+@pytest.mark.parametrize("kind", ["uniform", "const", "noise", "wide"])
+@pytest.mark.parametrize("h,pO2", GRIDS)
+def test_table_form_no_further_off_than_pair_by_pair(sph, monkeypatch, h, pO2, kind):
+    """The offset table holds the values that the kernel of each pair has, so its sums must be no
+    further from FP64 than those taken pair by pair (rms over eight fields)."""
+    err = {"pairs": [], "table": []}
+    for seed in range(8):
+        q = _weights(kind, seed)
+        ref = _exact(q, h, pO2)
+        err["pairs"].append(_near(sph, monkeypatch, PAIRS, q, h, pO2) / ref - 1)
+        err["table"].append(_near(sph, monkeypatch, TABLE, q, h, pO2) / ref - 1)
+    rms = {k: np.sqrt(np.mean(np.square(v))) for k, v in err.items()}
+    assert rms["table"] <= rms["pairs"], rms
