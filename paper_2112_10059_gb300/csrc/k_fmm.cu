@@ -1590,32 +1590,38 @@ void fmm_near_w(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int st
 }
 
 // ---------------------------------------------------------------- operands of the matrix near field
-__device__ __forceinline__ void split3(float x, uint32_t (&s)[NM_SPLIT]) {
+template <class T>
+__device__ __forceinline__ void split3(T x, uint32_t (&s)[NM_SPLIT]) {
 #pragma unroll
     for (int k = 0; k < NM_SPLIT; ++k) {             // each rest is exact
-        const __nv_bfloat16 b = __float2bfloat16_rn(x);
+        const __nv_bfloat16 b = __float2bfloat16_rn((float)x);
         s[k] = __bfloat16_as_ushort(b);
-        x -= __bfloat162float(b);
+        x -= (T)__bfloat162float(b);
     }
 }
 
 // Blocks below NP_G: the kernel's values of an offset between two leaves, [split][target][source]
 // (cells in local Morton order, K-major with the 128-byte swizzle); the others a warp per source
-// leaf: its weights on its 64 cells.  Weights and kernel values as the sums of three BF16 parts.
+// leaf: its weights on its 64 cells.  Weights and kernel values as the sums of three BF16 parts;
+// the kernel's 148 values come in FP64 from the host (formed here by the approximate functions of the
+// exp form they were 1.3e-7 to 2.6e-7 too small on average, most of a sum's error).
 constexpr int NP_G = NM_OFFS * NM_CELLS * NM_CELLS / 2 / 256, NP_WARPS = 8;
 
-template <bool TAYLOR>
-__global__ void __launch_bounds__(NP_WARPS * 32) k_near_pack(FmmDev F, P2PConst K, const int *__restrict__ list,
+__global__ void __launch_bounds__(NP_WARPS * 32) k_near_pack(FmmDev F, NearG G, const int *__restrict__ list,
                                                              const int *__restrict__ count, int row0,
                                                              uint16_t *__restrict__ rows, uint16_t *__restrict__ matrices,
                                                              int *__restrict__ near_max) {
     pdl_enter();
     __shared__ float cells[NP_WARPS][NM_CELLS];
+    __shared__ uint32_t gparts[NM_D2][NM_SPLIT];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if ((int)blockIdx.x < NP_G) {
+        if (tid < NM_D2) split3(G.g[tid], gparts[tid]);
+        __syncthreads();
         const int e = 2 * (blockIdx.x * 256 + tid);
         const int o = e / (NM_CELLS * NM_CELLS), t = e / NM_CELLS % NM_CELLS, s0 = e % NM_CELLS;
-        uint32_t tx, ty, tz, part[2][NM_SPLIT];
+        uint32_t tx, ty, tz;
+        int d2[2];
         demorton3((uint32_t)t, tx, ty, tz);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -1623,13 +1629,12 @@ __global__ void __launch_bounds__(NP_WARPS * 32) k_near_pack(FmmDev F, P2PConst 
             demorton3((uint32_t)(s0 + j), sx, sy, sz);
             const int dx = 4 * (o % 3 - 1) + (int)sx - (int)tx, dy = 4 * (o / 3 % 3 - 1) + (int)sy - (int)ty,
                       dz = 4 * (o / 9 - 1) + (int)sz - (int)tz;
-            const int d2 = dx * dx + dy * dy + dz * dz;
-            split3(d2 ? p2p_g<TAYLOR>((float)d2, K) : K.wself, part[j]);
+            d2[j] = dx * dx + dy * dy + dz * dz;
         }
         uint8_t *m = reinterpret_cast<uint8_t *>(matrices + (size_t)o * NM_MATRIX) + tc::sw128_offset(t, s0, NM_CELLS);
 #pragma unroll
         for (int k = 0; k < NM_SPLIT; ++k)
-            *reinterpret_cast<uint32_t *>(m + (size_t)k * NM_CELLS * NM_CELLS * 2) = part[0][k] | part[1][k] << 16;
+            *reinterpret_cast<uint32_t *>(m + (size_t)k * NM_CELLS * NM_CELLS * 2) = gparts[d2[0]][k] | gparts[d2[1]][k] << 16;
         return;
     }
     const float wsc = F.wscale * F.kp.C / (F.kp.h * F.kp.h * F.kp.h);
@@ -1658,14 +1663,10 @@ __global__ void __launch_bounds__(NP_WARPS * 32) k_near_pack(FmmDev F, P2PConst 
     if (lane == 0 && most) atomicMax(near_max, (int)most);
 }
 
-void fmm_near_pack(const FmmDev &F, const int *src_list, const int *src_count, int max_src, int row0, uint16_t *rows,
-                   uint16_t *matrices, int *near_max, cudaStream_t st) {
-    const P2PConst K = p2p_const(F);
+void fmm_near_pack(const FmmDev &F, const NearG &G, const int *src_list, const int *src_count, int max_src, int row0,
+                   uint16_t *rows, uint16_t *matrices, int *near_max, cudaStream_t st) {
     const int grid = NP_G + std::min((max_src + NP_WARPS - 1) / NP_WARPS, 152 * 8);
-    if (K.bma_h >= 0.5f)
-        launch_pdl(k_near_pack<false>, grid, NP_WARPS * 32, 0, st, F, K, src_list, src_count, row0, rows, matrices, near_max);
-    else
-        launch_pdl(k_near_pack<true>, grid, NP_WARPS * 32, 0, st, F, K, src_list, src_count, row0, rows, matrices, near_max);
+    launch_pdl(k_near_pack, grid, NP_WARPS * 32, 0, st, F, G, src_list, src_count, row0, rows, matrices, near_max);
 }
 
 void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, const int *near_max,

@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256, 1) k_m2l_tiles(FmmDev F, const int *__res
 // matrix near field (below)
 constexpr uint32_t NM_A = TCM * NM_CELLS * 2, NM_B = NM_CELLS * NM_CELLS * 2;   // one part of a step's operands
 constexpr uint32_t NM_STAGE = NM_SPLIT * (NM_A + NM_B);
-constexpr int NM_RING = 3, NM_ACCS = 6;          // steps in shared memory; accumulators of hi hi
+constexpr int NM_RING = 3, NM_KS = NM_CELLS / 16; // steps in shared memory; K slices (and accumulators) of a step
 constexpr uint32_t NM_SMEM = 1024 + NM_RING * NM_STAGE + 4 * TCM * 4 + 128;
 constexpr int NM_COPY = 256;                     // copying threads
 __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const int *__restrict__ p2p_list,
@@ -1862,9 +1862,10 @@ __global__ void __launch_bounds__(256, 1) k_m2l_tiles(FmmDev F, const int *__res
 // M = 128 leaves, N = 64 targets, K = 27 x 64 cells.  FP32 factors as sums of three BF16 parts
 // (24 bits); the products hi hi, hi mid, mid hi, hi lo, lo hi and mid mid are formed, the largest
 // left out is 2^-24 of the sum.  The tensor core's additions round towards zero (one accumulator for
-// everything: 8.5e-6 of a sum lost), so they are kept few: an offset's hi hi are a sum of four MMAs of
-// their own, in a ring of six accumulators, added up in FP32 registers; the parts below have two more
-// accumulators for the whole tile (8 x 64 columns of TMEM).
+// everything: 8.5e-6 of a sum lost), so they are kept few and small: every 16 source cells have an
+// accumulator of their own, into which the lower parts' products go first and hi hi last, the one
+// addition that rounds at the sum's own size; four accumulators an offset, two offsets' in TMEM, added
+// up in FP32 registers.
 // A step is an offset: 48 KB of rows gathered by 16-byte copies, 24 KB of matrices by a bulk copy,
 // 24 MMAs; three steps in shared memory.  A step takes 1.4 us against 0.6 us of MMAs, bound by the
 // latency of its copies (tensor pipe 27% active, L2 at 22%).  Eight warps look the leaves up an
@@ -1928,19 +1929,19 @@ __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const in
                     wait(bar_a + st, use);
                     tc::fence_after_sync();
                     const uint64_t a = tc::sdesc_sw128(ring + st * NM_STAGE), b = tc::sdesc_sw128(ring + st * NM_STAGE + NM_SPLIT * NM_A);
-                    const uint32_t big = tmem + (uint32_t)(o % NM_ACCS) * NM_CELLS;
-                    const uint32_t mid = tmem + NM_ACCS * NM_CELLS, low = mid + NM_CELLS;
+                    const uint32_t acc = tmem + (uint32_t)((o & 1) * NM_KS * NM_CELLS);
+                    auto product = [&](uint32_t pa, uint32_t pb, uint32_t accumulate) {   // part pa of the rows by pb
 #pragma unroll
-                    for (int ks = 0; ks < NM_CELLS / 16; ++ks) {
-                        const uint64_t ah = a + ((32 * ks) >> 4), am = ah + (NM_A >> 4), al = am + (NM_A >> 4);
-                        const uint64_t bh = b + ((32 * ks) >> 4), bm = bh + (NM_B >> 4), bl = bm + (NM_B >> 4);
-                        tc::mma_bf16(big, ah, bh, idesc, ks > 0);
-                        tc::mma_bf16(mid, ah, bm, idesc, o > 0 || ks > 0);
-                        tc::mma_bf16(mid, am, bh, idesc, 1);
-                        tc::mma_bf16(low, ah, bl, idesc, o > 0 || ks > 0);
-                        tc::mma_bf16(low, al, bh, idesc, 1);
-                        tc::mma_bf16(low, am, bm, idesc, 1);
-                    }
+                        for (int ks = 0; ks < NM_KS; ++ks)
+                            tc::mma_bf16(acc + (uint32_t)(ks * NM_CELLS), a + ((pa * NM_A + 32 * ks) >> 4),
+                                         b + ((pb * NM_B + 32 * ks) >> 4), idesc, accumulate);
+                    };
+                    product(2, 0, 0);
+                    product(0, 2, 1);
+                    product(1, 1, 1);
+                    product(1, 0, 1);
+                    product(0, 1, 1);
+                    product(0, 0, 1);
                     tc::mma_commit(tc::smem_u32(bar_e + st));
                 }
                 tc::mma_commit(tc::smem_u32(bar_d));
@@ -1958,13 +1959,20 @@ __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const in
         const int q = warp & 3, c0 = (warp >> 2) * 32;
         const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
         float sum[32];
-        auto add = [&](int k) {                   // accumulator k to the sums
+        auto add = [&](int o) {                   // offset o's accumulators to the sums
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                float v[16];
-                tc::tmem_ld16(acc + (uint32_t)k * NM_CELLS + 16 * h, v);
+                const uint32_t at = acc + (uint32_t)((o & 1) * NM_KS * NM_CELLS + 16 * h);
+                float s[16], v[16];
+                tc::tmem_ld16(at, s);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) sum[16 * h + j] += v[j];
+                for (int ks = 1; ks < NM_KS; ++ks) {
+                    tc::tmem_ld16(at + (uint32_t)(ks * NM_CELLS), v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) s[j] += v[j];
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) sum[16 * h + j] += s[j];
             }
         };
         int step = 0, turn = 0;
@@ -2008,8 +2016,8 @@ __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const in
                 tc::cp_async_commit();
                 if (o >= NM_RING) {               // the MMAs of offset o - NM_RING are done (waited for above)
                     tc::fence_after_sync();
-                    add((o - NM_RING) % NM_ACCS);
-                    tc::fence_before_sync();      // read before this thread's arrivals let its next MMAs begin
+                    add(o - NM_RING);
+                    tc::fence_before_sync();      // read before this thread's arrival lets offset o - 1's MMAs begin
                 }
                 if (o > 0) {                      // the step before has landed
                     tc::cp_async_wait<1>();
@@ -2018,15 +2026,18 @@ __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const in
                 }
                 asm volatile("bar.sync 1, %0;" ::"n"(NM_COPY) : "memory");   // the next offset's rows are in tab
             }
+            // as in the loop, for the last offset's MMAs
+            wait(bar_e + (step - NM_RING) % NM_RING, (step - NM_RING) / NM_RING);
+            tc::fence_after_sync();
+            add(NM_OFFS - NM_RING);
+            tc::fence_before_sync();
             tc::cp_async_wait<0>();
             tc::fence_proxy_async_smem();
             tc::mbar_arrive(tc::smem_u32(bar_a + (step - 1) % NM_RING));
             wait(bar_d, turn);
             tc::fence_after_sync();
-#pragma unroll
-            for (int o = NM_OFFS - NM_RING; o < NM_OFFS; ++o) add(o % NM_ACCS);
-            add(NM_ACCS);
-            add(NM_ACCS + 1);
+            add(NM_OFFS - 2);
+            add(NM_OFFS - 1);
             const int m = tile * TCM + 32 * q + lane;
             if (m < cnt) {
                 float *slot = F.near_buf + (size_t)(first + m) * F.near_s + c0;

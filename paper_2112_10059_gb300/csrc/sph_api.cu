@@ -117,6 +117,8 @@ struct sph_ctx {
     bool near_table = false;          // resolved for the current evaluation
     DevBuf b_gtab, b_dtab;            // near-field table; FP64 pair weights of the direct sum
     DevBuf b_nrows, b_nmat;           // operands of the matrix near field
+    NearG near_g;                     // its kernel values, of the grid and gas in near_g_key
+    double near_g_key[4] = {0, 0, 0, 0};
     // buffers
     DevBuf b_maxes, b_cnt, b_off, b_tot, b_skey, b_spc, b_sq, b_tkey, b_tpc, b_bstat;
     DevBuf b_boxat, b_flag, b_pos, b_rng, b_scan, b_lvl;
@@ -685,6 +687,7 @@ struct PassState {
     MtLevels ML;                 // target-stationary M2L: groups per level
     int *mt_groups = nullptr;    // [groups] scratch of that M2L
     bool fused = false;          // the last L2L and the L2P of the deepest level in one kernel
+    NearG G;                     // kernel values of the matrix near field
 };
 
 // the last L2L and the L2P of the deepest level fused (every box there a leaf of edge 4)
@@ -706,6 +709,21 @@ bool near_mma_pays(const sph_ctx *c, const PassState &S) {
     for (int l = 0; l <= c->Lmax; ++l) leaves += c->lvl_sleaf[l];
     const double mean = (double)c->ns / (double)std::max<int64_t>(leaves, 1);
     return mean >= 16.0 && (double)c->list_tot[0] * mean * 64.0 >= 2e8;
+}
+
+// The scaled kernel e^{-alpha R} (1 - e^{-(beta - alpha) R}) / s^3, R = h s, at s^2 = 0 .. NM_D2 - 1
+// (0: the self weight G_self h^3 / C), 148 values for as long as grid and gas stay.
+const NearG &near_kernel_values(sph_ctx *c) {
+    const double key[4] = {c->h, c->alpha, c->beta, c->self_mode ? c->self_int : 0.0};
+    if (memcmp(key, c->near_g_key, sizeof key) != 0) {
+        c->near_g.g[0] = key[3] * 4.0 * M_PI * std::log(c->beta / c->alpha) * (1.0 + NM_ROUND);
+        for (int d2 = 1; d2 < NM_D2; ++d2) {
+            const double s = std::sqrt((double)d2), R = c->h * s;
+            c->near_g.g[d2] = std::exp(-c->alpha * R) * -std::expm1(-(c->beta - c->alpha) * R) / (s * s * s) * (1.0 + NM_ROUND);
+        }
+        memcpy(c->near_g_key, key, sizeof key);
+    }
+    return c->near_g;
 }
 
 // Every buffer the passes need (so that fmm_queue allocates nothing and can be captured).
@@ -776,7 +794,10 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
         const int r = ensure(c, c->b_nrows, std::max<size_t>(c->lvl_count[L], 1) * NM_ROW * sizeof(uint16_t));
         const int r2 = r == SPH_OK ? ensure(c, c->b_nmat, NM_OFFS * NM_MATRIX * sizeof(uint16_t)) : r;
         if (c->poisoned) return SPH_ECUDA;
-        if (r2 == SPH_OK) F.near_mma_level = L;       // without room the other near-field form takes every leaf
+        if (r2 == SPH_OK) {                           // without room the other near-field form takes every leaf
+            F.near_mma_level = L;
+            S.G = near_kernel_values(c);
+        }
     }
     // the fused deepest level reads only the d rows of leaves with V or X entries: the rows of
     // that level are then cleared one by one by the work lists, the levels above by a memset
@@ -861,7 +882,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
             int *near_max = S.w_cnt + 33;
             if (L >= 0) {
                 uint16_t *rows = P<uint16_t>(c->b_nrows), *mat = P<uint16_t>(c->b_nmat);
-                fmm_near_pack(F, S.w_src + row0, S.w_cnt + L, c->lvl_src[L], row0, rows, mat, near_max, c->near_stream);
+                fmm_near_pack(F, S.G, S.w_src + row0, S.w_cnt + L, c->lvl_src[L], row0, rows, mat, near_max, c->near_stream);
                 fmm_near_mma(F, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), c->lvl_leaf[L], row0, rows, mat, near_max, S.err,
                              c->near_stream);
                 c->launches += 1 + (c->lvl_leaf[L] > 0);

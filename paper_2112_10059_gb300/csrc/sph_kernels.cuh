@@ -305,6 +305,14 @@ void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *
 // weights of the source leaves of level F.near_mma_level (src_list; rows by box - row0) and the
 // kernel's matrices, and leaves the bits of the largest |weight| in near_max (zeroed before)
 constexpr int NM_OFFS = 27, NM_CELLS = 64, NM_SPLIT = 3;
+constexpr int NM_D2 = 3 * 7 * 7 + 1;                                      // squared offsets between neighbouring leaves
+struct NearG {
+    double g[NM_D2];     // the near field's scaled kernel at squared offset d2, [0] the self weight
+};
+// k_near_mma's sums are rounded towards zero once at their own size, which takes half a unit in
+// the last place off them on average: 2^-24 (1 - 1/2) / ln 2 of a sum whose mantissa is spread
+// evenly over its logarithm.  The kernel values are larger by as much.
+constexpr double NM_ROUND = 4.3e-8;
 constexpr size_t NM_ROW = NM_SPLIT * NM_CELLS;                            // BF16 values of a leaf's row
 constexpr size_t NM_MATRIX = (size_t)NM_SPLIT * NM_CELLS * NM_CELLS;      // and of an offset's matrix
 #ifdef __CUDACC__
@@ -314,8 +322,8 @@ __device__ __forceinline__ bool near_mma_range(int max_bits) {
     return w >= 0x1p-80f && w <= 0x1p120f;                               // false for NaN
 }
 #endif
-void fmm_near_pack(const FmmDev &F, const int *src_list, const int *src_count, int max_src, int row0, uint16_t *rows,
-                   uint16_t *matrices, int *near_max, cudaStream_t st);
+void fmm_near_pack(const FmmDev &F, const NearG &G, const int *src_list, const int *src_count, int max_src, int row0,
+                   uint16_t *rows, uint16_t *matrices, int *near_max, cudaStream_t st);
 void fmm_near_mma(const FmmDev &F, const int *p2p_list, const int *p2p_cnt, int stride, int max_leaves, int row0,
                   const uint16_t *rows, const uint16_t *matrices, const int *near_max, int *err, cudaStream_t st);
 // the W-list part (Chebyshev far field) of the leaves in w_list (fmm_work_lists; at most max_w), added to the slots

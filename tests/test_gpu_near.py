@@ -77,3 +77,21 @@ def test_table_form_no_further_off_than_pair_by_pair(sph, monkeypatch, h, pO2, k
         err["table"].append(_near(sph, monkeypatch, TABLE, q, h, pO2) / ref - 1)
     rms = {k: np.sqrt(np.mean(np.square(v))) for k, v in err.items()}
     assert rms["table"] <= rms["pairs"], rms
+
+
+@pytest.mark.parametrize("kind", ["uniform", "const", "noise", "wide"])
+@pytest.mark.parametrize("h,pO2", GRIDS)
+def test_matrix_form_no_further_off_than_pair_by_pair(sph, monkeypatch, h, pO2, kind):
+    """The products of the three BF16 parts, summed by the tensor core, take the place of FP32 sums
+    pair by pair and must be no further from FP64 (rms over eight fields).  The form did run: the
+    table's sums of the same leaf differ from it in their last places."""
+    err = {"pairs": [], "matrix": []}
+    for seed in range(8):
+        q = _weights(kind, seed)
+        ref = _exact(q, h, pO2)
+        S = _near(sph, monkeypatch, MATRIX, q, h, pO2)
+        assert not np.array_equal(S, _near(sph, monkeypatch, TABLE, q, h, pO2))
+        err["pairs"].append(_near(sph, monkeypatch, PAIRS, q, h, pO2) / ref - 1)
+        err["matrix"].append(S / ref - 1)
+    rms = {k: np.sqrt(np.mean(np.square(v))) for k, v in err.items()}
+    assert rms["matrix"] <= rms["pairs"], rms
