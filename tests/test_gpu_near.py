@@ -95,3 +95,37 @@ def test_matrix_form_no_further_off_than_pair_by_pair(sph, monkeypatch, h, pO2, 
         err["matrix"].append(S / ref - 1)
     rms = {k: np.sqrt(np.mean(np.square(v))) for k, v in err.items()}
     assert rms["matrix"] <= rms["pairs"], rms
+
+
+def test_matrix_form_sums_every_part(sph, monkeypatch):
+    """Weights whose third BF16 part is nearly as large as it gets, and of one sign: 1 + 3 * 2^-10 +
+    2^-17 - 2^-21 is 1 (hi) + 3 * 2^-10 (mid) + 2^-17 - 2^-21 (lo), so that a sum without lo hi would be
+    7.1e-6 too small, one without lo hi and hi mid or mid hi far more.  What remains is at most a unit of
+    2^-23 for the four accumulators an offset, 27 FP32 additions of 2^-24 each and 2^-22 of the kernel
+    values' rounding and mean correction: 2e-6 in all."""
+    h, pO2 = 1.0 / 128, 150.0
+    # the near field multiplies the weights by C = 1 / (4 pi ln(chi ratio)): a scale that undoes it
+    q = _weights("const", 0) * np.float32(1 + 3 * 2.0 ** -10 + 2.0 ** -17 - 2.0 ** -21)
+    scale = 4 * np.pi * np.log(2.0 / 0.035)
+    S = _near(sph, monkeypatch, MATRIX, q, h, pO2, scale)
+    assert np.max(np.abs(S / _exact(q, h, pO2, scale) - 1)) < 2e-6
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, 2.0 ** 126, "small"])
+def test_weights_that_the_matrix_form_leaves_to_the_table(sph, monkeypatch, value):
+    """NaN, infinity, and weights whose BF16 parts would overflow or underflow: the table takes every
+    leaf, with the same bits as where the matrix form is off."""
+    q = _weights("uniform", 1)
+    if value == "small":
+        q = (q * np.float32(2.0 ** -90)).astype(np.float32)
+    else:
+        q = q.reshape(N, N, N)
+        q[1, 2, 3] = value
+        q = q.reshape(-1)
+    h, pO2 = 1.0 / 128, 150.0
+    a, b = _near(sph, monkeypatch, MATRIX, q, h, pO2), _near(sph, monkeypatch, TABLE, q, h, pO2)
+    assert np.array_equal(a, b, equal_nan=True)
+    if value == "small":
+        assert np.all(a > 0)
+    elif not np.isfinite(value):
+        assert not np.any(np.isfinite(a))
