@@ -825,18 +825,35 @@ bool m2l_target_tiles(const sph_ctx *c, const PassState &S) {
                     (c->m2l_tiles == 2 && (c->m2l_form >= 0 ? c->m2l_form == 1 : nV >= 32 * nb && nV >= 5000000)));
 }
 
-// CTAs per SM of the overlapped near field's U-list launch.  Five fit beside each other (37 KB of
-// shared memory each); where the far-field chain is the longer of the two, four leave slots to its
-// kernels (256^3 headline: 458 us with 4, 464 with 5, 467 with 6; uniform 128^3: 2830, 2813, 2811).
-// Estimates from the list totals: near-field pairs at most U entries x leaf size^2 at 5e12/s; far
-// field a fixed 150 us plus the M2L at its measured cost per V pair (0.18 ns).  The tabulated near field keeps its own figures (1.6e12/s, 16 and 6).
-int near_cap(const sph_ctx *c, const PassState &S) {
+// Whether the overlapped near field takes the U lists by the offset table (k_near_grid) or pair by
+// pair (k_p2p).  The table serves leaves of edge 4 or less; a coarser leaf takes k_near_grid's exp
+// form, which stages a leaf's sources anew for every 64 targets.  Near field alone, where no leaf
+// is that small: 512^2 cells in a plane 141 us by pairs and 222 by k_near_grid, wide streamer 192^3 at
+// leaf size 512 8.9 and 16.9 ms, all of 64^3 at 4096 70 and 259 ms; where all are: 92 and 61 us (adaptive
+// 256^3), 291 and 146 (all of 64^3); where a third are: 460 and 464.
+bool near_by_offsets(const sph_ctx *c, const FmmDev &F) {
+    if (F.gtab) return false;
+    int64_t all = 0, small = 0;
+    for (int l = 0; l <= c->Lmax; ++l) {
+        all += c->lvl_leaf[l];
+        if (c->D - l <= 2) small += c->lvl_leaf[l];
+    }
+    return F.near_mma_level >= 0 || 2 * small >= all;
+}
+
+// CTAs per SM of the overlapped near field's U-list launch.  Five of k_near_grid fit beside each
+// other (37 KB of shared memory each), and take as long as four (256^3 headline: 419 us with 4, 418
+// with 5, 431 with 6; wide 192^3: 978, 976, 983; uniform 128^3, whose leaves are k_near_mma's: 1615 with any).
+// k_p2p: 16 where the near field is the longer chain, else 6, which leaves slots to the far field's
+// kernels; estimated from the list totals, pairs at most U entries x leaf size^2 at 1.6e12/s, far field
+// a fixed 150 us plus the M2L at its measured cost per V pair (0.18 ns).
+int near_cap(const sph_ctx *c, bool by_offsets) {
     if (c->near_per_sm > 0) return c->near_per_sm;
+    if (by_offsets) return 5;
     const double s = c->leaf_eff;
-    const bool table = S.F.gtab != nullptr;
-    const double near_us = (double)c->list_tot[0] * s * s / (table ? 1.6e6 : 5e6);
+    const double near_us = (double)c->list_tot[0] * s * s / 1.6e6;
     const double far_us = 150.0 + (double)c->list_tot[1] * 0.18e-3;
-    return near_us > far_us ? (table ? 16 : 5) : (table ? 6 : 4);
+    return near_us > far_us ? 16 : 6;
 }
 
 // Queue the passes on c->stream: memsets and kernels only (no allocation, no sync).
@@ -875,8 +892,9 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
             ++c->launches;
         }
         if (tm) tm->mark_at(12, c->near_stream);
-        if (F.gtab)
-            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, S));
+        const bool by_offsets = near_by_offsets(c, F);
+        if (!by_offsets)
+            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, by_offsets));
         else {
             const int L = F.near_mma_level, row0 = L >= 0 ? c->lvl_base[L] : 0;
             int *near_max = S.w_cnt + 33;
@@ -887,7 +905,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
                              c->near_stream);
                 c->launches += 1 + (c->lvl_leaf[L] > 0);
             }
-            fmm_near_grid(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), near_max, c->near_stream, near_cap(c, S));
+            fmm_near_grid(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), near_max, c->near_stream, near_cap(c, by_offsets));
         }
         ++c->launches;
         if (tm) tm->mark_at(14, c->near_stream);

@@ -129,3 +129,24 @@ def test_weights_that_the_matrix_form_leaves_to_the_table(sph, monkeypatch, valu
         assert np.all(a > 0)
     elif not np.isfinite(value):
         assert not np.any(np.isfinite(a))
+
+
+@pytest.mark.parametrize("nx,ny,nz,leaf", [(16, 16, 16, 512), (16, 15, 13, 4096), (16, 16, 1, 64)])
+def test_coarse_leaves_go_pair_by_pair(sph, monkeypatch, nx, ny, nz, leaf):
+    """Leaves of edge 8 and 16, for which the offset table is not made: the near field beside the far
+    field sums them as the kernel after it does (SPH_NEAR_OVERLAP=0), to the same bits.  All boxes are
+    adjacent, so there is no far field."""
+    import torch
+    q = torch.from_numpy(np.random.default_rng(4).random(nx * ny * nz).astype(np.float32)).cuda()
+    out = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("SPH_NEAR_OVERLAP", flag)
+        c = sph.Context(0)
+        sph.set_grid(c, nx, ny, nz, 1.0 / 128, 150.0)
+        sph.set_sources(c, q, 1.0)
+        sph.set_targets(c)
+        sph.set_criteria(c, 0.0, leaf_size=leaf)
+        out.append(sph.eval_sph(c)[0].cpu().numpy())
+        assert sph.get_tree(c)["V"].size == 0
+        c.close()
+    assert np.array_equal(out[0], out[1]) and np.all(out[0] > 0)
