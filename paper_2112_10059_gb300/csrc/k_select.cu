@@ -283,7 +283,10 @@ __device__ __forceinline__ unsigned long long pack_state(unsigned st, unsigned n
 // fallback's block masks on 256^3 the count and emit passes had read every brick, 61 + 82 us a
 // selection, now 38 + 60 and 14 + 33 against 8 more here); the brick's maxima go into `out` (ordered uints, as k_grid_max).  Four threads per row of 16 cells, each one 16-byte load per array and
 // row, four rows per thread: all eight loads in flight at once.
+// MASK: with the mask's part (as an argument of one kernel it took the other selections from 46 to 64
+// registers, 2 us of 40 at 128^3).
 constexpr int STAT_T = 256;
+template <bool MASK>
 __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *__restrict__ q,
                                                         const float *__restrict__ e, const uint8_t *__restrict__ mk,
                                                         float4 *__restrict__ bstat, unsigned *__restrict__ out) {
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
     auto take = [&](float vq, float ve, bool in) {
         if (!in) return;
         if (q && vq == vq) mq = fmaxf(mq, vq);
-        if (e) {
+        if (!MASK && e) {
             if (ve == ve) {
                 lo = fminf(lo, ve);
                 hi = fmaxf(hi, ve);
@@ -313,7 +316,7 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
         hi = fmaxf(hi, m ? 1.f : 0.f);
     };
     const bool vec = x0 + 16 <= r.nx && (r.nx & 3) == 0 && (reinterpret_cast<uintptr_t>(q) & 15) == 0 &&
-                     (reinterpret_cast<uintptr_t>(e) & 15) == 0 && (reinterpret_cast<uintptr_t>(mk) & 3) == 0;
+                     (reinterpret_cast<uintptr_t>(e) & 15) == 0 && (!MASK || (reinterpret_cast<uintptr_t>(mk) & 3) == 0);
     if (vec) {
         float4 a[4], c[4];
         uint32_t m[4];
@@ -326,8 +329,8 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
             a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
             c[k] = a[k];
             if (in[k] && q) a[k] = __ldg(reinterpret_cast<const float4 *>(q + lin));
-            if (in[k] && e) c[k] = __ldg(reinterpret_cast<const float4 *>(e + lin));
-            m[k] = in[k] && mk ? __ldg(reinterpret_cast<const uint32_t *>(mk + lin)) : 0u;
+            if (!MASK && in[k] && e) c[k] = __ldg(reinterpret_cast<const float4 *>(e + lin));
+            if (MASK) m[k] = in[k] ? __ldg(reinterpret_cast<const uint32_t *>(mk + lin)) : 0u;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -335,34 +338,34 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
             take(a[k].y, c[k].y, in[k]);
             take(a[k].z, c[k].z, in[k]);
             take(a[k].w, c[k].w, in[k]);
-            if (in[k] && mk) {
+            if (MASK && in[k]) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) take_mask(m[k] >> (8 * j) & 255u);
             }
         }
     } else {
-        // an odd pitch: cell by cell, eight planes' loads in flight at a time (48 us on
-        // 222^3 one after another, 33 so)
+        // an odd pitch: cell by cell, four planes' loads in flight at a time (48 us on 222^3 one
+        // after another, 33 so)
         const int x = x0 + (tid & 15), y = y0 + (tid >> 4);
         const bool col = x < r.nx && y < r.ny;
+#pragma unroll 1
+        for (int h = 0; h < 4; ++h) {
+            float a[4], c[4];
+            uint32_t m[4];
+            bool in[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float a[8], c[8];
-            uint32_t m[8];
-            bool in[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int z = z0 + 8 * h + k;
+            for (int k = 0; k < 4; ++k) {
+                const int z = z0 + 4 * h + k;
                 in[k] = col && z < r.nz;
                 const int64_t lin = in[k] ? (int64_t)x + (int64_t)r.nx * ((int64_t)y + (int64_t)r.ny * z) : 0;
                 a[k] = in[k] && q ? __ldg(q + lin) : 0.f;
-                c[k] = in[k] && e ? __ldg(e + lin) : 0.f;
-                m[k] = in[k] && mk ? __ldg(mk + lin) : 0u;
+                c[k] = !MASK && in[k] && e ? __ldg(e + lin) : 0.f;
+                if (MASK) m[k] = in[k] ? __ldg(mk + lin) : 0u;
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < 4; ++k) {
                 take(a[k], c[k], in[k]);
-                if (in[k] && mk) take_mask(m[k]);
+                if (MASK && in[k]) take_mask(m[k]);
             }
         }
     }
@@ -393,6 +396,14 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
     }
 }
 
+// a brick of the enclosing cube that lies outside the grid
+__device__ __forceinline__ bool brick_outside(const SelRule &r, uint32_t brick) {
+    uint32_t bx, by, bz;
+    demorton3(brick, bx, by, bz);
+    const int b = r.brick_edge_log2;
+    return ((int)bx << b) >= r.nx || ((int)by << b) >= r.ny || ((int)bz << b) >= r.nz;
+}
+
 // Status of brick `brick` of 16^3 cells from its statistics (st, as k_brick_stats): 1 if none of
 // its cells inside the grid is a source and each of them a target, 2 if none is selected (a brick
 // outside the grid has none), 0 if the cells must be read.  The comparisons are those of the
@@ -402,9 +413,7 @@ __global__ void __launch_bounds__(STAT_T) k_brick_stats(SelRule r, const float *
 // and the emit pass 58, now 8 and 38.
 __device__ __forceinline__ int brick_mode(const SelRule &r, uint32_t brick, float4 st, float thr_q, float thr_e,
                                           bool qpos) {
-    uint32_t bx, by, bz;
-    demorton3(brick, bx, by, bz);
-    if (((int)bx << 4) >= r.nx || ((int)by << 4) >= r.ny || ((int)bz << 4) >= r.nz) return 2;
+    if (brick_outside(r, brick)) return 2;
     if (r.src_all || (qpos && st.x >= thr_q)) return 0;       // a source in the brick
     if (r.trg_mode == 0) return 1;
     if (r.trg_mode == 2) return st.y >= 0.5f ? 1 : (st.z < 0.5f ? 2 : 0);   // wholly inside or outside the mask
@@ -647,7 +656,7 @@ __device__ __forceinline__ void cube_emit(uint32_t brick, int b, int tid, int x0
 __device__ __forceinline__ void brick_emit_decided(const SelRule &r, uint32_t brick, int mode, int tid, int x0,
                                                    int y0, int z0, unsigned pt0, uint32_t *__restrict__ trg_key,
                                                    uint32_t *__restrict__ trg_pc, uint8_t *__restrict__ tmask) {
-    if (tmask) {
+    if (tmask && !brick_outside(r, brick)) {
         const uint8_t m = mode == 1 ? 1 : 0;
         if ((r.nx & 15) == 0 && (reinterpret_cast<uintptr_t>(tmask) & 15) == 0 &&
             brick_cells(r, x0, y0, z0) == 4096) {
@@ -717,7 +726,9 @@ __global__ void __launch_bounds__(SEL_T) k_select_onepass(
     if (tid == 0) {
         s_brick = (int)atomicAdd(ticket, 1u);
         block_thresholds(r, maxes, &s_thr_q, &s_thr_e, &s_qpos);
-        s_mode = bstat ? brick_mode(r, (uint32_t)s_brick, bstat[s_brick], s_thr_q, s_thr_e, s_qpos) : 0;
+        // 1024 x 1 x 1 cells, 64 of 262,144 bricks inside: 4.4 ms with all of them gone through, 2.8 so
+        s_mode = bstat ? brick_mode(r, (uint32_t)s_brick, bstat[s_brick], s_thr_q, s_thr_e, s_qpos)
+                       : (brick_outside(r, (uint32_t)s_brick) ? 2 : 0);
         if (s_mode == 1) {                         // targets of a brick that reaches past the grid: ranked below
             uint32_t ux, uy, uz;
             demorton3((uint32_t)s_brick, ux, uy, uz);
@@ -914,8 +925,11 @@ int select_launch(const SelectArgs &A, cudaStream_t st) {
     // one pass over bricks of 16^3 cells: the maxima with the per-brick statistics
     const bool stats = !A.two_pass && A.bstat != nullptr && b == 4 && (gq || ge);
     const float4 *bstat = reinterpret_cast<const float4 *>(A.bstat);
-    if (stats) launch_pdl(k_brick_stats, nbr, STAT_T, 0, st, r, gq, ge, (const uint8_t *)(r.trg_mode == 2 ? A.mask : nullptr),
-                          reinterpret_cast<float4 *>(A.bstat), A.maxes);
+    if (stats && r.trg_mode == 2)
+        launch_pdl(k_brick_stats<true>, nbr, STAT_T, 0, st, r, gq, ge, A.mask, reinterpret_cast<float4 *>(A.bstat), A.maxes);
+    else if (stats)
+        launch_pdl(k_brick_stats<false>, nbr, STAT_T, 0, st, r, gq, ge, (const uint8_t *)nullptr,
+                   reinterpret_cast<float4 *>(A.bstat), A.maxes);
     else if (gq || ge) launch_pdl(k_grid_max, gm, 256, 0, st, gq, ge, n, A.maxes);
     A.launched = (stats || gq || ge) ? 1 : 0;
     if (A.two_pass) {
