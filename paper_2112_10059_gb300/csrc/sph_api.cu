@@ -986,7 +986,6 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
             else fmm_l2l_gemm_level(F, l, c->lvl_base[l - 1], c->lvl_count[l - 1], c->stream);
             c->launches += c->lvl_count[l - 1] > 0;
         }
-        if (S.tc && !err_mapped) CK(cudaMemcpyAsync(c->pinned + 48, S.err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
         c->tc_used = S.tc;
     }
     if (tm) tm->mark_at(7, c->stream);
@@ -1036,8 +1035,6 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
                 ++c->launches;
             }
         }
-        if (l2p_tc && !err_mapped)
-            CK(cudaMemcpyAsync(c->pinned + 49, S.err + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
         c->l2p_tc_used = l2p_tc;
     }
     if (near_fork) CK(cudaEventRecord(c->near_join, c->near_stream));
@@ -1066,6 +1063,8 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
         fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->stream);
         c->launches += nb > 0;
     }
+    // after the near stream has joined: its matrix form sets the tiles' flag too
+    if (S.tc && !err_mapped) CK(cudaMemcpyAsync(c->pinned + 48, S.err, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     if (tm) tm->mark_at(9, c->stream);
     CK(cudaGetLastError());
     return SPH_OK;
