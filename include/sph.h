@@ -209,7 +209,8 @@ int eval_sph_host(sph_ctx *ctx, const float *q_host, const float *emag_host,
 
 /* Direct sum of Eq. summation over the same selected sets (no FMM):
  * fp64 == 0 writes float[nx*ny*nz] in FP32 arithmetic, fp64 == 1 writes
- * double[nx*ny*nz] in FP64 arithmetic.  0 at non-targets. */
+ * double[nx*ny*nz] in FP64 arithmetic, each term added with its rounding error kept
+ * (compensated summation).  0 at non-targets. */
 int eval_direct(sph_ctx *ctx, int fp64, void *s_dev);
 
 /* Selected sets of the last eval: canonical ascending linear indices.

@@ -232,6 +232,22 @@ __device__ __forceinline__ void neumaier(double &acc, double &comp, double term)
     acc = s;
 }
 
+// acc + comp += w q for w >= 0, the product unrounded.  eq: the biased exponent of q, less 1020.  Where |w q|
+// is at most half of |acc| by the exponents, acc and the fused sum are so close that their difference
+// is exact and one more FMA forms what the sum lost; the first terms, and one much larger than all
+// before it, go by Neumaier's rule with the product's own rounding error.
+__device__ __forceinline__ void add_product(double &acc, double &comp, double w, double q, int eq) {
+    if ((__double2hiint(w) >> 20) + eq <= (__double2hiint(acc) >> 20 & 0x7ff)) {
+        const double s = fma(w, q, acc);
+        comp += fma(w, q, acc - s);
+        acc = s;
+    } else {
+        const double t = w * q;
+        comp += fma(w, q, -t);
+        neumaier(acc, comp, t);
+    }
+}
+
 __global__ void k_pair_table(KParams64 kp, int self_mode, int entries, double *__restrict__ table) {
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < entries; d += gridDim.x * blockDim.x)
         table[d] = pair_weight(d, kp, self_mode);
@@ -240,10 +256,12 @@ __global__ void k_pair_table(KParams64 kp, int self_mode, int entries, double *_
 // On the grid a pair's weight depends on the integer d2 alone, so it is read from a table built
 // for the call (the same arithmetic) instead of two exponentials, a root and a division in FP64
 // per pair, about 250 instructions at 2 per SM and clock.  What is left is bound by the FP64 unit
-// too: one FMA a pair and one compensated addition per 16 (error against extended
-// precision as with one per pair: 1.8e-16 rms at 24^3, either way).  32 targets per CTA; its eight warps
-// take an eighth of each source tile and their sums are added in order.
-// 24^3 cells, all pairs (1.9e8): 68.6 ms with G per pair, 0.64 ms so.
+// too: two FMAs and two additions a pair, each product compensated (this is the library's own
+// reference: with one compensated addition per 16 products, 1.4 operations a pair, the rms error of
+// a sum of weights of both signs was 4.0e-15, of positive ones over twelve decades 6.0e-17; each for
+// itself, as pair by pair, 2.2e-15 and 5.1e-17, and with the products unrounded a tenth less).  32 targets per CTA; its eight warps take an
+// eighth of each source tile and their sums are added in order.
+// 24^3 cells, all pairs (1.9e8): 68.6 ms with G per pair, 0.64 with groups of 16, 1.5 ms so.
 constexpr int DW = 8;            // warps per CTA
 constexpr int DT64 = 512;        // sources per tile
 constexpr int TABLE_SMEM = 12288;   // entries of a table kept in shared memory (96 KB)
@@ -271,32 +289,17 @@ __global__ void __launch_bounds__(32 * DW) k_direct_f64_table(const uint32_t *__
         __syncthreads();
         for (int u = threadIdx.x; u < m; u += 32 * DW) {
             const uint32_t p = src_pc[s0 + u];
-            sp[u] = make_int4(pc_i(p), pc_j(p), pc_k(p), 0);
-            sq[u] = (double)src_q[s0 + u];
+            const double q = (double)src_q[s0 + u];
+            sp[u] = make_int4(pc_i(p), pc_j(p), pc_k(p), (__double2hiint(q) >> 20 & 0x7ff) - 1020);
+            sq[u] = q;
         }
         __syncthreads();
         const int u1 = min(m, (warp + 1) * (DT64 / DW));
-        for (int u = warp * (DT64 / DW); u < u1; u += 16) {
-            double c;
-            if (u + 16 <= u1) {
-                double c4[4];                  // four short chains, added in pairs: a rounding depth of 6
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int4 p = sp[u + j];
-                    const int di = ti - p.x, dj = tj - p.y, dk = tk - p.z;
-                    const double w = tab[di * di + dj * dj + dk * dk];
-                    c4[j & 3] = j < 4 ? w * sq[u + j] : fma(w, sq[u + j], c4[j & 3]);
-                }
-                c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
-            } else {
-                c = 0.0;
-                for (int j = u; j < u1; ++j) {
-                    const int4 p = sp[j];
-                    const int di = ti - p.x, dj = tj - p.y, dk = tk - p.z;
-                    c = fma(tab[di * di + dj * dj + dk * dk], sq[j], c);
-                }
-            }
-            neumaier(acc, comp, c);
+#pragma unroll 4
+        for (int u = warp * (DT64 / DW); u < u1; ++u) {
+            const int4 p = sp[u];
+            const int di = ti - p.x, dj = tj - p.y, dk = tk - p.z;
+            add_product(acc, comp, tab[di * di + dj * dj + dk * dk], sq[u], p.w);
         }
     }
     part[warp][lane][0] = acc;

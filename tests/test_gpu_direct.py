@@ -64,3 +64,36 @@ def test_direct_forms(sph, case):
     tol = J.size * 2.0 ** -24 + 8e-6
     assert np.max(np.abs(d32[S] / ref - 1)) < tol
     assert np.all(d32[off] == 0)
+
+
+@pytest.mark.parametrize("shape", [(16, 16, 16), (200, 9, 9)])     # weights in shared and in global memory
+def test_fp64_sums_keep_what_large_terms_of_both_signs_cancel(sph, shape):
+    """Weights +Q and -Q in cells opposite each other across the target cancel exactly, as their terms
+    are the same product: what is left is the sum of the others, 1e-12 of the size.  A sum that adds
+    several products before it compensates rounds them at the size of the largest, 1e-16 Q: 1e-5 of
+    the result.  Compensated one by one the bound is that of the other sums here."""
+    import torch
+    nx, ny, nz = shape
+    cx, cy, cz = nx // 2, ny // 2, nz // 2
+    small = si.uniform01(91, nx * ny * nz).astype(np.float32).reshape(nz, ny, nx) + np.float32(0.5)
+    small[cz, cy, cx] = 0.0
+    q = small.copy()
+    for k, (dx, dy, dz) in enumerate([(1, 0, 0), (2, 0, 0), (0, 1, 0), (0, 2, 1), (3, 1, 0)]):
+        for s in (1, -1):
+            small[cz + s * dz, cy + s * dy, cx + s * dx] = 0.0
+            q[cz + s * dz, cy + s * dy, cx + s * dx] = s * 1e12 / (k + 1)
+    mask = np.zeros((nz, ny, nx), np.uint8)
+    mask[cz, cy, cx] = 1
+    t = np.nonzero(mask.reshape(-1))[0].astype(np.int32)
+    h, pO2 = 0.01, si.pO2_of(760.0)
+    ctx = sph.Context(0)
+    sph.set_grid(ctx, nx, ny, nz, h, pO2)
+    qd, md = torch.from_numpy(q.reshape(-1)).cuda(), torch.from_numpy(mask.reshape(-1)).cuda()
+    sph.set_sources(ctx, qd, 1.0)
+    sph.set_targets(ctx, mask=md)
+    sph.set_criteria(ctx, 0.0)
+    d64 = sph.eval_direct(ctx, fp64=True).cpu().numpy()[t]
+    ctx.close()
+    alpha, beta = oracle.alpha_beta(pO2, 0.035, 2.0)
+    ref = oracle.sph(nx, ny, nz, h, alpha, beta, small.reshape(-1), 1.0, np.nonzero(small.reshape(-1))[0].astype(np.int32), t)
+    assert np.abs(d64 / ref - 1) < 1e-13
