@@ -64,9 +64,11 @@ struct DirectK {
     float bma_h;        // (beta - alpha) h
 };
 
-// G h^3 / C at squared distance d2 >= 1 (cells), for any R: both forms of 1 - e^{-x} and a selection,
-// so that the pairs of a chunk overlap (one_minus_exp_neg branches)
-__device__ __forceinline__ float general_g(float d2, const DirectK &k) {
+// w G h^3 / C at squared distance d2 >= 1 (cells), for any R: both forms of 1 - e^{-x} and a selection,
+// so that the pairs of a chunk overlap (one_minus_exp_neg branches).  Here and in the loops below
+// the weight multiplies the exponential first: e^{-alpha R} / R^3 by itself has lost bits to FP32's
+// smallest exponents at alpha R = 66 and a thousand cells, where w G has not.
+__device__ __forceinline__ float general_g(float d2, float w, const DirectK &k) {
     const float ir = rsqrt_approx(d2), R = d2 * ir, x = k.bma_h * R;
     float p = -2.4801587301587302e-05f;            // x (1 - x/2! + x^2/3! - ... - x^7/8!)
     p = fmaf(p, x, 1.9841269841269841e-04f);
@@ -77,7 +79,7 @@ __device__ __forceinline__ float general_g(float d2, const DirectK &k) {
     p = fmaf(p, x, -0.5f);
     p = fmaf(p, x, 1.0f) * x;
     const float em = x < 0.5f ? p : 1.f - ex2_approx(-k.b2 * R);
-    return ex2_approx(-k.a2 * R) * em * (ir * ir * ir);
+    return ex2_approx(-k.a2 * R) * w * em * (ir * ir * ir);
 }
 
 constexpr int WARPS = 4;
@@ -151,8 +153,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_direct_f32(const uint32_t *__res
                     const float2 dd = f2_get(d);
                     const F2 ir = f2(rsqrt_approx(dd.x), rsqrt_approx(dd.y));
                     const float2 e = f2_get(f2_mul(a2, f2_mul(d, ir)));
-                    const F2 g = f2_mul(f2(ex2_approx(e.x), ex2_approx(e.y)), f2_mul(f2_mul(ir, ir), ir));
-                    acc = f2_fma(g, f2(sw[u].x, sw[u].y), acc);
+                    const F2 ew = f2_mul(f2(ex2_approx(e.x), ex2_approx(e.y)), f2(sw[u].x, sw[u].y));
+                    acc = f2_fma(ew, f2_mul(f2_mul(ir, ir), ir), acc);
                 }
             } else if (g2 >= k.near2) {
 #pragma unroll 4
@@ -163,16 +165,17 @@ __global__ void __launch_bounds__(32 * WARPS) k_direct_f32(const uint32_t *__res
                     const F2 R = f2_mul(d, ir);
                     const float2 e = f2_get(f2_mul(a2, R)), q = f2_get(f2_mul(b2, R));
                     const F2 m1 = f2(1.f - ex2_approx(q.x), 1.f - ex2_approx(q.y));
-                    const F2 g = f2_mul(f2_mul(f2(ex2_approx(e.x), ex2_approx(e.y)), m1), f2_mul(f2_mul(ir, ir), ir));
-                    acc = f2_fma(g, f2(sw[u].x, sw[u].y), acc);
+                    const F2 ew = f2_mul(f2(ex2_approx(e.x), ex2_approx(e.y)), f2(sw[u].x, sw[u].y));
+                    acc = f2_fma(f2_mul(ew, m1), f2_mul(f2_mul(ir, ir), ir), acc);
                 }
             } else {
 #pragma unroll 4
                 for (int u = c; u < end; ++u) {
                     const float2 dd = f2_get(dist2(u));
-                    const float ga = dd.x > 0.f ? general_g(fmaxf(dd.x, 1.f), k) : k.self;
-                    const float gb = dd.y > 0.f ? general_g(fmaxf(dd.y, 1.f), k) : k.self;
-                    acc = f2_fma(f2(ga, gb), f2(sw[u].x, sw[u].y), acc);
+                    const float w = sw[u].x;
+                    const float ta = dd.x > 0.f ? general_g(fmaxf(dd.x, 1.f), w, k) : k.self * w;
+                    const float tb = dd.y > 0.f ? general_g(fmaxf(dd.y, 1.f), w, k) : k.self * w;
+                    acc = f2_add(acc, f2(ta, tb));
                 }
             }
         }
@@ -206,7 +209,7 @@ __global__ void __launch_bounds__(128) k_direct_f32_few(const uint32_t *__restri
         for (int u = 0; u < m; ++u) {
             const float4 p = sp[u];
             const float dx = tx - p.x, dy = ty - p.y, dz = tz - p.z, d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            acc = fmaf(d2 > 0.f ? general_g(fmaxf(d2, 1.f), k) : k.self, p.w, acc);
+            acc += d2 > 0.f ? general_g(fmaxf(d2, 1.f), p.w, k) : k.self * p.w;
         }
     }
     if (t < nt) out_dense[(int64_t)pc_i(tp) + (int64_t)nx * ((int64_t)pc_j(tp) + (int64_t)ny * pc_k(tp))] = acc;

@@ -97,3 +97,28 @@ def test_fp64_sums_keep_what_large_terms_of_both_signs_cancel(sph, shape):
     alpha, beta = oracle.alpha_beta(pO2, 0.035, 2.0)
     ref = oracle.sph(nx, ny, nz, h, alpha, beta, small.reshape(-1), 1.0, np.nonzero(small.reshape(-1))[0].astype(np.int32), t)
     assert np.abs(d64 / ref - 1) < 1e-13
+
+
+@pytest.mark.parametrize("ny,nz", [(3, 3), (12, 12)])     # one target a thread; pairs of targets
+def test_fp32_terms_of_strongly_absorbed_sources(sph, ny, nz):
+    """Sources at one end of 1024 cells of 0.0135 cm at atmospheric pressure: at the other end alpha R
+    is 72 and e^{-alpha R} / d^3 in cells 5e-41, below FP32's normal range, while S = w G stays far above
+    it.  The bound is that of the exponential's argument (105 in log2 units, 2^-24 of it, and the
+    constants' rounding) and of 20 FP32 additions."""
+    import torch
+    nx, h, pO2 = 1024, 0.0135, 150.0
+    q = np.zeros((nz, ny, nx), np.float32)
+    q[:, :, 0] = 1.0 + np.arange(ny * nz, dtype=np.float32).reshape(nz, ny) / (ny * nz)
+    ctx = sph.Context(0)
+    sph.set_grid(ctx, nx, ny, nz, h, pO2)
+    qd = torch.from_numpy(q.reshape(-1)).cuda()
+    sph.set_sources(ctx, qd, 1e20)
+    sph.set_targets(ctx)
+    sph.set_criteria(ctx, 0.5)
+    d32 = sph.eval_direct(ctx, fp64=False).cpu().numpy().astype(np.float64)
+    ctx.close()
+    alpha, beta = oracle.alpha_beta(pO2, 0.035, 2.0)
+    T = np.arange(1000, 1024, dtype=np.int32)
+    ref = oracle.sph(nx, ny, nz, h, alpha, beta, q.reshape(-1), 1e20, np.nonzero(q.reshape(-1))[0].astype(np.int32), T)
+    assert np.all(ref > 1e-25)
+    assert np.max(np.abs(d32[T] / ref - 1)) < 2 * 105 * 2.0 ** -24 + q[:, :, 0].size * 2.0 ** -24 + 2e-6
