@@ -1459,7 +1459,7 @@ __global__ void __launch_bounds__(LP_T, 1) k_l2lp_tc(FmmDev F, int level, int pa
 // leaf's cell values (and mask bytes) are read before its contraction, so that a warp's
 // loads overlap its arithmetic instead of following it.
 constexpr int OWN_W = 8;
-__global__ void __launch_bounds__(OWN_W * 32) k_l2p_own(FmmDev F, int level, const int *__restrict__ list,
+__global__ void __launch_bounds__(OWN_W * 32) k_l2p_own(FmmDev F, CellBasis B, int level, const int *__restrict__ list,
                                                         const int *__restrict__ count, float *__restrict__ out) {
     pdl_enter();
     const int cnt = *count;
@@ -1470,17 +1470,7 @@ __global__ void __launch_bounds__(OWN_W * 32) k_l2p_own(FmmDev F, int level, con
     __shared__ float tz[OWN_W][4 * P * P], ty[OWN_W][16 * P];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int np = F.O.npad;
-    if (threadIdx.x < 4 * P) {
-        const int k = threadIdx.x / 4;
-        const float x = (float)(2 * (int)(threadIdx.x & 3) - 3) * 0.25f, tk = F.O.cheb_t[k];
-        float num = 1.f, den = 1.f;
-        for (int j = 0; j < P; ++j)
-            if (j != k) {
-                num *= x - F.O.cheb_t[j];
-                den *= tk - F.O.cheb_t[j];
-            }
-        basis[k][threadIdx.x & 3] = num / den;
-    }
+    if (threadIdx.x < 4 * P) basis[threadIdx.x / 4][threadIdx.x & 3] = B.v[threadIdx.x / 4][threadIdx.x & 3];
     const TreeDev &T = F.T;
     const int stride = gridDim.x * OWN_W;
     int i = blockIdx.x * OWN_W + warp;
@@ -1582,7 +1572,7 @@ void fmm_l2p_own(const FmmDev &F, int level, const int *list, const int *count, 
                  cudaStream_t st) {
     if (max_count <= 0 || F.O.e_off[level] < 0 || F.O.npad > TCK || (1 << (F.D - level)) != 4) return;
     const int grid = std::max(1, std::min((max_count + OWN_W - 1) / OWN_W, 8 * sm_count()));
-    launch_pdl(k_l2p_own, grid, OWN_W * 32, 0, st, F, level, list, count, out);
+    launch_pdl(k_l2p_own, grid, OWN_W * 32, 0, st, F, cheb_cell_basis(), level, list, count, out);
 }
 
 bool tc_supported(const OpsDev &O) { return O.npad == TCK; }

@@ -1,6 +1,7 @@
 // Internal declarations shared by the libsph translation units (not part of the C ABI).
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include "sph_common.cuh"
 
@@ -344,6 +345,26 @@ void fmm_leaf(const FmmDev &F, int nboxes, const int *list, const int *count, fl
 // `level` must be a leaf (level == Lmax).  Replaces fmm_l2l_*_level(level) and the L2P of `level`.
 void fmm_l2lp_tc_level(const FmmDev &F, int level, int parent_begin, int parent_count, float *out, int *err,
                        cudaStream_t st);
+// value of the one-dimensional polynomial of Chebyshev node k (of 5) at cell i of a box of 4 cells, in
+// FP64 and rounded once, like the interpolation tables (formed in FP32 it was off by up to 4.4 units
+// of 2^-24, and the L2P axis by axis further off than by the table: rms 2.6e-7 and 2.0e-7 of random
+// expansions' values, 0.8e-7 so)
+struct CellBasis {
+    float v[5][4];
+};
+inline CellBasis cheb_cell_basis() {
+    CellBasis B;
+    double t[5];
+    for (int k = 0; k < 5; ++k) t[k] = cos((2.0 * k + 1.0) * 3.14159265358979323846 / 10.0);
+    for (int k = 0; k < 5; ++k)
+        for (int i = 0; i < 4; ++i) {
+            double v = 1.0;
+            for (int j = 0; j < 5; ++j)
+                if (j != k) v *= ((2 * i - 3) * 0.25 - t[j]) / (t[k] - t[j]);
+            B.v[k][i] = (float)v;
+        }
+    return B;
+}
 // the L2P of the own local terms of the leaves in list (count[0] <= max_count of them; leaves of
 // edge 4 at `level`), added into out at their targets (FP32); the part of the deepest level's
 // L2P that fmm_l2lp_tc_level leaves out
