@@ -1259,8 +1259,10 @@ __global__ void __launch_bounds__(2 * MAXPAD, 1) k_p2l(FmmDev F, P2PConst K, con
         uint32_t ux, uy, uz;
         demorton3(T.b_key[b], ux, uy, uz);
         const float r = 0.5f * (float)size, rad = F.O.method == FAR_CHEB ? r : (float)F.O.r.dc * r;
-        const float cx = (float)ux * size + r - 0.5f + rad * node.x, cy = (float)uy * size + r - 0.5f + rad * node.y,
-                    cz = (float)uz * size + r - 0.5f + rad * node.z;
+        // cells from the box's lowest one: a source's are whole numbers, a node's round at the box's
+        // size (at the grid's they were 3e-5 cells off at cell 1000, 7e-6 to 4e-5 of a sum)
+        const int bx = (int)ux * size, by = (int)uy * size, bz = (int)uz * size;
+        const float cx = r - 0.5f + rad * node.x, cy = r - 0.5f + rad * node.y, cz = r - 0.5f + rad * node.z;
         float acc = 0.f;
         const int x1 = F.L.x_off[b + 1];
         for (int x0 = F.L.x_off[b]; x0 < x1; x0 += 32) {     // lane k of every warp: entry x0 + k
@@ -1286,7 +1288,7 @@ __global__ void __launch_bounds__(2 * MAXPAD, 1) k_p2l(FmmDev F, P2PConst K, con
                     for (int q = lane; q < me; q += 32)
                         if ((unsigned)(at + q) < (unsigned)PX_CAP) {
                             const uint32_t pc = __ldg(F.src_pc + first + q);
-                            stage[at + q] = make_float4((float)pc_i(pc), (float)pc_j(pc), (float)pc_k(pc),
+                            stage[at + q] = make_float4((float)(pc_i(pc) - bx), (float)(pc_j(pc) - by), (float)(pc_k(pc) - bz),
                                                         __ldg(F.src_q + first + q) * wsc);
                         }
                 }
