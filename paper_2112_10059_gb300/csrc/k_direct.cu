@@ -70,15 +70,7 @@ struct DirectK {
 // smallest exponents at alpha R = 66 and a thousand cells, where w G has not.
 __device__ __forceinline__ float general_g(float d2, float w, const DirectK &k) {
     const float ir = rsqrt_approx(d2), R = d2 * ir, x = k.bma_h * R;
-    float p = -2.4801587301587302e-05f;            // x (1 - x/2! + x^2/3! - ... - x^7/8!)
-    p = fmaf(p, x, 1.9841269841269841e-04f);
-    p = fmaf(p, x, -1.3888888888888889e-03f);
-    p = fmaf(p, x, 8.3333333333333333e-03f);
-    p = fmaf(p, x, -4.1666666666666667e-02f);
-    p = fmaf(p, x, 1.6666666666666667e-01f);
-    p = fmaf(p, x, -0.5f);
-    p = fmaf(p, x, 1.0f) * x;
-    const float em = x < 0.5f ? p : 1.f - ex2_approx(-k.b2 * R);
+    const float em = x < 0.5f ? one_minus_exp_series(x) : 1.f - ex2_approx(-k.b2 * R);
     return ex2_approx(-k.a2 * R) * w * em * (ir * ir * ir);
 }
 

@@ -1010,12 +1010,11 @@ __global__ void k_near_table(P2PConst K, float *tab) {
 }
 
 // list: P2P_CLASSES lists of `stride` slots, count: their lengths; the leaves are taken class
-// by class, the heaviest first.  Passes [pass_lo, pass_hi) of 0 (U list) and 1 (W list).
+// by class, the heaviest first.  Passes: 1 (U lists), or 2 (U and W lists).
 template <bool TAYLOR, bool TABLE>
 __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p(FmmDev F, const int *__restrict__ list,
                                                          const int *__restrict__ count, int stride,
-                                                         float *__restrict__ out, P2PConst K, int pass_lo,
-                                                         int pass_hi) {
+                                                         float *__restrict__ out, P2PConst K, int max_passes) {
     pdl_enter();
     __shared__ float4 stage[P2P_CAP];
     __shared__ float tab[TABLE ? GTAB_N : 1];
@@ -1049,7 +1048,7 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p(FmmDev F, const int *__r
         // the leaf's sums: its slots of the scratch (cleared by the launch that starts with the
         // U list), or the output itself
         float *nslot = F.near_buf ? F.near_buf + (size_t)i * F.near_s : nullptr;
-        if (nslot && pass_lo == 0) {
+        if (nslot) {
             for (int t = tid; t < te - tb; t += blockDim.x) nslot[t] = 0.f;
             __syncthreads();
         }
@@ -1062,11 +1061,11 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p(FmmDev F, const int *__r
         const int k = warp % G;
         float acc[2] = {0.f, 0.f};        // the first two chunks of this warp; further chunks flush per round
         // pass 0: U list (point sources); pass 1: W list (Chebyshev nodes of the W boxes)
-        const int passes = min(pass_hi, F.O.method == FAR_CHEB ? 2 : 1);   // the surface form keeps M2P in k_leaf
+        const int passes = min(max_passes, F.O.method == FAR_CHEB ? 2 : 1);   // the surface form keeps M2P in k_leaf
         // strategy 3 applies to leaves whose every chunk stays in this warp's two sum slots
         const bool skip3 = F.r_s > 0.f && nch <= 2 * groups && F.L.w_off[b + 1] > F.L.w_off[b];
         float sest[2] = {0.f, 0.f};
-        for (int pass = pass_lo; pass < passes; ++pass) {
+        for (int pass = 0; pass < passes; ++pass) {
             const int l0 = pass == 0 ? F.L.u_off[b] : F.L.w_off[b];
             const int l1 = pass == 0 ? F.L.u_off[b + 1] : F.L.w_off[b + 1];
             if (pass == 1 && skip3) {
@@ -1718,24 +1717,20 @@ void fmm_near_table(const FmmDev &F, float *gtab, cudaStream_t st) {
 }
 
 void fmm_p2p(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,
-             cudaStream_t st, int pass_lo, int pass_hi, int per_sm) {
+             cudaStream_t st, int passes, int per_sm) {
     if (nboxes <= 0) return;
     const int cap = 152 * per_sm;
     const int grid = nboxes < cap ? nboxes : cap;
     const P2PConst K = p2p_const(F);
     const bool taylor = K.bma_h < 0.5f, table = F.gtab != nullptr;
     if (!taylor && !table)
-        launch_pdl(k_p2p<false, false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi);
+        launch_pdl(k_p2p<false, false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, passes);
     else if (taylor && !table)
-        launch_pdl(k_p2p<true, false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi);
+        launch_pdl(k_p2p<true, false>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, passes);
     else if (!taylor)
-        launch_pdl(k_p2p<false, true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi);
+        launch_pdl(k_p2p<false, true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, passes);
     else
-        launch_pdl(k_p2p<true, true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, pass_lo,
-                   pass_hi);
+        launch_pdl(k_p2p<true, true>, grid, P2P_WARPS * 32, 0, st, F, p2p_list, p2p_cnt, stride, out, K, passes);
 }
 
 void fmm_near_add(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,

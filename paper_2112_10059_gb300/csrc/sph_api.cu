@@ -894,7 +894,7 @@ int fmm_queue(sph_ctx *c, PassState &S, float *out, PhaseTimer *tm) {
         if (tm) tm->mark_at(12, c->near_stream);
         const bool by_offsets = near_by_offsets(c, F);
         if (!by_offsets)
-            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->near_stream, 0, 1, near_cap(c, by_offsets));
+            fmm_p2p(F, nb, S.w_p2p, S.w_cnt + 55, std::max(nb, 1), out, c->near_stream, 1, near_cap(c, by_offsets));
         else {
             const int L = F.near_mma_level, row0 = L >= 0 ? c->lvl_base[L] : 0;
             int *near_max = S.w_cnt + 33;
@@ -2170,7 +2170,6 @@ int eval_direct(sph_ctx *c, int fp64, void *s_dev) {
     A.ns = (int)c->ns;
     A.trg_key = P<uint32_t>(c->b_tkey);
     A.nt = (int)c->nt;
-    A.kp = make_kp(c);
     double L = std::log(c->beta / c->alpha);
     A.kp64.alpha = c->alpha; A.kp64.bma = c->beta - c->alpha; A.kp64.C = 1.0 / (4.0 * M_PI * L);
     A.kp64.h = c->h; A.kp64.vol = c->h * c->h * c->h; A.kp64.scale = c->source_scale;

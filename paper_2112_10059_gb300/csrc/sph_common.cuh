@@ -126,20 +126,23 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     return y;
 }
 
+// 1 - e^{-x} for 0 <= x < 1/2, by its series
+__device__ __forceinline__ float one_minus_exp_series(float x) {
+    // Horner form of x * (1 - x/2 + x^2/6 - x^3/24 + x^4/120 - x^5/720 + x^6/5040 - x^7/40320)
+    float p = -2.4801587301587302e-05f;            // -1/40320
+    p = fmaf(p, x, 1.9841269841269841e-04f);       //  1/5040
+    p = fmaf(p, x, -1.3888888888888889e-03f);      // -1/720
+    p = fmaf(p, x, 8.3333333333333333e-03f);       //  1/120
+    p = fmaf(p, x, -4.1666666666666667e-02f);      // -1/24
+    p = fmaf(p, x, 1.6666666666666667e-01f);       //  1/6
+    p = fmaf(p, x, -0.5f);
+    p = fmaf(p, x, 1.0f);
+    return p * x;
+}
+
 // 1 - e^{-x} for x >= 0.
 __device__ __forceinline__ float one_minus_exp_neg(float x, float x_log2e) {
-    if (x < 0.5f) {
-        // Horner form of x * (1 - x/2 + x^2/6 - x^3/24 + x^4/120 - x^5/720 + x^6/5040 - x^7/40320)
-        float p = -2.4801587301587302e-05f;            // -1/40320
-        p = fmaf(p, x, 1.9841269841269841e-04f);       //  1/5040
-        p = fmaf(p, x, -1.3888888888888889e-03f);      // -1/720
-        p = fmaf(p, x, 8.3333333333333333e-03f);       //  1/120
-        p = fmaf(p, x, -4.1666666666666667e-02f);      // -1/24
-        p = fmaf(p, x, 1.6666666666666667e-01f);       //  1/6
-        p = fmaf(p, x, -0.5f);
-        p = fmaf(p, x, 1.0f);
-        return p * x;
-    }
+    if (x < 0.5f) return one_minus_exp_series(x);
     return 1.0f - ex2_approx(-x_log2e);
 }
 

@@ -55,7 +55,6 @@ struct DirectArgs {
     int ns;
     const uint32_t *trg_key;         // Morton keys of the targets (cells by key_pc)
     int nt;
-    KParams kp;
     KParams64 kp64;
     int self_mode, nx, ny, fp64;
     void *out;
@@ -292,12 +291,11 @@ constexpr int64_t P2P_CLASS0 = 1 << 16;
 void fmm_work_lists(const FmmDev &F, int nboxes, int *src_list, int *src_cnt, int *leaf_list, int *leaf_cnt,
                     int *p2p_list, int *p2p_cnt, int p2p_stride, int *own_list, int *own_cnt, cudaStream_t st,
                     int *w_list, int *w_cnt, int *x_list, int *x_cnt);
-// near field over the U lists (pass 0) and W lists (pass 1) of the leaves in the class lists of
-// p2p_list, passes [pass_lo, pass_hi); adds into out, or into F.near_buf where it is set (pass 0
-// clears the leaf's slots; a launch of pass 1 alone must follow the one of pass 0).  At most
-// per_sm CTAs per SM (grid-stride over the leaves).
+// near field pair by pair over the U lists (passes 1), or the U and W lists (2), of the leaves in the
+// class lists of p2p_list; adds into out, or into F.near_buf where it is set (after clearing the
+// leaf's slots).  At most per_sm CTAs per SM (grid-stride over the leaves).
 void fmm_p2p(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, float *out,
-             cudaStream_t st, int pass_lo = 0, int pass_hi = 2, int per_sm = 16);
+             cudaStream_t st, int passes = 2, int per_sm = 16);
 // the U-list part into the leaves' slots of F.near_buf by the offset table, for the same lists
 // (class P2P_MMA is left out unless the weights' maximum near_max is outside fmm_near_mma's range)
 void fmm_near_grid(const FmmDev &F, int nboxes, const int *p2p_list, const int *p2p_cnt, int stride, const int *near_max,
