@@ -20,7 +20,9 @@ namespace sph {
 //   - far: e^{-(beta - alpha) R} < 2^-25, so that 1 - it is 1 in FP32 and its ex2 is left out;
 //   - near: both exponentials;
 //   - general: the boxes meet (a source may be the target's own cell) or R is small enough for
-//     the series form of 1 - e^{-x} (general_g, pair by pair).
+//     the series form of 1 - e^{-x} (general_term, pair by pair).
+// A chunk is summed by itself before it joins a target's sum: in one chain the error grows with the
+// sources (1,309 of them: 5e-6 of S, 2e-7 so).
 // 160^3 cells, 7,072 sources (2.9e10 pairs): 28.2 ms pair by pair with integer offsets (their
 // conversion is a fourth result of the same unit), 10.5 ms so.
 constexpr int DS = 256;    // sources per shared-memory tile
@@ -64,14 +66,16 @@ struct DirectK {
     float bma_h;        // (beta - alpha) h
 };
 
-// w G h^3 / C at squared distance d2 >= 1 (cells), for any R: both forms of 1 - e^{-x} and a selection,
-// so that the pairs of a chunk overlap (one_minus_exp_neg branches).  Here and in the loops below
-// the weight multiplies the exponential first: e^{-alpha R} / R^3 by itself has lost bits to FP32's
-// smallest exponents at alpha R = 66 and a thousand cells, where w G has not.
-__device__ __forceinline__ float general_g(float d2, float w, const DirectK &k) {
-    const float ir = rsqrt_approx(d2), R = d2 * ir, x = k.bma_h * R;
+// A term w G h^3 / C of squared distance d2 (cells; 0: the self term) as the product of a and b, for any
+// R: both forms of 1 - e^{-x} and selections, so that the pairs of a chunk overlap (one_minus_exp_neg
+// branches).  Here and in the loops below the weight multiplies the exponential first:
+// e^{-alpha R} / R^3 by itself has lost bits to FP32's smallest exponents at alpha R = 66 and a thousand
+// cells, where w G has not.
+__device__ __forceinline__ void general_term(float d2, float w, const DirectK &k, float &a, float &b) {
+    const float ir = rsqrt_approx(fmaxf(d2, 1.f)), R = fmaxf(d2, 1.f) * ir, x = k.bma_h * R;
     const float em = x < 0.5f ? one_minus_exp_series(x) : 1.f - ex2_approx(-k.b2 * R);
-    return ex2_approx(-k.a2 * R) * w * em * (ir * ir * ir);
+    a = d2 > 0.f ? ex2_approx(-k.a2 * R) * w * em : k.self;
+    b = d2 > 0.f ? ir * ir * ir : w;
 }
 
 constexpr int WARPS = 4;
@@ -138,6 +142,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_direct_f32(const uint32_t *__res
                 d = f2_fma(ty, f2(xy.z, xy.w), d);
                 return f2_fma(tz, f2(zs.x, zs.y), d);
             };
+            F2 part = f2(0.f, 0.f);            // a chunk by itself, then into the sum
             if (g2 >= k.far2) {                // uniform over the warp, as every choice here
 #pragma unroll 4
                 for (int u = c; u < end; ++u) {
@@ -146,7 +151,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_direct_f32(const uint32_t *__res
                     const F2 ir = f2(rsqrt_approx(dd.x), rsqrt_approx(dd.y));
                     const float2 e = f2_get(f2_mul(a2, f2_mul(d, ir)));
                     const F2 ew = f2_mul(f2(ex2_approx(e.x), ex2_approx(e.y)), f2(sw[u].x, sw[u].y));
-                    acc = f2_fma(ew, f2_mul(f2_mul(ir, ir), ir), acc);
+                    part = f2_fma(ew, f2_mul(f2_mul(ir, ir), ir), part);
                 }
             } else if (g2 >= k.near2) {
 #pragma unroll 4
@@ -158,18 +163,19 @@ __global__ void __launch_bounds__(32 * WARPS) k_direct_f32(const uint32_t *__res
                     const float2 e = f2_get(f2_mul(a2, R)), q = f2_get(f2_mul(b2, R));
                     const F2 m1 = f2(1.f - ex2_approx(q.x), 1.f - ex2_approx(q.y));
                     const F2 ew = f2_mul(f2(ex2_approx(e.x), ex2_approx(e.y)), f2(sw[u].x, sw[u].y));
-                    acc = f2_fma(f2_mul(ew, m1), f2_mul(f2_mul(ir, ir), ir), acc);
+                    part = f2_fma(f2_mul(ew, m1), f2_mul(f2_mul(ir, ir), ir), part);
                 }
             } else {
 #pragma unroll 4
                 for (int u = c; u < end; ++u) {
                     const float2 dd = f2_get(dist2(u));
-                    const float w = sw[u].x;
-                    const float ta = dd.x > 0.f ? general_g(fmaxf(dd.x, 1.f), w, k) : k.self * w;
-                    const float tb = dd.y > 0.f ? general_g(fmaxf(dd.y, 1.f), w, k) : k.self * w;
-                    acc = f2_add(acc, f2(ta, tb));
+                    float a0, a1, b0, b1;
+                    general_term(dd.x, sw[u].x, k, a0, b0);
+                    general_term(dd.y, sw[u].y, k, a1, b1);
+                    part = f2_fma(f2(a0, a1), f2(b0, b1), part);
                 }
             }
+            acc = f2_add(acc, part);
         }
     }
     const float2 r = f2_get(acc);
@@ -197,11 +203,18 @@ __global__ void __launch_bounds__(128) k_direct_f32_few(const uint32_t *__restri
             sp[u] = make_float4((float)pc_i(p), (float)pc_j(p), (float)pc_k(p), src_q[s0 + u] * k.wscale);
         }
         __syncthreads();
+        for (int c = 0; c < m; c += DC) {
+            const int end = min(c + DC, m);
+            float part = 0.f;
 #pragma unroll 4
-        for (int u = 0; u < m; ++u) {
-            const float4 p = sp[u];
-            const float dx = tx - p.x, dy = ty - p.y, dz = tz - p.z, d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            acc += d2 > 0.f ? general_g(fmaxf(d2, 1.f), p.w, k) : k.self * p.w;
+            for (int u = c; u < end; ++u) {
+                const float4 p = sp[u];
+                const float dx = tx - p.x, dy = ty - p.y, dz = tz - p.z, d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                float a, b;
+                general_term(d2, p.w, k, a, b);
+                part = fmaf(a, b, part);
+            }
+            acc += part;
         }
     }
     if (t < nt) out_dense[(int64_t)pc_i(tp) + (int64_t)nx * ((int64_t)pc_j(tp) + (int64_t)ny * pc_k(tp))] = acc;

@@ -122,3 +122,34 @@ def test_fp32_terms_of_strongly_absorbed_sources(sph, ny, nz):
     ref = oracle.sph(nx, ny, nz, h, alpha, beta, q.reshape(-1), 1e20, np.nonzero(q.reshape(-1))[0].astype(np.int32), T)
     assert np.all(ref > 1e-25)
     assert np.max(np.abs(d32[T] / ref - 1)) < 2 * 105 * 2.0 ** -24 + q[:, :, 0].size * 2.0 ** -24 + 2e-6
+
+
+@pytest.mark.parametrize("ft", [0.01, 1.0])     # one target a thread; pairs of targets
+def test_fp32_sums_of_many_small_terms_behind_a_large_one(sph, ft):
+    """A source of weight 1, the first in Morton order, and 16,383 of 3e-8: at targets as far from all of
+    them each small term is below half a unit in the last place of the sum, and one chain loses them all,
+    up to 5e-4 of it.  32 terms are summed at a time, and the sums of the chunks: 32 + 16384 / 32
+    roundings of 2^-24 one after another, whose errors add as squares, and 1e-6 at most for the
+    approximate root and exponentials of a term (2^-22.9, cubed, and 2^-22.5)."""
+    import torch
+    nx, ny, nz, h, pO2 = 64, 64, 32, 1e-3, 150.0
+    n = nx * ny * nz
+    q = np.zeros((nz, ny, nx), np.float32)
+    q[:16, :32, :32] = 3e-8 * (0.75 + 0.25 * si.uniform01(93, 16384).reshape(16, 32, 32))
+    q[0, 0, 0] = 1.0
+    mask = (si.uniform01(94, n) <= ft).astype(np.uint8)
+    ctx = sph.Context(0)
+    sph.set_grid(ctx, nx, ny, nz, h, pO2)
+    qd, md = torch.from_numpy(q.reshape(-1)).cuda(), torch.from_numpy(mask).cuda()
+    sph.set_sources(ctx, qd, 1.0)
+    sph.set_targets(ctx, mask=md)
+    sph.set_criteria(ctx, 1e-9)
+    d32 = sph.eval_direct(ctx, fp64=False).cpu().numpy().astype(np.float64)
+    ctx.close()
+    T = np.nonzero(mask)[0].astype(np.int32)
+    T = T[(T % nx >= 40) & (T // nx % ny >= 40)]
+    T = T[:: max(1, T.size // 500)]
+    J = np.nonzero(q.reshape(-1))[0].astype(np.int32)
+    alpha, beta = oracle.alpha_beta(pO2, 0.035, 2.0)
+    ref = oracle.sph(nx, ny, nz, h, alpha, beta, q.reshape(-1), 1.0, J, T)
+    assert np.sqrt(np.mean((d32[T] / ref - 1) ** 2)) < 2.0 ** -24 * np.sqrt(32 + J.size / 32) + 1e-6
