@@ -173,7 +173,7 @@ def measured_peaks():
 # DRAM bytes (read + write) per launch from one ncu capture each of the 256^3 adaptive workload
 # (dram__bytes_read.sum + dram__bytes_write.sum of the kernel); valid for that workload and the
 # kernels as profiled (removed once a kernel has changed since).
-NCU_TRAFFIC = {"m2l": (97.748 + 2.976) * 1e6, "l2lp": (26.381 + 9.930) * 1e6}
+NCU_TRAFFIC = {"m2l": (97.751 + 3.248) * 1e6, "l2lp": (26.255 + 9.648) * 1e6}
 
 
 def pipe_peaks(sph, dev, stream, f_mhz_nominal=2070.0):
@@ -190,7 +190,7 @@ def pipe_peaks(sph, dev, stream, f_mhz_nominal=2070.0):
                 "source": "nominal (measurement failed: %s)" % e}
 
 
-def rooflines(tree, step_stats, args, nt, ns, ncell, peaks, pipes, traffic_ok=True, order=None):
+def rooflines(tree, step_stats, args, nt, ns, ncell, peaks, pipes, traffic_ok=True, order=None, near_kernels="k_p2p"):
     """Achieved vs peak per kernel.  Work is ALGORITHMIC (what the method needs), not executed:
       m2l  (tensor, k_m2l_tc): 2 n^2 flops per V pair, n = order^3 (the BF16 x3 split executes
                      3 x 2 x 128^2);
@@ -202,10 +202,11 @@ def rooflines(tree, step_stats, args, nt, ns, ncell, peaks, pipes, traffic_ok=Tr
                   have V or X entries read (npad x 4 B each) with S read and written at their
                   targets (8 B per target), and the other levels' leaves (npad x 4 B per leaf
                   with targets + 4 B per target written) -- only where such leaves exist;
-      near (k_near_grid, k_near_mma, k_near_w): P2P pairs + M2P evaluations against the measured
-                  ex2 and rsqrt rates at 2 ex2 + 1 rsqrt each; an offset table and matrix products
-                  stand for most pairs' evaluations, so the fraction may pass 1;
-      select (HBM, k_brick_stats + k_select_onepass): 8 B per cell (q and |E| read once) + 4 B
+      near (near_kernels: k_p2p where the near field was timed after the far field): P2P pairs +
+                  M2P evaluations against the measured ex2 and rsqrt rates at 2 ex2 + 1 rsqrt each;
+                  beside the far field an offset table and matrix products stand for most pairs'
+                  evaluations, and the fraction may pass 1;
+      select (HBM, k_brick_stats + k_select_count + k_scan2 + k_select_emit): 8 B per cell (q and |E| read once) + 4 B
                   per selected index (sources and targets) -- the minimum of the operation: the
                   maxima pass reads every cell, the rules re-read only the bricks that the
                   maxima pass's per-brick statistics leave undecided.
@@ -276,10 +277,10 @@ def rooflines(tree, step_stats, args, nt, ns, ncell, peaks, pipes, traffic_ok=Tr
             "k_l2p_sep_small + k_l2p_sep", False, "hbm",
             4.0 * npad * (n_leaf_t + n_deep) + 4.0 * nt_other + 8.0 * nt_own, "bytes", med("ms_l2p") - ms_lp, hbm,
             "GB/s", hbm_basis)
-    add("near", "k_near_grid + k_near_mma + k_near_w", False, "alu", float(p2p + m2p), "kernel-evals", med("ms_near"), mufu_evals, "evals/s",
+    add("near", near_kernels, near_kernels == "k_p2p", "alu", float(p2p + m2p), "kernel-evals", med("ms_near"), mufu_evals, "evals/s",
         "MUFU: 2 ex2 + 1 rsqrt per evaluation at the measured %.3g ex2/s and %.3g rsqrt/s (%s)"
         % (pipes["ex2_per_s"], pipes["rsqrt_per_s"], pipes["source"]))
-    add("select", "k_brick_stats + k_select_onepass", False, "hbm", 8.0 * ncell + 4.0 * (nt + ns),
+    add("select", "k_brick_stats + k_select_count + k_scan2 + k_select_emit", False, "hbm", 8.0 * ncell + 4.0 * (nt + ns),
         "bytes", med("ms_select"), hbm, "GB/s", hbm_basis)
     return out
 
@@ -780,7 +781,8 @@ def run_full128(sph, torch, dev, stream, args, peaks, pipes, flush):
         S = out.cpu().numpy().astype(np.float64)
         tree = sph.get_tree(ctx)
         sub_args = argparse.Namespace(order=args.order, m2l=m2l)
-        roof = rooflines(tree, st, sub_args, p.ncell, p.ncell, p.ncell, peaks, pipes, traffic_ok=False)
+        roof = rooflines(tree, st, sub_args, p.ncell, p.ncell, p.ncell, peaks, pipes, traffic_ok=False,
+                         near_kernels="k_near_grid + k_near_pack + k_near_mma + k_near_w")   # beside the far field
         med = statistics.median(ms)
         res[name] = {"ms_per_step": med, "targets_per_s": p.ncell / (med * 1e-3),
                      "rel_l2_all_targets_vs_fft": oracle.rel_l2(S, fft),

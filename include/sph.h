@@ -110,7 +110,11 @@ typedef struct sph_stats {
     float ms_l2lp;             /* its GPU milliseconds (inside ms_l2p), 0 if not fused */
     int32_t m2l_tiles;         /* tensor-core M2L form of this eval: 1 target-stationary tiles (dense V
                                   lists of 5 million pairs or more), 0 tiles of V pairs; chosen by timing
-                                  both when the leaf size is autotuned (set_criteria leaf_size 0) */
+                                  both when the leaf size is autotuned (set_criteria leaf_size 0).  The
+                                  forms differ in the order of FP32 sums alone: S by pairs is within 4e-7
+                                  of FP32 translations, by target tiles within 5e-6 (rel-L2), where the
+                                  order-5 expansion is 2e-5 to 3e-5 off; SPH_M2L_TILES=0 or 1 in the
+                                  environment fixes the form */
 } sph_stats;
 
 /* Create a context on CUDA device `device`, queuing work on `cuda_stream`
@@ -154,9 +158,12 @@ int set_criteria(sph_ctx *ctx, double i_frac, double e_frac, double e_applied,
 int sph_set_far_field(sph_ctx *ctx, int method, int order);
 
 /* Near field (Eq. nearfar, the exact part): SPH_NEAR_EXP (default) uses the kernel's
- * exponential form: once per cell offset between leaves of edge 4 or less, whose offsets are few
- * (dense ones then sum on the tensor cores, values and weights as three BF16 parts), per
- * source-target pair elsewhere; SPH_NEAR_TABLE reads G for the integer
+ * exponential form: once per cell offset between leaves of edge 4 or less, whose offsets are few,
+ * where at least half the leaves are that small, per source-target pair elsewhere.  Dense leaves of
+ * edge 4 sum on the tensor cores: values and weights as three BF16 parts each (24 bits), the six
+ * products that reach 2^-24 of a sum, FP32 accumulators; its sums are no further from FP64 than FP32
+ * pair by pair (rms 1e-7 to 2.5e-7).  SPH_NEAR_MMA=0 in the environment (read by sph_create) keeps
+ * those leaves in FP32.  SPH_NEAR_TABLE reads G for the integer
  * squared cell offsets below 4096 from a table built per evaluation with the same arithmetic
  * (uniform grids make every offset an integer); SPH_NEAR_AUTO times both on the first eval
  * of each problem class and keeps the faster.  Takes effect at the next eval. */

@@ -339,9 +339,9 @@ __device__ __forceinline__ int warp_append(unsigned act, bool pred, int *counter
     return base + __popc(grp & ((1u << lane) - 1u));
 }
 
-// A leaf's near field costs the matrix form (k_near_mma) 2.5 ns of the whole chip whatever its
-// sources, the table form (k_near_grid) 12.6 ps a source (both measured on the uniform 128^3 tree): they are
-// level at 200 of the 1728 cells, more where tiles are few.
+// A leaf's near field costs the matrix form (k_near_mma) 2.8 ns of the whole chip whatever its
+// sources, the table form (k_near_grid) 11.8 ps a source (both measured on the uniform 128^3 tree): they are
+// level at 240 of the 1728 cells, more where tiles are few.
 constexpr int NEAR_MMA_MIN = 384;
 
 __global__ void k_work_lists(FmmDev F, int nboxes, int *__restrict__ src_list, int *__restrict__ src_cnt,
@@ -1322,8 +1322,9 @@ int fmm_p2l(const FmmDev &F, const int *list, const int *count, int max_boxes, c
 // of the source; 25 pairs per SM and clock) instead of three special-function results (8).  Four
 // warps share a leaf's sources, each lane sums two targets, and the warps' sums are added in
 // order.  Entries of larger leaves take the exp form (the staged points and p2p_sum below).
-// Uniform 128^3 (3.4e9 pairs): 2290 us by the exp form alone, 670 us so; wide streamer 192^3:
-// 996, 290 (39 since its dense leaves are k_near_mma's; all of the uniform tree's are).
+// Uniform 128^3 (3.4e9 pairs), without the matrix form: 2290 us by the exp form alone, 655 us so; wide
+// streamer 192^3: 996, 281 (34 beside the matrix form, which takes its dense leaves and all of the
+// uniform tree's).  Both kernels alone.
 constexpr int NG_PY = 20, NG_PZ = 304, NG_CENTRE = 7 * (1 + NG_PY + NG_PZ), NG_N = 2 * NG_CENTRE + 1;
 constexpr int NG_CAP = 2048;         // staged points per round (16 KiB; 1024 in the exp form)
 constexpr int NG_GROUP = 16;         // sources summed by themselves

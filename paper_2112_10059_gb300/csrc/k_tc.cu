@@ -1857,11 +1857,12 @@ __global__ void __launch_bounds__(256, 1) k_m2l_tiles(FmmDev F, const int *__res
 // addition that rounds at the sum's own size; four accumulators an offset, two offsets' in TMEM, added
 // up in FP32 registers.
 // A step is an offset: 48 KB of rows gathered by 16-byte copies, 24 KB of matrices by a bulk copy,
-// 24 MMAs; three steps in shared memory.  A step takes 1.4 us against 0.6 us of MMAs, bound by the
-// latency of its copies (tensor pipe 27% active, L2 at 22%).  Eight warps look the leaves up an
-// offset ahead, copy, add up and write results, one thread issues MMAs.
-// Uniform 128^3 (32,768 full leaves, 3.4e9 pairs): 712 us by the offset table, 82 so and 14 for its
-// operands; wide streamer 192^3 303, and 44 + 12 + 39 for the other leaves by the table.
+// 24 MMAs; three steps in shared memory.  A step takes 1.6 us against 0.6 us of MMAs, bound by the
+// latency of its copies (tensor pipe 24% active, L2 at 20%) and the reading of its accumulators (0.13 us).
+// Eight warps look the leaves up an offset ahead, copy, add up and write results, one thread issues MMAs.
+// Near field alone against FP64, rms: 0.9e-7 to 2.3e-7 of a sum, pair by pair in FP32 1.9e-7 to 4.7e-7.
+// Uniform 128^3 (32,768 full leaves, 3.4e9 pairs): 655 us by the offset table, 90 so and 10 to 14 for its
+// operands; wide streamer 192^3 281, and 48 + 11 + 34 for the other leaves by the table.
 __global__ void __launch_bounds__(NM_COPY + 32, 1) k_near_mma(FmmDev F, const int *__restrict__ p2p_list,
                                                              const int *__restrict__ p2p_cnt, int stride, int row0,
                                                              const uint16_t *__restrict__ rows,

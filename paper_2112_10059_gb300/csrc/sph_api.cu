@@ -698,7 +698,7 @@ bool l2lp_fusable(const sph_ctx *c, const PassState &S) {
 }
 
 // Whether dense leaves take their near field as a matrix product (k_near_mma).  A tile of 128
-// leaves takes 40 us, however few tiles there are, and its operands 12; the offset table is level
+// leaves takes 45 us, however few tiles there are, and its operands 10; the offset table is level
 // with it at 2e8 pairs (40 us at 5e12/s, 60 beside the far field).  Below 16 sources a source leaf
 // hardly a leaf has the sources that it takes (k_work_lists).
 bool near_mma_pays(const sph_ctx *c, const PassState &S) {
@@ -814,11 +814,18 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
 }
 
 // The M2L form (an autotuned choice overrides it).  The target-stationary tiles pay a round per
-// (group, offset) whatever the number of pairs in it: on all-source grids of n^3 cells they take
-// 134 / 251 / 274 / 688 / 1099 us for n = 24 / 48 / 64 / 96 / 128, the tile loop over V pairs 20 / 84 / 190 /
-// 434 / 1057 us.  They are taken where the lists are dense and so long that the two are level (6 M
-// pairs at 128^3).  Error against FP64 there: 2.1e-5 by the target tiles, 2.3e-5 by the pairs as by
-// FP32 translations (the tiles' long sums, rounded towards zero, cancel some of the expansion's own error).
+// (group, offset) whatever the number of pairs in it.  On all-source grids of n^3 cells:
+//     n                       24     48     64     96    112    128    144    160    192
+//     pairs, millions       0.02   0.24   0.64    2.4    4.0    6.0    8.8   12.2   21.5
+//     target tiles, us       137    255    288    700   1110   1110   2360   2650   3590
+//     tile loop, us           20     83    155    438    738   1067   1530   2110   3773
+//     error of S, target    2.32   3.21   2.08   2.15   2.13   2.10   2.05   1.99   1.91  x 1e-5
+//     error of S, loop      2.33   3.31   2.15   2.29   2.31   2.32   2.29   2.26   2.21  x 1e-5
+// The loop is the closer of the two to FP32 translations (3e-8 to 3e-7 of S, the target tiles 7e-7 to
+// 5e-6: their long sums are rounded towards zero), whose error is the loop's; the target tiles'
+// rounding happens to cancel some of the expansion's own error in the norm, not at its worst cell.  They
+// are taken for dense lists of 5 million pairs or more, where the two are level and the smaller norm
+// costs 4% of an evaluation (128^3); it costs more between 144^3 and 160^3, and nothing at 192^3.
 bool m2l_target_tiles(const sph_ctx *c, const PassState &S) {
     const int64_t nV = c->list_tot[1], nb = c->nboxes;
     return S.tc && (c->m2l_tiles == 1 ||
