@@ -112,7 +112,7 @@ typedef struct sph_stats {
                                   lists of 5 million pairs or more), 0 tiles of V pairs; chosen by timing
                                   both when the leaf size is autotuned (set_criteria leaf_size 0).  The
                                   forms differ in the order of FP32 sums alone: S by pairs is within 4e-7
-                                  of FP32 translations, by target tiles within 5e-6 (rel-L2), where the
+                                  of FP32 translations, by target tiles within 8e-6 (rel-L2), where the
                                   order-5 expansion is 2e-5 to 3e-5 off; SPH_M2L_TILES=0 or 1 in the
                                   environment fixes the form */
 } sph_stats;

@@ -821,8 +821,8 @@ int fmm_prepare(sph_ctx *c, PassState &S) {
 //     tile loop, us           20     83    155    438    738   1067   1530   2110   3773
 //     error of S, target    2.32   3.21   2.08   2.15   2.13   2.10   2.05   1.99   1.91  x 1e-5
 //     error of S, loop      2.33   3.31   2.15   2.29   2.31   2.32   2.29   2.26   2.21  x 1e-5
-// The loop is the closer of the two to FP32 translations (3e-8 to 3e-7 of S, the target tiles 7e-7 to
-// 5e-6: their long sums are rounded towards zero), whose error is the loop's; the target tiles'
+// The loop is the closer of the two to FP32 translations (3e-8 to 4e-7 of S, the target tiles 7e-7 to
+// 7e-6: their long sums are rounded towards zero), whose error is the loop's; the target tiles'
 // rounding happens to cancel some of the expansion's own error in the norm, not at its worst cell.  They
 // are taken for dense lists of 5 million pairs or more, where the two are level and the smaller norm
 // costs 4% of an evaluation (128^3); it costs more between 144^3 and 160^3, and nothing at 192^3.
