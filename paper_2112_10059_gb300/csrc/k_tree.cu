@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_onepass(ScanSet S, int n, int n
     tile_store<SCAN_T>(S.out[a], base, n, sh, v, s_pre + pre);
 }
 
-size_t scan_tmp_ints(int n) {
-    const int ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+size_t scan_tmp_ints(int64_t n) {
+    const int64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     return 2 * 4 * ((size_t)ntiles + 1) + 16;
 }
 

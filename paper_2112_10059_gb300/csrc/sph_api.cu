@@ -328,7 +328,8 @@ TreeDev tree_dev(sph_ctx *c) {
 ListDev list_dev(sph_ctx *c) {
     ListDev L;
     memset(static_cast<void *>(&L), 0, sizeof L);
-    int nb = std::max(c->list_cap, 1);
+    // 64 bits: on a grid of more than 512 cells at leaf sizes below 8 there are 1.2e9 slots
+    const size_t nb = std::max(c->list_cap, 1);
     int *cnt = P<int>(c->b_lcnt), *off = P<int>(c->b_loff);
     L.u_cnt = cnt; L.v_cnt = cnt + nb; L.w_cnt = cnt + 2 * nb; L.x_cnt = cnt + 3 * nb;
     L.u_off = off; L.v_off = off + (nb + 1); L.w_off = off + 2 * (nb + 1); L.x_off = off + 3 * (nb + 1);
@@ -378,9 +379,9 @@ int lmax_of(const sph_ctx *c) {
 
 // The scan scratch: the tree scan's region first, then the list scan's (separate look-back
 // states, so that both can be cleared before the evaluation)
-int64_t scan_list_off(int64_t dense_total) { return (int64_t)scan_tmp_ints((int)(4 * (dense_total + 1))); }
+int64_t scan_list_off(int64_t dense_total) { return (int64_t)scan_tmp_ints(4 * (dense_total + 1)); }
 size_t scan_scratch_bytes(int64_t dense_total) {
-    return (size_t)(scan_list_off(dense_total) + (int64_t)scan_tmp_ints((int)(dense_total + 1))) * sizeof(int) + 64;
+    return (size_t)(scan_list_off(dense_total) + (int64_t)scan_tmp_ints(dense_total + 1)) * sizeof(int) + 64;
 }
 
 int tree_queue(sph_ctx *c) {
@@ -1895,7 +1896,7 @@ int sph_scan_i32(int device, void *cuda_stream, int64_t n, const int32_t *in_dev
         return SPH_ECUDA;
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-    const size_t nt = scan_tmp_ints((int)n);
+    const size_t nt = scan_tmp_ints(n);
     int *tmp = nullptr;
     if (cudaMalloc(&tmp, (nt + 2) * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();

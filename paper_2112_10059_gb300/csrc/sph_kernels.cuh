@@ -128,7 +128,7 @@ void zero_set_launch(const ZeroSet &Z, cudaStream_t st);
 // bytes of state a look-back scan of k arrays of length n clears before it runs (0: the
 // single-CTA scan, which keeps no state)
 size_t scan_state_bytes(int k, int n);
-size_t scan_tmp_ints(int n);
+size_t scan_tmp_ints(int64_t n);
 void scan_exclusive(const int *in, int *out, int n, int *total, int *tmp, cudaStream_t st, int *err = nullptr,
                     unsigned wait_limit = SCAN_WAIT_LIMIT, bool state_zeroed = false);
 
